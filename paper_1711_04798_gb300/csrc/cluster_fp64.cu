@@ -10,6 +10,8 @@
 // arithmetic are those of the grid-wide kernels (kernels.cu, cholqr.cu).
 #include <cooperative_groups.h>
 
+#include <algorithm>
+
 #include "ctm_internal.h"
 
 namespace cg = cooperative_groups;
@@ -17,7 +19,6 @@ namespace cg = cooperative_groups;
 namespace {
 
 constexpr int CL_THREADS = 256;         // 8 warps per CTA (Cholesky): FP64 pipe occupancy
-constexpr int JC_THREADS = 256;         // Jacobi: 8 warps per CTA, two per row pair
 constexpr int CL_SMEM = 200 * 1024;     // dynamic shared memory bound per CTA
 int g_csize = 0;                        // CTAs per cluster (16 if schedulable, else 8)
 
@@ -25,24 +26,6 @@ __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
-}
-
-// Sums of four values over a warp with 6 FP64 additions per lane instead of
-// 20: the first two butterfly levels halve the values each lane carries.  On
-// return lane 0 holds the total of a, lane 8 of b, lane 16 of c, lane 24 of d.
-__device__ __forceinline__ double warp_sum4(double a, double b, double c, double d) {
-  const int lane = threadIdx.x & 31;
-  const bool up = lane & 16;
-  double k1 = up ? c : a, k2 = up ? d : b;
-  k1 += __shfl_xor_sync(0xffffffffu, up ? a : c, 16);
-  k2 += __shfl_xor_sync(0xffffffffu, up ? b : d, 16);
-  const bool b3 = lane & 8;
-  double k = b3 ? k2 : k1;
-  k += __shfl_xor_sync(0xffffffffu, b3 ? k1 : k2, 8);
-  k += __shfl_xor_sync(0xffffffffu, k, 4);
-  k += __shfl_xor_sync(0xffffffffu, k, 2);
-  k += __shfl_xor_sync(0xffffffffu, k, 1);
-  return k;
 }
 
 __device__ __forceinline__ void pair_of(int r, int p, int np, int rounds, int* i, int* j) {
@@ -113,58 +96,322 @@ __device__ __forceinline__ float4 df_elem(cplx x) {
   return make_float4(r.h, r.l, i.h, i.l);
 }
 
-__device__ __forceinline__ df2 warp_sum_df(df2 v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float oh = __shfl_xor_sync(0xffffffffu, v.h, o), ol = __shfl_xor_sync(0xffffffffu, v.l, o);
-    float s, t;
-    two_sum(v.h, oh, s, t);
-    v.h = s;
-    v.l = __fadd_rn(v.l, __fadd_rn(ol, t));
-  }
-  return df_norm(v);
+// a b, the leading product exactly, the cross terms in FP32
+__device__ __forceinline__ df2 df_mul(df2 a, df2 b) {
+  const float p = __fmul_rn(a.h, b.h);
+  float e = __fmaf_rn(a.h, b.h, -p);
+  e = __fmaf_rn(a.h, b.l, e);
+  e = __fmaf_rn(a.l, b.h, e);
+  return {p, e};
 }
 
-// One-sided Jacobi on the n rows of G (length m): rows and, with Vt, the rows
-// of the accumulated rotation (length n, from the identity, or from Vt itself
-// with warm) in the cluster's shared memory.  DF: the rows are held, dotted
-// and rotated in double-float arithmetic (the rotation angles stay FP64;
-// only with a rotation log, Vt being rebuilt from it in FP64).
+__device__ __forceinline__ df2 df_add(df2 a, df2 b) {
+  df2 r;
+  two_sum(a.h, b.h, r.h, r.l);
+  r.l = __fadd_rn(r.l, __fadd_rn(a.l, b.l));
+  return df_norm(r);
+}
+
+// 1/sqrt(a) of a normalised a > 0: an FP32 root refined by one step of third
+// order, x (1 + e/2 + 3 e^2/8) with e = 1 - a x^2 in double-float
+__device__ __forceinline__ df2 df_rsqrt(df2 a) {
+  const float x = rsqrtf(a.h);
+  const df2 xx = {x, 0.f};
+  const df2 ax2 = df_norm(df_mul(df_norm(df_mul(a, xx)), xx));
+  const float e = __fadd_rn(__fadd_rn(1.0f, -ax2.h), -ax2.l);
+  df2 r = {x, __fmul_rn(x, __fmul_rn(e, __fmaf_rn(0.375f, e, 0.5f)))};
+  return df_norm(r);
+}
+
+// 1/sqrt(a) of a finite a > 0 to FP64 rounding with five FP64 instructions:
+// the argument scaled into [1, 4) and converted on the integer pipe, an FP32
+// root, one step of third order (its error (5/16) e^3 with |e| < 2^-21)
+__device__ __forceinline__ double rsqrt64(double a) {
+  const long long b = __double_as_longlong(a);
+  const int ex = (int)(b >> 52) - 1023, half = ex >> 1;                  // a = m 4^half, m in [1, 4)
+  const double m = __longlong_as_double(b - ((long long)half << 53));
+  const double x = f2d_bits(rsqrtf(d2f_bits(m)));
+  const double e = fma(-(m * x), x, 1.0);
+  const double r = fma(x * e, fma(0.375, e, 0.5), x);
+  return __longlong_as_double(__double_as_longlong(r) - ((long long)half << 52));
+}
+
+// the sums of a and b over the warp, in every lane: after the first butterfly
+// level each half of the warp carries one of them
+__device__ __forceinline__ void warp_sum2(double& a, double& b) {
+  const bool up = threadIdx.x & 16;
+  double k = up ? b : a;
+  k += __shfl_xor_sync(0xffffffffu, up ? a : b, 16);
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
+  a = __shfl_sync(0xffffffffu, k, 0);
+  b = __shfl_sync(0xffffffffu, k, 16);
+}
+
+__device__ __forceinline__ void warp_sum2(df2& a, df2& b) {
+  const bool up = threadIdx.x & 16;
+  df2 k = up ? b : a;
+  const df2 o = up ? a : b;
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) {
+    const float oh = __shfl_xor_sync(0xffffffffu, d == 16 ? o.h : k.h, d);
+    const float ol = __shfl_xor_sync(0xffffffffu, d == 16 ? o.l : k.l, d);
+    float s, t;
+    two_sum(k.h, oh, s, t);
+    k.h = s;
+    k.l = __fadd_rn(k.l, __fadd_rn(ol, t));
+  }
+  k = df_norm(k);
+  a = {__shfl_sync(0xffffffffu, k.h, 0), __shfl_sync(0xffffffffu, k.l, 0)};
+  b = {__shfl_sync(0xffffffffu, k.h, 16), __shfl_sync(0xffffffffu, k.l, 16)};
+}
+
+// A rotation of rows i, j (the form of jac_rotate): a' = c a - q b,
+// b' = c b + conj(q) a with q = s e^{-i phi}, c^2 + |q|^2 = 1.
+template <class S>
+struct Rot {
+  S c, qr, qi;
+};
+
+// Row element types: FP64 complex, or two double-floats (Re hi, Re lo, Im hi,
+// Im lo) in the same 16 bytes.
 template <bool DF>
-__global__ void __launch_bounds__(JC_THREADS, 1)
-    jacobi_cluster_kernel(cplx* __restrict__ G, int n, int m, long long ldg, cplx* __restrict__ Vt, int max_sweeps,
-                          double tol, double4_16a* __restrict__ log, int* sweeps_used, DevStatus* st, int warm) {
+struct RowT {
+  typedef double S;
+  typedef cplx E;
+};
+template <>
+struct RowT<true> {
+  typedef df2 S;
+  typedef float4 E;
+};
+
+__device__ __forceinline__ void dot_acc(double& gr, double& gi, cplx x, cplx y) {  // conj(x) y
+  gr = fma(x.x, y.x, gr);
+  gr = fma(x.y, y.y, gr);
+  gi = fma(x.x, y.y, gi);
+  gi = fma(-x.y, y.x, gi);
+}
+__device__ __forceinline__ void dot_acc(df2& gr, df2& gi, float4 x, float4 y) {
+  const df2 xr = {x.x, x.y}, xi = {x.z, x.w}, yr = {y.x, y.y}, yi = {y.z, y.w};
+  acc_mul(gr, xr, yr);
+  acc_mul(gr, xi, yi);
+  acc_mul(gi, xr, yi);
+  acc_mul(gi, df_negate(xi), yr);
+}
+__device__ __forceinline__ void norm_acc(double& a, cplx x) {
+  a = fma(x.x, x.x, a);
+  a = fma(x.y, x.y, a);
+}
+__device__ __forceinline__ void norm_acc(df2& a, float4 x) {
+  acc_mul(a, {x.x, x.y}, {x.x, x.y});
+  acc_mul(a, {x.z, x.w}, {x.z, x.w});
+}
+__device__ __forceinline__ void rotate_elem(const Rot<double>& r, cplx& a, cplx& b) {
+  const cplx x = a, y = b;
+  a.x = fma(-r.qr, y.x, fma(r.qi, y.y, r.c * x.x));
+  a.y = fma(-r.qr, y.y, fma(-r.qi, y.x, r.c * x.y));
+  b.x = fma(r.qr, x.x, fma(r.qi, x.y, r.c * y.x));
+  b.y = fma(r.qr, x.y, fma(-r.qi, x.x, r.c * y.y));
+}
+__device__ __forceinline__ void rotate_elem(const Rot<df2>& r, float4& a, float4& b) {
+  const df2 xr = {a.x, a.y}, xi = {a.z, a.w}, yr = {b.x, b.y}, yi = {b.z, b.w};
+  const df2 nr = df_negate(r.qr), ni = df_negate(r.qi);
+  df2 ar = df_mul(r.c, xr), ai = df_mul(r.c, xi), br = df_mul(r.c, yr), bi = df_mul(r.c, yi);
+  acc_mul(ar, nr, yr);
+  acc_mul(ar, r.qi, yi);
+  acc_mul(ai, nr, yi);
+  acc_mul(ai, ni, yr);
+  acc_mul(br, r.qr, xr);
+  acc_mul(br, r.qi, xi);
+  acc_mul(bi, r.qr, xi);
+  acc_mul(bi, ni, xr);
+  ar = df_norm(ar);
+  ai = df_norm(ai);
+  br = df_norm(br);
+  bi = df_norm(bi);
+  a = make_float4(ar.h, ar.l, ai.h, ai.l);
+  b = make_float4(br.h, br.l, bi.h, bi.l);
+}
+
+// The rotation that makes rows of squared norms al, be and inner product
+// g = x^H y orthogonal: t = tan, c = 1/sqrt(1 + t^2), q = c t conj(g)/|g|; tg
+// = t |g| (the squared norms become al - tg, be + tg).  Returns 0: left alone
+// (|g| <= tol sqrt(al be)), 1: off-orthogonality and angle at most 1e-8, 2:
+// larger.  g is scaled by a power of two into [1, 2) first, so nothing under-
+// or overflows that the test does not settle.
+__device__ __forceinline__ int rotation(df2 al, df2 be, df2 gr, df2 gi, float tol, Rot<df2>& rot, df2& tg) {
+  const float big = fmaxf(fabsf(gr.h), fabsf(gi.h));
+  const int e = (int)(__float_as_uint(big) >> 23);
+  if (!(big > 0.f) || e >= 255 || e < 8) return 0;
+  const float S = __uint_as_float((unsigned)(254 - e) << 23), iS = __uint_as_float((unsigned)e << 23);  // 2^(127-e), 1/S
+  gr = {gr.h * S, gr.l * S};
+  gi = {gi.h * S, gi.l * S};
+  df2 g2 = df_mul(gr, gr);
+  acc_mul(g2, gi, gi);
+  g2 = df_norm(g2);
+  const float as = al.h * S, bs = be.h * S;
+  if (!(g2.h > (tol * as) * (tol * bs))) return 0;
+  const df2 ig = df_rsqrt(g2);
+  const df2 d = df_add(be, df_negate(al));
+  const float zf = 0.5f * (d.h * S) * ig.h;
+  // the tangent in FP32: an angle off by 2^-24 leaves that share of g behind
+  const float az = fabsf(zf);
+  const float t = copysignf(az < 1e15f ? 1.0f / (az + sqrtf(fmaf(zf, zf, 1.0f))) : 0.5f / az, zf);
+  const df2 tt = {t, 0.f};
+  df2 w = df_mul(tt, tt), one;
+  two_sum(1.0f, w.h, one.h, one.l);
+  one.l = __fadd_rn(one.l, w.l);
+  rot.c = df_rsqrt(df_norm(one));
+  const df2 u = df_norm(df_mul(df_norm(df_mul(rot.c, tt)), ig));
+  rot.qr = df_norm(df_mul(u, gr));
+  rot.qi = df_negate(df_norm(df_mul(u, gi)));
+  tg = df_mul(df_norm(df_mul(g2, ig)), tt);
+  tg = {tg.h * iS, tg.l * iS};
+  return (g2.h > (1e-8f * as) * (1e-8f * bs) || fabsf(t) > 1e-8f) ? 2 : 1;
+}
+
+// FP64 rows: the angle in double-float on the FP32 pipe (its tangent good to
+// 2^-45; FP32 alone raised the corner spectra's noise from 2e-11 to 1e-10),
+// then c and q from that tangent in FP64, so c^2 + |q|^2 = 1 to FP64 rounding
+// whatever the tangent's error.  Some 20 FP64 instructions instead of the
+// 100 of FP64 roots and divides, each of which holds the SM's FP64 unit for
+// about 18 cycles.
+__device__ __forceinline__ int rotation(double al, double be, double gr, double gi, float tol, Rot<double>& rot,
+                                        double& tg) {
+  // exponent of the larger part, by integer operations
+  const unsigned long long br = (unsigned long long)__double_as_longlong(gr) & 0x7fffffffffffffffull;
+  const unsigned long long bi = (unsigned long long)__double_as_longlong(gi) & 0x7fffffffffffffffull;
+  const int e = (int)((br > bi ? br : bi) >> 52);
+  if (e >= 2047 || e < 64) return 0;  // |g| below 2^-960 (or not finite): nothing to rotate
+  const int sh = 1023 - e;
+  auto scaled = [&](double v) {  // v 2^sh for v >= 0, clamped (v is a squared norm: compared and subtracted only)
+    const long long b = __double_as_longlong(v);
+    const int ev = (int)(b >> 52) + sh;
+    return b <= 0 || ev <= 0 ? 0.0 : (ev >= 2046 ? 1e308 : __longlong_as_double(b + ((long long)sh << 52)));
+  };
+  auto scale_s = [&](double v) {  // signed, |v| <= |g|'s larger part
+    const long long b = __double_as_longlong(v);
+    const int ev = (int)((b >> 52) & 0x7ff) + sh;
+    return (b << 1) == 0 || ev <= 0 ? 0.0 : __longlong_as_double(b + ((long long)sh << 52));
+  };
+  const double xr = scale_s(gr), xi = scale_s(gi), as = scaled(al), bs = scaled(be);
+  const float hr = d2f_bits(xr), hi = d2f_bits(xi);
+  const df2 dr = {hr, d2f_bits(xr - f2d_bits(hr))}, di = {hi, d2f_bits(xi - f2d_bits(hi))};
+  df2 g2 = df_mul(dr, dr);
+  acc_mul(g2, di, di);
+  g2 = df_norm(g2);
+  const float af = d2f_bits(as), bf = d2f_bits(bs);
+  if (!(g2.h > (tol * af) * (tol * bf))) return 0;
+  const df2 ig = df_rsqrt(g2);
+  const double dd = bs - as;
+  const float dh = d2f_bits(dd);
+  df2 z = df_norm(df_mul({dh, fabsf(dh) < 1e30f ? d2f_bits(dd - f2d_bits(dh)) : 0.f}, ig));
+  z = {0.5f * fabsf(z.h), dh >= 0.f ? 0.5f * z.l : -0.5f * z.l};
+  df2 t;
+  if (z.h < 1e8f) {
+    // 1 / (|z| + sqrt(1 + z^2)): the root as w / sqrt(w), the reciprocal refined once
+    df2 w = df_mul(z, z), w1;
+    two_sum(1.0f, w.h, w1.h, w1.l);
+    w1.l = __fadd_rn(w1.l, w.l);
+    w1 = df_norm(w1);
+    const df2 den = df_add(z, df_norm(df_mul(w1, df_rsqrt(w1))));
+    const float r0 = 1.0f / den.h;
+    const df2 p = df_norm(df_mul(den, {r0, 0.f}));
+    t = {r0, __fmul_rn(r0, __fadd_rn(__fadd_rn(1.0f, -p.h), -p.l))};
+  } else {
+    t = {0.5f / z.h, 0.f};  // 1/(2 z): below 5e-9, good to 2^-23 of itself
+  }
+  if (dh < 0.f) t = df_negate(t);
+  const df2 u = df_norm(df_mul(df_norm(t), ig));
+  const df2 ur = df_norm(df_mul(u, dr)), ui = df_norm(df_mul(u, di));
+  const double er = f2d_bits(ur.h) + f2d_bits(ur.l), ei = f2d_bits(ui.h) + f2d_bits(ui.l);  // t conj(phase), exactly
+  const double w = fma(er, er, fma(ei, ei, 1.0));
+  rot.c = rsqrt64(w);
+  rot.qr = rot.c * er;
+  rot.qi = -(rot.c * ei);
+  tg = fma(er, gr, ei * gi);
+  return (g2.h > (1e-8f * af) * (1e-8f * bf) || fabsf(t.h) > 1e-8f) ? 2 : 1;
+}
+
+__device__ __forceinline__ double s_zero(double) { return 0.0; }
+__device__ __forceinline__ df2 s_zero(df2) { return {0.f, 0.f}; }
+__device__ __forceinline__ double s_val(double x) { return x; }
+__device__ __forceinline__ double s_val(df2 x) { return df_val(x); }
+__device__ __forceinline__ double s_add(double a, double b) { return a + b; }
+__device__ __forceinline__ df2 s_add(df2 a, df2 b) { return df_add(a, b); }
+__device__ __forceinline__ double s_neg(double a) { return neg_bits(a); }
+__device__ __forceinline__ df2 s_neg(df2 a) { return df_negate(a); }
+__device__ __forceinline__ bool s_less(double a, double b) { return a < b; }       // for squared norms
+__device__ __forceinline__ bool s_less(df2 a, df2 b) { return a.h < b.h; }
+__device__ __forceinline__ double s_quarter(double a) { return 0.25 * a; }
+__device__ __forceinline__ df2 s_quarter(df2 a) { return {0.25f * a.h, 0.25f * a.l}; }
+
+constexpr int JC_MAXP = 32;  // row pairs of one round per CTA (n <= 2 * 16 * 32 with 16 CTAs, half with 8)
+
+// One-sided Jacobi (Hestenes) on the n rows of G (length m), one matrix per
+// cluster (cluster b: G + b * strideG), rows in the cluster's shared memory
+// (active row a in CTA a mod cs).  One warp per row pair: it holds both rows in
+// registers between the inner product and the rotation (NE elements per lane;
+// NE = 0: any length, read twice) and needs no block barrier; a cluster
+// barrier ends each round.  Rows below 1e-15 ||G||_F are rounding noise and
+// take part in no rotation: they are left out of the schedule, which covers
+// the other rows only.  The squared norms stay with their rows and follow the
+// rotations (al - t|g|, be + t|g|), formed anew at every sweep and where a
+// rotation takes most of one away, so a round's inner product is x^H y alone.
+//
+// Bound: FP64 rows by the FP64 units of the cluster's SMs (about 18 cycles per
+// warp instruction and SM: 16 for the inner product, 48 for the rotation and
+// some 25 for the reduction and angle, per pair and 128 columns); double-float
+// rows by the latency of a round (loads from the partner CTAs, reduction,
+// angle, rotation, cluster barrier).
+//
+// FP64 with a log: the rotations are logged and replayed onto Vt by
+// jacobi_replay_kernel across the GPU (rotating V here would double the FP64
+// work of these 16 SMs).  Double-float with Vt: the second half of the warps
+// rotates the rows of V (double-float, from Vt), one round behind the first
+// half, in the cycles the rounds leave idle.
+template <bool DF, int NE>
+__global__ void __launch_bounds__(512, 1)
+    jacobi_cluster_kernel(cplx* __restrict__ G0, int n, int m, long long ldg, long long strideG,
+                          cplx* __restrict__ Vt, int max_sweeps, float tol, double4_16a* __restrict__ log,
+                          int* __restrict__ amap, int* sweeps_used, DevStatus* st, int warm) {
+  typedef typename RowT<DF>::S S;
+  typedef typename RowT<DF>::E E;
   cg::cluster_group cl = cg::this_cluster();
   const int rank = (int)cl.block_rank(), cs = (int)cl.num_blocks();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = JC_THREADS / 32;
-  const int R = (n + cs - 1) / cs;  // row slots per CTA
-  extern __shared__ cplx sm[];      // [R x m] rows of G, then [R x n] rows of Vt
+  cplx* __restrict__ G = G0 + (long long)(blockIdx.x / cs) * strideG;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  const int R = (n + cs - 1) / cs;   // row slots per CTA
+  const bool with_v = DF && Vt != nullptr;
+  const int gwarps = with_v ? nwarps / 2 : nwarps;
+  extern __shared__ cplx sm[];       // [R x m] rows of G, then (with_v) [R x n] rows of V
+  __shared__ S s_nrm[JC_MAXP * 2];   // squared norm of each row slot
+  __shared__ int s_act[JC_MAXP * 2 * 16], s_nact;  // original row of each active row
   __shared__ double s_fro;
   __shared__ int s_rot, s_big;
-  __shared__ double s_part[JC_THREADS / 64][2][4];  // [pair slot][half][al, be, Re g, Im g]
-  __shared__ double s_rp[JC_THREADS / 64][4];       // [pair slot][c, s, Re ph, Im ph]
-  __shared__ float s_rf[JC_THREADS / 64][6];        // DF: c, Re sq, Im sq as double-float pairs
-  __shared__ int s_rr[JC_THREADS / 64];             // [pair slot] rotated
-  cplx* gl = sm;
-  cplx* vl = sm + (long long)R * m;
-  double f = 0.0;
-  for (int l = 0; l < R; ++l) {
-    const int i = l * cs + rank;
-    if (i >= n) break;
-    for (int t = threadIdx.x; t < m; t += JC_THREADS) {
+  __shared__ Rot<df2> s_rec[2][JC_MAXP];  // with_v: the last rounds' rotations
+  __shared__ int s_recij[2][JC_MAXP];     // their rows, i << 16 | j, or -1
+  __shared__ double s_w[16];
+  E* gl = (E*)sm;
+  E* vl = (E*)(sm + (long long)R * m);
+  // squared row norms of the whole matrix by every CTA: the Frobenius norm and
+  // the active rows, the same in each
+  double* rn = (double*)sm;  // n doubles before the rows arrive
+  for (int i = warp; i < n; i += nwarps) {
+    double f = 0.0;
+    for (int t = lane; t < m; t += 32) {
       const cplx x = G[(long long)i * ldg + t];
-      if constexpr (DF)
-        ((float4*)gl)[(long long)l * m + t] = df_elem(x);
-      else
-        gl[(long long)l * m + t] = x;
-      f += x.x * x.x + x.y * x.y;
+      f = fma(x.x, x.x, f);
+      f = fma(x.y, x.y, f);
     }
-    if (Vt)
-      for (int t = threadIdx.x; t < n; t += JC_THREADS)
-        vl[(long long)l * n + t] = warm ? Vt[(long long)i * n + t] : make_double2(t == i ? 1.0 : 0.0, 0.0);
+    f = warp_sum(f);
+    if (lane == 0) rn[i] = f;
   }
+  __syncthreads();
+  double f = 0.0;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) f += rn[i];
   f = warp_sum(f);
-  __shared__ double s_w[JC_THREADS / 32];
   if (lane == 0) s_w[warp] = f;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -174,169 +421,191 @@ __global__ void __launch_bounds__(JC_THREADS, 1)
     s_rot = 0;
     s_big = 0;
   }
-  cl.sync();
-  double fro2 = 0.0;
-  for (int r = 0; r < cs; ++r) fro2 += *cl.map_shared_rank(&s_fro, r);
-  const double negligible = fro2 * 1e-30;
-  auto grow = [&](int i) { return cl.map_shared_rank(gl, i % cs) + (long long)(i / cs) * m; };
-  auto vrow = [&](int i) { return cl.map_shared_rank(vl, i % cs) + (long long)(i / cs) * n; };
-  const int np = (n + 1) & ~1;
+  __syncthreads();
+  const double fro2 = s_fro;
+  if (warp == 0) {
+    int cnt = 0;
+    for (int i0 = 0; i0 < n; i0 += 32) {
+      const bool on = i0 + lane < n && rn[i0 + lane] > fro2 * 1e-30;
+      const unsigned mask = __ballot_sync(0xffffffffu, on);
+      if (on) s_act[cnt + __popc(mask & ((1u << lane) - 1u))] = i0 + lane;
+      cnt += __popc(mask);
+    }
+    if (lane == 0) s_nact = cnt;
+  }
+  __syncthreads();
+  const int na = s_nact;
+  // double-float rows are scaled by a power of two so that ||G||_F lies near
+  // 2^20: every squared norm that takes part is then far inside FP32's range
+  double sc = 1.0, isc = 1.0;
+  if (DF && fro2 > 0.0 && fro2 < 1e300) {
+    const int ef = ((int)(__double_as_longlong(fro2) >> 52) - 1023) / 2;
+    sc = __longlong_as_double((long long)(1023 + 20 - ef) << 52);
+    isc = __longlong_as_double((long long)(1023 - 20 + ef) << 52);
+  }
+  const double fros = DF ? fro2 * sc * sc : fro2;
+  for (int l = 0; l < R; ++l) {
+    const int a = l * cs + rank;
+    if (a >= na) break;
+    const int i = s_act[a];
+    for (int t = threadIdx.x; t < m; t += blockDim.x) {
+      const cplx x = G[(long long)i * ldg + t];
+      if constexpr (DF)
+        gl[(long long)l * m + t] = df_elem(make_double2(x.x * sc, x.y * sc));
+      else
+        gl[(long long)l * m + t] = x;
+    }
+    if constexpr (DF) {
+      if (with_v)
+        for (int t = threadIdx.x; t < n; t += blockDim.x)
+          vl[(long long)l * n + t] = df_elem(warm ? Vt[(long long)i * n + t] : make_double2(t == i ? 1.0 : 0.0, 0.0));
+    }
+  }
+  if constexpr (DF) {
+    for (int q = threadIdx.x; q < 2 * JC_MAXP; q += blockDim.x) (&s_recij[0][0])[q] = -1;
+  }
+  const float neg = DF ? (float)(fros * 1e-30) : 0.f;
+  const double negd = fros * 1e-30;
+  auto negligible = [&](S x) {
+    if constexpr (DF)
+      return !(x.h > neg);
+    else
+      return !(x > negd);
+  };
+  auto grow = [&](int a) { return cl.map_shared_rank(gl, a % cs) + (long long)(a / cs) * m; };
+  auto vrow = [&](int a) { return cl.map_shared_rank(vl, a % cs) + (long long)(a / cs) * n; };
+  auto nrm = [&](int a) { return cl.map_shared_rank(s_nrm, a % cs) + a / cs; };
+  const int np = (na + 1) & ~1;
   const int rounds = np - 1, npairs = np / 2;
-  bool converged = false;
-  int sweep = 0;
-  for (; sweep < max_sweeps; ++sweep) {
-    for (int r = 0; r < rounds; ++r) {
-      // two warps per pair: warp (slot, half) takes the columns of 32-wide
-      // chunks 2j + half; the halves' sums meet in shared memory (fixed order)
-      for (int p0 = rank * (nwarps / 2); p0 < npairs; p0 += cs * (nwarps / 2)) {
-        const int slot = warp % (nwarps / 2), half = warp / (nwarps / 2);
-        const int p = p0 + slot;
-        int i = 0, j = n;
-        if (p < npairs) pair_of(r, p, np, rounds, &i, &j);
-        const bool active = p < npairs && j < n;
-        cplx* gi = active ? grow(i) : nullptr;
-        cplx* gj = active ? grow(j) : nullptr;
-        if (active && DF) {
-          df2 al = {0.f, 0.f}, be = {0.f, 0.f}, gr = {0.f, 0.f}, gim = {0.f, 0.f};
-          const float4* fi = (const float4*)gi;
-          const float4* fj = (const float4*)gj;
-          for (int t = lane + 32 * half; t < m; t += 64) {
-            const float4 x4 = fi[t], y4 = fj[t];
-            const df2 xr = {x4.x, x4.y}, xi = {x4.z, x4.w}, yr = {y4.x, y4.y}, yi = {y4.z, y4.w};
-            acc_mul(al, xr, xr);
-            acc_mul(al, xi, xi);
-            acc_mul(be, yr, yr);
-            acc_mul(be, yi, yi);
-            acc_mul(gr, xr, yr);
-            acc_mul(gr, xi, yi);
-            acc_mul(gim, xr, yi);
-            acc_mul(gim, df_negate(xi), yr);
-          }
-          al = warp_sum_df(al);
-          be = warp_sum_df(be);
-          gr = warp_sum_df(gr);
-          gim = warp_sum_df(gim);
-          if (lane == 0) {
-            s_part[slot][half][0] = df_val(al);
-            s_part[slot][half][1] = df_val(be);
-            s_part[slot][half][2] = df_val(gr);
-            s_part[slot][half][3] = df_val(gim);
-          }
-        } else if (active) {
-          double al = 0.0, be = 0.0, gr = 0.0, gim = 0.0;
-          for (int t = lane + 32 * half; t < m; t += 64) {
-            const cplx x = gi[t], y = gj[t];
-            al += x.x * x.x + x.y * x.y;
-            be += y.x * y.x + y.y * y.y;
-            gr += x.x * y.x + x.y * y.y;
-            gim += x.x * y.y - x.y * y.x;
-          }
-          const double tot = warp_sum4(al, be, gr, gim);
-          if ((lane & 7) == 0) s_part[slot][half][lane >> 3] = tot;
-        }
-        __syncthreads();
-        // the pair's rotation, by one thread of the pair (a lone FP64
-        // instruction occupies the sub-partition's FP64 unit as long as a
-        // full warp's).  c = 1/sqrt(1 + t^2) and the phase g/|g| in FP64, so
-        // that c^2 + s^2 = 1 and |ph| = 1 to FP64 rounding; the tangent t in
-        // FP32 for double-float rows (their angles only steer a convergence
-        // judged at 48 bits), in FP64 otherwise (an FP32 tangent raised the
-        // FP64 path's corner-spectrum noise from 2e-11 to 1e-10)
-        if (active && half == 0 && lane == 0) {
-          double c = 1.0, sn = 0.0, phr = 1.0, phi = 0.0;
-          int rot = 0;
-          const double al = s_part[slot][0][0] + s_part[slot][1][0], be = s_part[slot][0][1] + s_part[slot][1][1];
-          const double gr = s_part[slot][0][2] + s_part[slot][1][2], gim = s_part[slot][0][3] + s_part[slot][1][3];
-          const double g2 = gr * gr + gim * gim;
-          if (al > negligible && be > negligible && g2 > tol * tol * al * be) {
-            const double ig = rsqrt(g2);
-            const double zeta = 0.5 * (be - al) * ig;
-            double t;
-            if (!DF) {
-              t = (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-            } else if (fabs(zeta) < 1e15) {
-              const float zf = (float)zeta;
-              t = (double)(copysignf(1.0f, zf) / (fabsf(zf) + sqrtf(fmaf(zf, zf, 1.0f))));
-            } else {
-              t = 0.5 / zeta;  // t -> 1/(2 zeta)
-            }
-            c = rsqrt(fma(t, t, 1.0));
-            sn = c * t;
-            phr = gr * ig;
-            phi = -gim * ig;
-            rot = 1;
-            atomicAdd(&s_rot, 1);
-            // a rotation with off-orthogonality or angle above 1e-8 keeps
-            // the sweep from being the last one
-            if (g2 > 1e-16 * al * be || fabs(sn) > 1e-8) s_big = 1;
-          }
-          s_rp[slot][0] = c;
-          s_rp[slot][1] = sn;
-          s_rp[slot][2] = phr;
-          s_rp[slot][3] = phi;
-          s_rr[slot] = rot;
-          if (DF) {
-            // the rotation's double-float factors once here, not in every thread
-            const df2 cd = df_of(c), qr = df_of(sn * phr), qi = df_of(sn * phi);
-            s_rf[slot][0] = cd.h;
-            s_rf[slot][1] = cd.l;
-            s_rf[slot][2] = qr.h;
-            s_rf[slot][3] = qr.l;
-            s_rf[slot][4] = qi.h;
-            s_rf[slot][5] = qi.l;
-          }
-          if (log)
-            log[((long long)sweep * rounds + r) * npairs + p] = rot ? make_double4_16a(c, sn, phr, phi)
-                                                                   : make_double4_16a(2.0, 0.0, 0.0, 0.0);
-        } else if (!active && lane == 0 && half == 0) {
-          s_rr[slot] = 0;
-          if (log && p < npairs)
-            log[((long long)sweep * rounds + r) * npairs + p] = make_double4_16a(2.0, 0.0, 0.0, 0.0);
-        }
-        __syncthreads();  // the rotation is published; partial sums read before the next pair overwrites them
-        if (s_rr[slot]) {
-          if constexpr (DF) {
-            // a' = c a - sq b, b' = c b + sp a (the form of jac_rotate), sp = conj(sq)
-            const df2 cd = {s_rf[slot][0], s_rf[slot][1]}, qr = {s_rf[slot][2], s_rf[slot][3]},
-                      qi = {s_rf[slot][4], s_rf[slot][5]}, pr = qr, pi = df_negate(qi);
-            float4* fi = (float4*)gi;
-            float4* fj = (float4*)gj;
-            for (int q = lane + 32 * half; q < m; q += 64) {
-              const float4 x4 = fi[q], y4 = fj[q];
-              const df2 xr = {x4.x, x4.y}, xi = {x4.z, x4.w}, yr = {y4.x, y4.y}, yi = {y4.z, y4.w};
-              df2 ar = {0.f, 0.f}, ai = {0.f, 0.f}, br = {0.f, 0.f}, bi = {0.f, 0.f};
-              acc_mul(ar, cd, xr);
-              acc_mul(ar, df_negate(qr), yr);
-              acc_mul(ar, qi, yi);
-              acc_mul(ai, cd, xi);
-              acc_mul(ai, df_negate(qr), yi);
-              acc_mul(ai, df_negate(qi), yr);
-              acc_mul(br, cd, yr);
-              acc_mul(br, pr, xr);
-              acc_mul(br, df_negate(pi), xi);
-              acc_mul(bi, cd, yi);
-              acc_mul(bi, pr, xi);
-              acc_mul(bi, pi, xr);
-              ar = df_norm(ar);
-              ai = df_norm(ai);
-              br = df_norm(br);
-              bi = df_norm(bi);
-              fi[q] = make_float4(ar.h, ar.l, ai.h, ai.l);
-              fj[q] = make_float4(br.h, br.l, bi.h, bi.l);
-            }
-          } else {
-            const double c = s_rp[slot][0], sn = s_rp[slot][1];
-            const cplx ph = make_double2(s_rp[slot][2], s_rp[slot][3]);
-            const cplx sq = make_double2(sn * ph.x, sn * ph.y), sp = make_double2(sn * ph.x, -sn * ph.y);
-            for (int q = lane + 32 * half; q < m; q += 64) jac_rotate(gi[q], gj[q], c, sq, sp);
-            if (Vt) {
-              cplx* vi = vrow(i);
-              cplx* vj = vrow(j);
-              for (int q = lane + 32 * half; q < n; q += 64) jac_rotate(vi[q], vj[q], c, sq, sp);
-            }
-          }
+  const int own = (npairs + cs - 1) / cs;  // pairs of this CTA: p = slot * cs + rank
+  bool converged = na < 2;
+  int sweep = 0, par = 0;
+  // with_v: the second half of the warps applies the rotations recorded in buffer b
+  auto rotate_v = [&](int b) {
+    if constexpr (DF) {
+      for (int slot = warp - gwarps; slot < own; slot += gwarps) {
+        const int ij = s_recij[b][slot];
+        if (ij < 0) continue;
+        float4* vi = vrow(ij >> 16);
+        float4* vj = vrow(ij & 0xffff);
+        const Rot<df2> rot = s_rec[b][slot];
+        for (int q = lane; q < n; q += 32) {
+          float4 x = vi[q], y = vj[q];
+          rotate_elem(rot, x, y);
+          vi[q] = x;
+          vj[q] = y;
         }
       }
+    }
+  };
+  cl.sync();
+  for (; sweep < max_sweeps && !converged; ++sweep) {
+    // squared norms formed anew
+    for (int l = warp; l < R; l += nwarps) {
+      if (l * cs + rank >= na) break;
+      S a = s_zero(S());
+      for (int t = lane; t < m; t += 32) norm_acc(a, gl[(long long)l * m + t]);
+      S b = a;
+      warp_sum2(a, b);
+      if (lane == 0) s_nrm[l] = a;
+    }
+    cl.sync();
+    for (int r = 0; r < rounds; ++r) {
+      if (warp < gwarps) {
+        for (int slot = warp; slot < own; slot += gwarps) {
+          const int p = slot * cs + rank;
+          int i = 0, j = na, kind = 0;
+          if (p < npairs) pair_of(r, p, np, rounds, &i, &j);
+          Rot<S> rot;
+          if (p < npairs && j < na) {
+            E* gi = grow(i);
+            E* gj = grow(j);
+            const S al = *nrm(i), be = *nrm(j);
+            S gr = s_zero(S()), gim = s_zero(S()), tg = s_zero(S());
+            constexpr int NR = NE > 0 ? NE : 1;
+            E x[NR], y[NR];
+            if constexpr (NE > 0) {
+#pragma unroll
+              for (int q = 0; q < NE; ++q) {
+                const int t = lane + 32 * q;
+                x[q] = E();
+                y[q] = E();
+                if (t < m) {
+                  x[q] = gi[t];
+                  y[q] = gj[t];
+                }
+              }
+#pragma unroll
+              for (int q = 0; q < NE; ++q) dot_acc(gr, gim, x[q], y[q]);
+            } else {
+              for (int t = lane; t < m; t += 32) dot_acc(gr, gim, gi[t], gj[t]);
+            }
+            warp_sum2(gr, gim);
+            if (!negligible(al) && !negligible(be)) kind = rotation(al, be, gr, gim, tol, rot, tg);
+            if (kind) {
+              S na_i = s_add(al, s_neg(tg)), na_j = s_add(be, tg);
+              const bool anew = !s_less(s_quarter(al), na_i) || !s_less(s_quarter(be), na_j);
+              S ni = s_zero(S()), nj = s_zero(S());
+              if constexpr (NE > 0) {
+#pragma unroll
+                for (int q = 0; q < NE; ++q) {
+                  const int t = lane + 32 * q;
+                  rotate_elem(rot, x[q], y[q]);
+                  if (t < m) {
+                    gi[t] = x[q];
+                    gj[t] = y[q];
+                  }
+                }
+                if (anew) {
+#pragma unroll
+                  for (int q = 0; q < NE; ++q) {
+                    norm_acc(ni, x[q]);
+                    norm_acc(nj, y[q]);
+                  }
+                }
+              } else {
+                for (int t = lane; t < m; t += 32) {
+                  E u = gi[t], v = gj[t];
+                  rotate_elem(rot, u, v);
+                  gi[t] = u;
+                  gj[t] = v;
+                  if (anew) {
+                    norm_acc(ni, u);
+                    norm_acc(nj, v);
+                  }
+                }
+              }
+              if (anew) {
+                warp_sum2(ni, nj);
+                na_i = ni;
+                na_j = nj;
+              }
+              if (lane == 0) {
+                *nrm(i) = na_i;
+                *nrm(j) = na_j;
+                atomicAdd(&s_rot, 1);
+                if (kind == 2) s_big = 1;
+              }
+            }
+          }
+          if (lane == 0) {
+            if constexpr (DF) {
+              if (with_v) {
+                s_recij[par][slot] = kind ? (i << 16 | j) : -1;
+                s_rec[par][slot] = rot;
+              }
+            }
+            if (log && p < npairs) {
+              double4_16a rec = make_double4_16a(2.0, 0.0, 0.0, 0.0);
+              if (kind) rec = make_double4_16a(s_val(rot.c), s_val(rot.qr), s_val(rot.qi), 0.0);
+              log[((long long)sweep * rounds + r) * npairs + p] = rec;
+            }
+          }
+        }
+      } else {
+        rotate_v(par ^ 1);
+      }
+      par ^= 1;
       cl.sync();
     }
     int total = 0, big = 0;
@@ -349,35 +618,54 @@ __global__ void __launch_bounds__(JC_THREADS, 1)
       s_rot = 0;
       s_big = 0;
     }
-    cl.sync();
     // No rotation: converged.  Only rotations with off-orthogonality and angle
     // <= 1e-8: each later rotation changed an earlier pair's inner product by at
     // most 1e-16 relative, so the rows are orthogonal to ~k * 1e-16 (the
     // m * eps tolerance) and the confirming sweep is skipped.
-    if (total == 0 || big == 0) {
-      converged = true;
-      break;
-    }
+    if (total == 0 || big == 0) converged = true;
+  }
+  if (with_v) {
+    if (warp >= gwarps) rotate_v(par ^ 1);  // the last round's rotations
+    cl.sync();
   }
   for (int l = 0; l < R; ++l) {
-    const int i = l * cs + rank;
-    if (i >= n) break;
-    for (int t = threadIdx.x; t < m; t += JC_THREADS) {
+    const int a = l * cs + rank;
+    if (a >= na) break;
+    const int i = s_act[a];
+    for (int t = threadIdx.x; t < m; t += blockDim.x) {
       if constexpr (DF) {
-        const float4 x4 = ((const float4*)gl)[(long long)l * m + t];
-        G[(long long)i * ldg + t] = make_double2(df_val({x4.x, x4.y}), df_val({x4.z, x4.w}));
+        const float4 x4 = gl[(long long)l * m + t];
+        G[(long long)i * ldg + t] = make_double2(df_val({x4.x, x4.y}) * isc, df_val({x4.z, x4.w}) * isc);
       } else {
         G[(long long)i * ldg + t] = gl[(long long)l * m + t];
       }
     }
-    if (Vt)
-      for (int t = threadIdx.x; t < n; t += JC_THREADS) Vt[(long long)i * n + t] = vl[(long long)l * n + t];
+    if constexpr (DF) {
+      if (with_v)
+        for (int t = threadIdx.x; t < n; t += blockDim.x) {
+          const float4 x4 = vl[(long long)l * n + t];
+          Vt[(long long)i * n + t] = make_double2(df_val({x4.x, x4.y}), df_val({x4.z, x4.w}));
+        }
+    }
   }
-  if (rank == 0 && threadIdx.x == 0) {
-    if (sweeps_used) *sweeps_used = converged ? sweep + 1 : max_sweeps;
-    atomicAdd(&st->jacobi_calls, 1);
-    atomicAdd(&st->jacobi_sweeps, converged ? sweep + 1 : max_sweeps);
-    if (!converged) atomicAdd(&st->jacobi_unconverged, 1);
+  if (with_v && !warm)  // rows that took part in no rotation: the identity's
+    for (int i = rank; i < n; i += cs) {
+      bool on = false;
+      for (int a = threadIdx.x; a < na; a += blockDim.x) on |= s_act[a] == i;
+      if (!__syncthreads_or(on))
+        for (int t = threadIdx.x; t < n; t += blockDim.x) Vt[(long long)i * n + t] = make_double2(t == i ? 1.0 : 0.0, 0.0);
+    }
+  if (rank == 0) {
+    if (amap) {
+      for (int a = threadIdx.x; a < na; a += blockDim.x) amap[1 + a] = s_act[a];
+      if (threadIdx.x == 0) amap[0] = na;
+    }
+    if (threadIdx.x == 0) {
+      if (sweeps_used) *sweeps_used = sweep;
+      atomicAdd(&st->jacobi_calls, 1);
+      atomicAdd(&st->jacobi_sweeps, sweep);
+      if (!converged) atomicAdd(&st->jacobi_unconverged, 1);
+    }
   }
   cl.sync();  // no CTA leaves while another may still read its shared memory
 }
@@ -385,78 +673,54 @@ __global__ void __launch_bounds__(JC_THREADS, 1)
 // Vt (n x n) = the logged rotations applied to the identity (warm: to Vt as
 // it is, in place), one CTA per column q (columns are independent: a CTA
 // reads and writes its own column only): thread p applies pair p of every
-// round, rounds in order, the column held in shared memory.  Rotation c = 2
-// marks a pair that was not rotated.  DF (the precision form): the column in
-// double-float arithmetic on the FP32 pipe; the unitarity of V then holds to
-// about 2^-48 per rotation instead of 2^-53, some 1e-12 after thousands of
-// visits of a cut, far below the precision form's 1e-6 truncation.
-template <bool DF>
+// round, rounds in order, the column held in shared memory.  The log covers
+// the active rows (amap[0] of them, amap[1 + a] the row of active row a).
+// Rotation c = 2 marks a pair that was not rotated.  The next LOOK rounds'
+// records are on their way while one is applied: a round is a load from
+// memory, a rotation and a block barrier, and the load is the longest.
 __global__ void jacobi_replay_kernel(cplx* __restrict__ Vt, int n, const double4_16a* __restrict__ log,
-                                     const int* __restrict__ sweeps_used, int warm) {
-  extern __shared__ cplx col[];  // DF: (Re hi, Re lo, Im hi, Im lo) per element, the same 16 bytes
-  float4* colf = (float4*)col;
+                                     const int* __restrict__ amap, const int* __restrict__ sweeps_used, int warm) {
+  extern __shared__ cplx col[];
   const int q = blockIdx.x;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const cplx v = warm ? Vt[(long long)i * n + q] : make_double2(i == q ? 1.0 : 0.0, 0.0);
-    if constexpr (DF)
-      colf[i] = df_elem(v);
-    else
-      col[i] = v;
+  const int na = amap[0];
+  for (int a = threadIdx.x; a < na; a += blockDim.x) {
+    const int i = amap[1 + a];
+    col[a] = warm ? Vt[(long long)i * n + q] : make_double2(i == q ? 1.0 : 0.0, 0.0);
   }
+  if (!warm)  // rows left out keep the identity's
+    for (int i = threadIdx.x; i < n; i += blockDim.x) Vt[(long long)i * n + q] = make_double2(i == q ? 1.0 : 0.0, 0.0);
   __syncthreads();
   const int sweeps = *sweeps_used;
-  const int np = (n + 1) & ~1;
+  const int np = (na + 1) & ~1;
   const int rounds = np - 1, npairs = np / 2;
   const int p = threadIdx.x;
-  const long long steps = (long long)sweeps * rounds;
-  // the next round's record is loaded while this round's rotation runs
-  double4_16a next = make_double4_16a(2.0, 0.0, 0.0, 0.0);
-  if (p < npairs && steps > 0) next = log[p];
-  for (long long st = 0; st < steps; ++st) {
-    const int r = (int)(st % rounds);
-    const double4_16a rec = next;
-    if (p < npairs && st + 1 < steps) next = log[(st + 1) * npairs + p];
-    if (p < npairs && rec.x < 1.5) {
-      int i, j;
-      pair_of(r, p, np, rounds, &i, &j);
-      const double c = rec.x, s = rec.y;
-      if constexpr (DF) {
-        const df2 cd = df_of(c), qr = df_of(s * rec.z), qi = df_of(s * rec.w), pr = qr, pi = df_negate(qi);
-        const float4 x4 = colf[i], y4 = colf[j];
-        const df2 xr = {x4.x, x4.y}, xi = {x4.z, x4.w}, yr = {y4.x, y4.y}, yi = {y4.z, y4.w};
-        df2 ar = {0.f, 0.f}, ai = {0.f, 0.f}, br = {0.f, 0.f}, bi = {0.f, 0.f};
-        acc_mul(ar, cd, xr);
-        acc_mul(ar, df_negate(qr), yr);
-        acc_mul(ar, qi, yi);
-        acc_mul(ai, cd, xi);
-        acc_mul(ai, df_negate(qr), yi);
-        acc_mul(ai, df_negate(qi), yr);
-        acc_mul(br, cd, yr);
-        acc_mul(br, pr, xr);
-        acc_mul(br, df_negate(pi), xi);
-        acc_mul(bi, cd, yi);
-        acc_mul(bi, pr, xi);
-        acc_mul(bi, pi, xr);
-        ar = df_norm(ar);
-        ai = df_norm(ai);
-        br = df_norm(br);
-        bi = df_norm(bi);
-        colf[i] = make_float4(ar.h, ar.l, ai.h, ai.l);
-        colf[j] = make_float4(br.h, br.l, bi.h, bi.l);
-      } else {
-        jac_rotate(col[i], col[j], c, make_double2(s * rec.z, s * rec.w), make_double2(s * rec.z, -s * rec.w));
+  const long long steps = na < 2 ? 0 : (long long)sweeps * rounds;
+  constexpr int LOOK = 8;
+  double4_16a rec[LOOK];
+#pragma unroll
+  for (int u = 0; u < LOOK; ++u) {
+    rec[u] = make_double4_16a(2.0, 0.0, 0.0, 0.0);
+    if (p < npairs && u < steps) rec[u] = log[(long long)u * npairs + p];
+  }
+  int r = 0;
+  for (long long st0 = 0; st0 < steps; st0 += LOOK) {
+#pragma unroll
+    for (int u = 0; u < LOOK; ++u) {
+      const long long st = st0 + u;
+      if (st < steps) {
+        const double4_16a c = rec[u];
+        if (p < npairs && st + LOOK < steps) rec[u] = log[(st + LOOK) * npairs + p];
+        if (p < npairs && c.x < 1.5) {
+          int i, j;
+          pair_of(r, p, np, rounds, &i, &j);
+          rotate_elem(Rot<double>{c.x, c.y, c.z}, col[i], col[j]);
+        }
+        if (++r == rounds) r = 0;
+        __syncthreads();
       }
     }
-    __syncthreads();
   }
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    if constexpr (DF) {
-      const float4 x4 = colf[i];
-      Vt[(long long)i * n + q] = make_double2(df_val({x4.x, x4.y}), df_val({x4.z, x4.w}));
-    } else {
-      Vt[(long long)i * n + q] = col[i];
-    }
-  }
+  for (int a = threadIdx.x; a < na; a += blockDim.x) Vt[(long long)amap[1 + a] * n + q] = col[a];
 }
 
 // Right-looking Cholesky of the Hermitian n x n G (upper triangle used) with
@@ -591,11 +855,19 @@ __global__ void __launch_bounds__(CL_THREADS)
 
 }  // namespace
 
+static const void* jacobi_fn(bool df, int m) {
+  if (df)
+    return m <= 128 ? (const void*)jacobi_cluster_kernel<true, 4>
+                    : (m <= 256 ? (const void*)jacobi_cluster_kernel<true, 8> : (const void*)jacobi_cluster_kernel<true, 0>);
+  return m <= 128 ? (const void*)jacobi_cluster_kernel<false, 4>
+                  : (m <= 256 ? (const void*)jacobi_cluster_kernel<false, 8> : (const void*)jacobi_cluster_kernel<false, 0>);
+}
+
 static cudaError_t cluster_init() {
   if (g_csize) return cudaSuccess;
   cudaError_t e;
-  const void* fns[3] = {(const void*)jacobi_cluster_kernel<false>, (const void*)jacobi_cluster_kernel<true>,
-                        (const void*)chol_cluster_kernel};
+  const void* fns[7] = {jacobi_fn(false, 128), jacobi_fn(false, 256), jacobi_fn(false, 257), jacobi_fn(true, 128),
+                        jacobi_fn(true, 256),  jacobi_fn(true, 257),  (const void*)chol_cluster_kernel};
   for (const void* f : fns) {
     if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, CL_SMEM)) != cudaSuccess) return e;
@@ -609,13 +881,12 @@ static cudaError_t cluster_init() {
   attr.val.clusterDim.y = 1;
   attr.val.clusterDim.z = 1;
   cfg.gridDim = dim3(16);
-  cfg.blockDim = dim3(CL_THREADS);
+  cfg.blockDim = dim3(512);
   cfg.dynamicSmemBytes = CL_SMEM;
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
   int nclusters = 0;
-  if (cudaOccupancyMaxActiveClusters(&nclusters, (const void*)jacobi_cluster_kernel<false>, &cfg) == cudaSuccess &&
-      nclusters >= 1)
+  if (cudaOccupancyMaxActiveClusters(&nclusters, jacobi_fn(false, 257), &cfg) == cudaSuccess && nclusters >= 1)
     csize = 16;
   cudaGetLastError();  // a refused query leaves no error behind
   g_csize = csize;
@@ -624,15 +895,16 @@ static cudaError_t cluster_init() {
 
 cudaError_t fp64_cluster_init() { return cluster_init(); }
 
-static cudaError_t launch_cluster(const void* fn, void** args, size_t smem, cudaStream_t s,
-                                  int threads = CL_THREADS) {
+static cudaError_t launch_cluster(const void* fn, void** args, size_t smem, cudaStream_t s, int threads = CL_THREADS,
+                                  int csize = 0, int nclusters = 1) {
+  if (csize == 0) csize = g_csize;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr;
   attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = g_csize;
+  attr.val.clusterDim.x = csize;
   attr.val.clusterDim.y = 1;
   attr.val.clusterDim.z = 1;
-  cfg.gridDim = dim3(g_csize);
+  cfg.gridDim = dim3(csize * nclusters);
   cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
@@ -641,49 +913,86 @@ static cudaError_t launch_cluster(const void* fn, void** args, size_t smem, cuda
   return cudaLaunchKernelExC(&cfg, fn, args);
 }
 
-bool jacobi_cluster_fits(int n, int m, bool vt_in_smem) {
-  if (n < 32) return false;
-  if (cluster_init() != cudaSuccess) return false;
-  const long long R = (n + g_csize - 1) / g_csize;
-  return R * ((long long)m + (vt_in_smem ? n : 0)) * (long long)sizeof(cplx) <= CL_SMEM;
+// dynamic shared memory of a CTA, 0 where the rows do not fit a cluster of cs
+static size_t jacobi_smem(int n, int m, bool vt_in_smem, int cs) {
+  const long long R = (n + cs - 1) / cs, npairs = (n + 1) / 2;
+  if (R > 2 * JC_MAXP || (npairs + cs - 1) / cs > JC_MAXP || n > JC_MAXP * 2 * 16) return 0;
+  const long long b =
+      std::max(R * ((long long)m + (vt_in_smem ? n : 0)) * (long long)sizeof(cplx), n * (long long)sizeof(double));
+  return b <= CL_SMEM ? (size_t)b : 0;
 }
 
-long long jacobi_log_elems(int n, int max_sweeps) {
+bool jacobi_cluster_fits(int n, int m) {
+  if (n < 32) return false;
+  if (cluster_init() != cudaSuccess) return false;
+  return jacobi_smem(n, m, false, g_csize) > 0;
+}
+
+// the rotation records (one double4_16a = two complex slots per pair), then
+// the map of the active rows
+static long long jacobi_log_slots(int n, int max_sweeps) {
   const long long np = (n + 1) & ~1;
-  return (long long)max_sweeps * (np - 1) * (np / 2) * 2;  // one double4_16a = two complex slots per pair
+  return (long long)max_sweeps * (np - 1) * (np / 2) * 2;
+}
+long long jacobi_log_elems(int n, int max_sweeps) {
+  return jacobi_log_slots(n, max_sweeps) + (n + 1 + 3) / 4;
+}
+
+static int jacobi_threads(int n, int cs, bool with_v) {
+  const int own = ((n + 1) / 2 + cs - 1) / cs;  // pairs per CTA, a warp each (two with V)
+  return (with_v ? 2 * own : own) <= 8 ? 256 : 512;
 }
 
 cudaError_t jacobi_cluster(cudaStream_t s, cplx* G, int n, int m, long long ldg, cplx* Vt, int max_sweeps,
                            DevStatus* st, cplx* rotlog, int* sweeps_used, bool warm_v, bool dfloat) {
   cudaError_t e;
   if ((e = cluster_init()) != cudaSuccess) return e;
-  const bool replay = Vt && rotlog && sweeps_used && n <= 2048;
-  cplx* Vin = replay ? nullptr : Vt;  // with a log, Vt is rebuilt afterwards across the GPU
+  if (Vt && !rotlog) return cudaErrorInvalidValue;
+  // double-float rows only where a V comes with them (the projector cores);
+  // their dot products resolve orthogonality to about m 2^-48, so pairs are
+  // left alone below m 2^-44 (FP64: m eps)
+  const bool df = dfloat && Vt;
+  const bool v_in = df && jacobi_smem(n, m, true, g_csize) > 0;  // V beside the rows; else replayed from the log
+  const bool replay = Vt && !v_in;
+  cplx* Vin = v_in ? Vt : nullptr;
   double4_16a* logp = replay ? (double4_16a*)rotlog : nullptr;
+  int* amap = replay ? (int*)(rotlog + jacobi_log_slots(n, max_sweeps)) : nullptr;
   int* su = replay ? sweeps_used : nullptr;
-  const long long R = (n + g_csize - 1) / g_csize;
-  const size_t smem = (size_t)(R * ((long long)m + (Vin ? n : 0)) * sizeof(cplx));
-  // double-float rows only where Vt is rebuilt from the log in FP64; their
-  // dot products resolve orthogonality to about m 2^-48, so pairs are left
-  // alone below m 2^-44 (FP64: m eps)
-  const bool df = dfloat && replay;
-  double tol = df ? (double)m * 0x1p-44 : (double)m * 2.220446049250313e-16;
-  int warm = warm_v && Vin ? 1 : 0;
-  void* args[] = {&G, &n, &m, &ldg, &Vin, &max_sweeps, &tol, &logp, &su, &st, &warm};
-  e = launch_cluster(df ? (const void*)jacobi_cluster_kernel<true> : (const void*)jacobi_cluster_kernel<false>, args,
-                     smem, s, JC_THREADS);
+  size_t smem = jacobi_smem(n, m, v_in, g_csize);
+  float tol = df ? (float)((double)m * 0x1p-44) : (float)((double)m * 2.220446049250313e-16);
+  int warm = warm_v && Vt ? 1 : 0;
+  long long stride = 0;
+  void* args[] = {&G, &n, &m, &ldg, &stride, &Vin, &max_sweeps, &tol, &logp, &amap, &su, &st, &warm};
+  e = launch_cluster(jacobi_fn(df, m), args, smem, s, jacobi_threads(n, g_csize, v_in));
   count_launch();
   if (e != cudaSuccess || !replay) return e;
   const int npairs = ((n + 1) & ~1) / 2;
   const int threads = (npairs + 31) / 32 * 32;
-  if (df)
-    jacobi_replay_kernel<true><<<n, threads, n * sizeof(cplx), s>>>(Vt, n, (const double4_16a*)rotlog, sweeps_used,
-                                                                  warm_v ? 1 : 0);
-  else
-    jacobi_replay_kernel<false><<<n, threads, n * sizeof(cplx), s>>>(Vt, n, (const double4_16a*)rotlog, sweeps_used,
-                                                                   warm_v ? 1 : 0);
+  jacobi_replay_kernel<<<n, threads, n * sizeof(cplx), s>>>(Vt, n, (const double4_16a*)rotlog, amap, sweeps_used,
+                                                          warm);
   count_launch();
   return cudaGetLastError();
+}
+
+// Singular values only of `count` matrices (matrix b at G + b * strideG), one
+// cluster each in one launch.  Clusters of 8 where 16-CTA ones would not all
+// be resident: the FP64 units of the SMs in use bound the kernel, and 16
+// corners on 8 CTAs each take 128 SMs at once.
+cudaError_t jacobi_cluster_batch(cudaStream_t s, cplx* G, int n, int m, long long ldg, long long strideG, int count,
+                                 int max_sweeps, DevStatus* st) {
+  cudaError_t e;
+  if ((e = cluster_init()) != cudaSuccess) return e;
+  int cs = g_csize;
+  if (count * cs > 144 && jacobi_smem(n, m, false, 8) > 0) cs = 8;
+  size_t smem = jacobi_smem(n, m, false, cs);
+  cplx* Vin = nullptr;
+  double4_16a* logp = nullptr;
+  int *amap = nullptr, *su = nullptr, warm = 0;
+  float tol = (float)((double)m * 2.220446049250313e-16);
+  void* args[] = {&G, &n, &m, &ldg, &strideG, &Vin, &max_sweeps, &tol, &logp, &amap, &su, &st, &warm};
+  e = launch_cluster(jacobi_fn(false, m), args, smem, s, jacobi_threads(n, cs, false), cs, count);
+  count_launch();
+  return e;
 }
 
 bool chol_cluster_fits(int n) {

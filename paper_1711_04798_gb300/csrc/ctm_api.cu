@@ -1764,19 +1764,38 @@ void ctm_set_sequential_cuts(ipeps_ctm h, bool on) {
 // spectra / convergence
 // ---------------------------------------------------------------------------
 static ipeps_status spectra_device(ipeps_ctm h, double* host) {
-  const int c = h->chi;
-  cplx* w = scratch_alloc(h, (long long)c * c);
-  if (!w) return fail(IPEPS_ENOMEM, "scratch exhausted (spectra)");
-  const int ncell = h->Lx * h->Ly;
-  for (int j = 0; j < 4; ++j)
-    for (int i = 0; i < ncell; ++i) {
-      CK(cudaMemcpyAsync(w, h->C[j][i], (size_t)c * c * sizeof(cplx), cudaMemcpyDeviceToDevice, h->stream));
+  const int c = h->chi, ncell = h->Lx * h->Ly, nc = 4 * ncell;
+  const size_t cb = (size_t)c * c * sizeof(cplx);
+  // all corners in one launch, a cluster each, where the scratch holds them
+  // (the corners' SVDs are independent; one after another each used 16 SMs)
+  const long long mark = h->scratch_top;
+  cplx* w = scratch_alloc(h, (long long)nc * c * c);
+  cplx* v = w ? scratch_alloc(h, (long long)nc * c) : nullptr;  // sigma and its selection, nc * c doubles each
+  cplx* pm = v ? scratch_alloc(h, (long long)nc * c / 4 + 1) : nullptr;
+  bool done = false;
+  if (pm) {
+    double* sig = (double*)v;
+    double* sel = sig + (size_t)nc * c;
+    for (int q = 0; q < nc; ++q)
+      CK(cudaMemcpyAsync(w + (size_t)q * c * c, h->C[q / ncell][q % ncell], cb, cudaMemcpyDeviceToDevice, h->stream));
+    CK(jacobi_rows_batch(h->stream, w, c, nc, sig, h->opt.jacobi_max_sweeps, h->st, &done));
+    if (done) {
+      CK(select_top(h->stream, sig, c, c, 0.0, (int*)pm, sel, nc));
+      CK(cudaMemcpyAsync(host, sel, (size_t)nc * c * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+    }
+  }
+  if (!done) {
+    h->scratch_top = mark;
+    w = scratch_alloc(h, (long long)c * c);
+    if (!w) return fail(IPEPS_ENOMEM, "scratch exhausted (spectra)");
+    for (int q = 0; q < nc; ++q) {
+      CK(cudaMemcpyAsync(w, h->C[q / ncell][q % ncell], cb, cudaMemcpyDeviceToDevice, h->stream));
       CK(jacobi_rows(h->stream, w, c, c, c, nullptr, h->sigma, h->opt.jacobi_max_sweeps, h->dwork,
                      h->counters, h->st, nullptr, 0, h->opt.wait_cycles));
       CK(select_top(h->stream, h->sigma, c, c, 0.0, h->perm, h->s_sel));
-      CK(cudaMemcpyAsync(host + (size_t)(j * ncell + i) * c, h->s_sel, c * sizeof(double),
-                         cudaMemcpyDeviceToHost, h->stream));
+      CK(cudaMemcpyAsync(host + (size_t)q * c, h->s_sel, c * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     }
+  }
   h->scratch_top = 0;
   CK(cudaStreamSynchronize(h->stream));
   for (int q = 0; q < 4 * ncell; ++q) {

@@ -114,29 +114,36 @@ cudaError_t set_zero(cudaStream_t s, cplx* x, long long n);
 // same rotations starting from the identity.  sigma[i] = ||row i|| on return.
 // counters: 4 ints of scratch (sweep counters and, for m <= 256, a grid barrier);
 // work: 1 double of scratch.
-// rotlog (optional, jacobi_log_elems(n, max_sweeps) complex slots): lets the
-// cluster path rebuild Vt from logged rotations instead of holding it.
+// rotlog (jacobi_log_elems(n, max_sweeps) complex slots): lets the cluster path
+// rebuild Vt from logged rotations; without it a call with Vt takes the
+// grid-wide kernels.
 // wait_cycles: limit of each grid-barrier wait of the small-row kernel (<= 0:
 // about 2 s of clock); a wait that runs out is counted in st->barrier_timeouts
 // and its CTA stops.
 // warm_v: Vt holds a unitary n x n start V0^T on entry (the rotations are
 // accumulated onto it, Vt = J^T V0^T) instead of starting from the identity.
-// dfloat: where the cluster path rebuilds Vt from the rotation log, hold,
-// dot and rotate the rows in double-float arithmetic (about 48 bits; the
-// rotations themselves and Vt stay FP64), for the precision form.
+// dfloat: on the cluster path with Vt, hold, dot and rotate the rows (and Vt)
+// in double-float arithmetic (about 48 bits), for the precision form.
 cudaError_t jacobi_rows(cudaStream_t s, cplx* G, int n, int m, long long ldg, cplx* Vt,
                         double* sigma, int max_sweeps, double* work, int* counters,
                         DevStatus* st, cplx* rotlog = nullptr, long long rotlog_elems = 0,
                         long long wait_cycles = 0, bool warm_v = false, bool dfloat = false);
+// The singular values alone of `count` n x n matrices stored one after another
+// (rows made orthogonal in place): sigma[b n + i] = ||row i of matrix b||.
+// One launch, a cluster per matrix, where jacobi_cluster_fits(n, n); false
+// returned in *done (nothing launched) otherwise.
+cudaError_t jacobi_rows_batch(cudaStream_t s, cplx* G, int n, int count, double* sigma, int max_sweeps, DevStatus* st,
+                              bool* done);
 // V (n x n) = identity
 cudaError_t set_identity(cudaStream_t s, cplx* V, int n);
 // rows of G scaled to unit norm where sigma > tol*max(sigma), zero otherwise
 cudaError_t orth_rows_finish(cudaStream_t s, cplx* G, int n, int m, long long ldg,
                              const double* sigma, double tol);
 // descending selection of the top chi of sigma[0..n) above cutoff*max:
-// perm[0..chi) (or -1), s_sel[0..chi) (or 0)
+// perm[0..chi) (or -1), s_sel[0..chi) (or 0); `count` such selections, sigma n
+// and perm, s_sel chi apart
 cudaError_t select_top(cudaStream_t s, const double* sigma, int n, int chi, double cutoff,
-                       int* perm, double* s_sel);
+                       int* perm, double* s_sel, int count = 1);
 // out[a, :] = scale_a * in[perm[a], :] (row length m); scale_a = 1/sigma[perm[a]] if
 // normalize_by_sigma, else 1; rows with perm[a] < 0 are zero.
 cudaError_t gather_rows(cudaStream_t s, const cplx* in, long long ldi, cplx* out,
@@ -192,14 +199,16 @@ cudaError_t kernels_init();
 // FP64 Jacobi / Cholesky on one thread-block cluster (cluster_fp64.cu): rows
 // in distributed shared memory, hardware cluster barriers between steps.
 cudaError_t fp64_cluster_init();
-bool jacobi_cluster_fits(int n, int m, bool vt_in_smem);
-// With rotlog (jacobi_log_elems(n, max_sweeps) complex slots) and sweeps_used
-// (one int), Vt is not held in the cluster: the rotations are logged and
-// replayed onto the identity (onto Vt itself with warm_v) by one CTA per
-// column afterwards.
+bool jacobi_cluster_fits(int n, int m);
+// Vt needs rotlog (jacobi_log_elems(n, max_sweeps) complex slots) and
+// sweeps_used (one int): FP64 rotations are logged and replayed onto the
+// identity (onto Vt itself with warm_v) by one CTA per column afterwards.
 cudaError_t jacobi_cluster(cudaStream_t s, cplx* G, int n, int m, long long ldg, cplx* Vt, int max_sweeps,
                            DevStatus* st, cplx* rotlog, int* sweeps_used, bool warm_v = false,
                            bool dfloat = false);
+// the rows of `count` matrices (strideG apart) made orthogonal, one cluster each
+cudaError_t jacobi_cluster_batch(cudaStream_t s, cplx* G, int n, int m, long long ldg, long long strideG, int count,
+                                 int max_sweeps, DevStatus* st);
 long long jacobi_log_elems(int n, int max_sweeps);
 bool chol_cluster_fits(int n);
 cudaError_t chol_cluster(cudaStream_t s, const cplx* G, cplx* R, int n, double tol);

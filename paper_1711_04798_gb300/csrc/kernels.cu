@@ -450,6 +450,9 @@ __global__ void select_top_kernel(const double* __restrict__ sigma, int n, int c
                                   double cutoff, int* perm, double* s_sel) {
   __shared__ double sh[32];
   __shared__ int cnt_sh;
+  sigma += (long long)blockIdx.x * n;
+  perm += (long long)blockIdx.x * chi;
+  s_sel += (long long)blockIdx.x * chi;
   double mx = 0.0;
   for (int i = threadIdx.x; i < n; i += blockDim.x) mx = fmax(mx, sigma[i]);
   mx = block_max(mx, sh);
@@ -612,8 +615,8 @@ cudaError_t jacobi_rows(cudaStream_t s, cplx* G, int n, int m, long long ldg, cp
   cudaError_t e;
   if ((e = kernels_init()) != cudaSuccess) return e;
   const bool logged = Vt && rotlog && n <= 2048 && rotlog_elems >= jacobi_log_elems(n, max_sweeps);
-  if (jacobi_cluster_fits(n, m, Vt != nullptr && !logged)) {
-    // rows (and Vt unless logged) fit in one cluster's shared memory: no grid-wide barrier
+  if (jacobi_cluster_fits(n, m) && (!Vt || logged)) {
+    // the rows fit in one cluster's shared memory: no grid-wide barrier
     if ((e = jacobi_cluster(s, G, n, m, ldg, Vt, max_sweeps, st, logged ? rotlog : nullptr,
                             logged ? counters : nullptr, warm_v, dfloat)) != cudaSuccess)
       return e;
@@ -660,6 +663,16 @@ cudaError_t jacobi_rows(cudaStream_t s, cplx* G, int n, int m, long long ldg, cp
   return cudaGetLastError();
 }
 
+cudaError_t jacobi_rows_batch(cudaStream_t s, cplx* G, int n, int count, double* sigma, int max_sweeps, DevStatus* st,
+                              bool* done) {
+  cudaError_t e;
+  if ((e = kernels_init()) != cudaSuccess) return e;
+  *done = jacobi_cluster_fits(n, n);
+  if (!*done) return cudaSuccess;
+  if ((e = jacobi_cluster_batch(s, G, n, n, n, (long long)n * n, count, max_sweeps, st)) != cudaSuccess) return e;
+  return row_norms(s, G, n * count, n, n, sigma);
+}
+
 cudaError_t set_identity(cudaStream_t s, cplx* V, int n) {
   init_identity_kernel<<<grid_for((long long)n * n), 256, 0, s>>>(V, n);
   count_launch();
@@ -674,8 +687,8 @@ cudaError_t orth_rows_finish(cudaStream_t s, cplx* G, int n, int m, long long ld
 }
 
 cudaError_t select_top(cudaStream_t s, const double* sigma, int n, int chi, double cutoff,
-                       int* perm, double* s_sel) {
-  select_top_kernel<<<1, 1024, 0, s>>>(sigma, n, chi, cutoff, perm, s_sel);
+                       int* perm, double* s_sel, int count) {
+  select_top_kernel<<<count, 1024, 0, s>>>(sigma, n, chi, cutoff, perm, s_sel);
   count_launch();
   return cudaGetLastError();
 }
