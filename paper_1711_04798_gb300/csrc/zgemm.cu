@@ -2,9 +2,7 @@
 // contractions) and the generic index permutation that feeds it.
 #include "ctm_internal.h"
 
-#include <algorithm>
 #include <atomic>
-#include <cmath>
 
 static std::atomic<uint64_t> g_launches{0};
 void count_launch(int n) { g_launches += (uint64_t)n; }
@@ -22,24 +20,26 @@ __device__ __forceinline__ cplx ld_op(const cplx* p, bool cj) {
   return v;
 }
 
-// TM x TN output tile per CTA (64 x 64 with 256 threads, or 32 x 32 with 64
-// threads for small outputs), each thread a 4x4 block of outputs strided by
-// TM/4 (TN/4) so that shared-memory reads are broadcast / conflict-free.
-template <int TM, int TN>
-__global__ void __launch_bounds__((TM / 4) * (TN / 4)) zgemm_kernel(int M, int N, int K, cplx alpha,
-                                                   const cplx* __restrict__ A, long long lda,
-                                                   int opA, const cplx* __restrict__ B,
-                                                   long long ldb, int opB, cplx beta,
-                                                   cplx* __restrict__ C, long long ldc,
-                                                   long long sA, long long sB, long long sC,
-                                                   int ksplit, int flags) {
-  constexpr int BM = TM, BN = TN, NT = (TM / 4) * (TN / 4), SX = TN / 4, SY = TM / 4;
-  __shared__ cplx As[BK][BM + 1];
-  __shared__ cplx Bs[BK][BN + 1];
+// T x T output tile per CTA of 256 threads, each thread MI x MI outputs (T =
+// 16 MI) strided by 16 so that shared-memory reads are broadcast /
+// conflict-free.  The FP64 units bound every tile (about 1.75 multiply-adds
+// per cycle and SM; even MI = 1 needs only 2 shared loads for the 4 that hold
+// the SM's units for some 70 cycles), so the tile only sets how evenly the
+// product covers the SMs and how much of it is padding: a 32 x 32 tile with K =
+// 64 is 70 us of one SM's FP64 time.
+template <int MI>
+__global__ void __launch_bounds__(256) zgemm_kernel(int M, int N, int K, cplx alpha, const cplx* __restrict__ A,
+                                                    long long lda, int opA, const cplx* __restrict__ B,
+                                                    long long ldb, int opB, cplx beta, cplx* __restrict__ C,
+                                                    long long ldc, long long sA, long long sB, long long sC,
+                                                    int ksplit, int flags) {
+  constexpr int T = 16 * MI, NT = 256;
+  __shared__ cplx As[BK][T + 1];
+  __shared__ cplx Bs[BK][T + 1];
   const long long bz = blockIdx.z;
-  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+  const int m0 = blockIdx.y * T, n0 = blockIdx.x * T;
   if ((flags & ZG_UPPER_TILES) && blockIdx.y > blockIdx.x) return;  // tile below the diagonal: not needed
-  const int tx = threadIdx.x % SX, ty = threadIdx.x / SX;
+  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
   const bool tA = opA & OP_T, cA = opA & OP_CONJ;
   const bool tB = opB & OP_T, cB = opB & OP_CONJ;
   if (ksplit > 0) {
@@ -48,65 +48,70 @@ __global__ void __launch_bounds__((TM / 4) * (TN / 4)) zgemm_kernel(int M, int N
     A += tA ? kb * lda : kb;
     B += tB ? kb : kb * ldb;
     K = (int)min((long long)ksplit, (long long)K - kb);
-    if (flags & ZG_A_LOWER) K = (int)max(0LL, min((long long)K, (long long)(m0 + BM) - kb));
+    if (flags & ZG_A_LOWER) K = (int)max(0LL, min((long long)K, (long long)(m0 + T) - kb));
     C += bz * sC;
   } else {
-    if (flags & ZG_A_LOWER) K = min(K, m0 + BM);  // A[m, k] = 0 for k > m: later k-tiles add nothing
+    if (flags & ZG_A_LOWER) K = min(K, m0 + T);  // A[m, k] = 0 for k > m: later k-tiles add nothing
     A += bz * sA;
     B += bz * sB;
     C += bz * sC;
   }
-  double cr[4][4], ci[4][4];
+  double cr[MI][MI], ci[MI][MI];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < MI; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) cr[i][j] = ci[i][j] = 0.0;
+    for (int j = 0; j < MI; ++j) cr[i][j] = ci[i][j] = 0.0;
 
+  auto step = [&](int kk) {
+    cplx a[MI], b[MI];
+#pragma unroll
+    for (int i = 0; i < MI; ++i) a[i] = As[kk][ty + 16 * i];
+#pragma unroll
+    for (int j = 0; j < MI; ++j) b[j] = Bs[kk][tx + 16 * j];
+#pragma unroll
+    for (int i = 0; i < MI; ++i)
+#pragma unroll
+      for (int j = 0; j < MI; ++j) {
+        cr[i][j] = fma(a[i].x, b[j].x, cr[i][j]);
+        cr[i][j] = fma(-a[i].y, b[j].y, cr[i][j]);
+        ci[i][j] = fma(a[i].x, b[j].y, ci[i][j]);
+        ci[i][j] = fma(a[i].y, b[j].x, ci[i][j]);
+      }
+  };
   for (int k0 = 0; k0 < K; k0 += BK) {
-    for (int e = threadIdx.x; e < BM * BK; e += NT) {
+    for (int e = threadIdx.x; e < T * BK; e += NT) {
       int mm, kk;
-      if (tA) { mm = e % BM; kk = e / BM; } else { kk = e % BK; mm = e / BK; }
+      if (tA) { mm = e % T; kk = e / T; } else { kk = e % BK; mm = e / BK; }
       const int m = m0 + mm, k = k0 + kk;
       cplx v = make_double2(0.0, 0.0);
       if (m < M && k < K) v = ld_op(tA ? A + (long long)k * lda + m : A + (long long)m * lda + k, cA);
       As[kk][mm] = v;
     }
-    for (int e = threadIdx.x; e < BN * BK; e += NT) {
+    for (int e = threadIdx.x; e < T * BK; e += NT) {
       int nn, kk;
-      if (tB) { kk = e % BK; nn = e / BK; } else { nn = e % BN; kk = e / BN; }
+      if (tB) { kk = e % BK; nn = e / BK; } else { nn = e % T; kk = e / T; }
       const int n = n0 + nn, k = k0 + kk;
       cplx v = make_double2(0.0, 0.0);
       if (n < N && k < K) v = ld_op(tB ? B + (long long)n * ldb + k : B + (long long)k * ldb + n, cB);
       Bs[kk][nn] = v;
     }
     __syncthreads();
+    if (K - k0 >= BK) {
 #pragma unroll 4
-    for (int kk = 0; kk < BK; ++kk) {
-      cplx a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + SY * i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx + SX * j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          cr[i][j] = fma(a[i].x, b[j].x, cr[i][j]);
-          cr[i][j] = fma(-a[i].y, b[j].y, cr[i][j]);
-          ci[i][j] = fma(a[i].x, b[j].y, ci[i][j]);
-          ci[i][j] = fma(a[i].y, b[j].x, ci[i][j]);
-        }
+      for (int kk = 0; kk < BK; ++kk) step(kk);
+    } else {  // no FP64 work for the padding of a short last k-tile
+      for (int kk = 0; kk < K - k0; ++kk) step(kk);
     }
     __syncthreads();
   }
   const bool use_beta = (beta.x != 0.0 || beta.y != 0.0);
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int m = m0 + ty + SY * i;
+  for (int i = 0; i < MI; ++i) {
+    const int m = m0 + ty + 16 * i;
     if (m >= M) continue;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int n = n0 + tx + SX * j;
+    for (int j = 0; j < MI; ++j) {
+      const int n = n0 + tx + 16 * j;
       if (n >= N) continue;
       cplx* cp = C + (long long)m * ldc + n;
       double r = alpha.x * cr[i][j] - alpha.y * ci[i][j];
@@ -182,31 +187,34 @@ cudaError_t zgemm(cudaStream_t s, int M, int N, int K, cplx alpha, const cplx* A
                   long long ldc, GemmBatch batch, cplx* work, long long work_elems, int flags) {
   if (M <= 0 || N <= 0 || batch.count <= 0) return cudaSuccess;
   if ((flags & ZG_UPPER_TILES) && M != N) return cudaErrorInvalidValue;
-  // Tile size and K split from a cost model of the FP64 pipe: every SM's FP64
-  // units carry the product; an SM runs at full rate with >= 16 resident warps
-  // and, measured on GB300, at 0.61x with one 8-warp CTA (rate ~ (warps/16)^0.72
-  // below 16).  Cost = k-tiles per CTA x CTAs on the busiest SM x tile work /
-  // rate; splits keep whole k-tiles.
-  const long long kb = (K + BK - 1) / BK;
-  int best_T = 64;
-  long long best_S = 1;
+  // Tile size and K split from a cost model, in microseconds: the busiest
+  // SM's share of the multiply-adds at the FP64 units' rate (a k step of a 64 x
+  // 64 tile takes them 4.5 us; 0.61 of the rate with one CTA on the SM, measured
+  // on GB300, its loads not hidden), a load latency (1 us) for each of its
+  // k-tiles as far as other CTAs do not cover it,
+  // and for a split the second kernel with the partials' round trip.
+  int best_T = 64, best_k = 0;  // best_k: k per split, 0 = unsplit
   double best_cost = -1.0;
-  for (int T : {64, 32}) {
-    if (batch.count != 1 && T != 64) continue;
+  const bool can_split = batch.count == 1 && work && K >= 16;
+  for (int T : {64, 32, 16}) {
+    if (T != 64 && (batch.count != 1 || M > 65535LL * T)) continue;
     const long long tm = (M + T - 1) / T, tn = (N + T - 1) / T;
     const long long tiles = (flags & ZG_UPPER_TILES) ? tm * (tm + 1) / 2 : tm * tn;
-    const double unit = T == 64 ? 1.0 : 0.25;
-    const int warps = T == 64 ? 8 : 2;
-    const bool can_split = batch.count == 1 && work && K >= 2 * BK;
-    for (long long S = 1; S <= (can_split ? 160 : 1) && S <= kb; ++S) {
-      const long long kps = (kb + S - 1) / S, Se = (kb + kps - 1) / kps;
+    const double per_k = 4.5 * (T / 64.0) * (T / 64.0);
+    int last = -1;
+    for (int S = 1; S <= (can_split ? 160 : 1); ++S) {
+      const int kps = S == 1 ? K : ((K + S - 1) / S + 7) / 8 * 8;
+      if (kps < 8 || kps == last) continue;
+      last = kps;
+      const long long Se = (K + kps - 1) / kps;
       if (Se > 1 && Se * M * N > work_elems) break;
       const long long busy = (tiles * Se * batch.count + 151) / 152;
-      const double rate = std::min(1.0, std::pow((double)(busy * warps) / 16.0, 0.72));
-      const double cost = (double)kps * (double)busy * unit / rate + 1e-4 * (double)Se;
+      const double rate = busy == 1 ? 0.61 : 1.0;
+      double cost = (double)kps * (double)busy * per_k / rate + (double)((kps + BK - 1) / BK) / (double)busy;
+      if (Se > 1) cost += 4.0 + (double)Se * (double)M * (double)N * 32.0 / 5e6;
       if (best_cost < 0.0 || cost < best_cost) {
         best_cost = cost;
-        best_S = Se;
+        best_k = Se > 1 ? kps : 0;
         best_T = T;
       }
     }
@@ -214,18 +222,21 @@ cudaError_t zgemm(cudaStream_t s, int M, int N, int K, cplx alpha, const cplx* A
   const int T = best_T;
   const long long tm = (M + T - 1) / T, tn = (N + T - 1) / T;
   auto launch = [&](dim3 grid, cplx al, cplx be, cplx* out, long long ldo, long long sC, int ksplit, int fl) {
+    auto go = [&](auto kern) {
+      kern<<<grid, 256, 0, s>>>(M, N, K, al, A, lda, opA, B, ldb, opB, be, out, ldo, batch.sA, batch.sB, sC, ksplit,
+                                fl);
+    };
     if (T == 64)
-      zgemm_kernel<64, 64><<<grid, 256, 0, s>>>(M, N, K, al, A, lda, opA, B, ldb, opB, be, out, ldo, batch.sA,
-                                                batch.sB, sC, ksplit, fl);
+      go(zgemm_kernel<4>);
+    else if (T == 32)
+      go(zgemm_kernel<2>);
     else
-      zgemm_kernel<32, 32><<<grid, 64, 0, s>>>(M, N, K, al, A, lda, opA, B, ldb, opB, be, out, ldo, batch.sA,
-                                               batch.sB, sC, ksplit, fl);
+      go(zgemm_kernel<1>);
   };
-  if (best_S >= 2) {
-    const long long kps = (kb + best_S - 1) / best_S;
-    const int ksplit = (int)(kps * BK);
-    const long long S = (K + ksplit - 1) / ksplit;
-    launch(dim3((unsigned)tn, (unsigned)tm, (unsigned)S), ONE_C, ZERO_C, work, N, (long long)M * N, ksplit, flags);
+  if (tm > 65535) return cudaErrorInvalidConfiguration;
+  if (best_k > 0) {
+    const long long S = (K + best_k - 1) / best_k;
+    launch(dim3((unsigned)tn, (unsigned)tm, (unsigned)S), ONE_C, ZERO_C, work, N, (long long)M * N, best_k, flags);
     long long blocks = ((long long)M * N + 255) / 256;
     if (blocks > 152 * 16) blocks = 152 * 16;
     splitk_sum_kernel<<<(unsigned)blocks, 256, 0, s>>>(work, (int)S, M, N, alpha, beta, C, ldc, flags, T, T);
