@@ -290,13 +290,27 @@ static bool tc_form(int prec) {
   return prec == IPEPS_PREC_TF32 || prec == IPEPS_PREC_BF16X3 || prec == IPEPS_PREC_BF16X6;
 }
 
+// The range finder's bases by shifted CholeskyQR3 and the SVD of W through its
+// k x k core (all forms but plain FP64 always).  Plain FP64 takes the same
+// route for the truncations it resolves: its Grams see directions down to
+// about 1e-12 of the largest, so a cutoff below 1e-9, an orth_tol that asks
+// for directions to be dropped, or a Jacobi budget beyond the rotation log's
+// keeps one-sided Jacobi on the full rows.  At D = 4, chi = 64 that Jacobi took
+// 14 ms for each of the six k x K bases of a cut (80 rows of 1024) and 75 % of
+// the sweep; a CholeskyQR3 takes about 1 ms (sweep and spectra 1180 -> 522 ms).
+constexpr int CHOL_MAX_SWEEPS = 64;
+static bool chol_route(const ipeps_options& o) {
+  return o.prec != IPEPS_PREC_FP64 ||
+         (o.orth_tol <= 1e-14 && o.svd_cutoff >= 1e-9 && o.jacobi_max_sweeps <= CHOL_MAX_SWEEPS);
+}
+
 // sizes of everything a handle carves from its memory
 struct Sizes {
   long long tens, a, C, T, Q, thin, proj, scratch;
   size_t total;
 };
 
-static Sizes plan_sizes(int Lx, int Ly, int d, int D, int chi, int k, int ntens, int prec) {
+static Sizes plan_sizes(int Lx, int Ly, int d, int D, int chi, int k, int ntens, int prec, int max_sweeps) {
   Sizes s;
   const long long D2 = (long long)D * D, K = chi * D2;
   s.tens = (long long)d * D2 * D2;
@@ -316,6 +330,10 @@ static Sizes plan_sizes(int Lx, int Ly, int d, int D, int chi, int k, int ntens,
   // digit planes of the FP64-accurate products: 28 B per complex element of
   // the A side, 56 B of the B side, and the exact split partials
   if (prec == IPEPS_PREC_FP64TC) s.scratch = s.scratch * 3 + (1 << 22);
+  // plain FP64: per projector lane the rotation log, the factors and the bases
+  // of the SVD of W beside the Grams' split sums
+  if (prec == IPEPS_PREC_FP64 && max_sweeps <= CHOL_MAX_SWEEPS)
+    s.scratch += 2 * (jacobi_log_elems(k, max_sweeps) + 10LL * k * k + 3 * s.thin);
   size_t tot = 0;
   auto add = [&](long long n, size_t el) { tot += align_up((size_t)n * el); };
   for (int i = 0; i < 2 * 4 * ntens; ++i) add(s.tens, 16);
@@ -824,7 +842,8 @@ extern "C" ipeps_status ipeps_ctm_workspace_size(const ipeps_cell* c, const ipep
                                                  size_t* bytes) {
   CKS(validate(c, o));
   if (!bytes) return fail(IPEPS_EINVAL, "null bytes");
-  Sizes s = plan_sizes(c->Lx, c->Ly, c->d, c->D, o->chi, o->chi + o->rsvd_oversample, c->n_tensors, o->prec);
+  Sizes s = plan_sizes(c->Lx, c->Ly, c->d, c->D, o->chi, o->chi + o->rsvd_oversample, c->n_tensors, o->prec,
+                       o->jacobi_max_sweeps);
   *bytes = s.total;
   return IPEPS_OK;
 }
@@ -937,7 +956,7 @@ extern "C" ipeps_status ipeps_ctm_create(const ipeps_cell* c, const ipeps_option
   if (!(h->opt.svd_cutoff > 0.0))  // automatic: above the noise floor of the contraction arithmetic
     h->opt.svd_cutoff = !tc_form(o->prec) ? 1e-8 : (o->prec == IPEPS_PREC_TF32 ? 1e-5 : 1e-6);
   h->stream = (cudaStream_t)o->stream;
-  Sizes sz = plan_sizes(h->Lx, h->Ly, h->d, h->D, h->chi, h->k, h->ntens, o->prec);
+  Sizes sz = plan_sizes(h->Lx, h->Ly, h->d, h->D, h->chi, h->k, h->ntens, o->prec, o->jacobi_max_sweeps);
   if (o->workspace) {
     if (o->workspace_bytes < sz.total) {
       delete h;
@@ -1320,19 +1339,24 @@ static ipeps_status orth(ipeps_ctm h, cplx* G) {
   return IPEPS_OK;
 }
 
-// FP64 GEMM of the precision form's projector step (CholeskyQR Grams and
-// applies, the core products): FP64-accurate products on the tensor cores
-// (exact digit splitting, ozaki.cu), bracketed as profiling class 2 with
-// their algorithmic flops (structure-aware: a Hermitian Gram counts its upper
-// triangle, a triangular factor its nonzero part; the digit products compute
-// the full rectangle, so `flags` only states the structure).
+// FP64 GEMM of the projector step (CholeskyQR Grams and applies, the core
+// products): FP64-accurate products on the tensor cores (exact digit
+// splitting, ozaki.cu; in plain FP64 the CUDA cores), bracketed as profiling
+// class 2 with their algorithmic flops (structure-aware: a Hermitian Gram
+// counts its upper triangle, a triangular factor its nonzero part; the digit
+// products compute the full rectangle, so there `flags` only states the
+// structure).
 static cudaError_t proj_zgemm(ipeps_ctm h, double flops, int M, int N, int K, const cplx* A, long long lda,
                               int opA, const cplx* B, long long ldb, int opB, cplx* C, long long ldc, int flags) {
-  (void)flags;
   cudaEvent_t ev = nullptr;
   prof_begin(h, &ev);
-  cudaError_t e = oz_zgemm(h->stream, M, N, K, A, lda, opA, B, ldb, opB, C, ldc, h->scratch + h->scratch_top,
-                           (size_t)(h->scratch_elems - h->scratch_top) * sizeof(cplx), &h->st->tc_timeouts);
+  cudaError_t e;
+  if (h->opt.prec == IPEPS_PREC_FP64)
+    e = zgemm(h->stream, M, N, K, ONE, A, lda, opA, B, ldb, opB, ZERO, C, ldc, GemmBatch{1, 0, 0, 0},
+              h->scratch + h->scratch_top, h->scratch_elems - h->scratch_top, flags);
+  else
+    e = oz_zgemm(h->stream, M, N, K, A, lda, opA, B, ldb, opB, C, ldc, h->scratch + h->scratch_top,
+                 (size_t)(h->scratch_elems - h->scratch_top) * sizeof(cplx), &h->st->tc_timeouts);
   prof_end(h, ev, flops, 2);
   return e;
 }
@@ -1367,8 +1391,8 @@ static ipeps_status cholqr_pass(ipeps_ctm h, const cplx* in, cplx* out, cplx* Ro
 // Precision form orthonormalisation: CholeskyQR2 (directions below ~1e-7 of
 // the largest singular value dropped in the first pass).
 static ipeps_status orth_chol(ipeps_ctm h, cplx* Y, cplx* tmp, bool twice) {
-  if (h->opt.prec == IPEPS_PREC_FP64TC) {
-    // FP64-accurate form: no direction of the basis is dropped for being
+  if (!tc_form(h->opt.prec)) {
+    // FP64 and the FP64-accurate form: no direction of the basis is dropped for being
     // small.  Shifted CholeskyQR (the shift keeps the Cholesky defined at any
     // condition number; the result spans the same space with condition below
     // about 1e5) and then one CholeskyQR pass (intermediate bases of the
@@ -1415,9 +1439,10 @@ static ipeps_status svd_rows_chol(ipeps_ctm h, const cplx* Wt, cplx* out, cplx* 
   cplx* R2 = scratch_alloc(h, (long long)k * k);
   cplx* Rt = scratch_alloc(h, (long long)k * k);
   if (!R1 || !R2 || !Rt) return fail(IPEPS_ENOMEM, "scratch exhausted (svd chol)");
-  const bool fp64tc = h->opt.prec == IPEPS_PREC_FP64TC;
+  const bool exact = !tc_form(h->opt.prec);          // FP64 and FP64TC
+  const bool warm = h->opt.prec != IPEPS_PREC_FP64;  // plain FP64 keeps nothing from visit to visit
   cplx* Q3 = nullptr;
-  if (fp64tc) {
+  if (exact) {
     // shifted CholeskyQR3: W = Q3 R3 R2 R1 (no direction dropped for being small)
     cplx* R3 = scratch_alloc(h, (long long)k * k);
     cplx* Q2 = scratch_alloc(h, (long long)k * K);
@@ -1437,7 +1462,10 @@ static ipeps_status svd_rows_chol(ipeps_ctm h, const cplx* Wt, cplx* out, cplx* 
     CK(proj_zgemm(h, 8.0 * k * (k + 1.0) * (k + 2.0) / 6.0, k, k, k, R1, k, OP_T, R2, k, OP_T, Rt, k, ZG_A_LOWER));
   }
   // R1 = V_prev^T Rt: rows are the columns of R V_prev
-  CK(proj_zgemm(h, 8.0 * k * (double)k * k, k, k, k, Vt, k, OP_N, Rt, k, OP_N, R1, k, 0));
+  if (warm)
+    CK(proj_zgemm(h, 8.0 * k * (double)k * k, k, k, k, Vt, k, OP_N, Rt, k, OP_N, R1, k, 0));
+  else
+    R1 = Rt;
   {
     cudaEvent_t a = nullptr;
     prof_begin(h, &a);
@@ -1445,10 +1473,10 @@ static ipeps_status svd_rows_chol(ipeps_ctm h, const cplx* Wt, cplx* out, cplx* 
     cplx* rotlog = scratch_alloc(h, nlog);
     if (!rotlog) return fail(IPEPS_ENOMEM, "scratch exhausted (rotation log)");
     CK(jacobi_rows(h->stream, R1, k, k, k, Vt, h->sigma, h->opt.jacobi_max_sweeps, h->dwork, h->counters,
-                   h->st, rotlog, nlog, h->opt.wait_cycles, true, !fp64tc));
+                   h->st, rotlog, nlog, h->opt.wait_cycles, warm, !exact));
     prof_end(h, a, 0.0, 1);
   }
-  if (fp64tc) {
+  if (exact) {
     // out = R1 Q3^T: rows (Q3 R v_i)^T = s_i (Q3 u_R,i)^T.  The left singular
     // vectors of W as the orthonormal basis Q3 times those of the core, rather
     // than W v_i / s_i, whose division by a small s_i magnifies the rounding
@@ -1467,14 +1495,13 @@ static ipeps_status svd_rows_chol(ipeps_ctm h, const cplx* Wt, cplx* out, cplx* 
 static ipeps_status projectors(ipeps_ctm h, int f, int x, int y, cplx* PT, cplx* Ptil) {
   CKS(enlarged_corners(h, f, x, y));
   const int k = h->k, K = h->K, chi = h->chi;
-  // the FP64 path orthonormalises by Jacobi; the other forms by CholeskyQR on
-  // FP64-accurate Grams (FP64TC: its products unpacked, on the digit planes)
-  const bool fp64 = h->opt.prec == IPEPS_PREC_FP64;
+  // CholeskyQR on FP64-accurate Grams, or Jacobi on the full rows (chol_route)
+  const bool jacobi_bases = !chol_route(h->opt);
   if (packed_path(h)) CKS(pack_corners(h));
   cplx* Qt = h->thin[0];
   cplx* Zt = h->thin[1];
   auto orth_any = [&](cplx* Y, bool last) -> ipeps_status {
-    return fp64 ? orth(h, Y) : orth_chol(h, Y, h->thin[2], last);
+    return jacobi_bases ? orth(h, Y) : orth_chol(h, Y, h->thin[2], last);
   };
   const int q = h->opt.rsvd_power;
   CKS(apply_XT(h, h->omt, Qt, k));
@@ -1489,7 +1516,7 @@ static ipeps_status projectors(ipeps_ctm h, int f, int x, int y, cplx* PT, cplx*
   CKS(apply_XHT(h, Qt, Zt, k));
   cplx* Wrot;  // rows sigma_i u_i^T
   cplx* Vt = h->Vt;  // rows = columns of V
-  if (fp64) {
+  if (jacobi_bases) {
     cudaEvent_t a = nullptr;
     prof_begin(h, &a);
     CK(jacobi_rows(h->stream, Zt, k, K, K, h->Vt, h->sigma, h->opt.jacobi_max_sweeps, h->dwork,
@@ -1499,7 +1526,7 @@ static ipeps_status projectors(ipeps_ctm h, int f, int x, int y, cplx* PT, cplx*
   } else {
     int lx, ly;
     frame_dims(h, f, &lx, &ly);
-    Vt = h->Vwarm[f][y * lx + x];
+    if (h->opt.prec != IPEPS_PREC_FP64) Vt = h->Vwarm[f][y * lx + x];
     CKS(svd_rows_chol(h, Zt, h->thin[2], Vt));
     Wrot = h->thin[2];
   }
