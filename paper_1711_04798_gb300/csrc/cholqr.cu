@@ -65,13 +65,14 @@ __global__ void __launch_bounds__(1024) chol_drop_kernel(const cplx* __restrict_
   }
 }
 
-// Rinv = inverse of the upper-triangular R on its kept block (zero rows and
-// columns where R[i,i] == 0).  One warp per column c: back substitution
-// R x = e_c, x_i for i = c .. 0, with x held in the warp's slice of shared
-// memory (each step reads the entries the previous steps wrote) and written
-// to Rinv at the end.
+// Linv = R^{-H}, R^{-1} the inverse of the upper-triangular R on its kept block
+// (zero rows and columns where R[i,i] == 0).  One warp per column c of R^{-1}:
+// back substitution R x = e_c, x_i for i = c .. 0, with x held in the warp's
+// slice of shared memory (each step reads the entries the previous steps
+// wrote) and written, conjugated, as row c of Linv at the end.  For the sizes
+// beside the cluster Cholesky, which forms Linv itself.
 constexpr int TRI_WARPS = 4;
-__global__ void tri_inv_kernel(const cplx* __restrict__ R, cplx* __restrict__ Rinv, int n) {
+__global__ void tri_inv_kernel(const cplx* __restrict__ R, cplx* __restrict__ Linv, int n) {
   extern __shared__ cplx xs_all[];  // [TRI_WARPS][n] solution columns, then [n] reciprocal diagonal
   double* rinv = (double*)(xs_all + (long long)TRI_WARPS * n);
   const int w = threadIdx.x >> 5;
@@ -105,7 +106,7 @@ __global__ void tri_inv_kernel(const cplx* __restrict__ R, cplx* __restrict__ Ri
       __syncwarp();
     }
   }
-  for (int i = lane; i < n; i += 32) Rinv[(long long)i * n + c] = xs[i];
+  for (int i = lane; i < n; i += 32) Linv[(long long)c * n + i] = make_double2(xs[i].x, neg_bits(xs[i].y));
 }
 
 // G += coef * tr(G) I (one CTA): the shift of shifted CholeskyQR (Fukaya,
@@ -133,16 +134,7 @@ cudaError_t gram_shift(cudaStream_t s, cplx* G, int n, double coef) {
   return cudaGetLastError();
 }
 
-cudaError_t chol_drop(cudaStream_t s, const cplx* G, cplx* work, cplx* R, int n, double tol) {
-  cudaError_t e;
-  if ((e = kernels_init()) != cudaSuccess) return e;
-  if (chol_cluster_fits(n)) return chol_cluster(s, G, R, n, tol);
-  chol_drop_kernel<<<1, 1024, 0, s>>>(G, work, R, n, tol);
-  count_launch();
-  return cudaGetLastError();
-}
-
-cudaError_t tri_inv(cudaStream_t s, const cplx* R, cplx* Rinv, int n) {
+static cudaError_t tri_inv(cudaStream_t s, const cplx* R, cplx* Linv, int n) {
   const size_t smem = (size_t)TRI_WARPS * n * sizeof(cplx) + (size_t)n * sizeof(double);
   if (smem > 200 * 1024) return cudaErrorInvalidValue;  // n above about 3000
   static size_t attr = 48 * 1024;
@@ -151,7 +143,17 @@ cudaError_t tri_inv(cudaStream_t s, const cplx* R, cplx* Rinv, int n) {
     if (e != cudaSuccess) return e;
     attr = 200 * 1024;
   }
-  tri_inv_kernel<<<(n + TRI_WARPS - 1) / TRI_WARPS, TRI_WARPS * 32, smem, s>>>(R, Rinv, n);
+  tri_inv_kernel<<<(n + TRI_WARPS - 1) / TRI_WARPS, TRI_WARPS * 32, smem, s>>>(R, Linv, n);
   count_launch();
   return cudaGetLastError();
+}
+
+cudaError_t chol_drop(cudaStream_t s, const cplx* G, cplx* work, cplx* R, cplx* Linv, int n, double tol) {
+  cudaError_t e;
+  if ((e = kernels_init()) != cudaSuccess) return e;
+  if (chol_cluster_fits(n)) return chol_cluster(s, G, R, Linv, n, tol);
+  chol_drop_kernel<<<1, 1024, 0, s>>>(G, work, R, n, tol);
+  count_launch();
+  if ((e = cudaGetLastError()) != cudaSuccess || !Linv) return e;
+  return tri_inv(s, R, Linv, n);
 }

@@ -136,6 +136,17 @@ __device__ __forceinline__ double rsqrt64(double a) {
   return __longlong_as_double(__double_as_longlong(r) - ((long long)half << 52));
 }
 
+// 1/a of a normal a > 0 the same way: an FP32 reciprocal, one step of third order
+__device__ __forceinline__ double rcp64(double a) {
+  const long long b = __double_as_longlong(a);
+  const int ex = (int)(b >> 52) - 1023;
+  const double m = __longlong_as_double(b - ((long long)ex << 52));  // [1, 2)
+  const double x = f2d_bits(__frcp_rn(d2f_bits(m)));
+  const double e = fma(-m, x, 1.0);
+  const double r = fma(x, fma(e, e, e), x);
+  return __longlong_as_double(__double_as_longlong(r) - ((long long)ex << 52));
+}
+
 // the sums of a and b over the warp, in every lane: after the first butterfly
 // level each half of the warp carries one of them
 __device__ __forceinline__ void warp_sum2(double& a, double& b) {
@@ -723,31 +734,43 @@ __global__ void jacobi_replay_kernel(cplx* __restrict__ Vt, int n, const double4
   for (int a = threadIdx.x; a < na; a += blockDim.x) Vt[(long long)amap[1 + a] * n + q] = col[a];
 }
 
-// Right-looking Cholesky of the Hermitian n x n G (upper triangle used) with
-// dropped pivots (d <= tol * max diagonal: row of R zero), blocked by CH_NB
-// rows.  Rows of the working copy W live in the cluster's shared memory (row
-// i in CTA i mod csize).  For the block of rows j0 .. j0+nb-1 each CTA
-// factors the nb x nb diagonal block (every CTA the same arithmetic, so the
-// same pivots) and, for the columns l >= j0+nb it owns (l mod csize = rank),
-// the block's entries of R; after a cluster barrier every CTA gathers the
-// block's rows of R and updates its own rows below the block, W[i,l] -=
-// conj(R[j,i]) R[j,l] for l >= i, j in order.  The operations and their order
-// per element are those of the column-by-column algorithm.
+// Right-looking Cholesky G = R^H R of the Hermitian n x n G (upper triangle
+// used) with dropped pivots (d <= tol * max diagonal: row of R zero), carried
+// out on the augmented rows [G | I], which leaves L^{-1} = R^{-H} beside R (zero
+// rows and columns for dropped pivots): row j of the working matrix holds the
+// Schur complement right of its diagonal and its row of L^{-1} left of it, so
+// the augmented part costs no storage and no further steps (a back
+// substitution of its own took 35 us, with no pivot dropped 196 us at n = 116,
+// a serial chain of n warp reductions per column).
+//
+// Blocked by CH_NB rows.  Rows of the working copy W live in the cluster's
+// shared memory (row i in CTA i mod csize).  For the block of rows j0 ..
+// j0+nb-1 each CTA factors the nb x nb diagonal block (every CTA the same
+// arithmetic, so the same pivots) and the block's entries in the other
+// columns it owns (l mod csize = rank), one barrier of four warps per row; after
+// a cluster barrier every CTA gathers the block's rows and updates its own
+// rows below the block.  Bound: the serial chain of pivots (each an FP64
+// reciprocal root and a rank-one update, some 0.4 us) and the trailing update
+// on the FP64 units of the cluster's SMs.
 constexpr int CH_NB = 8;
+constexpr int CH_PANEL = 128;  // threads of the panel's barrier
 
 __global__ void __launch_bounds__(CL_THREADS)
-    chol_cluster_kernel(const cplx* __restrict__ G, cplx* __restrict__ Rout, int n, double tol) {
+    chol_cluster_kernel(const cplx* __restrict__ G, cplx* __restrict__ Rout, cplx* __restrict__ Lout, int n,
+                        double tol) {
   cg::cluster_group cl = cg::this_cluster();
   const int rank = (int)cl.block_rank(), cs = (int)cl.num_blocks();
   const int R = (n + cs - 1) / cs;
-  extern __shared__ cplx sm[];  // [R x n] own rows of W, then [CH_NB x n] the block's rows of W, then of R
+  extern __shared__ cplx sm[];  // [R x n] own rows of W, then [CH_NB x n] the block's rows of W, then of [L^{-1} R]
   cplx* pan = sm + (long long)R * n;
   cplx* rpan = pan + (long long)CH_NB * n;
   __shared__ double s_max, s_rjj[CH_NB], s_inv[CH_NB];
+  __shared__ unsigned s_kept;  // pivots of the block that were not dropped
   for (int l = 0; l < R; ++l) {
     const int i = l * cs + rank;
     if (i >= n) break;
-    for (int t = threadIdx.x; t < n; t += CL_THREADS) sm[(long long)l * n + t] = G[(long long)i * n + t];
+    for (int t = threadIdx.x; t < n; t += CL_THREADS)
+      sm[(long long)l * n + t] = t >= i ? G[(long long)i * n + t] : make_double2(0.0, 0.0);
   }
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -763,91 +786,109 @@ __global__ void __launch_bounds__(CL_THREADS)
   double dmax = 0.0;
   for (int r = 0; r < cs; ++r) dmax = fmax(dmax, *cl.map_shared_rank(&s_max, r));
   const double thr = tol * dmax;
-  // columns of the block this CTA works on: the diagonal block (c < nb), then
-  // its own columns l >= j0 + nb (c >= nb: l = j0 + nb + (c - nb) * cs + off)
   for (int j0 = 0; j0 < n; j0 += CH_NB) {
     const int nb = min(CH_NB, n - j0), jn = j0 + nb;
+    // columns this CTA works on: the diagonal block (c < nb), then its own
+    // columns outside it, left ones first
+    const int nleft = j0 > rank ? (j0 - 1 - rank) / cs + 1 : 0;
     const int off = ((rank - jn) % cs + cs) % cs;  // first own column at or after jn is jn + off
-    const int nown = jn + off < n ? (n - 1 - (jn + off)) / cs + 1 : 0;
-    const int ncol = nb + nown;
-    auto col = [&](int c) { return c < nb ? j0 + c : jn + off + (c - nb) * cs; };
+    const int nright = jn + off < n ? (n - 1 - (jn + off)) / cs + 1 : 0;
+    const int ncol = nb + nleft + nright;
+    auto col = [&](int c) {
+      c -= nb;
+      return c < 0 ? jn + c : (c < nleft ? rank + c * cs : jn + off + (c - nleft) * cs);
+    };
     // the block's rows of W on those columns, from their owners
     for (int e = threadIdx.x; e < nb * ncol; e += CL_THREADS) {
       const int jj = e / ncol, l = col(e % ncol), j = j0 + jj;
       pan[(long long)jj * n + l] = cl.map_shared_rank(sm, j % cs)[(long long)(j / cs) * n + l];
     }
     __syncthreads();
-    for (int jj = 0; jj < nb; ++jj) {
-      const int j = j0 + jj;
-      cplx* pj = pan + (long long)jj * n;
-      // the pivot's reciprocal root once, r = d / sqrt(d) from it (FP64
-      // roots and divides are slow on this part, a lone thread's the more)
-      if (threadIdx.x == 0) {
+    if (threadIdx.x < CH_PANEL) {
+      // rows i > j of the block on every column: W[i,l] -= conj(W[j,i]) W[j,l] / d,
+      // for l >= i (the Schur complement) and l <= j (L^{-1}, whose column j
+      // starts here from 0 with a one in W[j,j]'s place).  Every thread forms 1/d
+      // itself: four FP64 instructions against a second barrier.
+      for (int jj = 0; jj < nb - 1; ++jj) {
+        const int j = j0 + jj;
+        const cplx* pj = pan + (long long)jj * n;
         const double d = pj[j].x;
-        const bool keep = d > thr;
-        const double inv = keep ? rsqrt(d) : 0.0;
-        s_inv[jj] = inv;
-        s_rjj[jj] = keep ? d * inv : 0.0;
-      }
-      __syncthreads();
-      const double rjj = s_rjj[jj], inv = s_inv[jj];
-      const bool keep = rjj > 0.0;
-      // row j of R on the CTA's columns into its own buffer (zero left of the
-      // diagonal, and for a dropped direction), and in the same phase the
-      // block's rows i > j: W[i,l] -= conj(R[j,i]) R[j,l] for l >= i, with
-      // R[j,.] = W[j,.] / r formed from row j of W, which this phase only reads
-      for (int c = threadIdx.x; c < ncol; c += CL_THREADS) {
-        const int l = col(c);
-        cplx v = make_double2(0.0, 0.0);
-        if (keep && l >= j) {
-          const cplx g = pj[l];
-          v = l == j ? make_double2(rjj, 0.0) : make_double2(g.x * inv, g.y * inv);
+        if (d > thr) {  // the same in every thread; a dropped direction updates nothing
+          const double inv = rcp64(d);
+          for (int e = threadIdx.x; e < (nb - 1 - jj) * ncol; e += CH_PANEL) {
+            const int i = j + 1 + e / ncol, l = col(e % ncol);
+            if (l > j && l < i) continue;
+            cplx* w = pan + (long long)(i - j0) * n + l;
+            const bool diag = l == j;
+            const cplx g = pj[i], h = diag ? make_double2(1.0, 0.0) : pj[l];
+            const cplx v = diag ? make_double2(0.0, 0.0) : *w;
+            const double ax = g.x * inv, ay = g.y * inv;
+            *w = make_double2(fma(-ax, h.x, fma(-ay, h.y, v.x)), fma(-ax, h.y, fma(ay, h.x, v.y)));
+          }
         }
+        asm volatile("bar.sync 1, %0;" ::"n"(CH_PANEL) : "memory");
+      }
+      if (threadIdx.x < nb) {  // r = d / sqrt(d) and 1/r, zero for a dropped direction
+        const double d = pan[(long long)threadIdx.x * n + j0 + threadIdx.x].x;
+        const bool keep = d > thr;
+        const double inv = keep ? rsqrt64(d) : 0.0;
+        s_inv[threadIdx.x] = inv;
+        s_rjj[threadIdx.x] = keep ? d * inv : 0.0;
+        const unsigned mask = __ballot_sync((1u << nb) - 1u, keep);
+        if (threadIdx.x == 0) s_kept = mask;
+      }
+      asm volatile("bar.sync 1, %0;" ::"n"(CH_PANEL) : "memory");
+      // the block's rows scaled: R right of the diagonal, L^{-1} left of it and on it
+      for (int e = threadIdx.x; e < nb * ncol; e += CH_PANEL) {
+        const int jj = e / ncol, l = col(e % ncol);
+        const double inv = s_inv[jj];
+        const cplx g = pan[(long long)jj * n + l];
+        cplx v = make_double2(g.x * inv, g.y * inv);
+        if (l == j0 + jj) v = make_double2(inv, 0.0);
+        if (!(s_kept >> jj & 1u)) v = make_double2(0.0, 0.0);
         rpan[(long long)jj * n + l] = v;
       }
-      if (keep) {
-        for (int e = threadIdx.x; e < (nb - 1 - jj) * ncol; e += CL_THREADS) {
-          const int i = j + 1 + e / ncol, l = col(e % ncol);
-          if (l < i) continue;
-          const cplx a = make_double2(pj[i].x * inv, pj[i].y * inv), b = make_double2(pj[l].x * inv, pj[l].y * inv);
-          cplx* wi = pan + (long long)(i - j0) * n;
-          wi[l].x -= a.x * b.x + a.y * b.y;
-          wi[l].y -= a.x * b.y - a.y * b.x;
-        }
-      }
-      __syncthreads();
     }
-    cl.sync();  // every CTA's columns of the block's rows of R are final
+    cl.sync();  // every CTA's columns of the block's rows are final
     // the other CTAs' columns of those rows
-    for (int e = threadIdx.x; e < nb * (n - jn); e += CL_THREADS) {
-      const int jj = e / (n - jn), l = jn + e % (n - jn);
+    for (int e = threadIdx.x; e < nb * (n - nb); e += CL_THREADS) {
+      const int jj = e / (n - nb), q = e % (n - nb), l = q < j0 ? q : q + nb;
       const int o = l % cs;
       if (o != rank) rpan[(long long)jj * n + l] = cl.map_shared_rank(rpan, o)[(long long)jj * n + l];
     }
     __syncthreads();
-    // the owners store their rows of R
+    // the owners store their rows of R and L^{-1}
     for (int jj = 0; jj < nb; ++jj) {
       const int j = j0 + jj;
       if (j % cs != rank) continue;
-      for (int l = threadIdx.x; l < n; l += CL_THREADS)
-        Rout[(long long)j * n + l] = l < j0 ? make_double2(0.0, 0.0) : rpan[(long long)jj * n + l];
-    }
-    // own rows below the block
-    for (int l0 = 0; l0 < R; ++l0) {
-      const int i = l0 * cs + rank;
-      if (i >= n) break;
-      if (i < jn) continue;
-      cplx* wi = sm + (long long)l0 * n;
-      for (int l = i + threadIdx.x; l < n; l += CL_THREADS) {
-        cplx v = wi[l];
-        for (int jj = 0; jj < nb; ++jj) {
-          if (s_rjj[jj] == 0.0) continue;  // dropped direction: no update
-          const cplx a = rpan[(long long)jj * n + i], b = rpan[(long long)jj * n + l];
-          v.x -= a.x * b.x + a.y * b.y;
-          v.y -= a.x * b.y - a.y * b.x;
-        }
-        wi[l] = v;
+      for (int l = threadIdx.x; l < n; l += CL_THREADS) {
+        const cplx v = rpan[(long long)jj * n + l], z = make_double2(0.0, 0.0);
+        if (Rout) Rout[(long long)j * n + l] = l < j ? z : (l == j ? make_double2(s_rjj[jj], 0.0) : v);
+        if (Lout) Lout[(long long)j * n + l] = l > j ? z : v;
       }
+    }
+    // own rows below the block, on the columns l < jn (L^{-1}: the block's own
+    // columns start here, from the rows at and below them) and l >= i: the
+    // (row, column) pairs of all own rows spread over the threads
+    const unsigned kept = s_kept;
+    const int l0 = jn > rank ? (jn - rank + cs - 1) / cs : 0;  // first own row at or after jn
+    const int span = Lout ? n : n - jn;
+    const int todo = (R - l0) * span;
+    for (int e = threadIdx.x; e < todo; e += CL_THREADS) {
+      const int lr = l0 + e / span, i = lr * cs + rank, c = e % span, l = Lout ? c : jn + c;
+      if (i >= n || (l >= jn && l < i)) continue;
+      cplx* w = sm + (long long)lr * n + l;
+      const bool fresh = l >= j0 && l < jn;
+      cplx v = fresh ? make_double2(0.0, 0.0) : *w;
+      const unsigned use = fresh ? kept & ~((1u << (l - j0)) - 1u) : kept;
+#pragma unroll
+      for (int jj = 0; jj < CH_NB; ++jj) {
+        if (!(use >> jj & 1u)) continue;
+        const cplx a = rpan[(long long)jj * n + i], b = rpan[(long long)jj * n + l];
+        v.x = fma(-a.x, b.x, fma(-a.y, b.y, v.x));
+        v.y = fma(-a.x, b.y, fma(a.y, b.x, v.y));
+      }
+      *w = v;
     }
     cl.sync();  // rows updated before they are read as the next block; gathers done before rpan is rewritten
   }
@@ -1002,12 +1043,12 @@ bool chol_cluster_fits(int n) {
   return (R + 2 * CH_NB) * n * (long long)sizeof(cplx) <= CL_SMEM;
 }
 
-cudaError_t chol_cluster(cudaStream_t s, const cplx* G, cplx* R, int n, double tol) {
+cudaError_t chol_cluster(cudaStream_t s, const cplx* G, cplx* R, cplx* Linv, int n, double tol) {
   cudaError_t e;
   if ((e = cluster_init()) != cudaSuccess) return e;
   const long long rows = (n + g_csize - 1) / g_csize;
   const size_t smem = (size_t)((rows + 2 * CH_NB) * n * sizeof(cplx));
-  void* args[] = {&G, &R, &n, &tol};
+  void* args[] = {&G, &R, &Linv, &n, &tol};
   e = launch_cluster((const void*)chol_cluster_kernel, args, smem, s);
   count_launch();
   return e;

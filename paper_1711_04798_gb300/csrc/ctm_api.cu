@@ -1372,18 +1372,15 @@ static ipeps_status cholqr_pass(ipeps_ctm h, const cplx* in, cplx* out, cplx* Ro
   cplx* G = scratch_alloc(h, (long long)k * k);
   cplx* W = scratch_alloc(h, (long long)k * k);
   cplx* R = Rout ? Rout : scratch_alloc(h, (long long)k * k);
-  cplx* Ri = scratch_alloc(h, (long long)k * k);
-  if (!G || !W || !R || !Ri) return fail(IPEPS_ENOMEM, "scratch exhausted (cholqr)");
+  cplx* Li = scratch_alloc(h, (long long)k * k);
+  if (!G || !W || !R || !Li) return fail(IPEPS_ENOMEM, "scratch exhausted (cholqr)");
   // Hermitian Gram: the Cholesky reads its upper triangle only
   CK(proj_zgemm(h, 8.0 * K * (0.5 * k * (k + 1)), k, k, K, in, K, OP_C, in, K, OP_T, G, k, ZG_UPPER_TILES));
   // shifted CholeskyQR: s = 11 (m n + n (n + 1)) u ||Y||^2 with u = 2^-53
   if (shifted) CK(gram_shift(h->stream, G, k, 11.0 * ((double)K * k + (double)k * (k + 1)) * 0x1p-53));
-  CK(chol_drop(h->stream, G, W, R, k, tol));
-  if (apply) {
-    CK(tri_inv(h->stream, R, Ri, k));
-    // Q = Y R^{-1}  ->  Q^T = R^{-T} Y^T
-    CK(proj_zgemm(h, 8.0 * K * (0.5 * k * (k + 1)), k, K, k, Ri, k, OP_T, in, K, OP_N, out, K, ZG_A_LOWER));
-  }
+  CK(chol_drop(h->stream, G, W, R, apply ? Li : nullptr, k, tol));
+  // Q = Y R^{-1}  ->  Q^T = R^{-T} Y^T = conj(R^{-H}) Y^T
+  if (apply) CK(proj_zgemm(h, 8.0 * K * (0.5 * k * (k + 1)), k, K, k, Li, k, OP_C, in, K, OP_N, out, K, ZG_A_LOWER));
   h->scratch_top = mark;
   return IPEPS_OK;
 }

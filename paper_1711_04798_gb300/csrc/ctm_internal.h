@@ -157,11 +157,12 @@ cudaError_t trace_product(cudaStream_t s, const cplx* rho, const cplx* H, int n,
                           int idx, double w);
 cudaError_t trace_normalize(cudaStream_t s, cplx* rho, int n, double* work);
 
-// Cholesky with dropped pivots (d <= tol * max diagonal) of the Hermitian n x n G:
-// R upper triangular (dropped rows zero); work: n*n scratch.  One CTA.
-cudaError_t chol_drop(cudaStream_t s, const cplx* G, cplx* work, cplx* R, int n, double tol);
-// inverse of upper-triangular R on its kept block (zero where R[i,i] == 0)
-cudaError_t tri_inv(cudaStream_t s, const cplx* R, cplx* Rinv, int n);
+// Cholesky with dropped pivots (d <= tol * max diagonal) of the Hermitian n x n G
+// = R^H R: R upper triangular (dropped rows zero) and Linv = R^{-H} on the kept
+// block (lower triangular, zero rows and columns where a pivot was dropped);
+// Linv may be null, and R too where Linv is given and chol_cluster_fits(n).
+// work: n*n scratch.
+cudaError_t chol_drop(cudaStream_t s, const cplx* G, cplx* work, cplx* R, cplx* Linv, int n, double tol);
 // G += coef * tr(G) * I for the Hermitian n x n Gram G (device): the diagonal
 // shift of shifted CholeskyQR
 cudaError_t gram_shift(cudaStream_t s, cplx* G, int n, double coef);
@@ -211,7 +212,7 @@ cudaError_t jacobi_cluster_batch(cudaStream_t s, cplx* G, int n, int m, long lon
                                  int max_sweeps, DevStatus* st);
 long long jacobi_log_elems(int n, int max_sweeps);
 bool chol_cluster_fits(int n);
-cudaError_t chol_cluster(cudaStream_t s, const cplx* G, cplx* R, int n, double tol);
+cudaError_t chol_cluster(cudaStream_t s, const cplx* G, cplx* R, cplx* Linv, int n, double tol);
 
 // launch accounting (host counter incremented by every launcher)
 void count_launch(int n = 1);
