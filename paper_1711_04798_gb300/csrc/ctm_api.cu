@@ -118,7 +118,7 @@ struct ipeps_ctm_s {
   cplx* spareC[2][2]; // replacement buffers for renormalised C1 / C4, per row
   cplx* spareT[2];    // replacement T4 per row
   cplx* Q[4];
-  TcPacked Qp[4][2];  // precision form: corners packed once per cut, [op N, op T]
+  TcPacked Qp[4][2];  // precision form: corners packed once per cut, [as is, transposed]
   void* Qpmem[4][2];
   cplx* omt;
   cplx* thin[4];      // k x K work
@@ -343,7 +343,7 @@ static Sizes plan_sizes(int Lx, int Ly, int d, int D, int chi, int k, int ntens,
   for (int i = 0; i < 2; ++i) add(s.T, 16);
   for (int i = 0; i < 4; ++i) add(s.Q, 16);
   if (tc_form(prec))
-    for (int i = 0; i < 8; ++i) tot += align_up(tc_packed_bytes(prec, (int)K, (int)K));
+    for (int i = 0; i < 8; ++i) tot += align_up(tc_packed_bytes(prec, (int)K));
   add(s.thin, 16);
   for (int i = 0; i < 4; ++i) add(s.thin, 16);
   for (int i = 0; i < 4; ++i) add(s.proj, 16);
@@ -362,7 +362,7 @@ static Sizes plan_sizes(int Lx, int Ly, int d, int D, int chi, int k, int ntens,
   // second projector lane (the other cut of a column runs concurrently)
   for (int i = 0; i < 4; ++i) add(s.Q, 16);
   if (tc_form(prec))
-    for (int i = 0; i < 8; ++i) tot += align_up(tc_packed_bytes(prec, (int)K, (int)K));
+    for (int i = 0; i < 8; ++i) tot += align_up(tc_packed_bytes(prec, (int)K));
   for (int i = 0; i < 4; ++i) add(s.thin, 16);
   add((long long)k * k, 16);
   add((long long)chi * k, 16);
@@ -996,7 +996,7 @@ extern "C" ipeps_status ipeps_ctm_create(const ipeps_cell* c, const ipeps_option
   for (int i = 0; i < 4; ++i) need(h->Q[i] = carve<cplx>(h, sz.Q));
   if (tc_form(o->prec))
     for (int i = 0; i < 4; ++i)
-      for (int v = 0; v < 2; ++v) need(h->Qpmem[i][v] = carve<char>(h, tc_packed_bytes(o->prec, h->K, h->K)));
+      for (int v = 0; v < 2; ++v) need(h->Qpmem[i][v] = carve<char>(h, tc_packed_bytes(o->prec, h->K)));
   need(h->omt = carve<cplx>(h, sz.thin));
   for (int i = 0; i < 4; ++i) need(h->thin[i] = carve<cplx>(h, sz.thin));
   for (int i = 0; i < 2; ++i) {
@@ -1020,7 +1020,7 @@ extern "C" ipeps_status ipeps_ctm_create(const ipeps_cell* c, const ipeps_option
   for (int i = 0; i < 4; ++i) need(h->alt.Q[i] = carve<cplx>(h, sz.Q));
   if (tc_form(o->prec))
     for (int i = 0; i < 4; ++i)
-      for (int v = 0; v < 2; ++v) need(h->alt.Qpmem[i][v] = carve<char>(h, tc_packed_bytes(o->prec, h->K, h->K)));
+      for (int v = 0; v < 2; ++v) need(h->alt.Qpmem[i][v] = carve<char>(h, tc_packed_bytes(o->prec, h->K)));
   for (int i = 0; i < 4; ++i) need(h->alt.thin[i] = carve<cplx>(h, sz.thin));
   need(h->alt.Vt = carve<cplx>(h, (size_t)h->k * h->k));
   need(h->alt.Gsel = carve<cplx>(h, (size_t)h->chi * h->k));
@@ -1246,32 +1246,53 @@ static ipeps_status thin_mul(ipeps_ctm h, const cplx* in, int opin, cplx* out, c
   return gemm_dispatch(h, rows, h->K, h->K, in, h->K, opin, Qm, h->K, opQ, out, h->K, ONE);
 }
 
-// precision form: in (op opin) times the pre-packed corner q in variant v
-// (0: Q, 1: Q^T); the result is conjugated when conj_out.
-static ipeps_status thin_mul_packed(ipeps_ctm h, const cplx* in, int opin, cplx* out, int q, int v, int rows,
-                                    bool conj_out) {
+// precision form: in (conjugated with conj_in) times the packed corners
+// path[0], path[1], ... (corner q in variant v as 2 q + v; v = 0: Q, 1: Q^T); the
+// result is conjugated when conj_out.  Between the products the thin operand
+// exists in packed form only.
+static ipeps_status thin_chain(ipeps_ctm h, const cplx* in, bool conj_in, std::initializer_list<int> path, int rows,
+                               cplx* out, bool conj_out) {
+  const int prec = (int)h->opt.prec;
+  const long long mark = h->scratch_top, n = (long long)(tc_thin_bytes(prec, rows, h->K) / sizeof(cplx)) + 1;
+  TcThin t[2];
+  for (int i = 0; i < 2; ++i) {
+    cplx* mem = scratch_alloc(h, n);
+    if (!mem) return fail(IPEPS_ENOMEM, "scratch exhausted (thin products)");
+    CK(tc_thin_layout(prec, rows, h->K, mem, &t[i]));
+  }
   cudaEvent_t a = nullptr;
   prof_begin(h, &a);
-  TcProbe pr;
-  TcProbe* p = tc_probe_begin(h, &pr);
-  cudaError_t e = tc_zgemm_packed(h->stream, (int)h->opt.prec, rows, ONE, in, h->K, opin, h->Qp[q][v], out, h->K,
-                                  conj_out, h->scratch, h->scratch_elems, h->scratch_top, &h->st->tc_timeouts,
-                                  h->tuner, p);
-  prof_end(h, a, 8.0 * (double)rows * (double)h->K * (double)h->K, 0);
-  if (e == cudaSuccess) tc_probe_end(h, p, rows, h->K, h->K);
-  CK(e);
+  CK(tc_pack_thin(h->stream, in, h->K, conj_in, t[0]));
+  int i = 0;
+  for (int qv : path) {
+    const bool last = i + 1 == (int)path.size();
+    if (i > 0) prof_begin(h, &a);
+    TcProbe pr;
+    TcProbe* p = tc_probe_begin(h, &pr);
+    cudaError_t e = tc_thin(h->stream, t[i & 1], h->Qp[qv >> 1][qv & 1], last ? out : nullptr, h->K, last && conj_out,
+                            last ? nullptr : &t[(i + 1) & 1], h->scratch, h->scratch_elems, h->scratch_top,
+                            &h->st->tc_timeouts, h->tuner, p);
+    prof_end(h, a, 8.0 * (double)rows * (double)h->K * (double)h->K, 0);
+    if (e == cudaSuccess) tc_probe_end(h, p, rows, h->K, h->K);
+    CK(e);
+    ++i;
+  }
+  h->scratch_top = mark;
   return IPEPS_OK;
 }
 
 static ipeps_status pack_corners(ipeps_ctm h) {
   for (int q = 0; q < 4; ++q) {
     if (two_corners(h) && (q == 1 || q == 2)) continue;
-    for (int v = 0; v < 2; ++v)
-      CK(tc_pack_b(h->stream, (int)h->opt.prec, h->Q[q], h->K, v ? OP_T : OP_N, h->K, h->K, h->Qpmem[q][v],
-                   &h->Qp[q][v]));
+    CK(tc_pack_square(h->stream, (int)h->opt.prec, h->Q[q], h->K, h->Qpmem[q][0], h->Qpmem[q][1], &h->Qp[q][0],
+                      &h->Qp[q][1]));
   }
   return IPEPS_OK;
 }
+
+// corner q as it is, and transposed, in a thin chain
+constexpr int thinN(int q) { return 2 * q; }
+constexpr int thinT(int q) { return 2 * q + 1; }
 
 static bool packed_path(ipeps_ctm h) { return tc_form(h->opt.prec); }
 
@@ -1280,21 +1301,14 @@ static bool packed_path(ipeps_ctm h) { return tc_form(h->opt.prec); }
 static ipeps_status apply_XT(ipeps_ctm h, const cplx* in, cplx* out, int rows) {
   if (two_corners(h)) {
     if (packed_path(h)) {
-      CKS(thin_mul_packed(h, in, OP_N, h->thin[2], 3, 1, rows, false));
-      CKS(thin_mul_packed(h, h->thin[2], OP_N, out, 0, 0, rows, false));
+      CKS(thin_chain(h, in, false, {thinT(3), thinN(0)}, rows, out, false));
     } else {
       CKS(thin_mul(h, in, OP_N, h->thin[2], h->Q[3], OP_T, rows));
       CKS(thin_mul(h, h->thin[2], OP_N, out, h->Q[0], OP_N, rows));
     }
     return IPEPS_OK;
   }
-  if (packed_path(h)) {
-    CKS(thin_mul_packed(h, in, OP_N, h->thin[2], 2, 0, rows, false));
-    CKS(thin_mul_packed(h, h->thin[2], OP_N, h->thin[3], 3, 1, rows, false));
-    CKS(thin_mul_packed(h, h->thin[3], OP_N, h->thin[2], 0, 0, rows, false));
-    CKS(thin_mul_packed(h, h->thin[2], OP_N, out, 1, 0, rows, false));
-    return IPEPS_OK;
-  }
+  if (packed_path(h)) return thin_chain(h, in, false, {thinN(2), thinT(3), thinN(0), thinN(1)}, rows, out, false);
   CKS(thin_mul(h, in, OP_N, h->thin[2], h->Q[2], OP_N, rows));
   CKS(thin_mul(h, h->thin[2], OP_N, h->thin[3], h->Q[3], OP_T, rows));
   CKS(thin_mul(h, h->thin[3], OP_N, h->thin[2], h->Q[0], OP_N, rows));
@@ -1307,21 +1321,14 @@ static ipeps_status apply_XT(ipeps_ctm h, const cplx* in, cplx* out, int rows) {
 static ipeps_status apply_XHT(ipeps_ctm h, const cplx* in, cplx* out, int rows) {
   if (two_corners(h)) {
     if (packed_path(h)) {
-      CKS(thin_mul_packed(h, in, OP_C, h->thin[2], 0, 1, rows, false));
-      CKS(thin_mul_packed(h, h->thin[2], OP_N, out, 3, 0, rows, true));
+      CKS(thin_chain(h, in, true, {thinT(0), thinN(3)}, rows, out, true));
     } else {
       CKS(thin_mul(h, in, OP_N, h->thin[2], h->Q[0], OP_H, rows));
       CKS(thin_mul(h, h->thin[2], OP_N, out, h->Q[3], OP_C, rows));
     }
     return IPEPS_OK;
   }
-  if (packed_path(h)) {
-    CKS(thin_mul_packed(h, in, OP_C, h->thin[2], 1, 1, rows, false));
-    CKS(thin_mul_packed(h, h->thin[2], OP_N, h->thin[3], 0, 1, rows, false));
-    CKS(thin_mul_packed(h, h->thin[3], OP_N, h->thin[2], 3, 0, rows, false));
-    CKS(thin_mul_packed(h, h->thin[2], OP_N, out, 2, 1, rows, true));
-    return IPEPS_OK;
-  }
+  if (packed_path(h)) return thin_chain(h, in, true, {thinT(1), thinT(0), thinN(3), thinT(2)}, rows, out, true);
   CKS(thin_mul(h, in, OP_N, h->thin[2], h->Q[1], OP_H, rows));
   CKS(thin_mul(h, h->thin[2], OP_N, h->thin[3], h->Q[0], OP_H, rows));
   CKS(thin_mul(h, h->thin[3], OP_N, h->thin[2], h->Q[3], OP_C, rows));
@@ -1540,12 +1547,11 @@ static ipeps_status projectors(ipeps_ctm h, int f, int x, int y, cplx* PT, cplx*
   // (two corners: P^T = S^-1/2 V^T Q4^T ;  Ptil = S^-1/2 U^H Q1^T)
   if (two_corners(h)) {
     if (packed_path(h))
-      CKS(thin_mul_packed(h, Vt_chi, OP_N, PT, 3, 1, chi, false));
+      CKS(thin_chain(h, Vt_chi, false, {thinT(3)}, chi, PT, false));
     else
       CKS(thin_mul(h, Vt_chi, OP_N, PT, h->Q[3], OP_T, chi));
   } else if (packed_path(h)) {
-    CKS(thin_mul_packed(h, Vt_chi, OP_N, tmp, 2, 0, chi, false));
-    CKS(thin_mul_packed(h, tmp, OP_N, PT, 3, 1, chi, false));
+    CKS(thin_chain(h, Vt_chi, false, {thinN(2), thinT(3)}, chi, PT, false));
   } else {
     CKS(thin_mul(h, Vt_chi, OP_N, tmp, h->Q[2], OP_N, chi));
     CKS(thin_mul(h, tmp, OP_N, PT, h->Q[3], OP_T, chi));
@@ -1553,12 +1559,11 @@ static ipeps_status projectors(ipeps_ctm h, int f, int x, int y, cplx* PT, cplx*
   CK(scale_rows_isqrt(h->stream, PT, chi, K, K, h->s_sel));
   if (two_corners(h)) {
     if (packed_path(h))
-      CKS(thin_mul_packed(h, Ut_chi, OP_C, Ptil, 0, 1, chi, false));
+      CKS(thin_chain(h, Ut_chi, true, {thinT(0)}, chi, Ptil, false));
     else
       CKS(thin_mul(h, Ut_chi, OP_C, Ptil, h->Q[0], OP_T, chi));
   } else if (packed_path(h)) {
-    CKS(thin_mul_packed(h, Ut_chi, OP_C, tmp, 1, 1, chi, false));
-    CKS(thin_mul_packed(h, tmp, OP_N, Ptil, 0, 1, chi, false));
+    CKS(thin_chain(h, Ut_chi, true, {thinT(1), thinT(0)}, chi, Ptil, false));
   } else {
     CKS(thin_mul(h, Ut_chi, OP_C, tmp, h->Q[1], OP_T, chi));
     CKS(thin_mul(h, tmp, OP_N, Ptil, h->Q[0], OP_T, chi));

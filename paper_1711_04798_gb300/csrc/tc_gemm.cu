@@ -553,6 +553,72 @@ __global__ void pack_b_tiled_kernel(TcView V, int N, int K, int Nrp, int Krp, in
   }
 }
 
+// A square K x K matrix Q as the wide operand of the thin products, in both
+// orientations from one read: oN holds rows n, columns k of Q[k, n] (for thin *
+// Q), oT rows n, columns k of Q[n, k] (for thin * Q^T), each Mp x Krp reals,
+// (Re, Im) pairs along k, padded with zeros.  32 x 32 complex tiles through
+// shared memory; both directions read and write 128-byte runs per warp.
+template <int PREC>
+__global__ void pack_square_kernel(const cplx* __restrict__ Q, int K, int Mp, int Krp, void* __restrict__ n0,
+                                   void* __restrict__ n1, void* __restrict__ n2, void* __restrict__ t0,
+                                   void* __restrict__ t1, void* __restrict__ t2) {
+  __shared__ cplx tile[32][33];
+  const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32, kc = Krp >> 1;
+  const int c = c0 + threadIdx.x;
+  for (int i = threadIdx.y; i < 32; i += blockDim.y) {
+    const int r = r0 + i;
+    cplx v = make_double2(0.0, 0.0);
+    if (r < K && c < K) v = Q[(long long)r * K + c];
+    tile[i][threadIdx.x] = v;
+    if (c < kc) store_pair(PREC, (long long)r * Krp + 2 * (long long)c, v.x, v.y, t0, t1, t2);
+  }
+  __syncthreads();
+  const int k = r0 + threadIdx.x;
+  if (k >= kc) return;
+  for (int i = threadIdx.y; i < 32; i += blockDim.y) {
+    const cplx v = tile[threadIdx.x][i];
+    store_pair(PREC, (long long)(c0 + i) * Krp + 2 * (long long)k, v.x, v.y, n0, n1, n2);
+  }
+}
+
+// The sum of a thin product's K-split partials, P[z][n][2m .. 2m+1] (the
+// product is computed transposed: rows n, real columns 2m + (Re, Im)), as C[m,
+// n] (FP32 sums widened to FP64) and / or as the packed thin operand of the next
+// product (rows 2m: (Re, -Im), 2m+1: (Im, Re) along n).  32 x 32 complex tiles:
+// reads run along m, writes along n.  The grid covers the packed operand with
+// its padding, where the partials are products of zeros.
+template <int PREC>
+__global__ void thin_reduce_kernel(const float* __restrict__ P, int S, long long pstride, int Nrp, int M, int N,
+                                   cplx* __restrict__ C, long long ldc, int conj_out, int Krp, void* __restrict__ o0,
+                                   void* __restrict__ o1, void* __restrict__ o2) {
+  __shared__ float2 tile[32][33];
+  const int n0 = blockIdx.x * 32, m0 = blockIdx.y * 32;
+  const int m = m0 + threadIdx.x;
+  for (int i = threadIdx.y; i < 32; i += blockDim.y) {
+    const float* p = P + (long long)(n0 + i) * Nrp + 2 * m;
+    float re = 0.0f, im = 0.0f;
+#pragma unroll 4
+    for (int z = 0; z < S; ++z) {
+      const float2 v = *(const float2*)(p + z * pstride);
+      re += v.x;
+      im += v.y;
+    }
+    tile[i][threadIdx.x] = make_float2(re, im);
+  }
+  __syncthreads();
+  const int n = n0 + threadIdx.x;
+  for (int i = threadIdx.y; i < 32; i += blockDim.y) {
+    const float2 v = tile[threadIdx.x][i];
+    const double re = f2d_bits(v.x), im = f2d_bits(v.y);
+    if (C && m0 + i < M && n < N) C[(long long)(m0 + i) * ldc + n] = make_double2(re, conj_out ? neg_bits(im) : im);
+    if (o0 && 2 * n < Krp) {
+      const long long e = 2LL * (m0 + i) * Krp + 2 * (long long)n;
+      store_pair(PREC, e, re, neg_bits(im), o0, o1, o2);
+      store_pair(PREC, e + Krp, im, re, o0, o1, o2);
+    }
+  }
+}
+
 PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
 
 cudaError_t get_encoder() {
@@ -663,7 +729,7 @@ cudaError_t ensure_attr() {
 
 template <int PREC, int BN>
 cudaError_t launch_main(cudaStream_t s, const Operands& o, int S, int M, int N, cplx alpha, cplx* C, long long ldc,
-                        float* part, bool conj_out, int* timeouts, TcProbe* probe) {
+                        float* part, bool conj_out, int* timeouts, TcProbe* probe, bool partials_only = false) {
   using K_ = Cfg<PREC, BN>;
   cudaError_t e;
   if ((e = ensure_attr<PREC, BN>()) != cudaSuccess) return e;
@@ -707,11 +773,13 @@ cudaError_t launch_main(cudaStream_t s, const Operands& o, int S, int M, int N, 
   }
   tc_gemm_kernel<PREC, BN><<<grid, NTHREADS, K_::SMEM, s>>>(mA0, mA1, mA2, mB0, mB1, mB2, o.kb_total, kps, n_tiles,
                                                              m_tiles, (int)tiles, M, 2 * N, alpha, C, ldc,
-                                                             S > 1 ? part : nullptr, (int)o.Nrp, o.Mp * o.Nrp,
+                                                             S > 1 || partials_only ? part : nullptr, (int)o.Nrp,
+                                                             o.Mp * o.Nrp,
                                                              conj_out ? 1 : 0, unit, timeouts);
   count_launch();
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (probe && (e = cudaEventRecord(probe->ev[1], s)) != cudaSuccess) return e;
+  if (partials_only) return cudaSuccess;
   if (S > 1) {
     if (S >= 64)
       splitk_reduce_warp_kernel<<<grid_for(32LL * M * N), 256, 0, s>>>(part, S, o.Mp * o.Nrp, (int)o.Nrp, M, N, alpha,
@@ -742,8 +810,9 @@ cudaError_t launch_choice(cudaStream_t s, const Operands& o, TcChoice c, int M, 
 struct TcTuner {
   struct Key {
     int prec, M, N, K;
+    bool thin;  // a transposed thin product (its reduction and operands differ)
     bool operator<(const Key& o) const {
-      return std::tie(prec, M, N, K) < std::tie(o.prec, o.M, o.N, o.K);
+      return std::tie(prec, M, N, K, thin) < std::tie(o.prec, o.M, o.N, o.K, o.thin);
     }
   };
   struct Entry {
@@ -796,10 +865,66 @@ bool tc_tuner_entry(const TcTuner* t, int i, int fields[6], double us[2]) {
 
 namespace {
 
+// Time every candidate (best of two runs each) on the packed operands and
+// record the fastest: both tile widths, K splits in powers of two and the
+// counts that fill one to four whole waves.
+template <class Room, class Launch>
+cudaError_t tune_choice(cudaStream_t s, TcTuner* tuner, const TcTuner::Key& key, const Operands& o, TcChoice base,
+                        Room&& room, Launch&& launch, TcChoice* best_choice) {
+  cudaError_t e;
+  auto time_one = [&](TcChoice c, double* us) -> cudaError_t {
+    double best = 1e30;
+    for (int rep = 0; rep < 2; ++rep) {
+      cudaError_t r;
+      if ((r = cudaEventRecord(tuner->e0, s)) != cudaSuccess) return r;
+      if ((r = launch(c)) != cudaSuccess) return r;
+      if ((r = cudaEventRecord(tuner->e1, s)) != cudaSuccess) return r;
+      if ((r = cudaEventSynchronize(tuner->e1)) != cudaSuccess) return r;
+      float ms = 0;
+      if ((r = cudaEventElapsedTime(&ms, tuner->e0, tuner->e1)) != cudaSuccess) return r;
+      best = std::min(best, 1e3 * (double)ms);
+    }
+    *us = best;
+    return cudaSuccess;
+  };
+  TcTuner::Entry ent{base, 0.0, 0.0, 0};
+  if ((e = time_one(base, &ent.heuristic_us)) != cudaSuccess) return e;
+  ent.us = ent.heuristic_us;
+  ent.candidates = 1;
+  static const int bns[2] = {128, 256};
+  for (int bn : bns) {
+    if (o.Nrp % bn != 0) continue;
+    const long long tiles = (o.Mp / BM) * (o.Nrp / bn);
+    std::vector<int> splits = {1, 2, 4, 8, 16, 32};
+    for (int w = 1; w <= 4; ++w) {
+      const int S = (int)((long long)w * NSM / tiles);
+      if (S > 1 && std::find(splits.begin(), splits.end(), S) == splits.end()) splits.push_back(S);
+    }
+    for (int S0 : splits) {
+      const int S = eff_splits(o.kb_total, S0);
+      if (S != S0 && S0 != 1) continue;            // duplicate of a smaller split count
+      if (S > 1 && o.kb_total / S < 2) continue;  // splits of a single k-block
+      if (!room(S)) continue;
+      const TcChoice c{bn, S};
+      if (c.bn == base.bn && c.splits == eff_splits(o.kb_total, base.splits)) continue;
+      double us = 0;
+      if ((e = time_one(c, &us)) != cudaSuccess) return e;
+      ++ent.candidates;
+      if (us < ent.us) {
+        ent.us = us;
+        ent.choice = c;
+      }
+    }
+  }
+  tuner->table[key] = ent;
+  tuner->order.push_back(key);
+  *best_choice = ent.choice;
+  return cudaSuccess;
+}
+
 template <int PREC>
 cudaError_t run(cudaStream_t s, int M, int N, int K, cplx alpha, const cplx* A, long long lda, int opA,
-                const cplx* B, long long ldb, int opB, const TcPacked* pre, cplx* C, long long ldc, bool conj_out,
-                char* scratch, size_t scratch_bytes, TcTuner* tuner, const TcChoice* force, int* timeouts,
+                const cplx* B, long long ldb, int opB, cplx* C, long long ldc, char* scratch, size_t scratch_bytes, TcTuner* tuner, const TcChoice* force, int* timeouts,
                 TcProbe* probe, const TcView* va = nullptr, const TcView* vb = nullptr) {
   if (!timeouts) return cudaErrorInvalidValue;
   using K_ = Cfg<PREC, 128>;  // element size, k-block and parts do not depend on the tile width
@@ -809,7 +934,8 @@ cudaError_t run(cudaStream_t s, int M, int N, int K, cplx alpha, const cplx* A, 
   o.kb_total = (int)(o.Krp / K_::BK);
   auto al = [](size_t x) { return (x + 1023) & ~(size_t)1023; };
   const size_t abytes = al((size_t)o.Mp * o.Krp * K_::ELEM);
-  const size_t bbytes = pre ? 0 : al((size_t)o.Nrp * o.Krp * K_::ELEM);
+  const size_t bbytes = al((size_t)o.Nrp * o.Krp * K_::ELEM);
+  const bool conj_out = false;
   const size_t fixed = K_::NOPS * (abytes + bbytes) + 1024;
   if (fixed > scratch_bytes) return cudaErrorMemoryAllocation;
   const size_t part_room = scratch_bytes - fixed;
@@ -824,7 +950,7 @@ cudaError_t run(cudaStream_t s, int M, int N, int K, cplx alpha, const cplx* A, 
   float* part = (float*)((char*)o.b0 + K_::NOPS * bbytes);
 
   TcChoice choice = heuristic(o.Mp, o.Nrp, o.kb_total);
-  const TcTuner::Key key{PREC, M, N, K};
+  const TcTuner::Key key{PREC, M, N, K, false};
   bool tune_now = false;
   if (tuner) {
     auto it = tuner->table.find(key);
@@ -865,12 +991,7 @@ cudaError_t run(cudaStream_t s, int M, int N, int K, cplx alpha, const cplx* A, 
   }
   count_launch();
   cudaError_t e;
-  if (pre) {
-    if (pre->prec != PREC || pre->N != N || pre->K != K) return cudaErrorInvalidValue;
-    o.b0 = pre->b0;
-    o.b1 = pre->b1;
-    o.b2 = pre->b2;
-  } else if (vb) {
+  if (vb) {
     if (o.Nrp / 64 > 65535) return cudaErrorNotSupported;
     const int row_contig = vb->rstr[vb->nr - 1] == 1 && vb->cstr[vb->nc - 1] != 1;
     pack_b_tiled_kernel<PREC><<<dim3((unsigned)((o.Krp / 2 + 31) / 32), (unsigned)(o.Nrp / 64)), dim3(32, 8), 0, s>>>(
@@ -881,58 +1002,13 @@ cudaError_t run(cudaStream_t s, int M, int N, int K, cplx alpha, const cplx* A, 
     return e;
   }
   if (tune_now) {
-    // time every candidate (best of two runs each) on the packed operands
-    auto time_one = [&](TcChoice c, double* us) -> cudaError_t {
-      double best = 1e30;
-      for (int rep = 0; rep < 2; ++rep) {
-        cudaError_t r;
-        if ((r = cudaEventRecord(tuner->e0, s)) != cudaSuccess) return r;
-        if ((r = launch_choice<PREC>(s, o, c, M, N, alpha, C, ldc, part, conj_out, timeouts)) != cudaSuccess)
-          return r;
-        if ((r = cudaEventRecord(tuner->e1, s)) != cudaSuccess) return r;
-        if ((r = cudaEventSynchronize(tuner->e1)) != cudaSuccess) return r;
-        float ms = 0;
-        if ((r = cudaEventElapsedTime(&ms, tuner->e0, tuner->e1)) != cudaSuccess) return r;
-        best = std::min(best, 1e3 * (double)ms);
-      }
-      *us = best;
-      return cudaSuccess;
-    };
-    TcTuner::Entry ent{choice, 0.0, 0.0, 0};
-    if ((e = time_one(choice, &ent.heuristic_us)) != cudaSuccess) return e;
-    ent.us = ent.heuristic_us;
-    ent.candidates = 1;
-    static const int bns[2] = {128, 256};
-    for (int bn : bns) {
-      if (o.Nrp % bn != 0) continue;
-      // powers of two, and the counts that fill one to four whole waves
-      const long long tiles = (o.Mp / BM) * (o.Nrp / bn);
-      std::vector<int> splits = {1, 2, 4, 8, 16, 32};
-      for (int w = 1; w <= 4; ++w) {
-        const int S = (int)((long long)w * NSM / tiles);
-        if (S > 1 && std::find(splits.begin(), splits.end(), S) == splits.end()) splits.push_back(S);
-      }
-      for (int S0 : splits) {
-        const int S = eff_splits(o.kb_total, S0);
-        if (S != S0 && S0 != 1) continue;        // duplicate of a smaller split count
-        if (S > 1 && o.kb_total / S < 2) continue;  // splits of a single k-block
-        if (part_bytes(S) > part_room) continue;
-        const TcChoice c{bn, S};
-        if (c.bn == ent.choice.bn && c.splits == eff_splits(o.kb_total, choice.splits)) continue;
-        double us = 0;
-        if ((e = time_one(c, &us)) != cudaSuccess) return e;
-        ++ent.candidates;
-        if (us < ent.us) {
-          ent.us = us;
-          ent.choice = c;
-        }
-      }
-    }
-    tuner->table[key] = ent;
-    tuner->order.push_back(key);
-    choice = ent.choice;
+    e = tune_choice(s, tuner, key, o, choice, [&](int S) { return part_bytes(S) <= part_room; },
+                    [&](TcChoice c) {
+                      return launch_choice<PREC>(s, o, c, M, N, alpha, C, ldc, part, conj_out, timeouts);
+                    },
+                    &choice);
+    if (e != cudaSuccess) return e;
   }
-  if (probe) probe->packed_b = pre != nullptr;
   return launch_choice<PREC>(s, o, choice, M, N, alpha, C, ldc, part, conj_out, timeouts, probe);
 }
 
@@ -972,7 +1048,7 @@ cudaError_t tc_zgemm(cudaStream_t s, int prec, int M, int N, int K, cplx alpha, 
   char* base = (char*)(scratch + scratch_top);
   const size_t bytes = (size_t)(scratch_elems - scratch_top) * sizeof(cplx);
   return by_prec(prec, [&](auto P) {
-    return run<decltype(P)::value>(s, M, N, K, alpha, A, lda, opA, B, ldb, opB, nullptr, C, ldc, false, base, bytes,
+    return run<decltype(P)::value>(s, M, N, K, alpha, A, lda, opA, B, ldb, opB, C, ldc, base, bytes,
                                    tuner, force, timeouts, probe);
   });
 }
@@ -985,57 +1061,151 @@ cudaError_t tc_zgemm_views(cudaStream_t s, int prec, int M, int N, int K, cplx a
   char* base = (char*)(scratch + scratch_top);
   const size_t bytes = (size_t)(scratch_elems - scratch_top) * sizeof(cplx);
   return by_prec(prec, [&](auto P) {
-    return run<decltype(P)::value>(s, M, N, K, alpha, A, lda, opA, B, ldb, opB, nullptr, C, ldc, false, base, bytes,
+    return run<decltype(P)::value>(s, M, N, K, alpha, A, lda, opA, B, ldb, opB, C, ldc, base, bytes,
                                    tuner, nullptr, timeouts, probe, va, vb);
   });
 }
 
 static int n_parts(int prec) { return prec == PREC_TF32 ? 1 : (prec == PREC_BF16X3 ? 2 : 3); }
 
-size_t tc_packed_bytes(int prec, int N, int K) {
-  long long Nrp, Krp;
-  if (prec == PREC_TF32) {
-    padded<PREC_TF32>(N, K, &Nrp, &Krp);
-    return (size_t)Nrp * Krp * 4 + 2048;
-  }
-  padded<PREC_BF16X3>(N, K, &Nrp, &Krp);  // BF16 k-blocks: the same padding for x3 and x6
-  return (size_t)n_parts(prec) * ((size_t)Nrp * Krp * 2 + 1024) + 2048;
-}
+namespace {
 
-cudaError_t tc_pack_b(cudaStream_t s, int prec, const cplx* B, long long ldb, int opB, int N, int K, void* mem,
-                      TcPacked* out) {
-  long long Nrp, Krp;
+// parts of `each` bytes (1 KB aligned) from mem
+void carve_parts(int prec, void* mem, size_t each, void* (&b)[3]) {
   char* p = (char*)(((uintptr_t)mem + 1023) & ~(uintptr_t)1023);
-  out->prec = prec;
-  out->N = N;
-  out->K = K;
-  if (prec == PREC_TF32) {
-    padded<PREC_TF32>(N, K, &Nrp, &Krp);
-    out->b0 = out->b1 = out->b2 = p;
-    return pack_b_any<PREC_TF32>(s, B, ldb, opB, N, K, Nrp, Krp, out->b0, out->b1, out->b2);
-  }
-  if (prec == PREC_BF16X3 || prec == PREC_BF16X6) {
-    padded<PREC_BF16X3>(N, K, &Nrp, &Krp);
-    const size_t part = ((size_t)Nrp * Krp * 2 + 1023) & ~(size_t)1023;
-    out->b0 = p;
-    out->b1 = p + part;
-    out->b2 = prec == PREC_BF16X6 ? p + 2 * part : out->b1;
-    if (prec == PREC_BF16X3) return pack_b_any<PREC_BF16X3>(s, B, ldb, opB, N, K, Nrp, Krp, out->b0, out->b1, out->b2);
-    return pack_b_any<PREC_BF16X6>(s, B, ldb, opB, N, K, Nrp, Krp, out->b0, out->b1, out->b2);
-  }
-  return cudaErrorNotSupported;
+  each = (each + 1023) & ~(size_t)1023;
+  const int n = n_parts(prec);
+  b[0] = p;
+  b[1] = n >= 2 ? p + each : p;
+  b[2] = n == 3 ? p + 2 * each : b[1];
 }
 
-cudaError_t tc_zgemm_packed(cudaStream_t s, int prec, int M, cplx alpha, const cplx* A, long long lda, int opA,
-                            const TcPacked& B, cplx* C, long long ldc, bool conj_out, cplx* scratch,
-                            long long scratch_elems, long long scratch_top, int* timeouts, TcTuner* tuner,
-                            TcProbe* probe) {
-  if (M <= 0) return cudaSuccess;
+size_t parts_bytes(int prec, size_t each) { return (size_t)n_parts(prec) * (each + 1024) + 2048; }
+
+long long pad_k(int prec, int K) {
+  long long Nrp, Krp;
+  by_prec(prec, [&](auto P) {
+    padded<decltype(P)::value>(K, K, &Nrp, &Krp);
+    return cudaSuccess;
+  });
+  return Krp;
+}
+
+long long elem_bytes(int prec) { return prec == PREC_TF32 ? 4 : 2; }
+
+long long pad_to(long long x, long long q) { return (x + q - 1) / q * q; }
+
+}  // namespace
+
+size_t tc_packed_bytes(int prec, int K) {
+  return parts_bytes(prec, (size_t)(pad_to(K, BM) * pad_k(prec, K) * elem_bytes(prec)));
+}
+
+size_t tc_thin_bytes(int prec, int M, int K) {
+  return parts_bytes(prec, (size_t)(pad_to(2LL * M, NPAD) * pad_k(prec, K) * elem_bytes(prec)));
+}
+
+cudaError_t tc_pack_square(cudaStream_t s, int prec, const cplx* Q, int K, void* memN, void* memT, TcPacked* outN,
+                           TcPacked* outT) {
+  const long long Mp = pad_to(K, BM), Krp = pad_k(prec, K);
+  if (Mp / 32 > 65535) return cudaErrorNotSupported;
+  TcPacked* out[2] = {outN, outT};
+  void* mem[2] = {memN, memT};
+  for (int v = 0; v < 2; ++v) {
+    out[v]->prec = prec;
+    out[v]->K = K;
+    carve_parts(prec, mem[v], (size_t)(Mp * Krp * elem_bytes(prec)), out[v]->b);
+  }
+  return by_prec(prec, [&](auto P) {
+    pack_square_kernel<decltype(P)::value><<<dim3((unsigned)(Mp / 32), (unsigned)(Mp / 32)), dim3(32, 8), 0, s>>>(
+        Q, K, (int)Mp, (int)Krp, outN->b[0], outN->b[1], outN->b[2], outT->b[0], outT->b[1], outT->b[2]);
+    count_launch();
+    return cudaGetLastError();
+  });
+}
+
+cudaError_t tc_thin_layout(int prec, int M, int K, void* mem, TcThin* out) {
+  out->prec = prec;
+  out->M = M;
+  out->K = K;
+  carve_parts(prec, mem, (size_t)(pad_to(2LL * M, NPAD) * pad_k(prec, K) * elem_bytes(prec)), out->b);
+  return cudaSuccess;
+}
+
+cudaError_t tc_pack_thin(cudaStream_t s, const cplx* A, long long lda, bool conj, const TcThin& t) {
+  return by_prec(t.prec, [&](auto P) {
+    return pack_b_any<decltype(P)::value>(s, A, lda, OP_T | (conj ? OP_CONJ : 0), t.M, t.K, pad_to(2LL * t.M, NPAD),
+                                          pad_k(t.prec, t.K), t.b[0], t.b[1], t.b[2]);
+  });
+}
+
+namespace {
+
+template <int PREC>
+cudaError_t run_thin(cudaStream_t s, const TcThin& A, const TcPacked& Q, cplx* C, long long ldc, bool conj_out,
+                     const TcThin* next, char* scratch, size_t scratch_bytes, int* timeouts, TcTuner* tuner,
+                     TcProbe* probe) {
+  using K_ = Cfg<PREC, 128>;
+  if (!timeouts || A.prec != PREC || Q.prec != PREC || A.K != Q.K) return cudaErrorInvalidValue;
+  if (next && (next->prec != PREC || next->M != A.M || next->K != Q.K)) return cudaErrorInvalidValue;
+  const int M = A.M, N = Q.K;
+  Operands o;  // the transposed product: rows n of Q, real columns 2m + (Re, Im)
+  o.Mp = pad_to(N, BM);
+  o.Nrp = pad_to(2LL * M, NPAD);
+  o.Krp = pad_k(PREC, Q.K);
+  o.kb_total = (int)(o.Krp / K_::BK);
+  o.a0 = Q.b[0];
+  o.a1 = Q.b[1];
+  o.a2 = Q.b[2];
+  o.b0 = A.b[0];
+  o.b1 = A.b[1];
+  o.b2 = A.b[2];
+  float* part = (float*)(((uintptr_t)scratch + 1023) & ~(uintptr_t)1023);
+  auto room = [&](int S) { return (size_t)S * o.Mp * o.Nrp * 4 + 1024 <= scratch_bytes; };
+  auto launch = [&](TcChoice c, TcProbe* pr) -> cudaError_t {
+    const int S = eff_splits(o.kb_total, c.splits);
+    cudaError_t e;
+    if (c.bn == 128 || o.Nrp % 256 != 0)
+      e = launch_main<PREC, 128>(s, o, S, N, M, make_double2(1.0, 0.0), nullptr, 0, part, false, timeouts, pr, true);
+    else
+      e = launch_main<PREC, 256>(s, o, S, N, M, make_double2(1.0, 0.0), nullptr, 0, part, false, timeouts, pr, true);
+    if (e != cudaSuccess) return e;
+    const long long rows = next ? std::max<long long>(N, o.Krp / 2) : N, cols = next ? o.Nrp / 2 : M;
+    thin_reduce_kernel<PREC><<<dim3((unsigned)((rows + 31) / 32), (unsigned)((cols + 31) / 32)), dim3(32, 8), 0, s>>>(
+        part, S, o.Mp * o.Nrp, (int)o.Nrp, M, N, C, ldc, conj_out ? 1 : 0, (int)o.Krp, next ? next->b[0] : nullptr,
+        next ? next->b[1] : nullptr, next ? next->b[2] : nullptr);
+    count_launch();
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (pr) {
+      pr->splits = S;
+      return cudaEventRecord(pr->ev[2], s);
+    }
+    return cudaSuccess;
+  };
+  TcChoice choice = heuristic(o.Mp, o.Nrp, o.kb_total);
+  if (!room(eff_splits(o.kb_total, choice.splits))) return cudaErrorMemoryAllocation;
+  if (tuner) {
+    const TcTuner::Key key{PREC, N, M, Q.K, true};
+    auto it = tuner->table.find(key);
+    if (it != tuner->table.end()) {
+      choice = it->second.choice;
+    } else if (tuner->measuring) {
+      cudaError_t e = tune_choice(s, tuner, key, o, choice, room, [&](TcChoice c) { return launch(c, nullptr); }, &choice);
+      if (e != cudaSuccess) return e;
+    }
+  }
+  return launch(choice, probe);
+}
+
+}  // namespace
+
+cudaError_t tc_thin(cudaStream_t s, const TcThin& A, const TcPacked& Q, cplx* C, long long ldc, bool conj_out,
+                    const TcThin* next, cplx* scratch, long long scratch_elems, long long scratch_top, int* timeouts,
+                    TcTuner* tuner, TcProbe* probe) {
   char* base = (char*)(scratch + scratch_top);
   const size_t bytes = (size_t)(scratch_elems - scratch_top) * sizeof(cplx);
-  return by_prec(prec, [&](auto P) {
-    return run<decltype(P)::value>(s, M, (int)B.N, (int)B.K, alpha, A, lda, opA, nullptr, 0, 0, &B, C, ldc, conj_out,
-                                   base, bytes, tuner, nullptr, timeouts, probe);
+  return by_prec(A.prec, [&](auto P) {
+    return run_thin<decltype(P)::value>(s, A, Q, C, ldc, conj_out, next, base, bytes, timeouts, tuner, probe);
   });
 }
 
@@ -1046,5 +1216,6 @@ cudaError_t tc_init() {
   if ((e = ensure_attr<PREC_BF16X3, 128>()) != cudaSuccess) return e;
   if ((e = ensure_attr<PREC_BF16X3, 256>()) != cudaSuccess) return e;
   if ((e = ensure_attr<PREC_BF16X6, 128>()) != cudaSuccess) return e;
+  if ((e = ensure_attr<PREC_BF16X6, 256>()) != cudaSuccess) return e;
   return get_encoder();
 }

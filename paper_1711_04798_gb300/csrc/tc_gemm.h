@@ -23,7 +23,6 @@ struct TcProbe {
   cudaEvent_t ev[3];
   long long Mp, Nrp, Krp;  // padded real-embedded shape
   int splits, bn, parts, elem_bytes;
-  bool packed_b;           // B came pre-packed (not repacked by this call)
 };
 
 // An operand read through a strided view instead of a permuted copy: element
@@ -45,23 +44,34 @@ cudaError_t tc_zgemm(cudaStream_t s, int prec, int M, int N, int K, cplx alpha, 
                      int* timeouts, TcTuner* tuner = nullptr, const TcChoice* force = nullptr,
                      TcProbe* probe = nullptr);
 
-// A B-role operand (op(B) is K x N complex) packed once as Br^T (2N x 2K real,
-// K-major, padded), reusable across products.
-struct TcPacked {
-  int prec;
-  long long N, K;
-  void* b0;  // TF32 values, or the leading BF16 part
-  void* b1;  // second BF16 part (== b0 for TF32)
-  void* b2;  // third BF16 part of BF16x6 (== b1 otherwise)
+// Thin products: C (M x K) = A (M x K) times a square K x K matrix, with few
+// rows (the range finder, the projector assembly).  They are computed
+// transposed, C^T = Q^T A^T, so that the real embedding doubles the thin operand
+// and not the matrix, whose packed form (Re, Im pairs, 2 reals per complex
+// number and part) is what bounds them: at K = 2500 in three BF16 parts 75 MB
+// per product instead of 150 MB.  The partials' sum writes the next product's
+// packed operand itself, so a chain packs its first operand only.
+struct TcPacked {  // one orientation of Q
+  int prec, K;
+  void* b[3];      // parts (TF32: one)
 };
-size_t tc_packed_bytes(int prec, int N, int K);
-cudaError_t tc_pack_b(cudaStream_t s, int prec, const cplx* B, long long ldb, int opB, int N, int K, void* mem,
-                      TcPacked* out);
-// C = alpha opA(A) B  (or its complex conjugate when conj_out), B pre-packed
-cudaError_t tc_zgemm_packed(cudaStream_t s, int prec, int M, cplx alpha, const cplx* A, long long lda, int opA,
-                            const TcPacked& B, cplx* C, long long ldc, bool conj_out, cplx* scratch,
-                            long long scratch_elems, long long scratch_top, int* timeouts,
-                            TcTuner* tuner = nullptr, TcProbe* probe = nullptr);
+struct TcThin {    // a packed thin operand: 2M x 2K reals
+  int prec, M, K;
+  void* b[3];
+};
+size_t tc_packed_bytes(int prec, int K);
+size_t tc_thin_bytes(int prec, int M, int K);
+// Q (row-major) packed for thin * Q (outN) and thin * Q^T (outT), one read
+cudaError_t tc_pack_square(cudaStream_t s, int prec, const cplx* Q, int K, void* memN, void* memT, TcPacked* outN,
+                           TcPacked* outT);
+// a thin operand's parts in mem (tc_thin_bytes)
+cudaError_t tc_thin_layout(int prec, int M, int K, void* mem, TcThin* out);
+// t = A (M x K, row-major, conjugated with conj), packed
+cudaError_t tc_pack_thin(cudaStream_t s, const cplx* A, long long lda, bool conj, const TcThin& t);
+// A Q as C (optional; conjugated with conj_out) and / or packed as *next (optional)
+cudaError_t tc_thin(cudaStream_t s, const TcThin& A, const TcPacked& Q, cplx* C, long long ldc, bool conj_out,
+                    const TcThin* next, cplx* scratch, long long scratch_elems, long long scratch_top, int* timeouts,
+                    TcTuner* tuner = nullptr, TcProbe* probe = nullptr);
 
 // Tile choice of one product: output tile 128 x bn (bn = 128 or 256 real
 // columns) and the number of K splits (FP32 partials summed in a fixed order).
