@@ -60,8 +60,9 @@ static const cplx ZERO = {0.0, 0.0};
 // handle
 // ---------------------------------------------------------------------------
 struct TV {  // contiguous row-major tensor view
-  cplx* p;
+  cplx* p;   // f32: complex FP32 values at the same address
   int nd;
+  bool f32 = false;
   int dims[8];
   long long size() const {
     long long s = 1;
@@ -70,9 +71,10 @@ struct TV {  // contiguous row-major tensor view
   }
 };
 
-static TV tv(cplx* p, std::initializer_list<int> dims) {
+static TV tv(cplx* p, std::initializer_list<int> dims, bool f32 = false) {
   TV t;
   t.p = p;
+  t.f32 = f32;
   t.nd = 0;
   for (int d : dims) t.dims[t.nd++] = d;
   return t;
@@ -501,11 +503,28 @@ static bool make_view(const TV& X, const std::string& lx, const std::string& row
     return true;
   };
   v->p = X.p;
+  v->f32 = X.f32 ? 1 : 0;
   v->conj = cj ? 1 : 0;
   if (!side(rows, &v->nr, v->rdim, v->rstr) || !side(cols, &v->nc, v->cdim, v->cstr)) return false;
   if (v->nr == 0) { v->nr = 1; v->rdim[0] = 1; v->rstr[0] = 0; }
   if (v->nc == 0) { v->nc = 1; v->cdim[0] = 1; v->cstr[0] = 0; }
   return true;
+}
+
+// whether a product of these sizes runs on the precision form's tensor cores
+// with gathered operands (which index in 32 bits)
+static bool tc_product(ipeps_ctm h, long long M, long long N, long long K) {
+  return tc_form(h->opt.prec) && M >= 64 && N >= 32 && K >= 16 &&
+         (2 * std::max(M, N) + 512) * (2 * K + 128) < (1LL << 31);
+}
+
+// Whether the tensor between two products of a chain, one of M x N that makes
+// it and one with K2 summed and N2 free labels beside it, is kept as complex
+// FP32: both run on the tensor cores, whose FP32 sums and FP32 (at most 24
+// bit) operands then pass through it unchanged, at half of the bytes of
+// complex FP64.  M2: rows of the second product.
+static bool f32_between(ipeps_ctm h, long long M, long long N, long long K, long long M2, long long N2, long long K2) {
+  return tc_product(h, M, N, K) && tc_product(h, M2, N2, K2) && std::max(M, M2) <= 2000000 && N <= 2000000;
 }
 
 static ipeps_status contract(ipeps_ctm h, const char* spec, TV A, bool conjA, TV B, bool conjB,
@@ -567,9 +586,9 @@ static ipeps_status contract(ipeps_ctm h, const char* spec, TV A, bool conjA, TV
   // Tensor-core products: an operand that is not already in GEMM form is
   // gathered by the operand packing through a view (fused permute-and-pack)
   // instead of being permuted into a copy first.
-  const bool tc = tc_form(h->opt.prec) &&
-                  ((direct && swap) ? (N >= 64 && M >= 32 && Kd >= 16) : (M >= 64 && N >= 32 && Kd >= 16)) &&
-                  (2 * std::max(M, N) + 512) * (2 * Kd + 128) < (1LL << 31);  // gathers index in 32 bits
+  const bool tc = (direct && swap) ? tc_product(h, N, M, Kd) : tc_product(h, M, N, Kd);
+  if ((A.f32 || B.f32 || C.f32) && (!tc || (C.f32 && (!direct || alpha.x != 1.0 || alpha.y != 0.0))))
+    return fail(IPEPS_EINVAL, "FP32 operand or result outside the tensor cores in %s", spec);
   // arrange one operand as [free..., k...] (op N) or [k..., free...] (op T)
   auto arrange = [&](TV X, const std::string& lx, bool cj, const std::string& fo,
                      const std::string& ko, const cplx** out, long long* ld, int* op) -> ipeps_status {
@@ -613,14 +632,18 @@ static ipeps_status contract(ipeps_ctm h, const char* spec, TV A, bool conjA, TV
   int opa = OP_N, opb = OP_N;
   TcView va, vb;
   bool use_va = false, use_vb = false;
-  if (tc && !is_form(la, Mo, ko)) use_va = make_view(A, la, Mo, ko, conjA, &va);
+  if (tc && (A.f32 || C.f32 || !is_form(la, Mo, ko))) use_va = make_view(A, la, Mo, ko, conjA, &va);
+  if (A.f32 && !use_va) return fail(IPEPS_EINVAL, "FP32 operand of too many axes in %s", spec);
   if (!use_va) CKS(arrange(A, la, conjA, Mo, ko, &pa, &lda, &opa));
   // B must be [ko, No] (op N) or [No, ko] (op T); arrange() returns [No, ko] forms
   {
     long long fdim = 1, kdim = 1;
     for (char c : No) fdim *= dimB(c);
     for (char c : ko) kdim *= dimB(c);
-    if (lb == ko + No) {
+    if (B.f32) {
+      use_vb = make_view(B, lb, No, ko, conjB, &vb);
+      if (!use_vb) return fail(IPEPS_EINVAL, "FP32 operand of too many axes in %s", spec);
+    } else if (lb == ko + No) {
       pb = B.p; ldb = fdim; opb = OP_N | (conjB ? OP_CONJ : 0);
     } else if (lb == No + ko) {
       pb = B.p; ldb = kdim; opb = OP_T | (conjB ? OP_CONJ : 0);
@@ -641,6 +664,7 @@ static ipeps_status contract(ipeps_ctm h, const char* spec, TV A, bool conjA, TV
     // A role: element (m, k) of op(A); B role: element (n, k) of op(B)^T
     const bool t = (op & OP_T) != 0;
     v->p = p;
+    v->f32 = 0;
     v->conj = (op & OP_CONJ) ? 1 : 0;
     v->nr = v->nc = 1;
     v->rdim[0] = rows;
@@ -649,6 +673,7 @@ static ipeps_status contract(ipeps_ctm h, const char* spec, TV A, bool conjA, TV
     v->rstr[0] = row_major_rows ? ld : 1;
     v->cstr[0] = row_major_rows ? 1 : ld;
   };
+  if (C.f32 && !use_va && !use_vb) return fail(IPEPS_EINVAL, "FP32 result of plain operands in %s", spec);
   if (use_va || use_vb) {
     // at least one gathered operand: one tensor-core product with views
     const TcView* VA = use_va ? &va : nullptr;
@@ -663,7 +688,7 @@ static ipeps_status contract(ipeps_ctm h, const char* spec, TV A, bool conjA, TV
       TcProbe pr;
       TcProbe* p = tc_probe_begin(h, &pr);
       cudaError_t e = tc_zgemm_views(h->stream, (int)h->opt.prec, (int)N, (int)M, (int)Kd, alpha, &xa, nullptr, 0, 0,
-                                     &xb, nullptr, 0, 0, C.p, M, h->scratch, h->scratch_elems, h->scratch_top,
+                                     &xb, nullptr, 0, 0, C.p, M, C.f32, h->scratch, h->scratch_elems, h->scratch_top,
                                      &h->st->tc_timeouts, h->tuner, p);
       prof_end(h, ev, 8.0 * (double)M * (double)N * (double)Kd, 0);
       if (e == cudaSuccess) tc_probe_end(h, p, (int)N, (int)M, (int)Kd);
@@ -680,7 +705,7 @@ static ipeps_status contract(ipeps_ctm h, const char* spec, TV A, bool conjA, TV
       TcProbe pr;
       TcProbe* p = tc_probe_begin(h, &pr);
       cudaError_t e = tc_zgemm_views(h->stream, (int)h->opt.prec, (int)M, (int)N, (int)Kd, direct ? alpha : ONE, VA,
-                                     pa, lda, opa, VB, pb, ldb, opb, out, N, h->scratch, h->scratch_elems,
+                                     pa, lda, opa, VB, pb, ldb, opb, out, N, direct && C.f32, h->scratch, h->scratch_elems,
                                      h->scratch_top, &h->st->tc_timeouts, h->tuner, p);
       prof_end(h, ev, 8.0 * (double)M * (double)N * (double)Kd, 0);
       if (e == cudaSuccess) tc_probe_end(h, p, (int)M, (int)N, (int)Kd);
@@ -1196,46 +1221,60 @@ extern "C" ipeps_status ipeps_ctm_reset_env(ipeps_ctm h) {
 // the two-corner projector (ipeps_options.corners = 2): X = Q1^T Q4
 static bool two_corners(ipeps_ctm h) { return h->opt.corners == 2; }
 
-static ipeps_status enlarged_corners(ipeps_ctm h, int f, int x, int y) {
+// The corners the thin products take packed, as the last product leaves them:
+// complex FP32 in [x][y][a][b] order for Q[(x a), (y b)] (x, y < chi, a, b < D^2),
+// the order and the widening left to the packing that follows.
+static bool corners_f32(ipeps_ctm h) {
+  const long long c = h->chi, D4 = (long long)h->D2 * h->D2;
+  return tc_product(h, c * c, D4, D4) && c * c <= 2000000;
+}
+
+// raw: corners as corners_f32 states (the caller packs them), else matrices
+static ipeps_status enlarged_corners(ipeps_ctm h, int f, int x, int y, bool raw) {
   const int c = h->chi, D2 = h->D2;
-  const long long entry = h->scratch_top;
+  const long long entry = h->scratch_top, D4 = (long long)D2 * D2;
+  const bool q32 = raw && corners_f32(h);
+  // ((C T) T) between its two products
+  const bool w32 = f32_between(h, (long long)c * D2, (long long)c * D2, c, (long long)c * c, D4, D4);
   cplx* w1 = scratch_alloc(h, (long long)c * D2 * c);
   cplx* w2 = scratch_alloc(h, (long long)h->K * h->K);
   if (!w1 || !w2) return fail(IPEPS_ENOMEM, "scratch exhausted (corners)");
   const long long mark = h->scratch_top;
+  // the last product of corner q: `in` -> [x a, y b], or [x y a b] with q32
+  auto last = [&](const char* in, const char* xayb, const char* xyab, TV w, cplx* a, int q) -> ipeps_status {
+    const std::string spec = std::string(in) + "->" + (q32 ? xyab : xayb);
+    const TV A = tv(a, {D2, D2, D2, D2});
+    return contract(h, spec.c_str(), w, false, A, false, q32 ? tv(h->Q[q], {c, c, D2, D2}, true) : tv(h->Q[q], {c, D2, c, D2}));
+  };
   // Q1 = ((C1 T1) T4) a
   CKS(contract(h, "ab,bcr->acr", tv(envC(h, f, 0, x, y), {c, c}), false,
                tv(envT(h, f, 0, x, y), {c, D2, c}), false, tv(w1, {c, D2, c})));
   CKS(contract(h, "dea,acr->decr", tv(envT(h, f, 3, x, y), {c, D2, c}), false, tv(w1, {c, D2, c}),
-               false, tv(w2, {c, D2, D2, c})));
-  CKS(contract(h, "decr,ceDR->dDrR", tv(w2, {c, D2, D2, c}), false,
-               tv(site_a(h, f, x, y), {D2, D2, D2, D2}), false, tv(h->Q[0], {c, D2, c, D2})));
+               false, tv(w2, {c, D2, D2, c}, w32)));
+  CKS(last("decr,ceDR", "dDrR", "drDR", tv(w2, {c, D2, D2, c}, w32), site_a(h, f, x, y), 0));
   h->scratch_top = mark;
   if (two_corners(h)) goto lower_left;  // Q2 and Q3 are not part of the two-corner ring
   // Q2 = ((T1 C2) T2) a
   CKS(contract(h, "Ltg,gh->Lth", tv(envT(h, f, 0, x + 1, y), {c, D2, c}), false,
                tv(envC(h, f, 1, x + 1, y), {c, c}), false, tv(w1, {c, D2, c})));
   CKS(contract(h, "Lth,hmE->LtmE", tv(w1, {c, D2, c}), false, tv(envT(h, f, 1, x + 1, y), {c, D2, c}),
-               false, tv(w2, {c, D2, D2, c})));
-  CKS(contract(h, "LtmE,tKem->LKEe", tv(w2, {c, D2, D2, c}), false,
-               tv(site_a(h, f, x + 1, y), {D2, D2, D2, D2}), false, tv(h->Q[1], {c, D2, c, D2})));
+               false, tv(w2, {c, D2, D2, c}, w32)));
+  CKS(last("LtmE,tKem", "LKEe", "LEKe", tv(w2, {c, D2, D2, c}, w32), site_a(h, f, x + 1, y), 1));
   h->scratch_top = mark;
   // Q3 = ((T2 C3) T3) a
   CKS(contract(h, "Umh,hg->Umg", tv(envT(h, f, 1, x + 1, y + 1), {c, D2, c}), false,
                tv(envC(h, f, 2, x + 1, y + 1), {c, c}), false, tv(w1, {c, D2, c})));
   CKS(contract(h, "Umg,gtL->UmtL", tv(w1, {c, D2, c}), false,
-               tv(envT(h, f, 2, x + 1, y + 1), {c, D2, c}), false, tv(w2, {c, D2, D2, c})));
-  CKS(contract(h, "UmtL,uKtm->UuLK", tv(w2, {c, D2, D2, c}), false,
-               tv(site_a(h, f, x + 1, y + 1), {D2, D2, D2, D2}), false, tv(h->Q[2], {c, D2, c, D2})));
+               tv(envT(h, f, 2, x + 1, y + 1), {c, D2, c}), false, tv(w2, {c, D2, D2, c}, w32)));
+  CKS(last("UmtL,uKtm", "UuLK", "ULuK", tv(w2, {c, D2, D2, c}, w32), site_a(h, f, x + 1, y + 1), 2));
   h->scratch_top = mark;
 lower_left:
   // Q4 = ((C4 T4) T3) a
   CKS(contract(h, "gh,hmU->gmU", tv(envC(h, f, 3, x, y + 1), {c, c}), false,
                tv(envT(h, f, 3, x, y + 1), {c, D2, c}), false, tv(w1, {c, D2, c})));
   CKS(contract(h, "gmU,Rtg->mUtR", tv(w1, {c, D2, c}), false, tv(envT(h, f, 2, x, y + 1), {c, D2, c}),
-               false, tv(w2, {D2, c, D2, c})));
-  CKS(contract(h, "mUtR,umtr->UuRr", tv(w2, {D2, c, D2, c}), false,
-               tv(site_a(h, f, x, y + 1), {D2, D2, D2, D2}), false, tv(h->Q[3], {c, D2, c, D2})));
+               false, tv(w2, {D2, c, D2, c}, w32)));
+  CKS(last("mUtR,umtr", "UuRr", "URur", tv(w2, {D2, c, D2, c}, w32), site_a(h, f, x, y + 1), 3));
   h->scratch_top = entry;
   return IPEPS_OK;
 }
@@ -1284,7 +1323,7 @@ static ipeps_status thin_chain(ipeps_ctm h, const cplx* in, bool conj_in, std::i
 static ipeps_status pack_corners(ipeps_ctm h) {
   for (int q = 0; q < 4; ++q) {
     if (two_corners(h) && (q == 1 || q == 2)) continue;
-    CK(tc_pack_square(h->stream, (int)h->opt.prec, h->Q[q], h->K, h->Qpmem[q][0], h->Qpmem[q][1], &h->Qp[q][0],
+    CK(tc_pack_square(h->stream, (int)h->opt.prec, h->Q[q], h->K, corners_f32(h) ? h->D2 : 0, h->Qpmem[q][0], h->Qpmem[q][1], &h->Qp[q][0],
                       &h->Qp[q][1]));
   }
   return IPEPS_OK;
@@ -1497,7 +1536,7 @@ static ipeps_status svd_rows_chol(ipeps_ctm h, const cplx* Wt, cplx* out, cplx* 
 
 // Projectors of the left cut of plaquette (x,y): PT = P^T, Ptil (both chi x K).
 static ipeps_status projectors(ipeps_ctm h, int f, int x, int y, cplx* PT, cplx* Ptil) {
-  CKS(enlarged_corners(h, f, x, y));
+  CKS(enlarged_corners(h, f, x, y, packed_path(h)));
   const int k = h->k, K = h->K, chi = h->chi;
   // CholeskyQR on FP64-accurate Grams, or Jacobi on the full rows (chol_route)
   const bool jacobi_bases = !chol_route(h->opt);
@@ -1612,13 +1651,15 @@ static ipeps_status left_move(ipeps_ctm h, int f) {
       CKS(contract(h, "nas,asr->nr", tv(h->PT[ym], {c, c, D2}), false, tv(w1, {c, D2, c}), false,
                    tv(h->spareC[0][y], {c, c})));
       // T4'[b,r,a] = sum P[(e,h),b] T4[e,m,f] a[g,m,h,r] Ptil[a,(f,g)]
+      const long long cD = (long long)c * D2, cc = (long long)c * c, D4 = (long long)D2 * D2;
+      const bool w2f = f32_between(h, cD, cD, c, cc, D4, D4), w3f = f32_between(h, cc, D4, D4, cD, c, cD);
       CKS(contract(h, "emf,beh->mfhb", tv(envT(h, f, 3, x, y), {c, D2, c}), false,
-                   tv(h->PT[y], {c, c, D2}), false, tv(w2, {D2, c, D2, c})));
+                   tv(h->PT[y], {c, c, D2}), false, tv(w2, {D2, c, D2, c}, w2f)));
       cplx* w3 = scratch_alloc(h, (long long)c * D2 * c * D2);
       if (!w3) return fail(IPEPS_ENOMEM, "scratch exhausted (absorb)");
-      CKS(contract(h, "mfhb,gmhr->fbgr", tv(w2, {D2, c, D2, c}), false,
-                   tv(site_a(h, f, x, y), {D2, D2, D2, D2}), false, tv(w3, {c, c, D2, D2})));
-      CKS(contract(h, "fbgr,afg->bra", tv(w3, {c, c, D2, D2}), false, tv(h->Ptil[ym], {c, c, D2}),
+      CKS(contract(h, "mfhb,gmhr->fbgr", tv(w2, {D2, c, D2, c}, w2f), false,
+                   tv(site_a(h, f, x, y), {D2, D2, D2, D2}), false, tv(w3, {c, c, D2, D2}, w3f)));
+      CKS(contract(h, "fbgr,afg->bra", tv(w3, {c, c, D2, D2}, w3f), false, tv(h->Ptil[ym], {c, c, D2}),
                    false, tv(h->spareT[y], {c, D2, c})));
       // C4'[r,a] = sum (C4 T3)[r,s,u] Ptil[a,(u,s)]
       CKS(contract(h, "gu,rsg->rsu", tv(envC(h, f, 3, x, y), {c, c}), false,
@@ -1877,26 +1918,43 @@ extern "C" ipeps_status ipeps_ctm_converge(ipeps_ctm h, double tol, int max_swee
 // ---------------------------------------------------------------------------
 // RDMs and energy (frame f horizontal bond (x,y)-(x+1,y))
 // ---------------------------------------------------------------------------
+// The FP32 intermediates of an RDM half (f32_between) in its four products: C
+// T T (two, three), the ket tensor, the lower corner and edge, the bra tensor.
+// `open`: the half's own result, for the bond's last product.
+struct HalfF32 {
+  bool two, ket, low, open;
+};
+static HalfF32 half_f32(ipeps_ctm h) {
+  const long long c = h->chi, D = h->D, d = h->d, D2 = D * D, c2 = c * c;
+  const long long p2[3] = {c * D2, c * D2, c}, p3[3] = {c2 * D2, d * D2, D2}, p4[3] = {c * D2 * d * D, c * D, c * D},
+                  p5[3] = {c2 * d * D, d * D, D2 * D}, p6[3] = {d * d, d * d, c2 * D2};
+  auto between = [&](const long long* a, const long long* b) {
+    return f32_between(h, a[0], a[1], a[2], b[0], b[1], b[2]);
+  };
+  return {between(p2, p3), between(p3, p4), between(p4, p5), between(p5, p6)};
+}
+
 // Left half of the window of site (x,y) in frame f, its physical legs open:
-// C1 T1 / T4 [A, A*] / C4 T3 contracted into left[h, r, s, k, p, q] with h
+// C1 T1 / T4 [A, A*] / C4 T3 contracted into left[h, p, r, k, q, s] with h
 // T1's right leg, (r, s) the site's right double leg (ket, bra), k T3's right
-// leg and (p, q) the physical (ket, bra) pair.  L2, L3, L4, small are work.
+// leg and (p, q) the physical (ket, bra) pair: the order in which the last
+// product leaves them.  L2, L3, L4, small are work; F: which are FP32.
 static ipeps_status rdm_left_half(ipeps_ctm h, int f, int x, int y, cplx* L2, cplx* L3, cplx* L4, cplx* small,
-                                  cplx* left) {
+                                  cplx* left, HalfF32 F) {
   const int c = h->chi, D = h->D, d = h->d;
   const cplx* Aa = h->A[f][tensor_id(h, f, x, y)];
   CKS(contract(h, "ab,bUVh->aUVh", tv(envC(h, f, 0, x, y), {c, c}), false,
                tv(envT(h, f, 0, x, y), {c, D, D, c}), false, tv(small, {c, D, D, c})));
   CKS(contract(h, "eLMa,aUVh->eLMUVh", tv(envT(h, f, 3, x, y), {c, D, D, c}), false,
-               tv(small, {c, D, D, c}), false, tv(L2, {c, D, D, D, D, c})));
-  CKS(contract(h, "eLMUVh,pULSr->eMVhpSr", tv(L2, {c, D, D, D, D, c}), false,
-               tv((cplx*)Aa, {d, D, D, D, D}), false, tv(L3, {c, D, D, c, d, D, D})));
+               tv(small, {c, D, D, c}), false, tv(L2, {c, D, D, D, D, c}, F.two)));
+  CKS(contract(h, "eLMUVh,pULSr->eMVhpSr", tv(L2, {c, D, D, D, D, c}, F.two), false,
+               tv((cplx*)Aa, {d, D, D, D, D}), false, tv(L3, {c, D, D, c, d, D, D}, F.ket)));
   CKS(contract(h, "ge,kSTg->ekST", tv(envC(h, f, 3, x, y), {c, c}), false,
                tv(envT(h, f, 2, x, y), {c, D, D, c}), false, tv(small, {c, c, D, D})));
-  CKS(contract(h, "eMVhpSr,ekST->MVhprkT", tv(L3, {c, D, D, c, d, D, D}), false,
-               tv(small, {c, c, D, D}), false, tv(L4, {D, D, c, d, D, c, D})));
-  CKS(contract(h, "MVhprkT,qVMTs->hrskpq", tv(L4, {D, D, c, d, D, c, D}), false,
-               tv((cplx*)Aa, {d, D, D, D, D}), true, tv(left, {c, D, D, c, d, d})));
+  CKS(contract(h, "eMVhpSr,ekST->MVhprkT", tv(L3, {c, D, D, c, d, D, D}, F.ket), false,
+               tv(small, {c, c, D, D}), false, tv(L4, {D, D, c, d, D, c, D}, F.low)));
+  CKS(contract(h, "MVhprkT,qVMTs->hprkqs", tv(L4, {D, D, c, d, D, c, D}, F.low), false,
+               tv((cplx*)Aa, {d, D, D, D, D}), true, tv(left, {c, d, D, c, d, D}, F.open)));
   return IPEPS_OK;
 }
 
@@ -1904,6 +1962,7 @@ static ipeps_status rdm_horizontal(ipeps_ctm h, int f, int x, int y, cplx* rho) 
   const int c = h->chi, D = h->D, d = h->d;
   const cplx* Ab = h->A[f][tensor_id(h, f, x + 1, y)];
   const long long big = (long long)c * c * D * D * D * D * d;
+  const HalfF32 F = half_f32(h);
   cplx* L2 = scratch_alloc(h, (long long)c * c * D * D * D * D);
   cplx* L3 = scratch_alloc(h, big);
   cplx* L4 = scratch_alloc(h, big);
@@ -1911,22 +1970,22 @@ static ipeps_status rdm_horizontal(ipeps_ctm h, int f, int x, int y, cplx* rho) 
   cplx* right = scratch_alloc(h, (long long)c * c * D * D * d * d);
   cplx* small = scratch_alloc(h, (long long)c * c * D * D);
   if (!L2 || !L3 || !L4 || !left || !right || !small) return fail(IPEPS_ENOMEM, "scratch exhausted (rdm)");
-  CKS(rdm_left_half(h, f, x, y, L2, L3, L4, small, left));
-  // right half
+  CKS(rdm_left_half(h, f, x, y, L2, L3, L4, small, left, F));
+  // right half [h, p, l, k, q, m]
   CKS(contract(h, "hUVc,cf->hUVf", tv(envT(h, f, 0, x + 1, y), {c, D, D, c}), false,
                tv(envC(h, f, 1, x + 1, y), {c, c}), false, tv(small, {c, D, D, c})));
   CKS(contract(h, "hUVf,fRSg->hUVRSg", tv(small, {c, D, D, c}), false,
-               tv(envT(h, f, 1, x + 1, y), {c, D, D, c}), false, tv(L2, {c, D, D, D, D, c})));
-  CKS(contract(h, "hUVRSg,pUlXR->hVSgplX", tv(L2, {c, D, D, D, D, c}), false,
-               tv((cplx*)Ab, {d, D, D, D, D}), false, tv(L3, {c, D, D, c, d, D, D})));
+               tv(envT(h, f, 1, x + 1, y), {c, D, D, c}), false, tv(L2, {c, D, D, D, D, c}, F.two)));
+  CKS(contract(h, "hUVRSg,pUlXR->hVSgplX", tv(L2, {c, D, D, D, D, c}, F.two), false,
+               tv((cplx*)Ab, {d, D, D, D, D}), false, tv(L3, {c, D, D, c, d, D, D}, F.ket)));
   CKS(contract(h, "gi,iXYk->gXYk", tv(envC(h, f, 2, x + 1, y), {c, c}), false,
                tv(envT(h, f, 2, x + 1, y), {c, D, D, c}), false, tv(small, {c, D, D, c})));
-  CKS(contract(h, "hVSgplX,gXYk->hVSplYk", tv(L3, {c, D, D, c, d, D, D}), false,
-               tv(small, {c, D, D, c}), false, tv(L4, {c, D, D, d, D, D, c})));
-  CKS(contract(h, "hVSplYk,qVmYS->hlmkpq", tv(L4, {c, D, D, d, D, D, c}), false,
-               tv((cplx*)Ab, {d, D, D, D, D}), true, tv(right, {c, D, D, c, d, d})));
-  CKS(contract(h, "hrskpq,hrskPQ->pPqQ", tv(left, {c, D, D, c, d, d}), false,
-               tv(right, {c, D, D, c, d, d}), false, tv(rho, {d, d, d, d})));
+  CKS(contract(h, "hVSgplX,gXYk->hVSplYk", tv(L3, {c, D, D, c, d, D, D}, F.ket), false,
+               tv(small, {c, D, D, c}), false, tv(L4, {c, D, D, d, D, D, c}, F.low)));
+  CKS(contract(h, "hVSplYk,qVmYS->hplkqm", tv(L4, {c, D, D, d, D, D, c}, F.low), false,
+               tv((cplx*)Ab, {d, D, D, D, D}), true, tv(right, {c, d, D, c, d, D}, F.open)));
+  CKS(contract(h, "hprkqs,hPrkQs->pPqQ", tv(left, {c, d, D, c, d, D}, F.open), false,
+               tv(right, {c, d, D, c, d, D}, F.open), false, tv(rho, {d, d, d, d})));
   CK(trace_normalize(h->stream, rho, d * d, h->dwork));
   h->scratch_top = 0;
   return IPEPS_OK;
@@ -1944,12 +2003,14 @@ static ipeps_status rdm_site(ipeps_ctm h, int x, int y, cplx* rho) {
   cplx* small = scratch_alloc(h, (long long)c * c * D * D);
   cplx* col = scratch_alloc(h, (long long)c * c * D * D);
   if (!L2 || !L3 || !L4 || !left || !small || !col) return fail(IPEPS_ENOMEM, "scratch exhausted (site rdm)");
-  CKS(rdm_left_half(h, 0, x, y, L2, L3, L4, small, left));
+  HalfF32 F = half_f32(h);
+  F.open = false;  // its last product has one column: FP64 CUDA cores
+  CKS(rdm_left_half(h, 0, x, y, L2, L3, L4, small, left, F));
   CKS(contract(h, "hf,fRSg->hRSg", tv(envC(h, 0, 1, x, y), {c, c}), false,
                tv(envT(h, 0, 1, x, y), {c, D, D, c}), false, tv(small, {c, D, D, c})));
   CKS(contract(h, "hRSg,gk->hRSk", tv(small, {c, D, D, c}), false, tv(envC(h, 0, 2, x, y), {c, c}), false,
                tv(col, {c, D, D, c})));
-  CKS(contract(h, "hrskpq,hrsk->pq", tv(left, {c, D, D, c, d, d}), false, tv(col, {c, D, D, c}), false,
+  CKS(contract(h, "hprkqs,hrsk->pq", tv(left, {c, d, D, c, d, D}), false, tv(col, {c, D, D, c}), false,
                tv(rho, {d, d})));
   CK(trace_normalize(h->stream, rho, d, h->dwork));
   h->scratch_top = 0;
@@ -2160,7 +2221,7 @@ static ipeps_status window_contract(ipeps_ctm h, bool rows, bool cols, cplx* res
   const int c = h->chi, D2 = h->D2, Lx = h->Lx, Ly = h->Ly, W = 2;
   const long long mark = h->scratch_top;
   if (rows && cols) {
-    CKS(enlarged_corners(h, 0, 0, 0));
+    CKS(enlarged_corners(h, 0, 0, 0, false));
     const long long K = h->K;
     cplx* Rup = scratch_alloc(h, K * K);
     cplx* Rdn = scratch_alloc(h, K * K);

@@ -33,6 +33,7 @@ namespace {
 // padded N is a multiple of 256
 constexpr int BM = 128, NPAD = 128;
 constexpr int NTHREADS = 192;        // main kernel: producer warp, MMA warp, four epilogue warps
+constexpr int EPI_LD = 18, EPI_FLOATS = 32 * EPI_LD;  // an epilogue warp's 32 rows x 16 columns
 constexpr int PREC_TF32 = 1, PREC_BF16X3 = 2, PREC_BF16X6 = 3;
 
 
@@ -56,7 +57,8 @@ struct Cfg {
   static_assert(STAGES >= 2, "at least two pipeline stages");
   static constexpr int UMMA_K = PREC == PREC_TF32 ? 8 : 16;  // K of one MMA
   static constexpr int KSTEPS = BK / UMMA_K;
-  static constexpr int SMEM = STAGES * STAGE_BYTES + 1024 + 256;
+  // stages, alignment, barriers, the epilogue warps' transpose buffers
+  static constexpr int SMEM = STAGES * STAGE_BYTES + 1024 + 256 + 4 * EPI_FLOATS * 4;
   // instruction descriptor: FP32 accumulate, K-major A and B, N = BN, M = 128
   static constexpr uint32_t IDESC = (1u << 4) | ((PREC == PREC_TF32 ? 2u : 1u) << 7) |
                                     ((PREC == PREC_TF32 ? 2u : 1u) << 10) |
@@ -92,8 +94,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                    const __grid_constant__ CUtensorMap mA2, const __grid_constant__ CUtensorMap mB0,
                    const __grid_constant__ CUtensorMap mB1, const __grid_constant__ CUtensorMap mB2,
                    int kb_total, int kb_per_split, int n_tiles, int m_tiles, int tiles, int M, int Nr, cplx alpha,
-                   cplx* __restrict__ C, long long ldc, float* __restrict__ partial, int Nrp, long long pstride,
-                   int conj_out, int unit_alpha, int* __restrict__ timeouts) {
+                   void* __restrict__ Cv, long long ldc, float* __restrict__ partial, int Nrp, long long pstride,
+                   int conj_out, int unit_alpha, int out_f32, int* __restrict__ timeouts) {
   using K_ = Cfg<PREC, BN>;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -225,6 +227,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   } else if (warp >= 2) {
     // epilogue: warp w drains tensor-memory lanes 32 (w % 4) .. (the rows of its quarter)
     const int quad = warp & 3;
+    float* epi = (float*)(smem + K_::STAGES * K_::STAGE_BYTES + 256) + quad * EPI_FLOATS;
     int it = 0;
     for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++it) {
       const int split = t / (n_tiles * m_tiles);
@@ -237,34 +240,41 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         break;
       }
       fence_after();
-      const int row = m_tile * BM + quad * 32 + lane;
       const uint32_t trow = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(b * BN);
       for (int c0 = 0; c0 < BN; c0 += 16) {
+        // a lane drains 16 columns of its row; through shared memory eight lanes
+        // take a row's 8 complex numbers, so that a store instruction writes
+        // four runs of 64 (FP32) or 128 (FP64) bytes instead of 32 pieces of 16
         float v[16];
         tmem_ld16(trow + c0, v);
-        const int col = n_tile * BN + c0;  // real column
-        if (partial) {
-          float4* dst = (float4*)(partial + split * pstride + (long long)row * Nrp + col);
+        if (partial) {  // rows of whole 64-byte runs per lane: written as they are
+          float4* dst = (float4*)(partial + split * pstride + (long long)(m_tile * BM + quad * 32 + lane) * Nrp +
+                                  n_tile * BN + c0);
 #pragma unroll
           for (int q = 0; q < 4; ++q) dst[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-        } else if (row < M) {
-          if (unit_alpha) {
-            // alpha = 1: exact FP32 -> FP64 widening on the integer pipe
+          continue;
+        }
+        __syncwarp();
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-              if (col + 2 * u < Nr) {
-                const double re = f2d_bits(v[2 * u]), im = f2d_bits(v[2 * u + 1]);
-                C[(long long)row * ldc + (col >> 1) + u] = make_double2(re, conj_out ? neg_bits(im) : im);
-              }
-            }
-          } else {
+        for (int q = 0; q < 8; ++q) *(float2*)(epi + lane * EPI_LD + 2 * q) = make_float2(v[2 * q], v[2 * q + 1]);
+        __syncwarp();
+        const int u = lane & 7, col = n_tile * BN + c0 + 2 * u;  // real column
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-              if (col + 2 * u < Nr) {
-                const double re = v[2 * u], im = v[2 * u + 1];
-                const double orr = alpha.x * re - alpha.y * im, oi = alpha.x * im + alpha.y * re;
-                C[(long long)row * ldc + (col >> 1) + u] = make_double2(orr, conj_out ? -oi : oi);
-              }
+        for (int q = 0; q < 8; ++q) {
+          const int r = 4 * q + (lane >> 3), row = m_tile * BM + quad * 32 + r;
+          const float2 x = *(const float2*)(epi + r * EPI_LD + 2 * u);
+          if (row < M && col < Nr) {
+            const long long o = (long long)row * ldc + (col >> 1);
+            if (out_f32) {
+              ((float2*)Cv)[o] = x;
+            } else if (unit_alpha) {
+              // alpha = 1: exact FP32 -> FP64 widening on the integer pipe
+              const double re = f2d_bits(x.x), im = f2d_bits(x.y);
+              ((cplx*)Cv)[o] = make_double2(re, conj_out ? neg_bits(im) : im);
+            } else {
+              const double re = x.x, im = x.y;
+              const double orr = alpha.x * re - alpha.y * im, oi = alpha.x * im + alpha.y * re;
+              ((cplx*)Cv)[o] = make_double2(orr, conj_out ? -oi : oi);
             }
           }
         }
@@ -283,8 +293,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 
 // C[m,n] = alpha * sum_z P[z][m][2n .. 2n+1]  (fixed summation order)
 __global__ void splitk_reduce_kernel(const float* __restrict__ P, int S, long long pstride, int Nrp, int M,
-                                     int N, cplx alpha, cplx* __restrict__ C, long long ldc, int conj_out,
-                                     int unit_alpha) {
+                                     int N, cplx alpha, void* __restrict__ Cv, long long ldc, int conj_out,
+                                     int unit_alpha, int out_f32) {
+  cplx* C = (cplx*)Cv;
   const long long total = (long long)M * N;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
        e += (long long)gridDim.x * blockDim.x) {
@@ -293,10 +304,15 @@ __global__ void splitk_reduce_kernel(const float* __restrict__ P, int S, long lo
       // FP32 sum of the partials (the products carry ~16 significant bits),
       // widened to FP64 on the integer pipe
       float re = 0.0f, im = 0.0f;
-      for (int z = 0; z < S; ++z) {
+#pragma unroll 8
+      for (int z = 0; z < S; ++z) {  // eight loads in flight, added in order
         const float2 p = *(const float2*)(P + z * pstride + (long long)m * Nrp + 2 * n);
         re += p.x;
         im += p.y;
+      }
+      if (out_f32) {
+        ((float2*)Cv)[(long long)m * ldc + n] = make_float2(re, im);
+        continue;
       }
       const double dr = f2d_bits(re), di = f2d_bits(im);
       C[(long long)m * ldc + n] = make_double2(dr, conj_out ? neg_bits(di) : di);
@@ -316,8 +332,9 @@ __global__ void splitk_reduce_kernel(const float* __restrict__ P, int S, long lo
 // The same with a warp per output for many splits: lane l sums splits
 // l, l + 32, ... in order, then the lanes' sums meet in a fixed butterfly.
 __global__ void splitk_reduce_warp_kernel(const float* __restrict__ P, int S, long long pstride, int Nrp, int M,
-                                          int N, cplx alpha, cplx* __restrict__ C, long long ldc, int conj_out,
-                                          int unit_alpha) {
+                                          int N, cplx alpha, void* __restrict__ Cv, long long ldc, int conj_out,
+                                          int unit_alpha, int out_f32) {
+  cplx* C = (cplx*)Cv;
   const int lane = threadIdx.x & 31;
   const long long total = (long long)M * N;
   for (long long e = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; e < total;
@@ -335,7 +352,9 @@ __global__ void splitk_reduce_warp_kernel(const float* __restrict__ P, int S, lo
       im += __shfl_xor_sync(0xffffffffu, im, o);
     }
     if (lane != 0) continue;
-    if (unit_alpha) {
+    if (out_f32) {
+      ((float2*)Cv)[(long long)m * ldc + n] = make_float2(re, im);
+    } else if (unit_alpha) {
       const double dr = f2d_bits(re), di = f2d_bits(im);
       C[(long long)m * ldc + n] = make_double2(dr, conj_out ? neg_bits(di) : di);
     } else {
@@ -378,25 +397,42 @@ __device__ __forceinline__ void split3(float f, __nv_bfloat16& p0, __nv_bfloat16
   p2 = __float2bfloat16_rn(r1 - __bfloat162float(p1));
 }
 
-__device__ __forceinline__ void store_pair(int prec, long long e, double x0, double x1, void* o0, void* o1,
-                                           void* o2) {
+// the FP32 value of a packed real: rounded for the three-part split, which
+// keeps all 24 bits, truncated for the others
+template <int PREC>
+__device__ __forceinline__ float pack_f32(double x) {
+  return PREC == PREC_BF16X6 ? d2f_rn_bits(x) : d2f_bits(x);
+}
+
+template <int PREC>
+__device__ __forceinline__ void store_pair(long long e, float x0, float x1, void* o0, void* o1, void* o2) {
   // two consecutive packed reals at element e (e even)
-  if (prec == PREC_TF32) {
-    ((uint2*)o0)[e >> 1] = make_uint2(to_tf32(d2f_bits(x0)), to_tf32(d2f_bits(x1)));
-  } else if (prec == PREC_BF16X6) {
+  if (PREC == PREC_TF32) {
+    ((uint2*)o0)[e >> 1] = make_uint2(to_tf32(x0), to_tf32(x1));
+  } else if (PREC == PREC_BF16X6) {
     __nv_bfloat16 a0, a1, a2, c0, c1, c2;
-    split3(d2f_rn_bits(x0), a0, a1, a2);
-    split3(d2f_rn_bits(x1), c0, c1, c2);
+    split3(x0, a0, a1, a2);
+    split3(x1, c0, c1, c2);
     ((__nv_bfloat162*)o0)[e >> 1] = __halves2bfloat162(a0, c0);
     ((__nv_bfloat162*)o1)[e >> 1] = __halves2bfloat162(a1, c1);
     ((__nv_bfloat162*)o2)[e >> 1] = __halves2bfloat162(a2, c2);
   } else {
-    const float f0 = d2f_bits(x0), f1 = d2f_bits(x1);
-    const __nv_bfloat16 h0 = __float2bfloat16_rn(f0), h1 = __float2bfloat16_rn(f1);
-    const __nv_bfloat16 l0 = __float2bfloat16_rn(f0 - __bfloat162float(h0));
-    const __nv_bfloat16 l1 = __float2bfloat16_rn(f1 - __bfloat162float(h1));
+    const __nv_bfloat16 h0 = __float2bfloat16_rn(x0), h1 = __float2bfloat16_rn(x1);
+    const __nv_bfloat16 l0 = __float2bfloat16_rn(x0 - __bfloat162float(h0));
+    const __nv_bfloat16 l1 = __float2bfloat16_rn(x1 - __bfloat162float(h1));
     ((__nv_bfloat162*)o0)[e >> 1] = __halves2bfloat162(h0, h1);
     ((__nv_bfloat162*)o1)[e >> 1] = __halves2bfloat162(l0, l1);
+  }
+}
+
+// element at offset o of a complex FP64 (F32: complex FP32) source as FP32 parts
+template <int PREC, bool F32>
+__device__ __forceinline__ float2 load_f32(const void* p, long long o) {
+  if constexpr (F32) {
+    return ((const float2*)p)[o];
+  } else {
+    const cplx v = ((const cplx*)p)[o];
+    return make_float2(pack_f32<PREC>(v.x), pack_f32<PREC>(v.y));
   }
 }
 
@@ -410,7 +446,7 @@ __global__ void pack_a_kernel(const cplx* __restrict__ A, long long lda, int opA
     const Idx m = e / kc, k = e - m * kc;
     cplx v = make_double2(0.0, 0.0);
     if ((int)m < M && (int)k < K) v = load_op(A, lda, opA, (int)m, (int)k);
-    store_pair(PREC, (long long)m * Krp + 2 * (long long)k, v.x, v.y, o0, o1, o2);
+    store_pair<PREC>((long long)m * Krp + 2 * (long long)k, pack_f32<PREC>(v.x), pack_f32<PREC>(v.y), o0, o1, o2);
   }
 }
 
@@ -425,8 +461,9 @@ __global__ void pack_b_kernel(const cplx* __restrict__ B, long long ldb, int opB
     cplx v = make_double2(0.0, 0.0);
     if ((int)n < N && (int)k < K) v = load_op(B, ldb, opB, (int)k, (int)n);
     const long long r0 = (long long)(2 * n) * Krp + 2 * (long long)k;
-    store_pair(PREC, r0, v.x, neg_bits(v.y), o0, o1, o2);
-    store_pair(PREC, r0 + Krp, v.y, v.x, o0, o1, o2);
+    const float x = pack_f32<PREC>(v.x), y = pack_f32<PREC>(v.y);
+    store_pair<PREC>(r0, x, -y, o0, o1, o2);
+    store_pair<PREC>(r0 + Krp, y, x, o0, o1, o2);
   }
 }
 
@@ -436,14 +473,14 @@ __global__ void pack_b_kernel(const cplx* __restrict__ B, long long ldb, int opB
 template <int PREC>
 __global__ void pack_b_tr_kernel(const cplx* __restrict__ B, long long ldb, int conj, int N, int K, int Nrp,
                                  int Krp, void* __restrict__ o0, void* __restrict__ o1, void* __restrict__ o2) {
-  __shared__ cplx tile[32][33];
+  __shared__ float2 tile[32][33];
   const int k0 = blockIdx.y * 32, n0 = blockIdx.x * 32;
   for (int i = threadIdx.y; i < 32; i += blockDim.y) {
     const int k = k0 + i, n = n0 + threadIdx.x;
-    cplx v = make_double2(0.0, 0.0);
+    float2 v = make_float2(0.f, 0.f);
     if (k < K && n < N) {
-      v = B[(long long)k * ldb + n];
-      if (conj) v.y = neg_bits(v.y);
+      v = load_f32<PREC, false>(B, (long long)k * ldb + n);
+      if (conj) v.y = -v.y;
     }
     tile[i][threadIdx.x] = v;
   }
@@ -455,12 +492,12 @@ __global__ void pack_b_tr_kernel(const cplx* __restrict__ B, long long ldb, int 
   for (int r = threadIdx.y; r < 64; r += blockDim.y) {
     const int nr = 2 * n0 + r;
     if (nr >= Nrp) break;
-    const cplx v = tile[threadIdx.x][r >> 1];
+    const float2 v = tile[threadIdx.x][r >> 1];
     const long long e = (long long)nr * Krp + 2 * (long long)k;
     if (r & 1)
-      store_pair(PREC, e, v.y, v.x, o0, o1, o2);  // row 2n+1: (Im, Re)
+      store_pair<PREC>(e, v.y, v.x, o0, o1, o2);  // row 2n+1: (Im, Re)
     else
-      store_pair(PREC, e, v.x, neg_bits(v.y), o0, o1, o2);  // row 2n: (Re, -Im)
+      store_pair<PREC>(e, v.x, -v.y, o0, o1, o2);  // row 2n: (Re, -Im)
   }
 }
 
@@ -482,10 +519,10 @@ __device__ __forceinline__ long long view_off(unsigned idx, int n, const int* di
 // once per tile (the divisions of the index arithmetic would otherwise bound
 // the kernel); reads run along whichever of m or k is contiguous in the
 // source (row_contig: m), writes along k.
-template <int PREC>
+template <int PREC, bool F32>
 __global__ void pack_a_tiled_kernel(TcView V, int M, int K, int Mp, int Krp, int row_contig, void* __restrict__ o0,
                                     void* __restrict__ o1, void* __restrict__ o2) {
-  __shared__ cplx tile[32][33];
+  __shared__ float2 tile[32][33];
   __shared__ long long roff[32], coff[32];
   const int k0 = blockIdx.x * 32, m0 = blockIdx.y * 32;
   if (threadIdx.y == 0) {
@@ -496,10 +533,10 @@ __global__ void pack_a_tiled_kernel(TcView V, int M, int K, int Mp, int Krp, int
   __syncthreads();
   for (int i = threadIdx.y; i < 32; i += blockDim.y) {
     const int mi = row_contig ? (int)threadIdx.x : i, ki = row_contig ? i : (int)threadIdx.x;
-    cplx v = make_double2(0.0, 0.0);
+    float2 v = make_float2(0.f, 0.f);
     if (roff[mi] >= 0 && coff[ki] >= 0) {
-      v = V.p[roff[mi] + coff[ki]];
-      if (V.conj) v.y = neg_bits(v.y);
+      v = load_f32<PREC, F32>(V.p, roff[mi] + coff[ki]);
+      if (V.conj) v.y = -v.y;
     }
     tile[ki][mi] = v;
   }
@@ -509,18 +546,18 @@ __global__ void pack_a_tiled_kernel(TcView V, int M, int K, int Mp, int Krp, int
   for (int r = threadIdx.y; r < 32; r += blockDim.y) {
     const int m = m0 + r;
     if (m >= Mp) break;
-    const cplx v = tile[threadIdx.x][r];
-    store_pair(PREC, (long long)m * Krp + 2 * (long long)k, v.x, v.y, o0, o1, o2);
+    const float2 v = tile[threadIdx.x][r];
+    store_pair<PREC>((long long)m * Krp + 2 * (long long)k, v.x, v.y, o0, o1, o2);
   }
 }
 
 // Br^T[nr, kr] gathered through a view (rows n, columns k), padded to Nrp x Krp,
 // by 32 x 32 complex tiles as pack_a_tiled_kernel: complex (n, k) gives rows
 // 2n: (Re, -Im) and 2n+1: (Im, Re) at columns 2k, 2k+1
-template <int PREC>
+template <int PREC, bool F32>
 __global__ void pack_b_tiled_kernel(TcView V, int N, int K, int Nrp, int Krp, int row_contig, void* __restrict__ o0,
                                     void* __restrict__ o1, void* __restrict__ o2) {
-  __shared__ cplx tile[32][33];
+  __shared__ float2 tile[32][33];
   __shared__ long long roff[32], coff[32];
   const int k0 = blockIdx.x * 32, n0 = blockIdx.y * 32;
   if (threadIdx.y == 0) {
@@ -531,10 +568,10 @@ __global__ void pack_b_tiled_kernel(TcView V, int N, int K, int Nrp, int Krp, in
   __syncthreads();
   for (int i = threadIdx.y; i < 32; i += blockDim.y) {
     const int ni = row_contig ? (int)threadIdx.x : i, ki = row_contig ? i : (int)threadIdx.x;
-    cplx v = make_double2(0.0, 0.0);
+    float2 v = make_float2(0.f, 0.f);
     if (roff[ni] >= 0 && coff[ki] >= 0) {
-      v = V.p[roff[ni] + coff[ki]];
-      if (V.conj) v.y = neg_bits(v.y);
+      v = load_f32<PREC, F32>(V.p, roff[ni] + coff[ki]);
+      if (V.conj) v.y = -v.y;
     }
     tile[ki][ni] = v;
   }
@@ -544,12 +581,12 @@ __global__ void pack_b_tiled_kernel(TcView V, int N, int K, int Nrp, int Krp, in
   for (int r = threadIdx.y; r < 64; r += blockDim.y) {
     const int nr = 2 * n0 + r;
     if (nr >= Nrp) break;
-    const cplx v = tile[threadIdx.x][r >> 1];
+    const float2 v = tile[threadIdx.x][r >> 1];
     const long long e = (long long)nr * Krp + 2 * (long long)k;
     if (r & 1)
-      store_pair(PREC, e, v.y, v.x, o0, o1, o2);  // row 2n+1: (Im, Re)
+      store_pair<PREC>(e, v.y, v.x, o0, o1, o2);  // row 2n+1: (Im, Re)
     else
-      store_pair(PREC, e, v.x, neg_bits(v.y), o0, o1, o2);  // row 2n: (Re, -Im)
+      store_pair<PREC>(e, v.x, -v.y, o0, o1, o2);  // row 2n: (Re, -Im)
   }
 }
 
@@ -558,26 +595,38 @@ __global__ void pack_b_tiled_kernel(TcView V, int N, int K, int Nrp, int Krp, in
 // Q), oT rows n, columns k of Q[n, k] (for thin * Q^T), each Mp x Krp reals,
 // (Re, Im) pairs along k, padded with zeros.  32 x 32 complex tiles through
 // shared memory; both directions read and write 128-byte runs per warp.
-template <int PREC>
-__global__ void pack_square_kernel(const cplx* __restrict__ Q, int K, int Mp, int Krp, void* __restrict__ n0,
+template <int PREC, bool F32>
+__global__ void pack_square_kernel(const void* __restrict__ Q, int K, int D2, int Mp, int Krp, void* __restrict__ n0,
                                    void* __restrict__ n1, void* __restrict__ n2, void* __restrict__ t0,
                                    void* __restrict__ t1, void* __restrict__ t2) {
-  __shared__ cplx tile[32][33];
+  __shared__ float2 tile[32][33];
+  __shared__ long long roff[32], coff[32];
   const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32, kc = Krp >> 1;
   const int c = c0 + threadIdx.x;
+  if (threadIdx.y == 0) {
+    const int r = r0 + threadIdx.x;
+    if (F32) {  // [x][y][a][b]: row (x a), column (y b)
+      const long long d4 = (long long)D2 * D2;
+      roff[threadIdx.x] = r < K ? (long long)(r / D2) * (K / D2) * d4 + (long long)(r % D2) * D2 : -1;
+      coff[threadIdx.x] = c < K ? (long long)(c / D2) * d4 + c % D2 : -1;
+    } else {
+      roff[threadIdx.x] = r < K ? (long long)r * K : -1;
+      coff[threadIdx.x] = c < K ? c : -1;
+    }
+  }
+  __syncthreads();
   for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-    const int r = r0 + i;
-    cplx v = make_double2(0.0, 0.0);
-    if (r < K && c < K) v = Q[(long long)r * K + c];
+    float2 v = make_float2(0.f, 0.f);
+    if (roff[i] >= 0 && coff[threadIdx.x] >= 0) v = load_f32<PREC, F32>(Q, roff[i] + coff[threadIdx.x]);
     tile[i][threadIdx.x] = v;
-    if (c < kc) store_pair(PREC, (long long)r * Krp + 2 * (long long)c, v.x, v.y, t0, t1, t2);
+    if (c < kc) store_pair<PREC>((long long)(r0 + i) * Krp + 2 * (long long)c, v.x, v.y, t0, t1, t2);
   }
   __syncthreads();
   const int k = r0 + threadIdx.x;
   if (k >= kc) return;
   for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-    const cplx v = tile[threadIdx.x][i];
-    store_pair(PREC, (long long)(c0 + i) * Krp + 2 * (long long)k, v.x, v.y, n0, n1, n2);
+    const float2 v = tile[threadIdx.x][i];
+    store_pair<PREC>((long long)(c0 + i) * Krp + 2 * (long long)k, v.x, v.y, n0, n1, n2);
   }
 }
 
@@ -609,12 +658,14 @@ __global__ void thin_reduce_kernel(const float* __restrict__ P, int S, long long
   const int n = n0 + threadIdx.x;
   for (int i = threadIdx.y; i < 32; i += blockDim.y) {
     const float2 v = tile[threadIdx.x][i];
-    const double re = f2d_bits(v.x), im = f2d_bits(v.y);
-    if (C && m0 + i < M && n < N) C[(long long)(m0 + i) * ldc + n] = make_double2(re, conj_out ? neg_bits(im) : im);
+    if (C && m0 + i < M && n < N) {
+      const double re = f2d_bits(v.x), im = f2d_bits(v.y);
+      C[(long long)(m0 + i) * ldc + n] = make_double2(re, conj_out ? neg_bits(im) : im);
+    }
     if (o0 && 2 * n < Krp) {
       const long long e = 2LL * (m0 + i) * Krp + 2 * (long long)n;
-      store_pair(PREC, e, re, neg_bits(im), o0, o1, o2);
-      store_pair(PREC, e + Krp, im, re, o0, o1, o2);
+      store_pair<PREC>(e, v.x, -v.y, o0, o1, o2);
+      store_pair<PREC>(e + Krp, v.y, v.x, o0, o1, o2);
     }
   }
 }
@@ -728,8 +779,9 @@ cudaError_t ensure_attr() {
 }
 
 template <int PREC, int BN>
-cudaError_t launch_main(cudaStream_t s, const Operands& o, int S, int M, int N, cplx alpha, cplx* C, long long ldc,
-                        float* part, bool conj_out, int* timeouts, TcProbe* probe, bool partials_only = false) {
+cudaError_t launch_main(cudaStream_t s, const Operands& o, int S, int M, int N, cplx alpha, void* C, long long ldc,
+                        bool c_f32, float* part, int* timeouts, TcProbe* probe, bool partials_only = false) {
+  const int conj_out = 0;
   using K_ = Cfg<PREC, BN>;
   cudaError_t e;
   if ((e = ensure_attr<PREC, BN>()) != cudaSuccess) return e;
@@ -774,8 +826,7 @@ cudaError_t launch_main(cudaStream_t s, const Operands& o, int S, int M, int N, 
   tc_gemm_kernel<PREC, BN><<<grid, NTHREADS, K_::SMEM, s>>>(mA0, mA1, mA2, mB0, mB1, mB2, o.kb_total, kps, n_tiles,
                                                              m_tiles, (int)tiles, M, 2 * N, alpha, C, ldc,
                                                              S > 1 || partials_only ? part : nullptr, (int)o.Nrp,
-                                                             o.Mp * o.Nrp,
-                                                             conj_out ? 1 : 0, unit, timeouts);
+                                                             o.Mp * o.Nrp, conj_out, unit, c_f32 ? 1 : 0, timeouts);
   count_launch();
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (probe && (e = cudaEventRecord(probe->ev[1], s)) != cudaSuccess) return e;
@@ -783,10 +834,10 @@ cudaError_t launch_main(cudaStream_t s, const Operands& o, int S, int M, int N, 
   if (S > 1) {
     if (S >= 64)
       splitk_reduce_warp_kernel<<<grid_for(32LL * M * N), 256, 0, s>>>(part, S, o.Mp * o.Nrp, (int)o.Nrp, M, N, alpha,
-                                                                      C, ldc, conj_out ? 1 : 0, unit);
+                                                                      C, ldc, conj_out, unit, c_f32 ? 1 : 0);
     else
       splitk_reduce_kernel<<<grid_for((long long)M * N), 256, 0, s>>>(part, S, o.Mp * o.Nrp, (int)o.Nrp, M, N,
-                                                                      alpha, C, ldc, conj_out ? 1 : 0, unit);
+                                                                      alpha, C, ldc, conj_out, unit, c_f32 ? 1 : 0);
     count_launch();
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
@@ -795,11 +846,11 @@ cudaError_t launch_main(cudaStream_t s, const Operands& o, int S, int M, int N, 
 }
 
 template <int PREC>
-cudaError_t launch_choice(cudaStream_t s, const Operands& o, TcChoice c, int M, int N, cplx alpha, cplx* C,
-                          long long ldc, float* part, bool conj_out, int* timeouts, TcProbe* probe = nullptr) {
+cudaError_t launch_choice(cudaStream_t s, const Operands& o, TcChoice c, int M, int N, cplx alpha, void* C,
+                          long long ldc, bool c_f32, float* part, int* timeouts, TcProbe* probe = nullptr) {
   if (c.bn == 128 || o.Nrp % 256 != 0)
-    return launch_main<PREC, 128>(s, o, c.splits, M, N, alpha, C, ldc, part, conj_out, timeouts, probe);
-  return launch_main<PREC, 256>(s, o, c.splits, M, N, alpha, C, ldc, part, conj_out, timeouts, probe);
+    return launch_main<PREC, 128>(s, o, c.splits, M, N, alpha, C, ldc, c_f32, part, timeouts, probe);
+  return launch_main<PREC, 256>(s, o, c.splits, M, N, alpha, C, ldc, c_f32, part, timeouts, probe);
 }
 
 }  // namespace
@@ -924,7 +975,7 @@ cudaError_t tune_choice(cudaStream_t s, TcTuner* tuner, const TcTuner::Key& key,
 
 template <int PREC>
 cudaError_t run(cudaStream_t s, int M, int N, int K, cplx alpha, const cplx* A, long long lda, int opA,
-                const cplx* B, long long ldb, int opB, cplx* C, long long ldc, char* scratch, size_t scratch_bytes, TcTuner* tuner, const TcChoice* force, int* timeouts,
+                const cplx* B, long long ldb, int opB, void* C, long long ldc, bool c_f32, char* scratch, size_t scratch_bytes, TcTuner* tuner, const TcChoice* force, int* timeouts,
                 TcProbe* probe, const TcView* va = nullptr, const TcView* vb = nullptr) {
   if (!timeouts) return cudaErrorInvalidValue;
   using K_ = Cfg<PREC, 128>;  // element size, k-block and parts do not depend on the tile width
@@ -935,7 +986,6 @@ cudaError_t run(cudaStream_t s, int M, int N, int K, cplx alpha, const cplx* A, 
   auto al = [](size_t x) { return (x + 1023) & ~(size_t)1023; };
   const size_t abytes = al((size_t)o.Mp * o.Krp * K_::ELEM);
   const size_t bbytes = al((size_t)o.Nrp * o.Krp * K_::ELEM);
-  const bool conj_out = false;
   const size_t fixed = K_::NOPS * (abytes + bbytes) + 1024;
   if (fixed > scratch_bytes) return cudaErrorMemoryAllocation;
   const size_t part_room = scratch_bytes - fixed;
@@ -971,6 +1021,7 @@ cudaError_t run(cudaStream_t s, int M, int N, int K, cplx alpha, const cplx* A, 
   if (!va) {
     const bool t = (opA & OP_T) != 0;
     pa.p = A;
+    pa.f32 = 0;
     pa.conj = (opA & OP_CONJ) ? 1 : 0;
     pa.nr = pa.nc = 1;
     pa.rdim[0] = M;
@@ -981,8 +1032,14 @@ cudaError_t run(cudaStream_t s, int M, int N, int K, cplx alpha, const cplx* A, 
   const TcView& av = va ? *va : pa;
   if (o.Mp / 32 <= 65535 && o.Mp * o.Krp < (1LL << 40)) {
     const int row_contig = av.rstr[av.nr - 1] == 1 && av.cstr[av.nc - 1] != 1;
-    pack_a_tiled_kernel<PREC><<<dim3((unsigned)((o.Krp / 2 + 31) / 32), (unsigned)(o.Mp / 32)), dim3(32, 8), 0, s>>>(
-        av, M, K, (int)o.Mp, (int)o.Krp, row_contig, o.a0, o.a1, o.a2);
+    auto go = [&](auto kern) {
+      kern<<<dim3((unsigned)((o.Krp / 2 + 31) / 32), (unsigned)(o.Mp / 32)), dim3(32, 8), 0, s>>>(
+          av, M, K, (int)o.Mp, (int)o.Krp, row_contig, o.a0, o.a1, o.a2);
+    };
+    if (av.f32)
+      go(pack_a_tiled_kernel<PREC, true>);
+    else
+      go(pack_a_tiled_kernel<PREC, false>);
   } else if (va) {
     return cudaErrorNotSupported;
   } else {
@@ -994,8 +1051,14 @@ cudaError_t run(cudaStream_t s, int M, int N, int K, cplx alpha, const cplx* A, 
   if (vb) {
     if (o.Nrp / 64 > 65535) return cudaErrorNotSupported;
     const int row_contig = vb->rstr[vb->nr - 1] == 1 && vb->cstr[vb->nc - 1] != 1;
-    pack_b_tiled_kernel<PREC><<<dim3((unsigned)((o.Krp / 2 + 31) / 32), (unsigned)(o.Nrp / 64)), dim3(32, 8), 0, s>>>(
-        *vb, N, K, (int)o.Nrp, (int)o.Krp, row_contig, o.b0, o.b1, o.b2);
+    auto go = [&](auto kern) {
+      kern<<<dim3((unsigned)((o.Krp / 2 + 31) / 32), (unsigned)(o.Nrp / 64)), dim3(32, 8), 0, s>>>(
+          *vb, N, K, (int)o.Nrp, (int)o.Krp, row_contig, o.b0, o.b1, o.b2);
+    };
+    if (vb->f32)
+      go(pack_b_tiled_kernel<PREC, true>);
+    else
+      go(pack_b_tiled_kernel<PREC, false>);
     count_launch();
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   } else if ((e = pack_b_any<PREC>(s, B, ldb, opB, N, K, o.Nrp, o.Krp, o.b0, o.b1, o.b2)) != cudaSuccess) {
@@ -1004,12 +1067,12 @@ cudaError_t run(cudaStream_t s, int M, int N, int K, cplx alpha, const cplx* A, 
   if (tune_now) {
     e = tune_choice(s, tuner, key, o, choice, [&](int S) { return part_bytes(S) <= part_room; },
                     [&](TcChoice c) {
-                      return launch_choice<PREC>(s, o, c, M, N, alpha, C, ldc, part, conj_out, timeouts);
+                      return launch_choice<PREC>(s, o, c, M, N, alpha, C, ldc, c_f32, part, timeouts);
                     },
                     &choice);
     if (e != cudaSuccess) return e;
   }
-  return launch_choice<PREC>(s, o, choice, M, N, alpha, C, ldc, part, conj_out, timeouts, probe);
+  return launch_choice<PREC>(s, o, choice, M, N, alpha, C, ldc, c_f32, part, timeouts, probe);
 }
 
 
@@ -1048,20 +1111,20 @@ cudaError_t tc_zgemm(cudaStream_t s, int prec, int M, int N, int K, cplx alpha, 
   char* base = (char*)(scratch + scratch_top);
   const size_t bytes = (size_t)(scratch_elems - scratch_top) * sizeof(cplx);
   return by_prec(prec, [&](auto P) {
-    return run<decltype(P)::value>(s, M, N, K, alpha, A, lda, opA, B, ldb, opB, C, ldc, base, bytes,
+    return run<decltype(P)::value>(s, M, N, K, alpha, A, lda, opA, B, ldb, opB, C, ldc, false, base, bytes,
                                    tuner, force, timeouts, probe);
   });
 }
 
 cudaError_t tc_zgemm_views(cudaStream_t s, int prec, int M, int N, int K, cplx alpha, const TcView* va,
                            const cplx* A, long long lda, int opA, const TcView* vb, const cplx* B, long long ldb,
-                           int opB, cplx* C, long long ldc, cplx* scratch, long long scratch_elems,
+                           int opB, void* C, long long ldc, bool c_f32, cplx* scratch, long long scratch_elems,
                            long long scratch_top, int* timeouts, TcTuner* tuner, TcProbe* probe) {
   if (M <= 0 || N <= 0 || K <= 0) return cudaErrorNotSupported;
   char* base = (char*)(scratch + scratch_top);
   const size_t bytes = (size_t)(scratch_elems - scratch_top) * sizeof(cplx);
   return by_prec(prec, [&](auto P) {
-    return run<decltype(P)::value>(s, M, N, K, alpha, A, lda, opA, B, ldb, opB, C, ldc, base, bytes,
+    return run<decltype(P)::value>(s, M, N, K, alpha, A, lda, opA, B, ldb, opB, C, ldc, c_f32, base, bytes,
                                    tuner, nullptr, timeouts, probe, va, vb);
   });
 }
@@ -1105,8 +1168,8 @@ size_t tc_thin_bytes(int prec, int M, int K) {
   return parts_bytes(prec, (size_t)(pad_to(2LL * M, NPAD) * pad_k(prec, K) * elem_bytes(prec)));
 }
 
-cudaError_t tc_pack_square(cudaStream_t s, int prec, const cplx* Q, int K, void* memN, void* memT, TcPacked* outN,
-                           TcPacked* outT) {
+cudaError_t tc_pack_square(cudaStream_t s, int prec, const void* Q, int K, int D2, void* memN, void* memT,
+                           TcPacked* outN, TcPacked* outT) {
   const long long Mp = pad_to(K, BM), Krp = pad_k(prec, K);
   if (Mp / 32 > 65535) return cudaErrorNotSupported;
   TcPacked* out[2] = {outN, outT};
@@ -1117,8 +1180,14 @@ cudaError_t tc_pack_square(cudaStream_t s, int prec, const cplx* Q, int K, void*
     carve_parts(prec, mem[v], (size_t)(Mp * Krp * elem_bytes(prec)), out[v]->b);
   }
   return by_prec(prec, [&](auto P) {
-    pack_square_kernel<decltype(P)::value><<<dim3((unsigned)(Mp / 32), (unsigned)(Mp / 32)), dim3(32, 8), 0, s>>>(
-        Q, K, (int)Mp, (int)Krp, outN->b[0], outN->b[1], outN->b[2], outT->b[0], outT->b[1], outT->b[2]);
+    auto go = [&](auto kern) {
+      kern<<<dim3((unsigned)(Mp / 32), (unsigned)(Mp / 32)), dim3(32, 8), 0, s>>>(
+          Q, K, D2, (int)Mp, (int)Krp, outN->b[0], outN->b[1], outN->b[2], outT->b[0], outT->b[1], outT->b[2]);
+    };
+    if (D2 > 0)
+      go(pack_square_kernel<decltype(P)::value, true>);
+    else
+      go(pack_square_kernel<decltype(P)::value, false>);
     count_launch();
     return cudaGetLastError();
   });
@@ -1166,9 +1235,9 @@ cudaError_t run_thin(cudaStream_t s, const TcThin& A, const TcPacked& Q, cplx* C
     const int S = eff_splits(o.kb_total, c.splits);
     cudaError_t e;
     if (c.bn == 128 || o.Nrp % 256 != 0)
-      e = launch_main<PREC, 128>(s, o, S, N, M, make_double2(1.0, 0.0), nullptr, 0, part, false, timeouts, pr, true);
+      e = launch_main<PREC, 128>(s, o, S, N, M, make_double2(1.0, 0.0), nullptr, 0, false, part, timeouts, pr, true);
     else
-      e = launch_main<PREC, 256>(s, o, S, N, M, make_double2(1.0, 0.0), nullptr, 0, part, false, timeouts, pr, true);
+      e = launch_main<PREC, 256>(s, o, S, N, M, make_double2(1.0, 0.0), nullptr, 0, false, part, timeouts, pr, true);
     if (e != cudaSuccess) return e;
     const long long rows = next ? std::max<long long>(N, o.Krp / 2) : N, cols = next ? o.Nrp / 2 : M;
     thin_reduce_kernel<PREC><<<dim3((unsigned)((rows + 31) / 32), (unsigned)((cols + 31) / 32)), dim3(32, 8), 0, s>>>(

@@ -31,7 +31,8 @@ struct TcProbe {
 // the A role rows are m and columns k; for the B role rows are n and columns
 // k (the transpose of op(B)).
 struct TcView {
-  const cplx* p;
+  const void* p;   // complex FP64, or complex FP32 with f32
+  int f32;
   int nr, nc;
   int rdim[4], cdim[4];
   long long rstr[4], cstr[4];
@@ -61,9 +62,11 @@ struct TcThin {    // a packed thin operand: 2M x 2K reals
 };
 size_t tc_packed_bytes(int prec, int K);
 size_t tc_thin_bytes(int prec, int M, int K);
-// Q (row-major) packed for thin * Q (outN) and thin * Q^T (outT), one read
-cudaError_t tc_pack_square(cudaStream_t s, int prec, const cplx* Q, int K, void* memN, void* memT, TcPacked* outN,
-                           TcPacked* outT);
+// Q packed for thin * Q (outN) and thin * Q^T (outT), one read.  D2 = 0: Q row-major
+// complex FP64.  D2 > 0: Q[(x a), (y b)] complex FP32 stored as [x][y][a][b] with a,
+// b < D2 and x, y < K / D2 (a corner as its last product leaves it).
+cudaError_t tc_pack_square(cudaStream_t s, int prec, const void* Q, int K, int D2, void* memN, void* memT,
+                           TcPacked* outN, TcPacked* outT);
 // a thin operand's parts in mem (tc_thin_bytes)
 cudaError_t tc_thin_layout(int prec, int M, int K, void* mem, TcThin* out);
 // t = A (M x K, row-major, conjugated with conj), packed
@@ -98,10 +101,11 @@ cudaError_t tc_init();
 
 // C[M,N] = alpha A B with either operand given as a view (the other, when the
 // view pointer is null, as (ptr, ld, op) like tc_zgemm): the operand packing
-// gathers straight from the source tensor (a fused permute-and-pack).
+// gathers straight from the source tensor (a fused permute-and-pack).  c_f32
+// (alpha 1): C as complex FP32, which is all that the FP32 sums carry.
 cudaError_t tc_zgemm_views(cudaStream_t s, int prec, int M, int N, int K, cplx alpha, const TcView* va,
                            const cplx* A, long long lda, int opA, const TcView* vb, const cplx* B, long long ldb,
-                           int opB, cplx* C, long long ldc, cplx* scratch, long long scratch_elems,
+                           int opB, void* C, long long ldc, bool c_f32, cplx* scratch, long long scratch_elems,
                            long long scratch_top, int* timeouts, TcTuner* tuner = nullptr,
                            TcProbe* probe = nullptr);
 
