@@ -47,25 +47,29 @@ namespace {
 constexpr int OZ_DIGITS = 7;                          // base-256 digits per element
 constexpr int OZ_GROUPS = 7;                          // weights g = s + t = 0..6
 constexpr int OZ_BM = 128;                            // output tile rows
-constexpr int OZ_BK = 64;                             // bf16 elements per k-block (128 bytes)
+constexpr int OZ_BK = 32;                             // bf16 elements per k-block
+constexpr int OZ_KB_BYTES = 2 * OZ_BK;                // 64-byte rows, 64-byte swizzle
 constexpr int OZ_CHUNK = 128;                         // reals of K per exact FP32 chunk
-constexpr int OZ_KB_PER_CHUNK = OZ_CHUNK / OZ_BK;     // 2
-constexpr int OZ_A_BYTES = OZ_BM * 128;               // one A plane k-block: 16 KB
+constexpr int OZ_KB_PER_CHUNK = OZ_CHUNK / OZ_BK;     // 4
+constexpr int OZ_A_BYTES = OZ_BM * OZ_KB_BYTES;       // one A plane k-block: 8 KB
 constexpr int OZ_TMEM_COLS = 512;
 static_assert(OZ_GROUPS == OZ_DIGITS, "weights 0..6 of the digit pairs s + t <= 6");
 
-// Output tiles of 128 x BN real columns.  BN = 32: two sets of the seven group
-// accumulators (224 of 256 columns each), so that a chunk's products run
-// while the epilogue drains the previous chunk; four 44 KB stages; four
+// Output tiles of 128 x BN real columns.  A pipeline stage holds a k-block of
+// all seven planes of both operands, so that each plane is loaded once per
+// tile and k-block (a stage per A plane with the B planes it meets loaded the
+// B planes four times over: 672 KB per 128-wide chunk and SM through L2, which
+// bound the 64-wide tile at 15 us a chunk).  BN = 32: two sets of the seven
+// group accumulators (224 of 256 columns each), so that a chunk's products run
+// while the epilogue drains the previous chunk; three 70 KB stages; four
 // epilogue warps.  BN = 64: one set (448 columns), the products of a chunk
-// wait for the previous chunk's drain, but each MMA does twice the work (the
-// narrow MMAs' issue bounds the 32-wide tile); three 72 KB stages; eight
-// epilogue warps (two per lane quarter, 32 columns each).
+// wait for the previous chunk's drain, but each MMA does twice the work; two
+// 84 KB stages; eight epilogue warps (two per lane quarter, 32 columns each).
 template <int BN>
 struct OzTile {
-  static constexpr int B_BYTES = BN * 128;                       // one B plane k-block
-  static constexpr int STAGE = OZ_A_BYTES + OZ_DIGITS * B_BYTES;  // 44 KB / 72 KB
-  static constexpr int STAGES = BN == 32 ? 4 : 3;
+  static constexpr int B_BYTES = BN * OZ_KB_BYTES;                   // one B plane k-block
+  static constexpr int STAGE = OZ_DIGITS * (OZ_A_BYTES + B_BYTES);  // 70 KB / 84 KB
+  static constexpr int STAGES = BN == 32 ? 3 : 2;
   static constexpr int SETS = BN == 32 ? 2 : 1;
   static constexpr int ACC_COLS = BN == 32 ? 256 : 512;          // columns per accumulator set
   static constexpr int EPI_WARPS = BN / 8;
@@ -245,7 +249,7 @@ __global__ void __launch_bounds__(OzTile<BN>::THREADS, 1)
   const int n_tile = blockIdx.x, m_tile = blockIdx.y, split = blockIdx.z;
   const int c0 = split * chunks_per_split;
   const int nch = min(chunks_total, c0 + chunks_per_split) - c0;  // >= 1 by construction
-  const int nstage = nch * OZ_KB_PER_CHUNK * OZ_DIGITS;             // (chunk, k-block, A digit)
+  const int nstage = nch * OZ_KB_PER_CHUNK;  // (chunk, k-block)
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < OZ_STAGES; ++s) {
@@ -271,20 +275,21 @@ __global__ void __launch_bounds__(OzTile<BN>::THREADS, 1)
   const uint32_t tmem = *tmem_slot;
 
   if (warp == 0 && lane == 0) {
-    // producer: stage q = (chunk, k-block, s) holds A plane s and B planes 0..6-s
+    // producer: stage q = (chunk, k-block) holds the seven planes of A, then of B
     int issued = 0;
     for (int q = 0; q < nstage; ++q) {
       const int slot = q % OZ_STAGES, round = q / OZ_STAGES;
-      const int s = q % OZ_DIGITS, kb = (c0 * OZ_KB_PER_CHUNK) + q / OZ_DIGITS;
+      const int kx = (c0 * OZ_KB_PER_CHUNK + q) * OZ_BK;
       if (!mbar_wait(&empty[slot], (round & 1) ^ 1)) {
         atomicAdd(timeouts, 1);
         break;
       }
       unsigned char* st = smem + slot * OZ_STAGE;
-      mbar_expect_tx(&full[slot], OZ_A_BYTES + (OZ_DIGITS - s) * OZ_B_BYTES);
-      tma_load_2d(st, &mA, &full[slot], kb * OZ_BK, s * Mp + m_tile * OZ_BM);
-      for (int t = 0; t < OZ_DIGITS - s; ++t)
-        tma_load_2d(st + OZ_A_BYTES + t * OZ_B_BYTES, &mB, &full[slot], kb * OZ_BK, t * Nrp + n_tile * BN);
+      mbar_expect_tx(&full[slot], OZ_STAGE);
+      for (int s = 0; s < OZ_DIGITS; ++s) {
+        tma_load_2d(st + s * OZ_A_BYTES, &mA, &full[slot], kx, s * Mp + m_tile * OZ_BM);
+        tma_load_2d(st + OZ_DIGITS * OZ_A_BYTES + s * OZ_B_BYTES, &mB, &full[slot], kx, s * Nrp + n_tile * BN);
+      }
       issued = q + 1;
     }
     // the last loads of every slot have landed before the CTA can leave
@@ -297,10 +302,9 @@ __global__ void __launch_bounds__(OzTile<BN>::THREADS, 1)
     bool ok = true;
     for (int q = 0; q < nstage && ok; ++q) {
       const int slot = q % OZ_STAGES, round = q / OZ_STAGES;
-      const int s = q % OZ_DIGITS, kbc = (q / OZ_DIGITS) % OZ_KB_PER_CHUNK, c = q / (OZ_DIGITS * OZ_KB_PER_CHUNK);
-      const bool chunk_start = kbc == 0 && s == 0;
+      const int kbc = q % OZ_KB_PER_CHUNK, c = q / OZ_KB_PER_CHUNK;
       // the set was drained: chunk c - SETS was that set's drain number c/SETS - 1
-      if (chunk_start && c >= SETS && !mbar_wait(&acc_empty[c % SETS], ((c / SETS) - 1) & 1)) {
+      if (kbc == 0 && c >= SETS && !mbar_wait(&acc_empty[c % SETS], ((c / SETS) - 1) & 1)) {
         atomicAdd(timeouts, 1);
         ok = false;
         break;
@@ -311,28 +315,34 @@ __global__ void __launch_bounds__(OzTile<BN>::THREADS, 1)
         break;
       }
       fence_after();
-      const uint32_t a = smem_u32(smem + slot * OZ_STAGE);
+      const uint32_t st = smem_u32(smem + slot * OZ_STAGE);
+      const uint32_t d = tmem + (uint32_t)((c % SETS) * T::ACC_COLS);
       // per k-step, A plane s meets the B planes t = 0 .. 6 - s in turn (group
       // s + t each): A is read from shared memory once per k-step and kept in
-      // the collector buffer for the other B planes
-      const int nt = OZ_DIGITS - s;
-      const uint32_t d0 = tmem + (uint32_t)((c % SETS) * T::ACC_COLS + s * BN);
+      // the collector buffer for the other B planes.  The plane s = 0 of a
+      // chunk's first k-step starts every group.
 #pragma unroll
       for (int ks = 0; ks < OZ_BK / 16; ++ks) {
-        const uint64_t ad = sdesc(a + ks * 32);
-        const uint32_t acc = (chunk_start && ks == 0) ? 0u : 1u;
-        const uint32_t b0 = a + OZ_A_BYTES + ks * 32;
-        if (nt == 1) {
-          umma_bf16(d0, ad, sdesc(b0), T::IDESC, acc);
-          continue;
+        const uint32_t bb = st + OZ_DIGITS * OZ_A_BYTES + ks * 32;
+#pragma unroll
+        for (int s = 0; s < OZ_DIGITS; ++s) {
+          const uint64_t ad = sdesc_kb<OZ_KB_BYTES>(st + s * OZ_A_BYTES + ks * 32);
+          const uint32_t acc = (kbc == 0 && ks == 0 && s == 0) ? 0u : 1u;
+          constexpr int ND = OZ_DIGITS;
+          auto bd = [&](int t) { return sdesc_kb<OZ_KB_BYTES>(bb + t * OZ_B_BYTES); };
+          if (s == ND - 1) {
+            umma_bf16(d + s * BN, ad, bd(0), T::IDESC, acc);
+            continue;
+          }
+          umma_bf16_coll<COLL_FILL>(d + s * BN, ad, bd(0), T::IDESC, acc);
+#pragma unroll
+          for (int t = 1; t < ND - 1 - s; ++t)
+            umma_bf16_coll<COLL_USE>(d + (s + t) * BN, ad, bd(t), T::IDESC, acc);
+          umma_bf16_coll<COLL_LAST>(d + (ND - 1) * BN, ad, bd(ND - 1 - s), T::IDESC, acc);
         }
-        umma_bf16_coll<COLL_FILL>(d0, ad, sdesc(b0), T::IDESC, acc);
-        for (int t = 1; t < nt - 1; ++t)
-          umma_bf16_coll<COLL_USE>(d0 + t * BN, ad, sdesc(b0 + t * OZ_B_BYTES), T::IDESC, acc);
-        umma_bf16_coll<COLL_LAST>(d0 + (nt - 1) * BN, ad, sdesc(b0 + (nt - 1) * OZ_B_BYTES), T::IDESC, acc);
       }
       umma_commit(&empty[slot]);  // frees the slot when these MMAs are done
-      if (kbc == OZ_KB_PER_CHUNK - 1 && s == OZ_DIGITS - 1) umma_commit(&acc_full[c % SETS]);
+      if (kbc == OZ_KB_PER_CHUNK - 1) umma_commit(&acc_full[c % SETS]);
     }
     // every MMA issued has completed before the accumulators are released
     umma_commit(mma_done);
@@ -362,25 +372,36 @@ __global__ void __launch_bounds__(OzTile<BN>::THREADS, 1)
       }
       fence_after();
       const uint32_t tset = trow + (uint32_t)((c % SETS) * T::ACC_COLS);
-      // two halves of 16 columns (fewer live registers beside the running sums)
+      // two halves of 16 columns (fewer live registers beside the running sums),
+      // two or three groups' loads waited for together
 #pragma unroll
       for (int hf = 0; hf < 2; ++hf) {
-        float v[16], t[16];
-        // groups 0..3: exact integers (below 2^24) into the 64-bit sum
+        uint32_t v[3][16];
+        // groups 0..3: exact integers up to 2^21, 2^22, 1.5 2^22 and 2^23, so each
+        // pair combines in 32 bits before the 64-bit sum
 #pragma unroll
-        for (int g = 0; g < 4; ++g) {
-          tmem_ld16(tset + g * BN + 16 * hf, v);
+        for (int g = 0; g < 4; g += 2) {
+          tmem_ld16_issue(tset + g * BN + 16 * hf, v[0]);
+          tmem_ld16_issue(tset + (g + 1) * BN + 16 * hf, v[1]);
+          tmem_ld_wait(v[0]);
+          tmem_ld_after(v[1]);
 #pragma unroll
-          for (int j = 0; j < 16; ++j) I[16 * hf + j] += (long long)__float2int_rn(v[j]) << (8 * (3 - g));
+          for (int j = 0; j < 16; ++j) {
+            const int p = __float2int_rn(__uint_as_float(v[0][j])) * 256 + __float2int_rn(__uint_as_float(v[1][j]));
+            I[16 * hf + j] += g == 0 ? (long long)p * 65536 : (long long)p;
+          }
         }
         // groups 4..6 (weight 2^-32 and below relative to group 0): FP32
-        tmem_ld16(tset + 6 * BN + 16 * hf, t);
-        tmem_ld16(tset + 5 * BN + 16 * hf, v);
 #pragma unroll
-        for (int j = 0; j < 16; ++j) t[j] = fmaf(t[j], 1.0f / 256.0f, v[j]);
-        tmem_ld16(tset + 4 * BN + 16 * hf, v);
+        for (int g = 0; g < 3; ++g) tmem_ld16_issue(tset + (4 + g) * BN + 16 * hf, v[g]);
+        tmem_ld_wait(v[0]);
 #pragma unroll
-        for (int j = 0; j < 16; ++j) u[16 * hf + j] += fmaf(t[j], 1.0f / 256.0f, v[j]);
+        for (int g = 1; g < 3; ++g) tmem_ld_after(v[g]);
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+          const float t = fmaf(__uint_as_float(v[2][j]), 1.0f / 256.0f, __uint_as_float(v[1][j]));
+          u[16 * hf + j] += fmaf(t, 1.0f / 256.0f, __uint_as_float(v[0][j]));
+        }
       }
       fence_before();
       __syncwarp();
@@ -529,8 +550,10 @@ cudaError_t oz_zgemm(cudaStream_t s, int M, int N, int K, const cplx* A, long lo
   count_launch();
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   CUtensorMap mA, mB;
-  if ((e = tc_encode_bf16_map(&mA, pa, (long long)OZ_DIGITS * L.Mp, L.Krp, OZ_BM)) != cudaSuccess) return e;
-  if ((e = tc_encode_bf16_map(&mB, pb, (long long)OZ_DIGITS * L.Nrp, L.Krp, L.bn)) != cudaSuccess) return e;
+  if ((e = tc_encode_bf16_map(&mA, pa, (long long)OZ_DIGITS * L.Mp, L.Krp, OZ_BM, OZ_KB_BYTES)) != cudaSuccess)
+    return e;
+  if ((e = tc_encode_bf16_map(&mB, pb, (long long)OZ_DIGITS * L.Nrp, L.Krp, L.bn, OZ_KB_BYTES)) != cudaSuccess)
+    return e;
   dim3 grid((unsigned)(L.Nrp / L.bn), (unsigned)(L.Mp / OZ_BM), (unsigned)L.S);
   if (L.bn == 64)
     oz_gemm_kernel<64><<<grid, OzTile<64>::THREADS, OzTile<64>::SMEM, s>>>(mA, mB, L.Mp, L.Nrp, L.chunks, L.cps, M,

@@ -1078,10 +1078,11 @@ cudaError_t run(cudaStream_t s, int M, int N, int K, cplx alpha, const cplx* A, 
 
 }  // namespace
 
-cudaError_t tc_encode_bf16_map(CUtensorMap* map, void* base, long long rows, long long kcols, int box_rows) {
+cudaError_t tc_encode_bf16_map(CUtensorMap* map, void* base, long long rows, long long kcols, int box_rows,
+                               int kb_bytes) {
   cudaError_t e = get_encoder();
   if (e != cudaSuccess) return e;
-  return make_map(map, base, PREC_BF16X3, rows, kcols, box_rows);
+  return make_map(map, base, PREC_BF16X3, rows, kcols, box_rows, kb_bytes);
 }
 
 namespace {

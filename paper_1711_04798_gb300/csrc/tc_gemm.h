@@ -110,8 +110,10 @@ cudaError_t tc_zgemm_views(cudaStream_t s, int prec, int M, int N, int K, cplx a
                            TcProbe* probe = nullptr);
 
 // 2D tensor map of a K-major BF16 operand [rows x kcols] with boxes of
-// box_rows x 64 elements (128 bytes, 128-byte swizzle), for the tcgen05 kernels.
-cudaError_t tc_encode_bf16_map(CUtensorMap* map, void* base, long long rows, long long kcols, int box_rows);
+// box_rows x kb_bytes (128 or 64, swizzled over that many bytes), for the
+// tcgen05 kernels.
+cudaError_t tc_encode_bf16_map(CUtensorMap* map, void* base, long long rows, long long kcols, int box_rows,
+                               int kb_bytes);
 
 // FP64-accurate complex GEMM on the tensor cores (ozaki.cu): C = opA(A) opB(B)
 // (complex FP64 storage, alpha 1, beta 0).  `work` (device, work_bytes) holds
