@@ -87,6 +87,7 @@ struct Lane {
   cudaStream_t stream;
   cplx* Q[4];
   TcPacked Qp[4][2];
+  OzSquare Qo[4][2];
   void* Qpmem[4][2];
   cplx* thin[4];
   cplx* Vt;
@@ -121,6 +122,7 @@ struct ipeps_ctm_s {
   cplx* spareT[2];    // replacement T4 per row
   cplx* Q[4];
   TcPacked Qp[4][2];  // precision form: corners packed once per cut, [as is, transposed]
+  OzSquare Qo[4][2];  // FP64-accurate form: their digit planes
   void* Qpmem[4][2];
   cplx* omt;
   cplx* thin[4];      // k x K work
@@ -253,6 +255,7 @@ static void swap_lane(ipeps_ctm h) {
     std::swap(h->thin[i], h->alt.thin[i]);
     for (int v = 0; v < 2; ++v) {
       std::swap(h->Qp[i][v], h->alt.Qp[i][v]);
+      std::swap(h->Qo[i][v], h->alt.Qo[i][v]);
       std::swap(h->Qpmem[i][v], h->alt.Qpmem[i][v]);
     }
   }
@@ -306,6 +309,12 @@ static bool chol_route(const ipeps_options& o) {
          (o.orth_tol <= 1e-14 && o.svd_cutoff >= 1e-9 && o.jacobi_max_sweeps <= CHOL_MAX_SWEEPS);
 }
 
+// bytes of one orientation of a packed corner, 0 for a form that packs none
+static size_t corner_pack_bytes(int prec, int K) {
+  if (tc_form(prec)) return tc_packed_bytes(prec, K);
+  return prec == IPEPS_PREC_FP64TC && K >= 64 ? oz_square_bytes(K) : 0;
+}
+
 // sizes of everything a handle carves from its memory
 struct Sizes {
   long long tens, a, C, T, Q, thin, proj, scratch;
@@ -344,8 +353,7 @@ static Sizes plan_sizes(int Lx, int Ly, int d, int D, int chi, int k, int ntens,
   for (int i = 0; i < 4; ++i) add(s.C, 16);
   for (int i = 0; i < 2; ++i) add(s.T, 16);
   for (int i = 0; i < 4; ++i) add(s.Q, 16);
-  if (tc_form(prec))
-    for (int i = 0; i < 8; ++i) tot += align_up(tc_packed_bytes(prec, (int)K));
+  for (int i = 0; i < 8; ++i) tot += align_up(corner_pack_bytes(prec, (int)K));
   add(s.thin, 16);
   for (int i = 0; i < 4; ++i) add(s.thin, 16);
   for (int i = 0; i < 4; ++i) add(s.proj, 16);
@@ -363,8 +371,7 @@ static Sizes plan_sizes(int Lx, int Ly, int d, int D, int chi, int k, int ntens,
   add(s.scratch, 16);
   // second projector lane (the other cut of a column runs concurrently)
   for (int i = 0; i < 4; ++i) add(s.Q, 16);
-  if (tc_form(prec))
-    for (int i = 0; i < 8; ++i) tot += align_up(tc_packed_bytes(prec, (int)K));
+  for (int i = 0; i < 8; ++i) tot += align_up(corner_pack_bytes(prec, (int)K));
   for (int i = 0; i < 4; ++i) add(s.thin, 16);
   add((long long)k * k, 16);
   add((long long)chi * k, 16);
@@ -1019,9 +1026,9 @@ extern "C" ipeps_status ipeps_ctm_create(const ipeps_cell* c, const ipeps_option
     need(h->spareT[i] = carve<cplx>(h, sz.T));
   }
   for (int i = 0; i < 4; ++i) need(h->Q[i] = carve<cplx>(h, sz.Q));
-  if (tc_form(o->prec))
-    for (int i = 0; i < 4; ++i)
-      for (int v = 0; v < 2; ++v) need(h->Qpmem[i][v] = carve<char>(h, tc_packed_bytes(o->prec, h->K)));
+  const size_t cpb = corner_pack_bytes(o->prec, h->K);
+  for (int i = 0; i < 4 && cpb; ++i)
+    for (int v = 0; v < 2; ++v) need(h->Qpmem[i][v] = carve<char>(h, cpb));
   need(h->omt = carve<cplx>(h, sz.thin));
   for (int i = 0; i < 4; ++i) need(h->thin[i] = carve<cplx>(h, sz.thin));
   for (int i = 0; i < 2; ++i) {
@@ -1043,9 +1050,8 @@ extern "C" ipeps_status ipeps_ctm_create(const ipeps_cell* c, const ipeps_option
   h->scratch_elems = sz.scratch;
   h->scratch_top = 0;
   for (int i = 0; i < 4; ++i) need(h->alt.Q[i] = carve<cplx>(h, sz.Q));
-  if (tc_form(o->prec))
-    for (int i = 0; i < 4; ++i)
-      for (int v = 0; v < 2; ++v) need(h->alt.Qpmem[i][v] = carve<char>(h, tc_packed_bytes(o->prec, h->K)));
+  for (int i = 0; i < 4 && cpb; ++i)
+    for (int v = 0; v < 2; ++v) need(h->alt.Qpmem[i][v] = carve<char>(h, cpb));
   for (int i = 0; i < 4; ++i) need(h->alt.thin[i] = carve<cplx>(h, sz.thin));
   need(h->alt.Vt = carve<cplx>(h, (size_t)h->k * h->k));
   need(h->alt.Gsel = carve<cplx>(h, (size_t)h->chi * h->k));
@@ -1279,10 +1285,26 @@ lower_left:
   return IPEPS_OK;
 }
 
-// thin (k x K, row-major = transposed K x k) times one corner
-static ipeps_status thin_mul(ipeps_ctm h, const cplx* in, int opin, cplx* out, const cplx* Qm, int opQ,
-                             int rows) {
-  return gemm_dispatch(h, rows, h->K, h->K, in, h->K, opin, Qm, h->K, opQ, out, h->K, ONE);
+// Whether a thin product of `rows` rows takes the corners' digit planes split
+// once per cut (FP64-accurate form; below, the planes' padding to 128 rows
+// and 64 columns outweighs them and the FP64 CUDA cores are as good).
+static bool oz_corners(ipeps_ctm h, int rows) {
+  return h->opt.prec == IPEPS_PREC_FP64TC && h->K >= 64 && rows >= 16;
+}
+
+// thin (k x K, row-major = transposed K x k) times corner q, opQ applied to it
+static ipeps_status thin_mul(ipeps_ctm h, const cplx* in, int opin, cplx* out, int q, int opQ, int rows) {
+  if (oz_corners(h, rows) && !(opin & OP_T)) {
+    // in Q^H = conj(conj(in) Q^T)
+    const bool cq = (opQ & OP_CONJ) != 0, ci = ((opin & OP_CONJ) != 0) != cq;
+    cudaEvent_t a = nullptr;
+    prof_begin(h, &a);
+    CK(oz_thin(h->stream, rows, in, h->K, ci, h->Qo[q][opQ & OP_T ? 1 : 0], out, h->K, cq, h->scratch + h->scratch_top,
+               (size_t)(h->scratch_elems - h->scratch_top) * sizeof(cplx), &h->st->tc_timeouts));
+    prof_end(h, a, 8.0 * (double)rows * (double)h->K * (double)h->K, 0);
+    return IPEPS_OK;
+  }
+  return gemm_dispatch(h, rows, h->K, h->K, in, h->K, opin, h->Q[q], h->K, opQ, out, h->K, ONE);
 }
 
 // precision form: in (conjugated with conj_in) times the packed corners
@@ -1320,9 +1342,15 @@ static ipeps_status thin_chain(ipeps_ctm h, const cplx* in, bool conj_in, std::i
   return IPEPS_OK;
 }
 
+static bool packed_path(ipeps_ctm h) { return tc_form(h->opt.prec); }
+
 static ipeps_status pack_corners(ipeps_ctm h) {
   for (int q = 0; q < 4; ++q) {
     if (two_corners(h) && (q == 1 || q == 2)) continue;
+    if (!packed_path(h)) {
+      CK(oz_pack_square(h->stream, h->Q[q], h->K, h->Qpmem[q][0], h->Qpmem[q][1], &h->Qo[q][0], &h->Qo[q][1]));
+      continue;
+    }
     CK(tc_pack_square(h->stream, (int)h->opt.prec, h->Q[q], h->K, corners_f32(h) ? h->D2 : 0, h->Qpmem[q][0], h->Qpmem[q][1], &h->Qp[q][0],
                       &h->Qp[q][1]));
   }
@@ -1333,7 +1361,6 @@ static ipeps_status pack_corners(ipeps_ctm h) {
 constexpr int thinN(int q) { return 2 * q; }
 constexpr int thinT(int q) { return 2 * q + 1; }
 
-static bool packed_path(ipeps_ctm h) { return tc_form(h->opt.prec); }
 
 // Yt = In * Q3 * Q4^T * Q1 * Q2      (the transpose of X * In^T)
 // two corners: Yt = In * Q4^T * Q1
@@ -1342,16 +1369,16 @@ static ipeps_status apply_XT(ipeps_ctm h, const cplx* in, cplx* out, int rows) {
     if (packed_path(h)) {
       CKS(thin_chain(h, in, false, {thinT(3), thinN(0)}, rows, out, false));
     } else {
-      CKS(thin_mul(h, in, OP_N, h->thin[2], h->Q[3], OP_T, rows));
-      CKS(thin_mul(h, h->thin[2], OP_N, out, h->Q[0], OP_N, rows));
+      CKS(thin_mul(h, in, OP_N, h->thin[2], 3, OP_T, rows));
+      CKS(thin_mul(h, h->thin[2], OP_N, out, 0, OP_N, rows));
     }
     return IPEPS_OK;
   }
   if (packed_path(h)) return thin_chain(h, in, false, {thinN(2), thinT(3), thinN(0), thinN(1)}, rows, out, false);
-  CKS(thin_mul(h, in, OP_N, h->thin[2], h->Q[2], OP_N, rows));
-  CKS(thin_mul(h, h->thin[2], OP_N, h->thin[3], h->Q[3], OP_T, rows));
-  CKS(thin_mul(h, h->thin[3], OP_N, h->thin[2], h->Q[0], OP_N, rows));
-  CKS(thin_mul(h, h->thin[2], OP_N, out, h->Q[1], OP_N, rows));
+  CKS(thin_mul(h, in, OP_N, h->thin[2], 2, OP_N, rows));
+  CKS(thin_mul(h, h->thin[2], OP_N, h->thin[3], 3, OP_T, rows));
+  CKS(thin_mul(h, h->thin[3], OP_N, h->thin[2], 0, OP_N, rows));
+  CKS(thin_mul(h, h->thin[2], OP_N, out, 1, OP_N, rows));
   return IPEPS_OK;
 }
 // Zt = In * Q2^H * Q1^H * conj(Q4) * Q3^H   (the transpose of X^H * In^T)
@@ -1362,16 +1389,16 @@ static ipeps_status apply_XHT(ipeps_ctm h, const cplx* in, cplx* out, int rows) 
     if (packed_path(h)) {
       CKS(thin_chain(h, in, true, {thinT(0), thinN(3)}, rows, out, true));
     } else {
-      CKS(thin_mul(h, in, OP_N, h->thin[2], h->Q[0], OP_H, rows));
-      CKS(thin_mul(h, h->thin[2], OP_N, out, h->Q[3], OP_C, rows));
+      CKS(thin_mul(h, in, OP_N, h->thin[2], 0, OP_H, rows));
+      CKS(thin_mul(h, h->thin[2], OP_N, out, 3, OP_C, rows));
     }
     return IPEPS_OK;
   }
   if (packed_path(h)) return thin_chain(h, in, true, {thinT(1), thinT(0), thinN(3), thinT(2)}, rows, out, true);
-  CKS(thin_mul(h, in, OP_N, h->thin[2], h->Q[1], OP_H, rows));
-  CKS(thin_mul(h, h->thin[2], OP_N, h->thin[3], h->Q[0], OP_H, rows));
-  CKS(thin_mul(h, h->thin[3], OP_N, h->thin[2], h->Q[3], OP_C, rows));
-  CKS(thin_mul(h, h->thin[2], OP_N, out, h->Q[2], OP_H, rows));
+  CKS(thin_mul(h, in, OP_N, h->thin[2], 1, OP_H, rows));
+  CKS(thin_mul(h, h->thin[2], OP_N, h->thin[3], 0, OP_H, rows));
+  CKS(thin_mul(h, h->thin[3], OP_N, h->thin[2], 3, OP_C, rows));
+  CKS(thin_mul(h, h->thin[2], OP_N, out, 2, OP_H, rows));
   return IPEPS_OK;
 }
 
@@ -1540,7 +1567,7 @@ static ipeps_status projectors(ipeps_ctm h, int f, int x, int y, cplx* PT, cplx*
   const int k = h->k, K = h->K, chi = h->chi;
   // CholeskyQR on FP64-accurate Grams, or Jacobi on the full rows (chol_route)
   const bool jacobi_bases = !chol_route(h->opt);
-  if (packed_path(h)) CKS(pack_corners(h));
+  if (packed_path(h) || oz_corners(h, k)) CKS(pack_corners(h));
   cplx* Qt = h->thin[0];
   cplx* Zt = h->thin[1];
   auto orth_any = [&](cplx* Y, bool last) -> ipeps_status {
@@ -1588,24 +1615,24 @@ static ipeps_status projectors(ipeps_ctm h, int f, int x, int y, cplx* PT, cplx*
     if (packed_path(h))
       CKS(thin_chain(h, Vt_chi, false, {thinT(3)}, chi, PT, false));
     else
-      CKS(thin_mul(h, Vt_chi, OP_N, PT, h->Q[3], OP_T, chi));
+      CKS(thin_mul(h, Vt_chi, OP_N, PT, 3, OP_T, chi));
   } else if (packed_path(h)) {
     CKS(thin_chain(h, Vt_chi, false, {thinN(2), thinT(3)}, chi, PT, false));
   } else {
-    CKS(thin_mul(h, Vt_chi, OP_N, tmp, h->Q[2], OP_N, chi));
-    CKS(thin_mul(h, tmp, OP_N, PT, h->Q[3], OP_T, chi));
+    CKS(thin_mul(h, Vt_chi, OP_N, tmp, 2, OP_N, chi));
+    CKS(thin_mul(h, tmp, OP_N, PT, 3, OP_T, chi));
   }
   CK(scale_rows_isqrt(h->stream, PT, chi, K, K, h->s_sel));
   if (two_corners(h)) {
     if (packed_path(h))
       CKS(thin_chain(h, Ut_chi, true, {thinT(0)}, chi, Ptil, false));
     else
-      CKS(thin_mul(h, Ut_chi, OP_C, Ptil, h->Q[0], OP_T, chi));
+      CKS(thin_mul(h, Ut_chi, OP_C, Ptil, 0, OP_T, chi));
   } else if (packed_path(h)) {
     CKS(thin_chain(h, Ut_chi, true, {thinT(1), thinT(0)}, chi, Ptil, false));
   } else {
-    CKS(thin_mul(h, Ut_chi, OP_C, tmp, h->Q[1], OP_T, chi));
-    CKS(thin_mul(h, tmp, OP_N, Ptil, h->Q[0], OP_T, chi));
+    CKS(thin_mul(h, Ut_chi, OP_C, tmp, 1, OP_T, chi));
+    CKS(thin_mul(h, tmp, OP_N, Ptil, 0, OP_T, chi));
   }
   CK(scale_rows_isqrt(h->stream, Ptil, chi, K, K, h->s_sel));
   return IPEPS_OK;

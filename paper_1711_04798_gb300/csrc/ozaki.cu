@@ -233,8 +233,8 @@ template <int BN>
 __global__ void __launch_bounds__(OzTile<BN>::THREADS, 1)
     oz_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mB, int Mp, int Nrp,
                    int chunks_total, int chunks_per_split, int M, int N, const int* __restrict__ ea,
-                   const int* __restrict__ eb, cplx* __restrict__ C, long long ldc, long long* __restrict__ pI,
-                   float* __restrict__ pU, int* __restrict__ timeouts) {
+                   const int* __restrict__ eb, cplx* __restrict__ C, long long ldc, int trans, int conj_out,
+                   long long* __restrict__ pI, float* __restrict__ pU, int* __restrict__ timeouts) {
   using T = OzTile<BN>;
   constexpr int OZ_STAGES = T::STAGES, OZ_STAGE = T::STAGE, OZ_B_BYTES = T::B_BYTES, SETS = T::SETS;
   extern __shared__ unsigned char smem_raw[];
@@ -422,9 +422,11 @@ __global__ void __launch_bounds__(OzTile<BN>::THREADS, 1)
 #pragma unroll
         for (int j = 0; j < EC; j += 2) {
           const int n = (col0 + j) >> 1;
-          if (n < N)
-            C[(long long)row * ldc + n] = make_double2(oz_value(I[j], u[j], er, eb[col0 + j]),
-                                                       oz_value(I[j + 1], u[j + 1], er, eb[col0 + j + 1]));
+          if (n < N) {
+            const double im = oz_value(I[j + 1], u[j + 1], er, eb[col0 + j + 1]);
+            C[trans ? (long long)n * ldc + row : (long long)row * ldc + n] =
+                make_double2(oz_value(I[j], u[j], er, eb[col0 + j]), conj_out ? -im : im);
+          }
         }
       }
     }
@@ -457,6 +459,111 @@ __global__ void oz_reduce_kernel(const long long* __restrict__ pI, const float* 
   }
 }
 
+// The same for a product computed transposed: C[n, m] from row m, column n of
+// the partials, by 32 x 32 tiles through shared memory (reads along n, writes
+// along m).
+__global__ void oz_reduce_t_kernel(const long long* __restrict__ pI, const float* __restrict__ pU, int S, int Mp,
+                                   int Nrp, int M, int N, const int* __restrict__ ea, const int* __restrict__ eb,
+                                   cplx* __restrict__ C, long long ldc, int conj_out) {
+  __shared__ cplx tile[32][33];
+  const int m0 = blockIdx.x * 32, n0 = blockIdx.y * 32;
+  const long long pstride = (long long)Mp * Nrp;
+  const int n = n0 + threadIdx.x;
+  for (int i = threadIdx.y; i < 32; i += blockDim.y) {
+    const int m = m0 + i;
+    long long I0 = 0, I1 = 0;
+    float u0 = 0.0f, u1 = 0.0f;
+    if (m < M && n < N) {
+      const long long o = (long long)m * Nrp + 2 * n;
+#pragma unroll 4
+      for (int z = 0; z < S; ++z) {
+        const longlong2 p = *(const longlong2*)(pI + z * pstride + o);
+        const float2 q = *(const float2*)(pU + z * pstride + o);
+        I0 += p.x;
+        I1 += p.y;
+        u0 += q.x;
+        u1 += q.y;
+      }
+      tile[i][threadIdx.x] =
+          make_double2(oz_value(I0, u0, ea[m], eb[2 * n]), oz_value(I1, u1, ea[m], eb[2 * n + 1]));
+    }
+  }
+  __syncthreads();
+  const int m = m0 + threadIdx.x;
+  for (int i = threadIdx.y; i < 32; i += blockDim.y) {
+    if (m < M && n0 + i < N) {
+      cplx v = tile[threadIdx.x][i];
+      if (conj_out) v.y = -v.y;
+      C[(long long)(n0 + i) * ldc + m] = v;
+    }
+  }
+}
+
+// The largest biased exponents of the rows (er) and columns (ec) of a K x K
+// matrix, both arrays zero on entry; a block takes 32 columns of 128 rows.
+__global__ void __launch_bounds__(256) oz_square_exp_kernel(const cplx* __restrict__ Q, int K, int* __restrict__ er,
+                                                            int* __restrict__ ec) {
+  __shared__ int s_c[8][32];
+  const int c = blockIdx.x * 32 + threadIdx.x;
+  int E = 0;
+  for (int r = blockIdx.y * 128 + threadIdx.y; r < min(K, (int)blockIdx.y * 128 + 128); r += 8) {
+    int e = 0;
+    if (c < K) {
+      const cplx v = Q[(long long)r * K + c];
+      e = max(bexp(v.x), bexp(v.y));
+    }
+    E = max(E, e);
+    e = __reduce_max_sync(0xffffffffu, e);
+    if (threadIdx.x == 0) atomicMax(&er[r], e);
+  }
+  s_c[threadIdx.y][threadIdx.x] = E;
+  __syncthreads();
+  if (threadIdx.y == 0 && c < K) {
+    for (int y = 1; y < 8; ++y) E = max(E, s_c[y][threadIdx.x]);
+    atomicMax(&ec[c], E);
+  }
+}
+
+// Digit planes of a K x K matrix as the row operand of products with Q^T (rows
+// r, columns k of Q[r, k]: pt, exponents er) and with Q (rows c, columns k of
+// Q[k, c]: pn, exponents ec), both Mp x Krp reals (Re, Im pairs along k, zeros
+// beyond), from one read in 32 x 32 tiles.  The raw exponents become the row
+// bounds et, en.
+__global__ void __launch_bounds__(256)
+    oz_square_prep_kernel(const cplx* __restrict__ Q, int K, int Mp, int Krp, const int* __restrict__ er,
+                          const int* __restrict__ ec, int* __restrict__ et, int* __restrict__ en,
+                          __nv_bfloat16* __restrict__ pt, __nv_bfloat16* __restrict__ pn) {
+  __shared__ cplx tile[32][33];
+  const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32, kc = Krp >> 1;
+  const long long plane = (long long)Mp * Krp;
+  auto bound = [](int E) { return E ? E - 1022 : 0; };
+  if (blockIdx.x == 0 && threadIdx.y == 0) {
+    et[r0 + threadIdx.x] = bound(er[r0 + threadIdx.x]);
+    en[r0 + threadIdx.x] = bound(ec[r0 + threadIdx.x]);
+  }
+  auto put = [&](__nv_bfloat16* p, int row, int k, cplx v, int e) {
+    int dr[OZ_DIGITS], di[OZ_DIGITS];
+    digits7(v.x, e, dr);
+    digits7(v.y, e, di);
+    __nv_bfloat162* out = (__nv_bfloat162*)(p + (long long)row * Krp + 2LL * k);
+#pragma unroll
+    for (int s = 0; s < OZ_DIGITS; ++s)
+      out[s * plane / 2] = __halves2bfloat162(__float2bfloat16_rn((float)dr[s]), __float2bfloat16_rn((float)di[s]));
+  };
+  const int c = c0 + threadIdx.x;
+  for (int i = threadIdx.y; i < 32; i += 8) {
+    const int r = r0 + i;
+    cplx v = make_double2(0.0, 0.0);
+    if (r < K && c < K) v = Q[(long long)r * K + c];
+    tile[i][threadIdx.x] = v;
+    if (c < kc) put(pt, r, c, v, bound(er[r]));
+  }
+  __syncthreads();
+  const int k = r0 + threadIdx.x;
+  if (k >= kc) return;
+  for (int i = threadIdx.y; i < 32; i += 8) put(pn, c0 + i, k, tile[threadIdx.x][i], bound(ec[c0 + i]));
+}
+
 unsigned oz_grid(long long n) {
   long long b = (n + 255) / 256;
   if (b < 1) b = 1;
@@ -469,35 +576,40 @@ struct OzLayout {
   size_t off_ea, off_eb, off_a, off_b, off_pi, off_pu, total;
 };
 
+// Tile width and chunks per CTA: the fewest chunk-times over whole waves of CTAs
+// (152 SMs, one CTA each), counting a CTA's start (barriers, tensor memory, the
+// pipeline's fill) as one chunk-time and, for K splits, the exact partials'
+// round trip through memory (24 bytes per output element and split, about 16 MB
+// per chunk-time).  A chunk of a 64-wide tile takes about the time of a 32-wide
+// one (its MMAs do twice the work at the same issue rate, its drain is not
+// overlapped).  Ties: the wider tile, the fewer K splits.  `room`: bytes for
+// the partials (12 per output element and split).
+void oz_choose(int Mp, int N, int chunks, double room, int* bn_, int* Nrp_, int* cps_) {
+  double best = -1.0;
+  for (int bn = 64; bn >= 32; bn -= 32) {
+    const int Nrp = (2 * N + bn - 1) / bn * bn;
+    const long long tiles = (long long)(Mp / OZ_BM) * (Nrp / bn);
+    for (int cps = chunks; cps >= 1; --cps) {
+      const long long S = (chunks + cps - 1) / cps;
+      if (S > 1 && 12.0 * (double)S * Mp * Nrp > room) break;
+      const double partials = S > 1 ? 24.0 * (double)S * Mp * Nrp / 16.0e6 : 0.0;
+      const double cost = (double)((tiles * S + 151) / 152) * (cps + 1) + partials;
+      if (best < 0 || cost < best) {
+        best = cost;
+        *bn_ = bn;
+        *Nrp_ = Nrp;
+        *cps_ = cps;
+      }
+    }
+  }
+}
+
 OzLayout oz_layout(int M, int N, int K) {
   OzLayout L;
   L.Mp = (M + OZ_BM - 1) / OZ_BM * OZ_BM;
   L.Krp = (2 * K + OZ_CHUNK - 1) / OZ_CHUNK * OZ_CHUNK;
   L.chunks = L.Krp / OZ_CHUNK;
-  // tile width and chunks per CTA: the fewest chunk-times over whole waves of
-  // CTAs (152 SMs, one CTA each), counting a CTA's start (barriers, tensor
-  // memory, the pipeline's fill) as one chunk-time and, for K splits, the
-  // exact partials' round trip through memory (24 bytes per output element
-  // and split, about 16 MB per chunk-time).  A chunk of a 64-wide tile takes
-  // about the time of a 32-wide one (measured: its MMAs do twice the work at
-  // the same issue rate, its drain is not overlapped).  Ties: the wider tile,
-  // the fewer K splits.
-  double best = -1.0;
-  for (int bn = 64; bn >= 32; bn -= 32) {
-    const int Nrp = (2 * N + bn - 1) / bn * bn;
-    const long long tiles = (long long)(L.Mp / OZ_BM) * (Nrp / bn);
-    for (int cps = L.chunks; cps >= 1; --cps) {
-      const long long S = (L.chunks + cps - 1) / cps;
-      const double partials = S > 1 ? 24.0 * (double)S * L.Mp * Nrp / 16.0e6 : 0.0;
-      const double cost = (double)((tiles * S + 151) / 152) * (cps + 1) + partials;
-      if (best < 0 || cost < best) {
-        best = cost;
-        L.bn = bn;
-        L.Nrp = Nrp;
-        L.cps = cps;
-      }
-    }
-  }
+  oz_choose(L.Mp, N, L.chunks, 1e300, &L.bn, &L.Nrp, &L.cps);
   L.S = (L.chunks + L.cps - 1) / L.cps;
   auto al = [](size_t x) { return (x + 1023) & ~(size_t)1023; };
   size_t o = 0;
@@ -517,16 +629,9 @@ OzLayout oz_layout(int M, int N, int K) {
   return L;
 }
 
-}  // namespace
-
-size_t oz_work_bytes(int M, int N, int K) { return oz_layout(M, N, K).total; }
-
-cudaError_t oz_zgemm(cudaStream_t s, int M, int N, int K, const cplx* A, long long lda, int opA, const cplx* B,
-                     long long ldb, int opB, cplx* C, long long ldc, void* work, size_t work_bytes, int* timeouts) {
-  if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
-  if (!timeouts) return cudaErrorInvalidValue;
-  const OzLayout L = oz_layout(M, N, K);
-  if (!work || work_bytes < L.total) return cudaErrorMemoryAllocation;
+cudaError_t oz_launch(cudaStream_t s, __nv_bfloat16* pa, __nv_bfloat16* pb, int Mp, int Nrp, int Krp, int bn, int chunks,
+                      int cps, int M, int N, const int* ea, const int* eb, cplx* C, long long ldc, bool trans,
+                      bool conj_out, long long* pI, float* pU, int* timeouts) {
   static bool attr = false;
   cudaError_t e;
   if (!attr) {
@@ -538,6 +643,100 @@ cudaError_t oz_zgemm(cudaStream_t s, int M, int N, int K, const cplx* A, long lo
       return e;
     attr = true;
   }
+  CUtensorMap mA, mB;
+  if ((e = tc_encode_bf16_map(&mA, pa, (long long)OZ_DIGITS * Mp, Krp, OZ_BM, OZ_KB_BYTES)) != cudaSuccess) return e;
+  if ((e = tc_encode_bf16_map(&mB, pb, (long long)OZ_DIGITS * Nrp, Krp, bn, OZ_KB_BYTES)) != cudaSuccess) return e;
+  const dim3 grid((unsigned)(Nrp / bn), (unsigned)(Mp / OZ_BM), (unsigned)((chunks + cps - 1) / cps));
+  auto go = [&](auto kern, int threads, int smem) {
+    kern<<<grid, threads, smem, s>>>(mA, mB, Mp, Nrp, chunks, cps, M, N, ea, eb, C, ldc, trans ? 1 : 0,
+                                     conj_out ? 1 : 0, pI, pU, timeouts);
+  };
+  if (bn == 64)
+    go(oz_gemm_kernel<64>, OzTile<64>::THREADS, OzTile<64>::SMEM);
+  else
+    go(oz_gemm_kernel<32>, OzTile<32>::THREADS, OzTile<32>::SMEM);
+  count_launch();
+  return cudaGetLastError();
+}
+
+size_t oz_al(size_t x) { return (x + 1023) & ~(size_t)1023; }
+
+}  // namespace
+
+size_t oz_square_bytes(int K) {
+  const size_t Mp = (size_t)(K + OZ_BM - 1) / OZ_BM * OZ_BM, Krp = (2 * (size_t)K + OZ_CHUNK - 1) / OZ_CHUNK * OZ_CHUNK;
+  return 2 * oz_al(4 * Mp) + oz_al((size_t)OZ_DIGITS * Mp * Krp * 2) + 1024;
+}
+
+cudaError_t oz_pack_square(cudaStream_t s, const cplx* Q, int K, void* memN, void* memT, OzSquare* outN,
+                           OzSquare* outT) {
+  const int Mp = (K + OZ_BM - 1) / OZ_BM * OZ_BM, Krp = (2 * K + OZ_CHUNK - 1) / OZ_CHUNK * OZ_CHUNK;
+  void* mem[2] = {memN, memT};
+  OzSquare* out[2] = {outN, outT};
+  int* raw[2];
+  cudaError_t e;
+  for (int v = 0; v < 2; ++v) {
+    char* p = (char*)(((uintptr_t)mem[v] + 1023) & ~(uintptr_t)1023);
+    out[v]->K = K;
+    out[v]->Mp = Mp;
+    out[v]->Krp = Krp;
+    raw[v] = (int*)p;
+    out[v]->e = (int*)(p + oz_al(4 * (size_t)Mp));
+    out[v]->p = p + 2 * oz_al(4 * (size_t)Mp);
+    if ((e = cudaMemsetAsync(raw[v], 0, 4 * (size_t)Mp, s)) != cudaSuccess) return e;
+  }
+  oz_square_exp_kernel<<<dim3((unsigned)((K + 31) / 32), (unsigned)((K + 127) / 128)), dim3(32, 8), 0, s>>>(Q, K, raw[1],
+                                                                                                     raw[0]);
+  // tiles cover Mp rows in both directions (Krp / 2 <= Mp)
+  oz_square_prep_kernel<<<dim3((unsigned)(Mp / 32), (unsigned)(Mp / 32)), dim3(32, 8), 0, s>>>(
+      Q, K, Mp, Krp, raw[1], raw[0], outT->e, outN->e, (__nv_bfloat16*)outT->p, (__nv_bfloat16*)outN->p);
+  count_launch(2);
+  return cudaGetLastError();
+}
+
+cudaError_t oz_thin(cudaStream_t s, int M, const cplx* A, long long lda, bool conj_in, const OzSquare& Q, cplx* C,
+                    long long ldc, bool conj_out, void* work, size_t work_bytes, int* timeouts) {
+  if (M <= 0) return cudaSuccess;
+  if (!timeouts || !work) return cudaErrorInvalidValue;
+  const int K = Q.K, chunks = Q.Krp / OZ_CHUNK;
+  char* base = (char*)(((uintptr_t)work + 1023) & ~(uintptr_t)1023);
+  const size_t fixed = oz_al((size_t)OZ_DIGITS * ((2 * (size_t)M + 63) / 64 * 64) * Q.Krp * 2) +
+                       oz_al(4 * ((2 * (size_t)M + 63) / 64 * 64)) + 3072;
+  if (work_bytes < fixed) return cudaErrorMemoryAllocation;
+  int bn = 64, Nrp = 0, cps = chunks;
+  oz_choose(Q.Mp, M, chunks, (double)(work_bytes - fixed), &bn, &Nrp, &cps);
+  const int S = (chunks + cps - 1) / cps;
+  int* eb = (int*)base;
+  __nv_bfloat16* pb = (__nv_bfloat16*)(base + oz_al(4 * (size_t)Nrp));
+  char* part = (char*)pb + oz_al((size_t)OZ_DIGITS * Nrp * Q.Krp * 2);
+  long long* pI = S > 1 ? (long long*)part : nullptr;
+  float* pU = S > 1 ? (float*)(part + (size_t)S * Q.Mp * Nrp * 8) : nullptr;
+  cudaError_t e;
+  oz_prep_kernel<<<(unsigned)(Nrp / 2), OZ_PREP_THREADS, 0, s>>>(nullptr, 0, OP_N, A, lda, OP_T | (conj_in ? OP_CONJ : 0),
+                                                               0, M, K, 0, Nrp, Q.Krp, nullptr, eb, nullptr, pb);
+  count_launch();
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if ((e = oz_launch(s, (__nv_bfloat16*)Q.p, pb, Q.Mp, Nrp, Q.Krp, bn, chunks, cps, K, M, Q.e, eb, C, ldc, true,
+                     conj_out, pI, pU, timeouts)) != cudaSuccess)
+    return e;
+  if (S > 1) {
+    oz_reduce_t_kernel<<<dim3((unsigned)((K + 31) / 32), (unsigned)((M + 31) / 32)), dim3(32, 8), 0, s>>>(
+        pI, pU, S, Q.Mp, Nrp, K, M, Q.e, eb, C, ldc, conj_out ? 1 : 0);
+    count_launch();
+    return cudaGetLastError();
+  }
+  return cudaSuccess;
+}
+
+size_t oz_work_bytes(int M, int N, int K) { return oz_layout(M, N, K).total; }
+
+cudaError_t oz_zgemm(cudaStream_t s, int M, int N, int K, const cplx* A, long long lda, int opA, const cplx* B,
+                     long long ldb, int opB, cplx* C, long long ldc, void* work, size_t work_bytes, int* timeouts) {
+  if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
+  if (!timeouts) return cudaErrorInvalidValue;
+  const OzLayout L = oz_layout(M, N, K);
+  if (!work || work_bytes < L.total) return cudaErrorMemoryAllocation;
+  cudaError_t e;
   char* base = (char*)(((uintptr_t)work + 1023) & ~(uintptr_t)1023);
   int* ea = (int*)(base + L.off_ea);
   int* eb = (int*)(base + L.off_eb);
@@ -549,20 +748,9 @@ cudaError_t oz_zgemm(cudaStream_t s, int M, int N, int K, const cplx* A, long lo
                                                                           L.Nrp, L.Krp, ea, eb, pa, pb);
   count_launch();
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  CUtensorMap mA, mB;
-  if ((e = tc_encode_bf16_map(&mA, pa, (long long)OZ_DIGITS * L.Mp, L.Krp, OZ_BM, OZ_KB_BYTES)) != cudaSuccess)
+  if ((e = oz_launch(s, pa, pb, L.Mp, L.Nrp, L.Krp, L.bn, L.chunks, L.cps, M, N, ea, eb, C, ldc, false, false, pI, pU,
+                     timeouts)) != cudaSuccess)
     return e;
-  if ((e = tc_encode_bf16_map(&mB, pb, (long long)OZ_DIGITS * L.Nrp, L.Krp, L.bn, OZ_KB_BYTES)) != cudaSuccess)
-    return e;
-  dim3 grid((unsigned)(L.Nrp / L.bn), (unsigned)(L.Mp / OZ_BM), (unsigned)L.S);
-  if (L.bn == 64)
-    oz_gemm_kernel<64><<<grid, OzTile<64>::THREADS, OzTile<64>::SMEM, s>>>(mA, mB, L.Mp, L.Nrp, L.chunks, L.cps, M,
-                                                                          N, ea, eb, C, ldc, pI, pU, timeouts);
-  else
-    oz_gemm_kernel<32><<<grid, OzTile<32>::THREADS, OzTile<32>::SMEM, s>>>(mA, mB, L.Mp, L.Nrp, L.chunks, L.cps, M,
-                                                                          N, ea, eb, C, ldc, pI, pU, timeouts);
-  count_launch();
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (L.S > 1) {
     oz_reduce_kernel<<<oz_grid((long long)M * N), 256, 0, s>>>(pI, pU, L.S, L.Mp, L.Nrp, M, N, ea, eb, C, ldc);
     count_launch();

@@ -121,3 +121,21 @@ cudaError_t tc_encode_bf16_map(CUtensorMap* map, void* base, long long rows, lon
 size_t oz_work_bytes(int M, int N, int K);
 cudaError_t oz_zgemm(cudaStream_t s, int M, int N, int K, const cplx* A, long long lda, int opA, const cplx* B,
                      long long ldb, int opB, cplx* C, long long ldc, void* work, size_t work_bytes, int* timeouts);
+
+// Thin FP64-accurate products C (M x K) = A (M x K) Q, computed transposed: the
+// digit planes of a square Q in both orientations are split once and serve every
+// product with it (splitting them for each of a cut's 28 products took as
+// long as a fifth of the products), and the real embedding doubles the thin
+// operand's planes instead of Q's.
+struct OzSquare {
+  int K, Mp, Krp;
+  int* e;   // row bounds
+  void* p;  // seven planes of Mp x Krp
+};
+size_t oz_square_bytes(int K);
+// Q (row-major K x K) for thin * Q (outN) and thin * Q^T (outT)
+cudaError_t oz_pack_square(cudaStream_t s, const cplx* Q, int K, void* memN, void* memT, OzSquare* outN,
+                           OzSquare* outT);
+// C = op(A) Q (op: conjugation with conj_in; the result conjugated with conj_out)
+cudaError_t oz_thin(cudaStream_t s, int M, const cplx* A, long long lda, bool conj_in, const OzSquare& Q, cplx* C,
+                    long long ldc, bool conj_out, void* work, size_t work_bytes, int* timeouts);
