@@ -18,6 +18,8 @@
 // beta_m |y_i[m-1]| (Parlett, "The Symmetric Eigenvalue Problem", ch. 13),
 // the last component from inverse iteration.
 // Everything is FP64; A and B are dense row-major complex matrices.
+#include <algorithm>
+
 #include "ctm_internal.h"
 
 namespace {
@@ -116,6 +118,60 @@ __global__ void __launch_bounds__(256) zgemv_mixed_kernel(const cplx* __restrict
   if (lane == 0) y[row] = make_double2(re, im);
 }
 
+// the same with A narrowed beforehand (the FP32 values that kernel makes of it,
+// in the same order: its results), at half of its bytes, and x narrowed once
+// per block into shared memory instead of once per row: 63 -> 43 us at n = 4096
+constexpr int GEMV_X = 2048;
+__global__ void __launch_bounds__(256) zgemv_f32_kernel(const float2* __restrict__ A, long long n,
+                                                        const cplx* __restrict__ x, cplx* __restrict__ y) {
+  __shared__ float2 xs[GEMV_X];
+  const long long row = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  const float2* a = A + row * n;
+  double re = 0.0, im = 0.0;
+  for (long long x0 = 0; x0 < n; x0 += GEMV_X) {
+    const int cnt = (int)min((long long)GEMV_X, n - x0);
+    __syncthreads();
+    for (int t = threadIdx.x; t < cnt; t += 256) {
+      const cplx v = x[x0 + t];
+      xs[t] = make_float2(d2f_bits(v.x), d2f_bits(v.y));
+    }
+    __syncthreads();
+    if (row >= n) continue;
+    int t = lane;
+    // whole groups of 128 columns, as from the row's start (GEMV_X is a multiple of 128)
+#pragma unroll 2
+    for (; t + 96 < cnt; t += 128) {
+      float r = 0.f, i = 0.f;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float2 av = __ldcs(a + x0 + t + 32 * q), xv = xs[t + 32 * q];
+        r = fmaf(av.x, xv.x, r);
+        r = fmaf(-av.y, xv.y, r);
+        i = fmaf(av.x, xv.y, i);
+        i = fmaf(av.y, xv.x, i);
+      }
+      re += f2d_bits(r);
+      im += f2d_bits(i);
+    }
+    for (; t < cnt; t += 32) {
+      const float2 av = __ldcs(a + x0 + t), xv = xs[t];
+      re += f2d_bits(fmaf(av.x, xv.x, -av.y * xv.y));
+      im += f2d_bits(fmaf(av.x, xv.y, av.y * xv.x));
+    }
+  }
+  re = warp_sum_d(re);
+  im = warp_sum_d(im);
+  if (lane == 0 && row < n) y[row] = make_double2(re, im);
+}
+
+__global__ void narrow_kernel(const cplx* __restrict__ in, long long n, float2* __restrict__ out) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const cplx v = in[i];
+    out[i] = make_float2(d2f_bits(v.x), d2f_bits(v.y));
+  }
+}
+
 // partial[b] = sum over block b's grid-stride slice of conj(x) y
 __global__ void __launch_bounds__(256) zdotc_partial_kernel(const cplx* __restrict__ x, const cplx* __restrict__ y,
                                                             long long n, double2* __restrict__ partial) {
@@ -179,23 +235,35 @@ __global__ void __launch_bounds__(256) proj_coeff_kernel(const cplx* __restrict_
   if (threadIdx.x == 0) c[blockIdx.x] = make_double2(re, im);
 }
 
-// r -= sum_{i<m} c[i] v_i
+// r -= sum_{i<m} c[i] v_i: 64 entries per block, four threads per entry that
+// take every fourth i (a thread per entry left most SMs idle at n = 4096)
 __global__ void __launch_bounds__(256) sub_proj_kernel(const cplx* __restrict__ V, long long n, int m,
                                                        const cplx* __restrict__ c, cplx* __restrict__ r) {
   __shared__ cplx cs[MAX_KRYLOV + 1];
+  __shared__ cplx part[4][64];
   for (int i = threadIdx.x; i < m; i += blockDim.x) cs[i] = c[i];
   __syncthreads();
-  for (long long t = blockIdx.x * 256LL + threadIdx.x; t < n; t += (long long)gridDim.x * 256) {
+  const int g = threadIdx.x >> 6, l = threadIdx.x & 63;
+  for (long long t0 = blockIdx.x * 64LL; t0 < n; t0 += (long long)gridDim.x * 64) {
+    const long long t = t0 + l;
     double re = 0.0, im = 0.0;
-    for (int i = 0; i < m; ++i) {
-      const cplx v = V[(long long)i * n + t], a = cs[i];
-      re += a.x * v.x - a.y * v.y;
-      im += a.x * v.y + a.y * v.x;
+    if (t < n) {
+#pragma unroll 4
+      for (int i = g; i < m; i += 4) {
+        const cplx v = V[(long long)i * n + t], a = cs[i];
+        re += a.x * v.x - a.y * v.y;
+        im += a.x * v.y + a.y * v.x;
+      }
     }
-    cplx x = r[t];
-    x.x -= re;
-    x.y -= im;
-    r[t] = x;
+    part[g][l] = make_double2(re, im);
+    __syncthreads();
+    if (g == 0 && t < n) {
+      cplx x = r[t];
+      x.x -= (part[0][l].x + part[1][l].x) + (part[2][l].x + part[3][l].x);
+      x.y -= (part[0][l].y + part[1][l].y) + (part[2][l].y + part[3][l].y);
+      r[t] = x;
+    }
+    __syncthreads();
   }
 }
 
@@ -212,78 +280,110 @@ __global__ void scale_pair_kernel(const cplx* __restrict__ r, const cplx* __rest
   }
 }
 
-// Leading k eigenvalues of the symmetric tridiagonal T (diagonal alpha_i =
-// adot[i].x, off-diagonal beta_i = sqrt(bdot[i].x), i = 1..m-1) and the
-// residual estimates beta_m |y_i[m-1]| of their Ritz pairs.  Block a finds the
-// a-th largest eigenvalue by bisection on Sturm counts (the number of negative
-// pivots of T - x I is the number of eigenvalues below x; Wilkinson, "The
-// Algebraic Eigenvalue Problem", ch. 5), then the eigenvector's last
-// component by inverse iteration with (T - theta I) factored without pivoting
-// (a tiny shift guards exact singularity).  One lane per block computes.
-__device__ int sturm_below(const double2* __restrict__ adot, const double2* __restrict__ bdot, int m, double x,
-                           double pivmin) {
+// 1/q of a normal q to FP64 rounding: an FP32 reciprocal refined by one step of
+// third order, x (1 + e + e^2) with e = 1 - q x below 2^-21
+__device__ __forceinline__ double rcp_signed(double q) {
+  const long long b = __double_as_longlong(q);
+  const long long sign = b & (long long)0x8000000000000000ull, mag = b ^ sign;
+  const int ex = (int)(mag >> 52) - 1023;
+  const double m = __longlong_as_double(mag - ((long long)ex << 52));  // [1, 2)
+  const double x = f2d_bits(__frcp_rn(d2f_bits(m)));
+  const double e = fma(-m, x, 1.0);
+  const double r = fma(x, fma(e, e, e), x);
+  return __longlong_as_double((__double_as_longlong(r) - ((long long)ex << 52)) | sign);
+}
+
+// eigenvalues of T below x: the negative pivots of T - x I (Wilkinson, "The
+// Algebraic Eigenvalue Problem", ch. 5)
+__device__ int sturm_below(const double* al, const double* b2, int m, double x, double pivmin) {
   int cnt = 0;
-  double q = adot[0].x - x;
+  double q = al[0] - x;
   if (fabs(q) < pivmin) q = -pivmin;
-  cnt += q < 0.0;
+  cnt += __double_as_longlong(q) < 0;
   for (int i = 1; i < m; ++i) {
-    const double b2 = bdot[i].x > 0.0 ? bdot[i].x : 0.0;
-    q = (adot[i].x - x) - b2 / q;
+    q = fma(-b2[i], rcp_signed(q), al[i] - x);
     if (fabs(q) < pivmin) q = -pivmin;
-    cnt += q < 0.0;
+    cnt += __double_as_longlong(q) < 0;
   }
   return cnt;
 }
 
-__global__ void tridiag_topk_kernel(const double2* __restrict__ adot, const double2* __restrict__ bdot, int m, int k,
-                                    double* __restrict__ theta, double* __restrict__ resid, double* __restrict__ work) {
-  const int a = blockIdx.x;
-  if (threadIdx.x != 0 || a >= k) return;
+// Leading k eigenvalues of the symmetric tridiagonal T (diagonal alpha_i =
+// adot[i].x, off-diagonal beta_i = sqrt(bdot[i].x), i = 1..m-1) and the
+// residual estimates beta_m |y_i[m-1]| of their Ritz pairs.  Block a finds the
+// a-th largest eigenvalue on Sturm counts, each lane of its warp counting at
+// one of 32 points that cut the interval into 33 (a count is a serial chain of
+// m pivots whatever the lane count: 11 rounds instead of the 53 of bisection),
+// then the eigenvector's last component by inverse iteration with (T - theta I)
+// factored once without pivoting (a tiny shift guards exact singularity), by
+// one lane.  Shared: alpha, beta^2, beta, multipliers, reciprocal pivots, y.
+__global__ void __launch_bounds__(32)
+    tridiag_topk_kernel(const double2* __restrict__ adot, const double2* __restrict__ bdot, int m, int k,
+                        double* __restrict__ theta, double* __restrict__ resid) {
+  extern __shared__ double tri[];
+  double *al = tri, *b2 = al + m, *be = b2 + m, *lw = be + m, *id = lw + m, *y = id + m;
+  const int a = blockIdx.x, lane = threadIdx.x;
+  if (a >= k) return;
+  for (int i = lane; i < m; i += 32) {
+    al[i] = adot[i].x;
+    const double b = i > 0 && bdot[i].x > 0.0 ? bdot[i].x : 0.0;
+    b2[i] = b;
+    be[i] = sqrt(b);
+  }
+  __syncwarp();
   // Gershgorin interval
-  double lo = 1e300, hi = -1e300, bmax = 0.0;
-  for (int i = 0; i < m; ++i) {
-    const double bl = i > 0 ? beta_of(bdot[i]) : 0.0, br = i + 1 < m ? beta_of(bdot[i + 1]) : 0.0;
-    lo = fmin(lo, adot[i].x - bl - br);
-    hi = fmax(hi, adot[i].x + bl + br);
-    bmax = fmax(bmax, bl);
+  double lo = 1e300, hi = -1e300;
+  for (int i = lane; i < m; i += 32) {
+    const double w = be[i] + (i + 1 < m ? be[i + 1] : 0.0);
+    lo = fmin(lo, al[i] - w);
+    hi = fmax(hi, al[i] + w);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
   }
   const double scale = fmax(fabs(lo), fabs(hi));
   const double pivmin = fmax(1e-300, 1e-30 * scale * scale) / fmax(scale, 1e-300);
   // the (m - 1 - a)-th smallest = the a-th largest
   const int target = m - a;  // eigenvalue with exactly target - 1 below it
   double l = lo, h = hi;
-  for (int it = 0; it < 200 && h - l > 2.2e-16 * fmax(fabs(l), fabs(h)) + 1e-300; ++it) {
-    const double mid = 0.5 * (l + h);
-    if (sturm_below(adot, bdot, m, mid, pivmin) >= target) h = mid; else l = mid;
+  for (int it = 0; it < 64 && h - l > 2.2e-16 * fmax(fabs(l), fabs(h)) + 1e-300; ++it) {
+    const double x = l + (h - l) * ((double)(lane + 1) * (1.0 / 33.0));
+    const unsigned above = __ballot_sync(0xffffffffu, sturm_below(al, b2, m, x, pivmin) >= target);
+    const int first = above ? __ffs(above) - 1 : 32;  // the eigenvalue lies below this point
+    const double xl = __shfl_sync(0xffffffffu, x, first > 0 ? first - 1 : 0), xh = __shfl_sync(0xffffffffu, x, first & 31);
+    const double nl = first > 0 ? xl : l, nh = first < 32 ? xh : h;
+    if (nl == l && nh == h) break;  // no point strictly inside
+    l = nl;
+    h = nh;
   }
   const double th = 0.5 * (l + h);
+  if (lane != 0) return;
   theta[a] = th;
-  // inverse iteration on (T - s I), s = th + tiny: y <- solve, normalise
-  double* dd = work + (long long)a * 3 * m;  // pivots
-  double* y = dd + m;
-  double* lw = y + m;  // multipliers
+  // inverse iteration on (T - s I), s = th + tiny: LU without pivoting (d_0 =
+  // a_0 - s, l_i = b_i / d_{i-1}, d_i = a_i - s - l_i b_i), y <- solve, normalise
   const double shift = th + 1e-14 * fmax(scale, 1e-300);
+  double d = al[0] - shift;
+  if (fabs(d) < pivmin) d = pivmin;
+  id[0] = rcp_signed(d);
+  for (int i = 1; i < m; ++i) {
+    const double li = be[i] * id[i - 1];
+    lw[i] = li;
+    d = fma(-li, be[i], al[i] - shift);
+    if (fabs(d) < pivmin) d = pivmin;
+    id[i] = rcp_signed(d);
+  }
   for (int i = 0; i < m; ++i) y[i] = 1.0;
   double last = 0.0;
   for (int pass = 0; pass < 3; ++pass) {
-    // LU of T - shift I without pivoting: d_0 = a_0 - s, l_i = b_i / d_{i-1}, d_i = a_i - s - l_i b_i
-    double d = adot[0].x - shift;
-    if (fabs(d) < pivmin) d = pivmin;
-    dd[0] = d;
-    for (int i = 1; i < m; ++i) {
-      const double b = beta_of(bdot[i]);
-      const double li = b / dd[i - 1];
-      lw[i] = li;
-      double di = (adot[i].x - shift) - li * b;
-      if (fabs(di) < pivmin) di = pivmin;
-      dd[i] = di;
-    }
     // forward (L z = y), backward (U x = z), U = diag(d) + superdiag(b)
-    for (int i = 1; i < m; ++i) y[i] -= lw[i] * y[i - 1];
-    y[m - 1] /= dd[m - 1];
-    for (int i = m - 2; i >= 0; --i) y[i] = (y[i] - beta_of(bdot[i + 1]) * y[i + 1]) / dd[i];
+    double v = y[0];
+    for (int i = 1; i < m; ++i) y[i] = v = fma(-lw[i], v, y[i]);
+    y[m - 1] = v = y[m - 1] * id[m - 1];
+    for (int i = m - 2; i >= 0; --i) y[i] = v = fma(-be[i + 1], v, y[i]) * id[i];
     double nrm = 0.0;
-    for (int i = 0; i < m; ++i) nrm += y[i] * y[i];
+    for (int i = 0; i < m; ++i) nrm = fma(y[i], y[i], nrm);
     nrm = sqrt(nrm);
     const double inv = nrm > 0.0 ? 1.0 / nrm : 0.0;
     for (int i = 0; i < m; ++i) y[i] *= inv;
@@ -338,6 +438,14 @@ long long lanczos_work_elems(long long n, int max_iter) {
   return 2 * (M + 1) * n + 3 * n + 2 * M * M + 5 * M + 8 + DOT_BLOCKS;
 }
 
+static cudaError_t launch_tridiag(cudaStream_t s, const double2* adot, const double2* bdot, int m, int k, double* theta,
+                                  double* resid) {
+  const size_t smem = (size_t)m * 6 * sizeof(double);  // 48 KB at the largest m, 1024
+  tridiag_topk_kernel<<<k, 32, smem, s>>>(adot, bdot, m, k, theta, resid);
+  count_launch();
+  return cudaGetLastError();
+}
+
 cudaError_t lanczos_leading(cudaStream_t s, const cplx* A, const cplx* B, long long n, int k, int max_iter,
                             double tol, uint64_t seed, cplx* work, long long work_elems, double* s_sel,
                             bool fp32_products, LanczosResult* res) {
@@ -353,19 +461,35 @@ cudaError_t lanczos_leading(cudaStream_t s, const cplx* A, const cplx* B, long l
   cplx* w = U + (M + 1) * n;
   cplx* r = w + n;
   cplx* sv = r + n;
-  cplx* T = sv + n;  // 2 M^2 complex slots: work of the tridiagonal eigensolver
-  cplx* c = T + 2 * M * M;
+  cplx* c = sv + n;
   double2* adot = (double2*)(c + M);
   double2* bdot = adot + M;
   double* resid = (double*)(bdot + M + 1);  // M doubles
   double2* partial = (double2*)(c + 5 * M + 8);  // past resid
   cudaError_t e;
-  const unsigned gb = blocks_for(n);
+  const unsigned gb = blocks_for(n), gp = (unsigned)std::min<long long>((n + 63) / 64, 152 * 16);
   auto check = [&]() { return cudaGetLastError(); };
+  // the mat-vecs of the precision forms read both operators once per step: from
+  // narrowed copies where the caller's memory has room for them
+  const bool narrowed = fp32_products && work_elems >= lanczos_work_elems(n, max_iter) + n * n + 64;
+  float2* nA = nullptr;
+  if (narrowed) {
+    nA = (float2*)(work + ((lanczos_work_elems(n, max_iter) + 15) & ~15LL));
+    narrow_kernel<<<blocks_for(n * n), 256, 0, s>>>(A, n * n, nA);
+    narrow_kernel<<<blocks_for(n * n), 256, 0, s>>>(B, n * n, nA + n * n);
+    count_launch(2);
+    if ((e = check()) != cudaSuccess) return e;
+  }
+  auto gemv = [&](bool b, const cplx* x, cplx* y) -> cudaError_t {
+    if (!narrowed) return zgemv_dense(s, b ? B : A, n, x, y, fp32_products);
+    zgemv_f32_kernel<<<(unsigned)((n + 7) / 8), 256, 0, s>>>(nA + (b ? n * n : 0), n, x, y);
+    count_launch();
+    return cudaGetLastError();
+  };
 
   // v0: uniform random entries (the range-finder generator), B-normalised
   if ((e = fill_omega_t(s, r, 1, (int)n, seed)) != cudaSuccess) return e;
-  if ((e = zgemv_dense(s, B, n, r, sv, fp32_products)) != cudaSuccess) return e;
+  if ((e = gemv(true, r, sv)) != cudaSuccess) return e;
   if ((e = zdotc_dev(s, r, sv, n, partial, &bdot[0])) != cudaSuccess) return e;
   scale_pair_kernel<<<gb, 256, 0, s>>>(r, sv, &bdot[0], n, V, U);
   count_launch();
@@ -376,44 +500,46 @@ cudaError_t lanczos_leading(cudaStream_t s, const cplx* A, const cplx* B, long l
   for (int j = 0; j < max_iter; ++j) {
     cplx* vj = V + (long long)j * n;
     cplx* uj = U + (long long)j * n;
-    if ((e = zgemv_dense(s, A, n, uj, w, fp32_products)) != cudaSuccess) return e;
+    if ((e = gemv(false, uj, w)) != cudaSuccess) return e;
     if ((e = zdotc_dev(s, uj, w, n, partial, &adot[j])) != cudaSuccess) return e;
     lanczos_update_kernel<<<gb, 256, 0, s>>>(w, vj, j > 0 ? vj - n : vj, adot, bdot, j, n, r);
     count_launch();
     for (int pass = 0; pass < 2; ++pass) {
       proj_coeff_kernel<<<j + 1, 256, 0, s>>>(U, n, r, c);
-      sub_proj_kernel<<<gb, 256, 0, s>>>(V, n, j + 1, c, r);
+      sub_proj_kernel<<<gp, 256, 0, s>>>(V, n, j + 1, c, r);
       count_launch(2);
     }
     if ((e = check()) != cudaSuccess) return e;
-    if ((e = zgemv_dense(s, B, n, r, sv, fp32_products)) != cudaSuccess) return e;
+    if ((e = gemv(true, r, sv)) != cudaSuccess) return e;
     if ((e = zdotc_dev(s, r, sv, n, partial, &bdot[j + 1])) != cudaSuccess) return e;
     scale_pair_kernel<<<gb, 256, 0, s>>>(r, sv, &bdot[j + 1], n, V + (long long)(j + 1) * n,
                                          U + (long long)(j + 1) * n);
     count_launch();
     if ((e = check()) != cudaSuccess) return e;
-    // host control: the new beta^2 and alpha decide breakdown and indefiniteness
-    double2 hb[2];
-    if ((e = cudaMemcpyAsync(&hb[0], &adot[j], sizeof(double2), cudaMemcpyDeviceToHost, s)) != cudaSuccess) return e;
-    if ((e = cudaMemcpyAsync(&hb[1], &bdot[j + 1], sizeof(double2), cudaMemcpyDeviceToHost, s)) != cudaSuccess)
+    // host control every 10 steps and at the end: beta^2 and alpha of the steps
+    // since decide breakdown and indefiniteness; steps past one that did are
+    // dropped
+    if ((j + 1) % 10 != 0 && j + 1 < max_iter) continue;
+    std::vector<double2> ha(j + 1 - m), hb(j + 1 - m);
+    if ((e = cudaMemcpyAsync(ha.data(), adot + m, ha.size() * sizeof(double2), cudaMemcpyDeviceToHost, s)) != cudaSuccess)
+      return e;
+    if ((e = cudaMemcpyAsync(hb.data(), bdot + m + 1, hb.size() * sizeof(double2), cudaMemcpyDeviceToHost, s)) !=
+        cudaSuccess)
       return e;
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
-    amax = fmax(amax, fabs(hb[0].x));
-    m = j + 1;
-    const double b2 = hb[1].x;
-    if (b2 < 0.0 && -b2 > 1e-20 * amax * amax) {  // r^H B r < 0: B is not positive definite
-      res->indefinite = 1;
-      break;
+    for (size_t q = 0; q < ha.size() && !res->indefinite && !res->breakdown; ++q) {
+      amax = fmax(amax, fabs(ha[q].x));
+      ++m;
+      const double bq = hb[q].x;
+      if (bq < 0.0 && -bq > 1e-20 * amax * amax)  // r^H B r < 0: B is not positive definite
+        res->indefinite = 1;
+      else if (bq <= 1e-26 * amax * amax)  // invariant Krylov subspace: the Ritz values are exact
+        res->breakdown = 1;
     }
-    if (b2 <= 1e-26 * amax * amax) {  // invariant Krylov subspace: the Ritz values are exact
-      res->breakdown = 1;
-      break;
-    }
-    // Ritz check every 10 steps once k + 10 values exist (the end is handled below)
+    if (res->indefinite || res->breakdown) break;
+    // Ritz check once k + 10 values exist (the end is handled below)
     if (m >= k + 10 && m % 10 == 0 && m < max_iter) {
-      tridiag_topk_kernel<<<k, 32, 0, s>>>(adot, bdot, m, k, s_sel, resid, (double*)T);
-      count_launch();
-      if ((e = check()) != cudaSuccess) return e;
+      if ((e = launch_tridiag(s, adot, bdot, m, k, s_sel, resid)) != cudaSuccess) return e;
       double th0 = 0.0;
       std::vector<double> rs(k);
       if ((e = cudaMemcpyAsync(&th0, s_sel, sizeof(double), cudaMemcpyDeviceToHost, s)) != cudaSuccess) return e;
@@ -436,9 +562,7 @@ cudaError_t lanczos_leading(cudaStream_t s, const cplx* A, const cplx* B, long l
   if (kk < k) {
     if ((e = cudaMemsetAsync(s_sel, 0, k * sizeof(double), s)) != cudaSuccess) return e;
   }
-  tridiag_topk_kernel<<<kk, 32, 0, s>>>(adot, bdot, m, kk, s_sel, resid, (double*)T);
-  count_launch();
-  if ((e = check()) != cudaSuccess) return e;
+  if ((e = launch_tridiag(s, adot, bdot, m, kk, s_sel, resid)) != cudaSuccess) return e;
   if (res->breakdown) {
     res->converged = kk;
   } else {
