@@ -633,40 +633,50 @@ __global__ void pack_square_kernel(const void* __restrict__ Q, int K, int D2, in
 // The sum of a thin product's K-split partials, P[z][n][2m .. 2m+1] (the
 // product is computed transposed: rows n, real columns 2m + (Re, Im)), as C[m,
 // n] (FP32 sums widened to FP64) and / or as the packed thin operand of the next
-// product (rows 2m: (Re, -Im), 2m+1: (Im, Re) along n).  32 x 32 complex tiles:
-// reads run along m, writes along n.  The grid covers the packed operand with
-// its padding, where the partials are products of zeros.
+// product (rows 2m: (Re, -Im), 2m+1: (Im, Re) along n).  A block takes 32 m x 8
+// n, reads running along m and writes along n, the splits in four groups of
+// warps (as one serial loop per output in 32 x 32 tiles the 38 splits of an 80
+// row, K = 1024 product took 60 us: too few loads in flight; 8.5 us so).  The grid covers
+// the packed operand with its padding, where the partials are products of
+// zeros.
+constexpr int THIN_ZG = 4;
 template <int PREC>
-__global__ void thin_reduce_kernel(const float* __restrict__ P, int S, long long pstride, int Nrp, int M, int N,
-                                   cplx* __restrict__ C, long long ldc, int conj_out, int Krp, void* __restrict__ o0,
-                                   void* __restrict__ o1, void* __restrict__ o2) {
-  __shared__ float2 tile[32][33];
-  const int n0 = blockIdx.x * 32, m0 = blockIdx.y * 32;
-  const int m = m0 + threadIdx.x;
-  for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-    const float* p = P + (long long)(n0 + i) * Nrp + 2 * m;
+__global__ void __launch_bounds__(256 * THIN_ZG)
+    thin_reduce_kernel(const float* __restrict__ P, int S, long long pstride, int Nrp, int M, int N,
+                       cplx* __restrict__ C, long long ldc, int conj_out, int Krp, void* __restrict__ o0,
+                       void* __restrict__ o1, void* __restrict__ o2) {
+  __shared__ float2 part[THIN_ZG][8][33];
+  const int n0 = blockIdx.x * 8, m0 = blockIdx.y * 32;
+  {
+    const float* p = P + (long long)(n0 + threadIdx.y) * Nrp + 2 * (m0 + threadIdx.x);
+    const int per = (S + THIN_ZG - 1) / THIN_ZG, z1 = min(S, (int)(threadIdx.z + 1) * per);
     float re = 0.0f, im = 0.0f;
-#pragma unroll 4
-    for (int z = 0; z < S; ++z) {
+#pragma unroll 8
+    for (int z = threadIdx.z * per; z < z1; ++z) {
       const float2 v = *(const float2*)(p + z * pstride);
       re += v.x;
       im += v.y;
     }
-    tile[i][threadIdx.x] = make_float2(re, im);
+    part[threadIdx.z][threadIdx.y][threadIdx.x] = make_float2(re, im);
   }
   __syncthreads();
-  const int n = n0 + threadIdx.x;
-  for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-    const float2 v = tile[threadIdx.x][i];
-    if (C && m0 + i < M && n < N) {
-      const double re = f2d_bits(v.x), im = f2d_bits(v.y);
-      C[(long long)(m0 + i) * ldc + n] = make_double2(re, conj_out ? neg_bits(im) : im);
-    }
-    if (o0 && 2 * n < Krp) {
-      const long long e = 2LL * (m0 + i) * Krp + 2 * (long long)n;
-      store_pair<PREC>(e, v.x, -v.y, o0, o1, o2);
-      store_pair<PREC>(e + Krp, v.y, v.x, o0, o1, o2);
-    }
+  const int t = threadIdx.y * 32 + threadIdx.x, i = t & 7, n = n0 + i, m = m0 + (t >> 3);
+  if (threadIdx.z != 0) return;
+  float2 v = part[0][i][t >> 3];
+#pragma unroll
+  for (int q = 1; q < THIN_ZG; ++q) {
+    const float2 w = part[q][i][t >> 3];
+    v.x += w.x;
+    v.y += w.y;
+  }
+  if (C && m < M && n < N) {
+    const double re = f2d_bits(v.x), im = f2d_bits(v.y);
+    C[(long long)m * ldc + n] = make_double2(re, conj_out ? neg_bits(im) : im);
+  }
+  if (o0 && 2 * n < Krp) {
+    const long long e = 2LL * m * Krp + 2 * (long long)n;
+    store_pair<PREC>(e, v.x, -v.y, o0, o1, o2);
+    store_pair<PREC>(e + Krp, v.y, v.x, o0, o1, o2);
   }
 }
 
@@ -1241,7 +1251,8 @@ cudaError_t run_thin(cudaStream_t s, const TcThin& A, const TcPacked& Q, cplx* C
       e = launch_main<PREC, 256>(s, o, S, N, M, make_double2(1.0, 0.0), nullptr, 0, false, part, timeouts, pr, true);
     if (e != cudaSuccess) return e;
     const long long rows = next ? std::max<long long>(N, o.Krp / 2) : N, cols = next ? o.Nrp / 2 : M;
-    thin_reduce_kernel<PREC><<<dim3((unsigned)((rows + 31) / 32), (unsigned)((cols + 31) / 32)), dim3(32, 8), 0, s>>>(
+    thin_reduce_kernel<PREC><<<dim3((unsigned)((rows + 7) / 8), (unsigned)((cols + 31) / 32)), dim3(32, 8, THIN_ZG), 0,
+                               s>>>(
         part, S, o.Mp * o.Nrp, (int)o.Nrp, M, N, C, ldc, conj_out ? 1 : 0, (int)o.Krp, next ? next->b[0] : nullptr,
         next ? next->b[1] : nullptr, next ? next->b[2] : nullptr);
     count_launch();
@@ -1260,7 +1271,10 @@ cudaError_t run_thin(cudaStream_t s, const TcThin& A, const TcPacked& Q, cplx* C
     if (it != tuner->table.end()) {
       choice = it->second.choice;
     } else if (tuner->measuring) {
-      cudaError_t e = tune_choice(s, tuner, key, o, choice, room, [&](TcChoice c) { return launch(c, nullptr); }, &choice);
+      // never summing more than twice the default's run in FP32: the sums'
+      // error grows with their length, and the timings do not see it
+      const int S0 = eff_splits(o.kb_total, choice.splits);
+      cudaError_t e = tune_choice(s, tuner, key, o, choice, [&](int S) { return 2 * S >= S0 && room(S); }, [&](TcChoice c) { return launch(c, nullptr); }, &choice);
       if (e != cudaSuccess) return e;
     }
   }
