@@ -1015,6 +1015,8 @@ cudaError_t jacobi_cluster(cudaStream_t s, cplx* G, int n, int m, long long ldg,
   return cudaGetLastError();
 }
 
+bool jacobi_batch_fits(int n) { return n >= 1 && cluster_init() == cudaSuccess && jacobi_smem(n, n, false, g_csize) > 0; }
+
 // Singular values only of `count` matrices (matrix b at G + b * strideG), one
 // cluster each in one launch.  Clusters of 8 where 16-CTA ones would not all
 // be resident: the FP64 units of the SMs in use bound the kernel, and 16

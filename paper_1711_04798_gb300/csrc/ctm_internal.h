@@ -130,7 +130,7 @@ cudaError_t jacobi_rows(cudaStream_t s, cplx* G, int n, int m, long long ldg, cp
                         long long wait_cycles = 0, bool warm_v = false, bool dfloat = false);
 // The singular values alone of `count` n x n matrices stored one after another
 // (rows made orthogonal in place): sigma[b n + i] = ||row i of matrix b||.
-// One launch, a cluster per matrix, where jacobi_cluster_fits(n, n); false
+// One launch, a cluster per matrix, where the rows fit a cluster; false
 // returned in *done (nothing launched) otherwise.
 cudaError_t jacobi_rows_batch(cudaStream_t s, cplx* G, int n, int count, double* sigma, int max_sweeps, DevStatus* st,
                               bool* done);
@@ -207,6 +207,7 @@ bool jacobi_cluster_fits(int n, int m);
 cudaError_t jacobi_cluster(cudaStream_t s, cplx* G, int n, int m, long long ldg, cplx* Vt, int max_sweeps,
                            DevStatus* st, cplx* rotlog, int* sweeps_used, bool warm_v = false,
                            bool dfloat = false);
+bool jacobi_batch_fits(int n);
 // the rows of `count` matrices (strideG apart) made orthogonal, one cluster each
 cudaError_t jacobi_cluster_batch(cudaStream_t s, cplx* G, int n, int m, long long ldg, long long strideG, int count,
                                  int max_sweeps, DevStatus* st);

@@ -667,7 +667,7 @@ cudaError_t jacobi_rows_batch(cudaStream_t s, cplx* G, int n, int count, double*
                               bool* done) {
   cudaError_t e;
   if ((e = kernels_init()) != cudaSuccess) return e;
-  *done = jacobi_cluster_fits(n, n);
+  *done = jacobi_batch_fits(n);
   if (!*done) return cudaSuccess;
   if ((e = jacobi_cluster_batch(s, G, n, n, n, (long long)n * n, count, max_sweeps, st)) != cudaSuccess) return e;
   return row_norms(s, G, n * count, n, n, sigma);
