@@ -1,5 +1,7 @@
 // Complex FP64 GEMM on the CUDA cores (the plain-FP64 path of the CTM
 // contractions) and the generic index permutation that feeds it.
+#include <cooperative_groups.h>
+
 #include "ctm_internal.h"
 
 #include <atomic>
@@ -7,6 +9,8 @@
 static std::atomic<uint64_t> g_launches{0};
 void count_launch(int n) { g_launches += (uint64_t)n; }
 uint64_t launch_counter() { return g_launches.load(); }
+
+namespace cg = cooperative_groups;
 
 namespace {
 
@@ -27,7 +31,9 @@ __device__ __forceinline__ cplx ld_op(const cplx* p, bool cj) {
 // the SM's units for some 70 cycles), so the tile only sets how evenly the
 // product covers the SMs and how much of it is padding: a 32 x 32 tile with K =
 // 64 is 70 us of one SM's FP64 time.
-template <int MI>
+// FUSED (MI = 1): the K splits of a tile are the CTAs of a cluster, whose sums meet
+// in shared memory, in split order, without a second kernel.
+template <int MI, bool FUSED = false>
 __global__ void __launch_bounds__(256) zgemm_kernel(int M, int N, int K, cplx alpha, const cplx* __restrict__ A,
                                                     long long lda, int opA, const cplx* __restrict__ B,
                                                     long long ldb, int opB, cplx beta, cplx* __restrict__ C,
@@ -38,8 +44,11 @@ __global__ void __launch_bounds__(256) zgemm_kernel(int M, int N, int K, cplx al
   __shared__ cplx Bs[BK][T + 1];
   const long long bz = blockIdx.z;
   const int m0 = blockIdx.y * T, n0 = blockIdx.x * T;
-  if ((flags & ZG_UPPER_TILES) && blockIdx.y > blockIdx.x) return;  // tile below the diagonal: not needed
   const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+  if ((flags & ZG_UPPER_TILES) && blockIdx.y > blockIdx.x) {  // tile below the diagonal: not needed
+    if (FUSED && blockIdx.z == 0 && m0 + ty < M && n0 + tx < N) C[(long long)(m0 + ty) * ldc + n0 + tx] = ZERO_C;
+    return;
+  }
   const bool tA = opA & OP_T, cA = opA & OP_CONJ;
   const bool tB = opB & OP_T, cB = opB & OP_CONJ;
   if (ksplit > 0) {
@@ -49,7 +58,7 @@ __global__ void __launch_bounds__(256) zgemm_kernel(int M, int N, int K, cplx al
     B += tB ? kb : kb * ldb;
     K = (int)min((long long)ksplit, (long long)K - kb);
     if (flags & ZG_A_LOWER) K = (int)max(0LL, min((long long)K, (long long)(m0 + T) - kb));
-    C += bz * sC;
+    if (!FUSED) C += bz * sC;
   } else {
     if (flags & ZG_A_LOWER) K = min(K, m0 + T);  // A[m, k] = 0 for k > m: later k-tiles add nothing
     A += bz * sA;
@@ -105,6 +114,33 @@ __global__ void __launch_bounds__(256) zgemm_kernel(int M, int N, int K, cplx al
     __syncthreads();
   }
   const bool use_beta = (beta.x != 0.0 || beta.y != 0.0);
+  if constexpr (FUSED) {
+    cg::cluster_group cl = cg::this_cluster();
+    const int S = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+    cplx* tile = &As[0][0];  // 256 sums; the last k-tile's reads ended at a block barrier
+    tile[threadIdx.x] = make_double2(cr[0][0], ci[0][0]);
+    cl.sync();
+    const int per = (256 + S - 1) / S, e = rank * per + threadIdx.x;
+    const int m = m0 + e / 16, n = n0 + e % 16;
+    if (threadIdx.x < per && e < 256 && m < M && n < N) {
+      double r = 0.0, i = 0.0;
+      for (int z = 0; z < S; ++z) {
+        const cplx v = cl.map_shared_rank(tile, z)[e];
+        r += v.x;
+        i += v.y;
+      }
+      cplx* cp = C + (long long)m * ldc + n;
+      double orr = alpha.x * r - alpha.y * i, oi = alpha.x * i + alpha.y * r;
+      if (use_beta) {
+        const cplx o = *cp;
+        orr += beta.x * o.x - beta.y * o.y;
+        oi += beta.x * o.y + beta.y * o.x;
+      }
+      *cp = make_double2(orr, oi);
+    }
+    cl.sync();  // no CTA leaves while another reads its sums
+    return;
+  }
 #pragma unroll
   for (int i = 0; i < MI; ++i) {
     const int m = m0 + ty + 16 * i;
@@ -195,7 +231,7 @@ cudaError_t zgemm(cudaStream_t s, int M, int N, int K, cplx alpha, const cplx* A
   // and for a split the second kernel with the partials' round trip.
   int best_T = 64, best_k = 0;  // best_k: k per split, 0 = unsplit
   double best_cost = -1.0;
-  const bool can_split = batch.count == 1 && work && K >= 16;
+  const bool can_split = batch.count == 1 && K >= 16;
   for (int T : {64, 32, 16}) {
     if (T != 64 && (batch.count != 1 || M > 65535LL * T)) continue;
     const long long tm = (M + T - 1) / T, tn = (N + T - 1) / T;
@@ -207,11 +243,17 @@ cudaError_t zgemm(cudaStream_t s, int M, int N, int K, cplx alpha, const cplx* A
       if (kps < 8 || kps == last) continue;
       last = kps;
       const long long Se = (K + kps - 1) / kps;
-      if (Se > 1 && Se * M * N > work_elems) break;
+      if (Se > 1 && Se * M * N > work_elems && !(T == 16 && Se <= 8)) continue;
       const long long busy = (tiles * Se * batch.count + 151) / 152;
       const double rate = busy == 1 ? 0.61 : 1.0;
       double cost = (double)kps * (double)busy * per_k / rate + (double)((kps + BK - 1) / BK) / (double)busy;
-      if (Se > 1) cost += 4.0 + (double)Se * (double)M * (double)N * 32.0 / 5e6;
+      // up to eight splits of 16-wide tiles meet in a cluster's shared memory
+      // (1.5 us), others in a second kernel with the partials' round trip
+      const bool fused = T == 16 && Se > 1 && Se <= 8;
+      if (fused)
+        cost += 1.5;
+      else if (Se > 1)
+        cost += 4.0 + (double)Se * (double)M * (double)N * 32.0 / 5e6;
       if (best_cost < 0.0 || cost < best_cost) {
         best_cost = cost;
         best_k = Se > 1 ? kps : 0;
@@ -236,6 +278,23 @@ cudaError_t zgemm(cudaStream_t s, int M, int N, int K, cplx alpha, const cplx* A
   if (tm > 65535) return cudaErrorInvalidConfiguration;
   if (best_k > 0) {
     const long long S = (K + best_k - 1) / best_k;
+    if (T == 16 && S <= 8) {
+      cudaLaunchConfig_t cfg = {};
+      cudaLaunchAttribute attr;
+      attr.id = cudaLaunchAttributeClusterDimension;
+      attr.val.clusterDim.x = 1;
+      attr.val.clusterDim.y = 1;
+      attr.val.clusterDim.z = (unsigned)S;
+      cfg.gridDim = dim3((unsigned)tn, (unsigned)tm, (unsigned)S);
+      cfg.blockDim = dim3(256);
+      cfg.stream = s;
+      cfg.attrs = &attr;
+      cfg.numAttrs = 1;
+      const cudaError_t e = cudaLaunchKernelEx(&cfg, zgemm_kernel<1, true>, M, N, K, alpha, A, lda, opA, B, ldb, opB, beta,
+                                               C, ldc, 0LL, 0LL, 0LL, best_k, flags);
+      count_launch();
+      return e;
+    }
     launch(dim3((unsigned)tn, (unsigned)tm, (unsigned)S), ONE_C, ZERO_C, work, N, (long long)M * N, best_k, flags);
     long long blocks = ((long long)M * N + 255) / 256;
     if (blocks > 152 * 16) blocks = 152 * 16;
