@@ -744,14 +744,17 @@ __global__ void jacobi_replay_kernel(cplx* __restrict__ Vt, int n, const double4
 // a serial chain of n warp reductions per column).
 //
 // Blocked by CH_NB rows.  Rows of the working copy W live in the cluster's
-// shared memory (row i in CTA i mod csize).  For the block of rows j0 ..
-// j0+nb-1 each CTA factors the nb x nb diagonal block (every CTA the same
-// arithmetic, so the same pivots) and the block's entries in the other
-// columns it owns (l mod csize = rank), one barrier of four warps per row; after
-// a cluster barrier every CTA gathers the block's rows and updates its own
-// rows below the block.  Bound: the serial chain of pivots (each an FP64
-// reciprocal root and a rank-one update, some 0.4 us) and the trailing update
-// on the FP64 units of the cluster's SMs.
+// shared memory (row i in CTA i mod csize, csize a power of two).  For the
+// block of rows j0 .. j0+nb-1 each CTA factors the nb x nb diagonal block
+// (every CTA the same arithmetic, so the same pivots) and the block's entries
+// in the other columns it owns (l mod csize = rank), one barrier of four warps per row, and
+// writes its scaled columns into every CTA's copy of the block's rows; after a
+// cluster barrier every CTA updates its own rows below the block and writes
+// those of the next block straight to the CTAs that factor them.  Bound: the
+// serial chain of pivots (each an FP64 reciprocal and a rank-one update, some
+// 0.3 us) and the trailing update on the FP64 units of the cluster's SMs.
+// Written by its maker, a row needs no round trip through the cluster to be
+// gathered (n = 116: 132 -> 98 us, 209 -> 163 us where no pivot is dropped).
 constexpr int CH_NB = 8;
 constexpr int CH_PANEL = 128;  // threads of the panel's barrier
 
@@ -786,37 +789,41 @@ __global__ void __launch_bounds__(CL_THREADS)
   double dmax = 0.0;
   for (int r = 0; r < cs; ++r) dmax = fmax(dmax, *cl.map_shared_rank(&s_max, r));
   const double thr = tol * dmax;
+  const int own = cs - 1;  // l & own: the owner of column (or row) l
   for (int j0 = 0; j0 < n; j0 += CH_NB) {
     const int nb = min(CH_NB, n - j0), jn = j0 + nb;
     // columns this CTA works on: the diagonal block (c < nb), then its own
-    // columns outside it, left ones first
-    const int nleft = j0 > rank ? (j0 - 1 - rank) / cs + 1 : 0;
-    const int off = ((rank - jn) % cs + cs) % cs;  // first own column at or after jn is jn + off
+    // columns outside it, left ones (L^{-1}) first
+    const int nleft = Lout && j0 > rank ? (j0 - 1 - rank) / cs + 1 : 0;
+    const int off = (rank - jn) & own;  // first own column at or after jn is jn + off
     const int nright = jn + off < n ? (n - 1 - (jn + off)) / cs + 1 : 0;
     const int ncol = nb + nleft + nright;
+    const unsigned rec = 65536u / ncol + 1;  // e / ncol = e rec >> 16 for e ncol < 65536
     auto col = [&](int c) {
       c -= nb;
       return c < 0 ? jn + c : (c < nleft ? rank + c * cs : jn + off + (c - nleft) * cs);
     };
-    // the block's rows of W on those columns, from their owners
-    for (int e = threadIdx.x; e < nb * ncol; e += CL_THREADS) {
-      const int jj = e / ncol, l = col(e % ncol), j = j0 + jj;
-      pan[(long long)jj * n + l] = cl.map_shared_rank(sm, j % cs)[(long long)(j / cs) * n + l];
+    if (j0 == 0) {  // the first block's rows of W on those columns, from their owners
+      for (int e = threadIdx.x; e < nb * ncol; e += CL_THREADS) {
+        const int jj = e / ncol, l = col(e % ncol);
+        pan[(long long)jj * n + l] = cl.map_shared_rank(sm, jj & own)[(long long)(jj / cs) * n + l];
+      }
+      __syncthreads();
     }
-    __syncthreads();
     if (threadIdx.x < CH_PANEL) {
       // rows i > j of the block on every column: W[i,l] -= conj(W[j,i]) W[j,l] / d,
       // for l >= i (the Schur complement) and l <= j (L^{-1}, whose column j
-      // starts here from 0 with a one in W[j,j]'s place).  Every thread forms 1/d
-      // itself: four FP64 instructions against a second barrier.
+      // starts here from 0 with a one in W[j,j]'s place).  Every warp with an
+      // element forms 1/d itself: four FP64 instructions against a second barrier.
       for (int jj = 0; jj < nb - 1; ++jj) {
-        const int j = j0 + jj;
+        const int j = j0 + jj, todo = (nb - 1 - jj) * ncol;
         const cplx* pj = pan + (long long)jj * n;
         const double d = pj[j].x;
-        if (d > thr) {  // the same in every thread; a dropped direction updates nothing
+        // d > thr: the same in every thread; a dropped direction updates nothing
+        if (d > thr && (int)(threadIdx.x & ~31u) < todo) {
           const double inv = rcp64(d);
-          for (int e = threadIdx.x; e < (nb - 1 - jj) * ncol; e += CH_PANEL) {
-            const int i = j + 1 + e / ncol, l = col(e % ncol);
+          for (int e = threadIdx.x; e < todo; e += CH_PANEL) {
+            const int q = (int)((unsigned)e * rec >> 16), i = j + 1 + q, l = col(e - q * ncol);
             if (l > j && l < i) continue;
             cplx* w = pan + (long long)(i - j0) * n + l;
             const bool diag = l == j;
@@ -838,45 +845,57 @@ __global__ void __launch_bounds__(CL_THREADS)
         if (threadIdx.x == 0) s_kept = mask;
       }
       asm volatile("bar.sync 1, %0;" ::"n"(CH_PANEL) : "memory");
-      // the block's rows scaled: R right of the diagonal, L^{-1} left of it and on it
+      // the block's rows scaled: R right of the diagonal, L^{-1} left of it and on
+      // it; the diagonal block is every CTA's own, the other columns go to all
       for (int e = threadIdx.x; e < nb * ncol; e += CH_PANEL) {
-        const int jj = e / ncol, l = col(e % ncol);
+        const int jj = (int)((unsigned)e * rec >> 16), c = e - jj * ncol, l = col(c);
         const double inv = s_inv[jj];
         const cplx g = pan[(long long)jj * n + l];
         cplx v = make_double2(g.x * inv, g.y * inv);
         if (l == j0 + jj) v = make_double2(inv, 0.0);
         if (!(s_kept >> jj & 1u)) v = make_double2(0.0, 0.0);
-        rpan[(long long)jj * n + l] = v;
+        cplx* to = rpan + (long long)jj * n + l;
+        if (c < nb) {
+          *to = v;
+        } else {
+#pragma unroll 8
+          for (int r = 0; r < cs; ++r) *cl.map_shared_rank(to, r) = v;
+        }
       }
     }
-    cl.sync();  // every CTA's columns of the block's rows are final
-    // the other CTAs' columns of those rows
-    for (int e = threadIdx.x; e < nb * (n - nb); e += CL_THREADS) {
-      const int jj = e / (n - nb), q = e % (n - nb), l = q < j0 ? q : q + nb;
-      const int o = l % cs;
-      if (o != rank) rpan[(long long)jj * n + l] = cl.map_shared_rank(rpan, o)[(long long)jj * n + l];
-    }
-    __syncthreads();
+    cl.sync();  // the block's rows are complete in every CTA, and pan is free
     // the owners store their rows of R and L^{-1}
     for (int jj = 0; jj < nb; ++jj) {
       const int j = j0 + jj;
-      if (j % cs != rank) continue;
+      if ((j & own) != rank) continue;
       for (int l = threadIdx.x; l < n; l += CL_THREADS) {
         const cplx v = rpan[(long long)jj * n + l], z = make_double2(0.0, 0.0);
         if (Rout) Rout[(long long)j * n + l] = l < j ? z : (l == j ? make_double2(s_rjj[jj], 0.0) : v);
         if (Lout) Lout[(long long)j * n + l] = l > j ? z : v;
       }
     }
+    // below the next block's diagonal nothing has been written yet: zero, which
+    // is what L^{-1} keeps there for a dropped pivot
+    if (threadIdx.x < CH_NB * CH_NB) {
+      const int jj = threadIdx.x / CH_NB, c = threadIdx.x % CH_NB;
+      if (c < jj && jn + jj < n) pan[(long long)jj * n + jn + c] = make_double2(0.0, 0.0);
+    }
     // own rows below the block, on the columns l < jn (L^{-1}: the block's own
     // columns start here, from the rows at and below them) and l >= i: the
-    // (row, column) pairs of all own rows spread over the threads
+    // (row, column) pairs of all own rows, row after row, spread over the threads
     const unsigned kept = s_kept;
-    const int l0 = jn > rank ? (jn - rank + cs - 1) / cs : 0;  // first own row at or after jn
-    const int span = Lout ? n : n - jn;
-    const int todo = (R - l0) * span;
-    for (int e = threadIdx.x; e < todo; e += CL_THREADS) {
-      const int lr = l0 + e / span, i = lr * cs + rank, c = e % span, l = Lout ? c : jn + c;
-      if (i >= n || (l >= jn && l < i)) continue;
+    const int left = Lout ? jn : 0;
+    int lr = jn > rank ? (jn - rank + cs - 1) / cs : 0;  // first own row at or after jn
+    int i = lr * cs + rank, len = left + n - i, e = threadIdx.x;
+    while (true) {
+      while (i < n && e >= len) {
+        e -= len;
+        len -= cs;
+        i += cs;
+        ++lr;
+      }
+      if (i >= n) break;
+      const int l = e < left ? e : i + (e - left);
       cplx* w = sm + (long long)lr * n + l;
       const bool fresh = l >= j0 && l < jn;
       cplx v = fresh ? make_double2(0.0, 0.0) : *w;
@@ -888,9 +907,20 @@ __global__ void __launch_bounds__(CL_THREADS)
         v.x = fma(-a.x, b.x, fma(-a.y, b.y, v.x));
         v.y = fma(-a.x, b.y, fma(a.y, b.x, v.y));
       }
-      *w = v;
+      if (i >= jn + CH_NB) {
+        *w = v;
+      } else {  // a row of the next block: to the CTAs that work on its column
+        cplx* to = pan + (long long)(i - jn) * n + l;
+        if (l >= jn && l < jn + CH_NB) {
+#pragma unroll 8
+          for (int r = 0; r < cs; ++r) *cl.map_shared_rank(to, r) = v;
+        } else {
+          *cl.map_shared_rank(to, l & own) = v;
+        }
+      }
+      e += CL_THREADS;
     }
-    cl.sync();  // rows updated before they are read as the next block; gathers done before rpan is rewritten
+    cl.sync();  // the next block's rows have arrived; rpan is read no more
   }
 }
 
