@@ -112,8 +112,8 @@ __device__ __forceinline__ df2 df_add(df2 a, df2 b) {
   return df_norm(r);
 }
 
-// 1/sqrt(a) of a normalised a > 0: an FP32 root refined by one step of third
-// order, x (1 + e/2 + 3 e^2/8) with e = 1 - a x^2 in double-float
+// 1/sqrt(a) of a normalised a > 0: an FP32 root refined by one Householder step
+// of third order, x (1 + e/2 + 3 e^2/8) with e = 1 - a x^2 in double-float
 __device__ __forceinline__ df2 df_rsqrt(df2 a) {
   const float x = rsqrtf(a.h);
   const df2 xx = {x, 0.f};
@@ -125,7 +125,7 @@ __device__ __forceinline__ df2 df_rsqrt(df2 a) {
 
 // 1/sqrt(a) of a finite a > 0 to FP64 rounding with five FP64 instructions:
 // the argument scaled into [1, 4) and converted on the integer pipe, an FP32
-// root, one step of third order (its error (5/16) e^3 with |e| < 2^-21)
+// root, one Householder step of third order (its error (5/16) e^3 with |e| < 2^-21)
 __device__ __forceinline__ double rsqrt64(double a) {
   const long long b = __double_as_longlong(a);
   const int ex = (int)(b >> 52) - 1023, half = ex >> 1;                  // a = m 4^half, m in [1, 4)
@@ -136,7 +136,8 @@ __device__ __forceinline__ double rsqrt64(double a) {
   return __longlong_as_double(__double_as_longlong(r) - ((long long)half << 52));
 }
 
-// 1/a of a normal a > 0 the same way: an FP32 reciprocal, one step of third order
+// 1/a of a normal a > 0 the same way: an FP32 reciprocal, one Householder
+// step of third order
 __device__ __forceinline__ double rcp64(double a) {
   const long long b = __double_as_longlong(a);
   const int ex = (int)(b >> 52) - 1023;

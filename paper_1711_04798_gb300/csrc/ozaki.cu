@@ -32,8 +32,8 @@
 // without a wide spread of magnitudes, as the projector step's are.
 //
 // One CTA computes a 128 x 32 or 128 x 64 tile of Cr over a range of K
-// chunks: warp 0 issues the TMA loads (per stage one A digit plane and the B
-// planes it pairs with), warp 1 the tcgen05.mma, the other warps (four or
+// chunks: warp 0 issues the TMA loads (per stage a k-block of all planes of
+// both operands), warp 1 the tcgen05.mma, the other warps (four or
 // eight) drain the seven group accumulators after each chunk.  Ranges of K
 // are split over the grid; the exact partials (I, u) are summed by a second
 // kernel.
@@ -166,33 +166,46 @@ __device__ __forceinline__ cplx oz_load(const cplx* X, long long ld, int op, int
 // row 2n (Re, -Im) and row 2n+1 (Im, Re) at columns 2k, 2k+1 of each plane of
 // Br^T [Nrp x Krp].  The block first reduces the row's largest exponent, then
 // writes its digits; the row is read twice, the second time from cache.
+// WARP: a warp per row, four rows to a block, for many short rows (a block's
+// start and its two barriers took longer than the at most four elements per
+// lane: 19456 rows of 27 took 38 us, 18 us so).
+// A row with an infinity or a NaN gets the bound OZ_NONFINITE (its digits are
+// zero then), which makes every output of that row NaN.
 constexpr int OZ_PREP_THREADS = 128;
+constexpr int OZ_NONFINITE = 1 << 20;
+template <bool WARP>
 __global__ void __launch_bounds__(OZ_PREP_THREADS)
     oz_prep_kernel(const cplx* __restrict__ A, long long lda, int opA, const cplx* __restrict__ B, long long ldb,
                    int opB, int M, int N, int K, int Mp, int Nrp, int Krp, int* __restrict__ ea, int* __restrict__ eb,
                    __nv_bfloat16* __restrict__ pa, __nv_bfloat16* __restrict__ pb) {
   __shared__ int s_e[OZ_PREP_THREADS / 32];
-  const bool is_a = (int)blockIdx.x < Mp;
-  const int r = is_a ? (int)blockIdx.x : (int)blockIdx.x - Mp;  // row of op(A), or column of op(B)
+  constexpr int NT = WARP ? 32 : OZ_PREP_THREADS;
+  const int row = WARP ? (int)blockIdx.x * (OZ_PREP_THREADS / 32) + (int)(threadIdx.x >> 5) : (int)blockIdx.x;
+  const int tid = WARP ? threadIdx.x & 31 : threadIdx.x;
+  if (WARP && row >= Mp + Nrp / 2) return;
+  const bool is_a = row < Mp;
+  const int r = is_a ? row : row - Mp;  // row of op(A), or column of op(B)
   const bool live = is_a ? r < M : r < N;
   auto load = [&](int c) {
     return is_a ? oz_load(A, lda, opA, r, c) : oz_load(B, ldb, opB, c, r);
   };
   int E = 0;
   if (live)
-    for (int c = threadIdx.x; c < K; c += OZ_PREP_THREADS) {
+    for (int c = tid; c < K; c += NT) {
       const cplx v = load(c);
       E = max(E, max(bexp(v.x), bexp(v.y)));
     }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, o));
-  if ((threadIdx.x & 31) == 0) s_e[threadIdx.x >> 5] = E;
-  __syncthreads();
-  E = s_e[0];
+  if constexpr (!WARP) {
+    if ((threadIdx.x & 31) == 0) s_e[threadIdx.x >> 5] = E;
+    __syncthreads();
+    E = s_e[0];
 #pragma unroll
-  for (int w = 1; w < OZ_PREP_THREADS / 32; ++w) E = max(E, s_e[w]);
-  const int e = E ? E - 1022 : 0;
-  if (threadIdx.x == 0) {
+    for (int w = 1; w < OZ_PREP_THREADS / 32; ++w) E = max(E, s_e[w]);
+  }
+  const int e = E == 0x7FF ? OZ_NONFINITE : (E ? E - 1022 : 0);
+  if (tid == 0) {
     if (is_a)
       ea[r] = e;
     else
@@ -200,7 +213,7 @@ __global__ void __launch_bounds__(OZ_PREP_THREADS)
   }
   const long long kc = Krp / 2;
   const long long plane = is_a ? (long long)Mp * Krp : (long long)Nrp * Krp;
-  for (int c = threadIdx.x; c < kc; c += OZ_PREP_THREADS) {
+  for (int c = tid; c < kc; c += NT) {
     cplx v = make_double2(0.0, 0.0);
     if (live && c < K) v = load(c);
     int dr[OZ_DIGITS], di[OZ_DIGITS];
@@ -224,8 +237,10 @@ __global__ void __launch_bounds__(OZ_PREP_THREADS)
   }
 }
 
-// Cr element from its exact sums: 2^(ea + eb - 38) (I + 2^-8 u)
+// Cr element from its exact sums: 2^(ea + eb - 38) (I + 2^-8 u), NaN where a
+// bound is OZ_NONFINITE
 __device__ __forceinline__ double oz_value(long long I, float u, int ea, int eb) {
+  if (ea + eb > OZ_NONFINITE / 2) return __longlong_as_double(0x7FF8000000000000LL);
   return ((double)I + (double)u * (1.0 / 256.0)) * pow2(ea + eb - 38);
 }
 
@@ -712,7 +727,7 @@ cudaError_t oz_thin(cudaStream_t s, int M, const cplx* A, long long lda, bool co
   long long* pI = S > 1 ? (long long*)part : nullptr;
   float* pU = S > 1 ? (float*)(part + (size_t)S * Q.Mp * Nrp * 8) : nullptr;
   cudaError_t e;
-  oz_prep_kernel<<<(unsigned)(Nrp / 2), OZ_PREP_THREADS, 0, s>>>(nullptr, 0, OP_N, A, lda, OP_T | (conj_in ? OP_CONJ : 0),
+  oz_prep_kernel<false><<<(unsigned)(Nrp / 2), OZ_PREP_THREADS, 0, s>>>(nullptr, 0, OP_N, A, lda, OP_T | (conj_in ? OP_CONJ : 0),
                                                                0, M, K, 0, Nrp, Q.Krp, nullptr, eb, nullptr, pb);
   count_launch();
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -744,8 +759,16 @@ cudaError_t oz_zgemm(cudaStream_t s, int M, int N, int K, const cplx* A, long lo
   __nv_bfloat16* pb = (__nv_bfloat16*)(base + L.off_b);
   long long* pI = L.S > 1 ? (long long*)(base + L.off_pi) : nullptr;
   float* pU = L.S > 1 ? (float*)(base + L.off_pu) : nullptr;
-  oz_prep_kernel<<<(unsigned)(L.Mp + L.Nrp / 2), OZ_PREP_THREADS, 0, s>>>(A, lda, opA, B, ldb, opB, M, N, K, L.Mp,
-                                                                          L.Nrp, L.Krp, ea, eb, pa, pb);
+  const int rows = L.Mp + L.Nrp / 2, per = OZ_PREP_THREADS / 32;
+  auto prep = [&](auto kern, int blocks) {
+    kern<<<(unsigned)blocks, OZ_PREP_THREADS, 0, s>>>(A, lda, opA, B, ldb, opB, M, N, K, L.Mp, L.Nrp, L.Krp, ea, eb, pa,
+                                                      pb);
+  };
+  // a warp per row where the rows are short and fill the chip several times so
+  if (L.Krp <= 256 && rows >= 152 * 32)
+    prep(oz_prep_kernel<true>, (rows + per - 1) / per);
+  else
+    prep(oz_prep_kernel<false>, rows);
   count_launch();
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if ((e = oz_launch(s, pa, pb, L.Mp, L.Nrp, L.Krp, L.bn, L.chunks, L.cps, M, N, ea, eb, C, ldc, false, false, pI, pU,

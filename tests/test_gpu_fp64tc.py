@@ -182,3 +182,22 @@ def test_batch_of_uneven_instances():
         assert abs(e[i] - e_ref) < TOL * abs(e_ref), (i, e[i], e_ref)
         assert spectra_err(b.instance(i).spectra(), O.corner_spectra(st)) < TOL, i
     b.close()
+
+
+@pytest.mark.parametrize("chi", [11, 12, 20, 33])
+def test_tall_narrow_readout_products_match_fp64(chi):
+    """D = 3 bond readouts end in products of 72 chi^2 rows, 24 columns, K = 27:
+    on the FP64 CUDA cores at chi = 11, from chi = 12 digit-split in slabs of
+    19456 rows (one short one, two and five with a rest).  The same environment
+    read in plain FP64: every RDM element is a sum of positive weight one whose
+    few contractions round at 1e-15 of it."""
+    t = [synth.product_plus_noise(5, i, 4, 3) for i in range(2)]
+    a = gpu_ctm(t, [[0, 1]], chi)
+    a.sweep(2)
+    b = gpu_ctm(t, [[0, 1]], chi, prec="fp64tc")
+    b.copy_env_from(a)
+    ra, rb = a.rdms(), b.rdms()
+    a.close()
+    b.close()
+    for bond in ra:
+        assert np.abs(np.asarray(ra[bond]) - np.asarray(rb[bond])).max() < 1e-13
