@@ -10,10 +10,9 @@
 // tensor memory: 16 significand bits per operand) or in BF16 hi/mid/lo
 // triples (x = p0 + p1 + p2, the six products p_i q_j with i + j <= 2: 24
 // significand bits, the FP32 class).  One CTA computes a 128 x BN tile of Cr: warp 0
-// issues the TMA loads (128-byte swizzle), warp 1 issues tcgen05.mma, all four
-// warps drain the accumulator with tcgen05.ld.  Thin products (few output
-// tiles) split K over the grid's z dimension into FP32 partials, summed in a
-// fixed order by a second kernel.
+// issues the TMA loads, warp 1 issues tcgen05.mma, four more warps drain the
+// accumulators with tcgen05.ld.  Products of few output tiles split K into FP32
+// partials, summed in a fixed order by a second kernel.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cudaTypedefs.h>
@@ -57,6 +56,18 @@ struct Cfg {
   static_assert(STAGES >= 2, "at least two pipeline stages");
   static constexpr int UMMA_K = PREC == PREC_TF32 ? 8 : 16;  // K of one MMA
   static constexpr int KSTEPS = BK / UMMA_K;
+  // Accumulators.  The tensor cores round every FP32 accumulation towards zero, so
+  // a run of n of them loses up to n ulps of the sum, always in the same direction.
+  // BF16x6 keeps the five products with a low part (2^-8 of the result and below)
+  // in an accumulator of their own, added at the end: one accumulation of the
+  // result's size per k-step instead of six.  69 x 848 x 848 complex, rms of the
+  // result: 1.2e-5 -> 1.7e-6 in one K split, 4.1e-7 -> 1.3e-7 in 27; RDMs of a 2x1
+  // cell at D = 4, chi = 53 with two-corner projectors, mean of 40 states: 1.2e-6 ->
+  // 5.7e-7 (largest 4.2e-6 -> 2.1e-6).  At BN = 256 that leaves tensor memory for one
+  // set, whose drain the next tile waits for: 1 to 2 % of a sweep.
+  static constexpr bool SPLIT_ACC = PREC == PREC_BF16X6;
+  static constexpr int ACC_COLS = SPLIT_ACC ? 2 * BN : BN;  // tensor-memory columns of a set
+  static constexpr int SETS = 2 * ACC_COLS <= 512 ? 2 : 1;  // 2: a tile drains under the next one's MMAs
   // stages, alignment, barriers, the epilogue warps' transpose buffers
   static constexpr int SMEM = STAGES * STAGE_BYTES + 1024 + 256 + 4 * EPI_FLOATS * 4;
   // instruction descriptor: FP32 accumulate, K-major A and B, N = BN, M = 128
@@ -85,9 +96,9 @@ __device__ __forceinline__ void umma(uint32_t dtmem, uint64_t a, uint64_t b, uin
 // Persistent main kernel: CTA b takes the output tiles t = b, b + grid, ...
 // (t = n_tile + n_tiles * (m_tile + m_tiles * split)).  Warp 0 streams the
 // k-blocks of its tiles through the shared-memory stages (TMA), warp 1 issues
-// the MMAs of tile i into accumulator set i % 2 (tensor-memory columns
-// BN (i % 2) ..), warps 2..5 drain set i % 2 to global memory while the MMAs
-// of tile i + 1 run in the other set.
+// the MMAs of tile i into accumulator set i % SETS (tensor-memory columns
+// ACC_COLS (i % SETS) ..), warps 2..5 drain that set to global memory, with two
+// sets while the MMAs of tile i + 1 run in the other one.
 template <int PREC, int BN>
 __global__ void __launch_bounds__(NTHREADS, 1)
     tc_gemm_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ CUtensorMap mA1,
@@ -126,7 +137,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                 "r"(2 * BN)
+                 "r"(K_::SETS * K_::ACC_COLS)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -177,15 +188,16 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++it) {
       int kb0;
       const int nkb = kblocks(t, &kb0);
-      const int b = it & 1;
-      // the set was drained: tile it - 2 was that set's drain number it/2 - 1
-      if (it >= 2 && !mbar_wait(&acc_empty[b], ((it >> 1) - 1) & 1)) {
+      const int b = it % K_::SETS;
+      // the set was drained: tile it - SETS was that set's drain number it / SETS - 1
+      if (it >= K_::SETS && !mbar_wait(&acc_empty[b], (it / K_::SETS - 1) & 1)) {
         atomicAdd(timeouts, 1);
         ok = false;
         break;
       }
       fence_after();
-      const uint32_t d = tmem + (uint32_t)(b * BN);
+      const uint32_t d = tmem + (uint32_t)(b * K_::ACC_COLS);
+      const uint32_t dl = d + (K_::SPLIT_ACC ? BN : 0);  // the low parts' products
       for (int i = 0; i < nkb; ++i, ++q) {
         const int s = q % K_::STAGES, r = q / K_::STAGES;
         if (!mbar_wait(&full[s], r & 1)) {
@@ -203,12 +215,12 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           const uint32_t acc = (i > 0 || j > 0) ? 1u : 0u;
           if (K_::NOPS == 3) {
             // smallest parts first: p_i q_j with i + j = 2, then 1, then 0
-            umma<PREC, K_::IDESC>(d, sdesc_kb<K_::KB_BYTES>(a0 + ko), sdesc_kb<K_::KB_BYTES>(b2 + ko), acc);
-            umma<PREC, K_::IDESC>(d, sdesc_kb<K_::KB_BYTES>(a1 + ko), sdesc_kb<K_::KB_BYTES>(b1 + ko), 1u);
-            umma<PREC, K_::IDESC>(d, sdesc_kb<K_::KB_BYTES>(a2 + ko), sdesc_kb<K_::KB_BYTES>(b0 + ko), 1u);
-            umma<PREC, K_::IDESC>(d, sdesc_kb<K_::KB_BYTES>(a0 + ko), sdesc_kb<K_::KB_BYTES>(b1 + ko), 1u);
-            umma<PREC, K_::IDESC>(d, sdesc_kb<K_::KB_BYTES>(a1 + ko), sdesc_kb<K_::KB_BYTES>(b0 + ko), 1u);
-            umma<PREC, K_::IDESC>(d, sdesc_kb<K_::KB_BYTES>(a0 + ko), sdesc_kb<K_::KB_BYTES>(b0 + ko), 1u);
+            umma<PREC, K_::IDESC>(dl, sdesc_kb<K_::KB_BYTES>(a0 + ko), sdesc_kb<K_::KB_BYTES>(b2 + ko), acc);
+            umma<PREC, K_::IDESC>(dl, sdesc_kb<K_::KB_BYTES>(a1 + ko), sdesc_kb<K_::KB_BYTES>(b1 + ko), 1u);
+            umma<PREC, K_::IDESC>(dl, sdesc_kb<K_::KB_BYTES>(a2 + ko), sdesc_kb<K_::KB_BYTES>(b0 + ko), 1u);
+            umma<PREC, K_::IDESC>(dl, sdesc_kb<K_::KB_BYTES>(a0 + ko), sdesc_kb<K_::KB_BYTES>(b1 + ko), 1u);
+            umma<PREC, K_::IDESC>(dl, sdesc_kb<K_::KB_BYTES>(a1 + ko), sdesc_kb<K_::KB_BYTES>(b0 + ko), 1u);
+            umma<PREC, K_::IDESC>(d, sdesc_kb<K_::KB_BYTES>(a0 + ko), sdesc_kb<K_::KB_BYTES>(b0 + ko), acc);
           } else {
             umma<PREC, K_::IDESC>(d, sdesc_kb<K_::KB_BYTES>(a0 + ko), sdesc_kb<K_::KB_BYTES>(b0 + ko), acc);
             if (K_::NOPS == 2) {
@@ -232,21 +244,31 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++it) {
       const int split = t / (n_tiles * m_tiles);
       const int n_tile = t % n_tiles, m_tile = (t / n_tiles) % m_tiles;
-      const int b = it & 1;
+      const int b = it % K_::SETS;
       // every lane saw the set complete, or the warp stops (a wait that ran out)
-      const bool ready = __all_sync(0xffffffffu, mbar_wait(&acc_full[b], (it >> 1) & 1));
+      const bool ready = __all_sync(0xffffffffu, mbar_wait(&acc_full[b], (it / K_::SETS) & 1));
       if (!ready) {
         if (lane == 0) atomicAdd(timeouts, 1);
         break;
       }
       fence_after();
-      const uint32_t trow = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(b * BN);
+      const uint32_t trow = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(b * K_::ACC_COLS);
       for (int c0 = 0; c0 < BN; c0 += 16) {
         // a lane drains 16 columns of its row; through shared memory eight lanes
         // take a row's 8 complex numbers, so that a store instruction writes
         // four runs of 64 (FP32) or 128 (FP64) bytes instead of 32 pieces of 16
         float v[16];
-        tmem_ld16(trow + c0, v);
+        if constexpr (K_::SPLIT_ACC) {
+          uint32_t hi[16], lo[16];
+          tmem_ld16_issue(trow + c0, hi);
+          tmem_ld16_issue(trow + BN + c0, lo);
+          tmem_ld_wait(hi);
+          tmem_ld_after(lo);
+#pragma unroll
+          for (int q = 0; q < 16; ++q) v[q] = __uint_as_float(hi[q]) + __uint_as_float(lo[q]);
+        } else {
+          tmem_ld16(trow + c0, v);
+        }
         if (partial) {  // rows of whole 64-byte runs per lane: written as they are
           float4* dst = (float4*)(partial + split * pstride + (long long)(m_tile * BM + quad * 32 + lane) * Nrp +
                                   n_tile * BN + c0);
@@ -287,7 +309,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   fence_before();
   __syncthreads();
   if (warp == 0) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * BN) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(K_::SETS * K_::ACC_COLS) : "memory");
   }
 }
 
