@@ -378,11 +378,11 @@ constexpr int JC_MAXP = 32;  // row pairs of one round per CTA (n <= 2 * 16 * 32
 // rows by the latency of a round (loads from the partner CTAs, reduction,
 // angle, rotation, cluster barrier).
 //
-// FP64 with a log: the rotations are logged and replayed onto Vt by
-// jacobi_replay_kernel across the GPU (rotating V here would double the FP64
-// work of these 16 SMs).  Double-float with Vt: the second half of the warps
-// rotates the rows of V (double-float, from Vt), one round behind the first
-// half, in the cycles the rounds leave idle.
+// With a log: the rotations are logged and replayed onto Vt by
+// jacobi_replay_kernel across the GPU (rotating FP64 rows of V here would double
+// the FP64 work of these 16 SMs).  With Vt: the second half of the warps rotates
+// the rows of V (from Vt, in the rows' arithmetic), one round behind the first
+// half; for double-float rows in cycles that the rounds leave idle.
 template <bool DF, int NE>
 __global__ void __launch_bounds__(512, 1)
     jacobi_cluster_kernel(cplx* __restrict__ G0, int n, int m, long long ldg, long long strideG,
@@ -395,14 +395,14 @@ __global__ void __launch_bounds__(512, 1)
   cplx* __restrict__ G = G0 + (long long)(blockIdx.x / cs) * strideG;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
   const int R = (n + cs - 1) / cs;   // row slots per CTA
-  const bool with_v = DF && Vt != nullptr;
+  const bool with_v = Vt != nullptr;
   const int gwarps = with_v ? nwarps / 2 : nwarps;
   extern __shared__ cplx sm[];       // [R x m] rows of G, then (with_v) [R x n] rows of V
   __shared__ S s_nrm[JC_MAXP * 2];   // squared norm of each row slot
   __shared__ int s_act[JC_MAXP * 2 * 16], s_nact;  // original row of each active row
   __shared__ double s_fro;
   __shared__ int s_rot, s_big;
-  __shared__ Rot<df2> s_rec[2][JC_MAXP];  // with_v: the last rounds' rotations
+  __shared__ Rot<S> s_rec[2][JC_MAXP];  // with_v: the last rounds' rotations
   __shared__ int s_recij[2][JC_MAXP];     // their rows, i << 16 | j, or -1
   __shared__ double s_w[16];
   E* gl = (E*)sm;
@@ -467,15 +467,16 @@ __global__ void __launch_bounds__(512, 1)
       else
         gl[(long long)l * m + t] = x;
     }
-    if constexpr (DF) {
-      if (with_v)
-        for (int t = threadIdx.x; t < n; t += blockDim.x)
-          vl[(long long)l * n + t] = df_elem(warm ? Vt[(long long)i * n + t] : make_double2(t == i ? 1.0 : 0.0, 0.0));
-    }
+    if (with_v)
+      for (int t = threadIdx.x; t < n; t += blockDim.x) {
+        const cplx v = warm ? Vt[(long long)i * n + t] : make_double2(t == i ? 1.0 : 0.0, 0.0);
+        if constexpr (DF)
+          vl[(long long)l * n + t] = df_elem(v);
+        else
+          vl[(long long)l * n + t] = v;
+      }
   }
-  if constexpr (DF) {
-    for (int q = threadIdx.x; q < 2 * JC_MAXP; q += blockDim.x) (&s_recij[0][0])[q] = -1;
-  }
+  for (int q = threadIdx.x; q < 2 * JC_MAXP; q += blockDim.x) (&s_recij[0][0])[q] = -1;
   const float neg = DF ? (float)(fros * 1e-30) : 0.f;
   const double negd = fros * 1e-30;
   auto negligible = [&](S x) {
@@ -494,19 +495,17 @@ __global__ void __launch_bounds__(512, 1)
   int sweep = 0, par = 0;
   // with_v: the second half of the warps applies the rotations recorded in buffer b
   auto rotate_v = [&](int b) {
-    if constexpr (DF) {
-      for (int slot = warp - gwarps; slot < own; slot += gwarps) {
-        const int ij = s_recij[b][slot];
-        if (ij < 0) continue;
-        float4* vi = vrow(ij >> 16);
-        float4* vj = vrow(ij & 0xffff);
-        const Rot<df2> rot = s_rec[b][slot];
-        for (int q = lane; q < n; q += 32) {
-          float4 x = vi[q], y = vj[q];
-          rotate_elem(rot, x, y);
-          vi[q] = x;
-          vj[q] = y;
-        }
+    for (int slot = warp - gwarps; slot < own; slot += gwarps) {
+      const int ij = s_recij[b][slot];
+      if (ij < 0) continue;
+      E* vi = vrow(ij >> 16);
+      E* vj = vrow(ij & 0xffff);
+      const Rot<S> rot = s_rec[b][slot];
+      for (int q = lane; q < n; q += 32) {
+        E x = vi[q], y = vj[q];
+        rotate_elem(rot, x, y);
+        vi[q] = x;
+        vj[q] = y;
       }
     }
   };
@@ -601,11 +600,9 @@ __global__ void __launch_bounds__(512, 1)
             }
           }
           if (lane == 0) {
-            if constexpr (DF) {
-              if (with_v) {
-                s_recij[par][slot] = kind ? (i << 16 | j) : -1;
-                s_rec[par][slot] = rot;
-              }
+            if (with_v) {
+              s_recij[par][slot] = kind ? (i << 16 | j) : -1;
+              s_rec[par][slot] = rot;
             }
             if (log && p < npairs) {
               double4_16a rec = make_double4_16a(2.0, 0.0, 0.0, 0.0);
@@ -652,13 +649,15 @@ __global__ void __launch_bounds__(512, 1)
         G[(long long)i * ldg + t] = gl[(long long)l * m + t];
       }
     }
-    if constexpr (DF) {
-      if (with_v)
-        for (int t = threadIdx.x; t < n; t += blockDim.x) {
+    if (with_v)
+      for (int t = threadIdx.x; t < n; t += blockDim.x) {
+        if constexpr (DF) {
           const float4 x4 = vl[(long long)l * n + t];
           Vt[(long long)i * n + t] = make_double2(df_val({x4.x, x4.y}), df_val({x4.z, x4.w}));
+        } else {
+          Vt[(long long)i * n + t] = vl[(long long)l * n + t];
         }
-    }
+      }
   }
   if (with_v && !warm)  // rows that took part in no rotation: the identity's
     for (int i = rank; i < n; i += cs) {
@@ -994,10 +993,10 @@ static size_t jacobi_smem(int n, int m, bool vt_in_smem, int cs) {
   return b <= CL_SMEM ? (size_t)b : 0;
 }
 
-bool jacobi_cluster_fits(int n, int m) {
+bool jacobi_cluster_fits(int n, int m, bool vt_in_smem) {
   if (n < 32) return false;
   if (cluster_init() != cudaSuccess) return false;
-  return jacobi_smem(n, m, false, g_csize) > 0;
+  return jacobi_smem(n, m, vt_in_smem, g_csize) > 0;
 }
 
 // the rotation records (one double4_16a = two complex slots per pair), then
@@ -1019,12 +1018,13 @@ cudaError_t jacobi_cluster(cudaStream_t s, cplx* G, int n, int m, long long ldg,
                            DevStatus* st, cplx* rotlog, int* sweeps_used, bool warm_v, bool dfloat) {
   cudaError_t e;
   if ((e = cluster_init()) != cudaSuccess) return e;
-  if (Vt && !rotlog) return cudaErrorInvalidValue;
   // double-float rows only where a V comes with them (the projector cores);
   // their dot products resolve orthogonality to about m 2^-48, so pairs are
   // left alone below m 2^-44 (FP64: m eps)
   const bool df = dfloat && Vt;
-  const bool v_in = df && jacobi_smem(n, m, true, g_csize) > 0;  // V beside the rows; else replayed from the log
+  // V beside the rows (double-float, or no log to replay it from)
+  const bool v_in = Vt && (df || !rotlog) && jacobi_smem(n, m, true, g_csize) > 0;
+  if (Vt && !v_in && !rotlog) return cudaErrorInvalidValue;
   const bool replay = Vt && !v_in;
   cplx* Vin = v_in ? Vt : nullptr;
   double4_16a* logp = replay ? (double4_16a*)rotlog : nullptr;

@@ -114,9 +114,8 @@ cudaError_t set_zero(cudaStream_t s, cplx* x, long long n);
 // same rotations starting from the identity.  sigma[i] = ||row i|| on return.
 // counters: 4 ints of scratch (sweep counters and, for m <= 256, a grid barrier);
 // work: 1 double of scratch.
-// rotlog (jacobi_log_elems(n, max_sweeps) complex slots): lets the cluster path
-// rebuild Vt from logged rotations; without it a call with Vt takes the
-// grid-wide kernels.
+// rotlog (optional, jacobi_log_elems(n, max_sweeps) complex slots): lets the
+// cluster path rebuild Vt from logged rotations instead of holding it.
 // wait_cycles: limit of each grid-barrier wait of the small-row kernel (<= 0:
 // about 2 s of clock); a wait that runs out is counted in st->barrier_timeouts
 // and its CTA stops.
@@ -200,10 +199,11 @@ cudaError_t kernels_init();
 // FP64 Jacobi / Cholesky on one thread-block cluster (cluster_fp64.cu): rows
 // in distributed shared memory, hardware cluster barriers between steps.
 cudaError_t fp64_cluster_init();
-bool jacobi_cluster_fits(int n, int m);
-// Vt needs rotlog (jacobi_log_elems(n, max_sweeps) complex slots) and
-// sweeps_used (one int): FP64 rotations are logged and replayed onto the
-// identity (onto Vt itself with warm_v) by one CTA per column afterwards.
+bool jacobi_cluster_fits(int n, int m, bool vt_in_smem);
+// With rotlog (jacobi_log_elems(n, max_sweeps) complex slots) and sweeps_used
+// (one int) FP64 rotations are logged and replayed onto the identity (onto Vt
+// itself with warm_v) by one CTA per column afterwards; without them Vt is held
+// beside the rows.
 cudaError_t jacobi_cluster(cudaStream_t s, cplx* G, int n, int m, long long ldg, cplx* Vt, int max_sweeps,
                            DevStatus* st, cplx* rotlog, int* sweeps_used, bool warm_v = false,
                            bool dfloat = false);

@@ -615,8 +615,8 @@ cudaError_t jacobi_rows(cudaStream_t s, cplx* G, int n, int m, long long ldg, cp
   cudaError_t e;
   if ((e = kernels_init()) != cudaSuccess) return e;
   const bool logged = Vt && rotlog && n <= 2048 && rotlog_elems >= jacobi_log_elems(n, max_sweeps);
-  if (jacobi_cluster_fits(n, m) && (!Vt || logged)) {
-    // the rows fit in one cluster's shared memory: no grid-wide barrier
+  if (jacobi_cluster_fits(n, m, Vt && !logged)) {
+    // the rows (and Vt unless logged) fit in one cluster's shared memory: no grid-wide barrier
     if ((e = jacobi_cluster(s, G, n, m, ldg, Vt, max_sweeps, st, logged ? rotlog : nullptr,
                             logged ? counters : nullptr, warm_v, dfloat)) != cudaSuccess)
       return e;
