@@ -157,6 +157,12 @@ __device__ __forceinline__ cplx oz_load(const cplx* X, long long ld, int op, int
   return v;
 }
 
+// The power-of-two bound of a row (or column) whose largest biased exponent is E:
+// 0 for zeros; OZ_NONFINITE with an infinity or a NaN among them, which leaves the
+// digits zero and makes every output of the row NaN (oz_value).
+constexpr int OZ_NONFINITE = 1 << 20;
+__device__ __forceinline__ int row_bound(int E) { return E == 0x7FF ? OZ_NONFINITE : (E ? E - 1022 : 0); }
+
 // Both operands' exponents and digit planes in one launch.  Block b < Mp takes
 // row b of op(A) (M x K complex): e = (largest biased exponent of the row) -
 // 1022, the power-of-two bound of that row of Ar (0 for rows at or beyond M
@@ -169,10 +175,7 @@ __device__ __forceinline__ cplx oz_load(const cplx* X, long long ld, int op, int
 // WARP: a warp per row, four rows to a block, for many short rows (a block's
 // start and its two barriers took longer than the at most four elements per
 // lane: 19456 rows of 27 took 38 us, 18 us so).
-// A row with an infinity or a NaN gets the bound OZ_NONFINITE (its digits are
-// zero then), which makes every output of that row NaN.
 constexpr int OZ_PREP_THREADS = 128;
-constexpr int OZ_NONFINITE = 1 << 20;
 template <bool WARP>
 __global__ void __launch_bounds__(OZ_PREP_THREADS)
     oz_prep_kernel(const cplx* __restrict__ A, long long lda, int opA, const cplx* __restrict__ B, long long ldb,
@@ -204,7 +207,7 @@ __global__ void __launch_bounds__(OZ_PREP_THREADS)
 #pragma unroll
     for (int w = 1; w < OZ_PREP_THREADS / 32; ++w) E = max(E, s_e[w]);
   }
-  const int e = E == 0x7FF ? OZ_NONFINITE : (E ? E - 1022 : 0);
+  const int e = row_bound(E);
   if (tid == 0) {
     if (is_a)
       ea[r] = e;
@@ -551,10 +554,9 @@ __global__ void __launch_bounds__(256)
   __shared__ cplx tile[32][33];
   const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32, kc = Krp >> 1;
   const long long plane = (long long)Mp * Krp;
-  auto bound = [](int E) { return E ? E - 1022 : 0; };
   if (blockIdx.x == 0 && threadIdx.y == 0) {
-    et[r0 + threadIdx.x] = bound(er[r0 + threadIdx.x]);
-    en[r0 + threadIdx.x] = bound(ec[r0 + threadIdx.x]);
+    et[r0 + threadIdx.x] = row_bound(er[r0 + threadIdx.x]);
+    en[r0 + threadIdx.x] = row_bound(ec[r0 + threadIdx.x]);
   }
   auto put = [&](__nv_bfloat16* p, int row, int k, cplx v, int e) {
     int dr[OZ_DIGITS], di[OZ_DIGITS];
@@ -571,12 +573,12 @@ __global__ void __launch_bounds__(256)
     cplx v = make_double2(0.0, 0.0);
     if (r < K && c < K) v = Q[(long long)r * K + c];
     tile[i][threadIdx.x] = v;
-    if (c < kc) put(pt, r, c, v, bound(er[r]));
+    if (c < kc) put(pt, r, c, v, row_bound(er[r]));
   }
   __syncthreads();
   const int k = r0 + threadIdx.x;
   if (k >= kc) return;
-  for (int i = threadIdx.y; i < 32; i += 8) put(pn, c0 + i, k, tile[threadIdx.x][i], bound(ec[c0 + i]));
+  for (int i = threadIdx.y; i < 32; i += 8) put(pn, c0 + i, k, tile[threadIdx.x][i], row_bound(ec[c0 + i]));
 }
 
 unsigned oz_grid(long long n) {
