@@ -86,6 +86,8 @@ struct GemmBatch {
 // triangle), ZG_A_LOWER (opA(A) is lower triangular: k-tiles beyond a tile
 // row's diagonal are skipped).
 enum { ZG_UPPER_TILES = 1, ZG_A_LOWER = 2 };
+// the tile width (64, 32 or 16) and K split that zgemm takes (host only)
+void zgemm_plan(int M, int N, int K, int count, long long work_elems, int flags, int* tile, int* ksplit);
 cudaError_t zgemm(cudaStream_t s, int M, int N, int K, cplx alpha, const cplx* A, long long lda,
                   int opA, const cplx* B, long long ldb, int opB, cplx beta, cplx* C,
                   long long ldc, GemmBatch batch = {1, 0, 0, 0}, cplx* work = nullptr,

@@ -218,33 +218,35 @@ __global__ void permute_kernel(const cplx* __restrict__ in, cplx* __restrict__ o
 
 }  // namespace
 
-cudaError_t zgemm(cudaStream_t s, int M, int N, int K, cplx alpha, const cplx* A, long long lda,
-                  int opA, const cplx* B, long long ldb, int opB, cplx beta, cplx* C,
-                  long long ldc, GemmBatch batch, cplx* work, long long work_elems, int flags) {
-  if (M <= 0 || N <= 0 || batch.count <= 0) return cudaSuccess;
-  if ((flags & ZG_UPPER_TILES) && M != N) return cudaErrorInvalidValue;
-  // Tile size and K split from a cost model, in microseconds: the busiest
-  // SM's share of the multiply-adds at the FP64 units' rate (a k step of a 64 x
-  // 64 tile takes them 4.5 us; 0.61 of the rate with one CTA on the SM, measured
-  // on GB300, its loads not hidden), a load latency (1 us) for each of its
-  // k-tiles as far as other CTAs do not cover it,
-  // and for a split the second kernel with the partials' round trip.
-  int best_T = 64, best_k = 0;  // best_k: k per split, 0 = unsplit
+// Tile size and K split from a cost model, in microseconds: the busiest SM's
+// share of the multiply-adds at the FP64 units' rate (a k step of a 64 x 64 tile
+// takes them 4.5 us; 0.61 of the rate with one CTA on the SM, measured on GB300,
+// its loads not hidden), a load latency (1 us) for each of its k-tiles as far as
+// other CTAs do not cover it, and for a split the second kernel with the
+// partials' round trip.  ksplit: k per split, 0 = unsplit (no minimum there: with
+// the splits' minimum of 8 on it too, every product of K < 8 fell to 64-wide tiles,
+// 1024 x 32 x 4 to 16 CTAs and 23 us).  For sums that short a narrow tile has to
+// be the better one by its waves: where all widths fill the chip, each CTA's
+// start and stores count for more than the model's latency term.
+void zgemm_plan(int M, int N, int K, int count, long long work_elems, int flags, int* tile, int* ksplit) {
+  *tile = 64;
+  *ksplit = 0;
   double best_cost = -1.0;
-  const bool can_split = batch.count == 1 && K >= 16;
+  const bool can_split = count == 1 && K >= 16;
   for (int T : {64, 32, 16}) {
-    if (T != 64 && (batch.count != 1 || M > 65535LL * T)) continue;
+    if (T != 64 && (count != 1 || M > 65535LL * T)) continue;
     const long long tm = (M + T - 1) / T, tn = (N + T - 1) / T;
-    const long long tiles = (flags & ZG_UPPER_TILES) ? tm * (tm + 1) / 2 : tm * tn;
     const double per_k = 4.5 * (T / 64.0) * (T / 64.0);
     int last = -1;
     for (int S = 1; S <= (can_split ? 160 : 1); ++S) {
       const int kps = S == 1 ? K : ((K + S - 1) / S + 7) / 8 * 8;
-      if (kps < 8 || kps == last) continue;
+      if ((S > 1 && kps < 8) || kps == last) continue;
       last = kps;
       const long long Se = (K + kps - 1) / kps;
       if (Se > 1 && Se * M * N > work_elems && !(T == 16 && Se <= 8)) continue;
-      const long long busy = (tiles * Se * batch.count + 151) / 152;
+      // an unsplit product computes the tiles below the diagonal too
+      const long long tiles = Se > 1 && (flags & ZG_UPPER_TILES) ? tm * (tm + 1) / 2 : tm * tn;
+      const long long busy = (tiles * Se * count + 151) / 152;
       const double rate = busy == 1 ? 0.61 : 1.0;
       double cost = (double)kps * (double)busy * per_k / rate + (double)((kps + BK - 1) / BK) / (double)busy;
       // up to eight splits of 16-wide tiles meet in a cluster's shared memory
@@ -254,14 +256,22 @@ cudaError_t zgemm(cudaStream_t s, int M, int N, int K, cplx alpha, const cplx* A
         cost += 1.5;
       else if (Se > 1)
         cost += 4.0 + (double)Se * (double)M * (double)N * 32.0 / 5e6;
-      if (best_cost < 0.0 || cost < best_cost) {
+      if (best_cost < 0.0 || cost < best_cost * (K < 8 ? 0.95 : 1.0)) {
         best_cost = cost;
-        best_k = Se > 1 ? kps : 0;
-        best_T = T;
+        *ksplit = Se > 1 ? kps : 0;
+        *tile = T;
       }
     }
   }
-  const int T = best_T;
+}
+
+cudaError_t zgemm(cudaStream_t s, int M, int N, int K, cplx alpha, const cplx* A, long long lda,
+                  int opA, const cplx* B, long long ldb, int opB, cplx beta, cplx* C,
+                  long long ldc, GemmBatch batch, cplx* work, long long work_elems, int flags) {
+  if (M <= 0 || N <= 0 || batch.count <= 0) return cudaSuccess;
+  if ((flags & ZG_UPPER_TILES) && M != N) return cudaErrorInvalidValue;
+  int T, best_k;
+  zgemm_plan(M, N, K, batch.count, work_elems, flags, &T, &best_k);
   const long long tm = (M + T - 1) / T, tn = (N + T - 1) / T;
   auto launch = [&](dim3 grid, cplx al, cplx be, cplx* out, long long ldo, long long sC, int ksplit, int fl) {
     auto go = [&](auto kern) {
