@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                    const __grid_constant__ CUtensorMap mB1, const __grid_constant__ CUtensorMap mB2,
                    int kb_total, int kb_per_split, int n_tiles, int m_tiles, int tiles, int M, int Nr, cplx alpha,
                    void* __restrict__ Cv, long long ldc, float* __restrict__ partial, int Nrp, long long pstride,
-                   int conj_out, int unit_alpha, int out_f32, int* __restrict__ timeouts) {
+                   int unit_alpha, int out_f32, int* __restrict__ timeouts) {
   using K_ = Cfg<PREC, BN>;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -291,12 +291,10 @@ __global__ void __launch_bounds__(NTHREADS, 1)
               ((float2*)Cv)[o] = x;
             } else if (unit_alpha) {
               // alpha = 1: exact FP32 -> FP64 widening on the integer pipe
-              const double re = f2d_bits(x.x), im = f2d_bits(x.y);
-              ((cplx*)Cv)[o] = make_double2(re, conj_out ? neg_bits(im) : im);
+              ((cplx*)Cv)[o] = make_double2(f2d_bits(x.x), f2d_bits(x.y));
             } else {
               const double re = x.x, im = x.y;
-              const double orr = alpha.x * re - alpha.y * im, oi = alpha.x * im + alpha.y * re;
-              ((cplx*)Cv)[o] = make_double2(orr, conj_out ? -oi : oi);
+              ((cplx*)Cv)[o] = make_double2(alpha.x * re - alpha.y * im, alpha.x * im + alpha.y * re);
             }
           }
         }
@@ -315,7 +313,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 
 // C[m,n] = alpha * sum_z P[z][m][2n .. 2n+1]  (fixed summation order)
 __global__ void splitk_reduce_kernel(const float* __restrict__ P, int S, long long pstride, int Nrp, int M,
-                                     int N, cplx alpha, void* __restrict__ Cv, long long ldc, int conj_out,
+                                     int N, cplx alpha, void* __restrict__ Cv, long long ldc,
                                      int unit_alpha, int out_f32) {
   cplx* C = (cplx*)Cv;
   const long long total = (long long)M * N;
@@ -336,8 +334,7 @@ __global__ void splitk_reduce_kernel(const float* __restrict__ P, int S, long lo
         ((float2*)Cv)[(long long)m * ldc + n] = make_float2(re, im);
         continue;
       }
-      const double dr = f2d_bits(re), di = f2d_bits(im);
-      C[(long long)m * ldc + n] = make_double2(dr, conj_out ? neg_bits(di) : di);
+      C[(long long)m * ldc + n] = make_double2(f2d_bits(re), f2d_bits(im));
       continue;
     }
     double re = 0.0, im = 0.0;
@@ -346,15 +343,14 @@ __global__ void splitk_reduce_kernel(const float* __restrict__ P, int S, long lo
       re += p.x;
       im += p.y;
     }
-    const double oi = alpha.x * im + alpha.y * re;
-    C[(long long)m * ldc + n] = make_double2(alpha.x * re - alpha.y * im, conj_out ? -oi : oi);
+    C[(long long)m * ldc + n] = make_double2(alpha.x * re - alpha.y * im, alpha.x * im + alpha.y * re);
   }
 }
 
 // The same with a warp per output for many splits: lane l sums splits
 // l, l + 32, ... in order, then the lanes' sums meet in a fixed butterfly.
 __global__ void splitk_reduce_warp_kernel(const float* __restrict__ P, int S, long long pstride, int Nrp, int M,
-                                          int N, cplx alpha, void* __restrict__ Cv, long long ldc, int conj_out,
+                                          int N, cplx alpha, void* __restrict__ Cv, long long ldc,
                                           int unit_alpha, int out_f32) {
   cplx* C = (cplx*)Cv;
   const int lane = threadIdx.x & 31;
@@ -377,12 +373,10 @@ __global__ void splitk_reduce_warp_kernel(const float* __restrict__ P, int S, lo
     if (out_f32) {
       ((float2*)Cv)[(long long)m * ldc + n] = make_float2(re, im);
     } else if (unit_alpha) {
-      const double dr = f2d_bits(re), di = f2d_bits(im);
-      C[(long long)m * ldc + n] = make_double2(dr, conj_out ? neg_bits(di) : di);
+      C[(long long)m * ldc + n] = make_double2(f2d_bits(re), f2d_bits(im));
     } else {
       const double r = re, i = im;
-      const double oi = alpha.x * i + alpha.y * r;
-      C[(long long)m * ldc + n] = make_double2(alpha.x * r - alpha.y * i, conj_out ? -oi : oi);
+      C[(long long)m * ldc + n] = make_double2(alpha.x * r - alpha.y * i, alpha.x * i + alpha.y * r);
     }
   }
 }
@@ -813,7 +807,6 @@ cudaError_t ensure_attr() {
 template <int PREC, int BN>
 cudaError_t launch_main(cudaStream_t s, const Operands& o, int S, int M, int N, cplx alpha, void* C, long long ldc,
                         bool c_f32, float* part, int* timeouts, TcProbe* probe, bool partials_only = false) {
-  const int conj_out = 0;
   using K_ = Cfg<PREC, BN>;
   cudaError_t e;
   if ((e = ensure_attr<PREC, BN>()) != cudaSuccess) return e;
@@ -858,7 +851,7 @@ cudaError_t launch_main(cudaStream_t s, const Operands& o, int S, int M, int N, 
   tc_gemm_kernel<PREC, BN><<<grid, NTHREADS, K_::SMEM, s>>>(mA0, mA1, mA2, mB0, mB1, mB2, o.kb_total, kps, n_tiles,
                                                              m_tiles, (int)tiles, M, 2 * N, alpha, C, ldc,
                                                              S > 1 || partials_only ? part : nullptr, (int)o.Nrp,
-                                                             o.Mp * o.Nrp, conj_out, unit, c_f32 ? 1 : 0, timeouts);
+                                                             o.Mp * o.Nrp, unit, c_f32 ? 1 : 0, timeouts);
   count_launch();
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (probe && (e = cudaEventRecord(probe->ev[1], s)) != cudaSuccess) return e;
@@ -866,10 +859,10 @@ cudaError_t launch_main(cudaStream_t s, const Operands& o, int S, int M, int N, 
   if (S > 1) {
     if (S >= 64)
       splitk_reduce_warp_kernel<<<grid_for(32LL * M * N), 256, 0, s>>>(part, S, o.Mp * o.Nrp, (int)o.Nrp, M, N, alpha,
-                                                                      C, ldc, conj_out, unit, c_f32 ? 1 : 0);
+                                                                      C, ldc, unit, c_f32 ? 1 : 0);
     else
       splitk_reduce_kernel<<<grid_for((long long)M * N), 256, 0, s>>>(part, S, o.Mp * o.Nrp, (int)o.Nrp, M, N,
-                                                                      alpha, C, ldc, conj_out, unit, c_f32 ? 1 : 0);
+                                                                      alpha, C, ldc, unit, c_f32 ? 1 : 0);
     count_launch();
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
