@@ -382,8 +382,9 @@ constexpr int JC_MAXP = 32;  // row pairs of one round per CTA (n <= 2 * 16 * 32
 // jacobi_replay_kernel across the GPU (rotating FP64 rows of V here would double
 // the FP64 work of these 16 SMs).  With Vt: the second half of the warps rotates
 // the rows of V (from Vt, in the rows' arithmetic), one round behind the first
-// half; for double-float rows in cycles that the rounds leave idle.
-template <bool DF, int NE>
+// half; for double-float rows in cycles that the rounds leave idle.  V = false:
+// without that half's code, which costs the FP64 kernel 5 % by its registers.
+template <bool DF, int NE, bool V>
 __global__ void __launch_bounds__(512, 1)
     jacobi_cluster_kernel(cplx* __restrict__ G0, int n, int m, long long ldg, long long strideG,
                           cplx* __restrict__ Vt, int max_sweeps, float tol, double4_16a* __restrict__ log,
@@ -395,7 +396,7 @@ __global__ void __launch_bounds__(512, 1)
   cplx* __restrict__ G = G0 + (long long)(blockIdx.x / cs) * strideG;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
   const int R = (n + cs - 1) / cs;   // row slots per CTA
-  const bool with_v = Vt != nullptr;
+  const bool with_v = V && Vt != nullptr;
   const int gwarps = with_v ? nwarps / 2 : nwarps;
   extern __shared__ cplx sm[];       // [R x m] rows of G, then (with_v) [R x n] rows of V
   __shared__ S s_nrm[JC_MAXP * 2];   // squared norm of each row slot
@@ -476,7 +477,8 @@ __global__ void __launch_bounds__(512, 1)
           vl[(long long)l * n + t] = v;
       }
   }
-  for (int q = threadIdx.x; q < 2 * JC_MAXP; q += blockDim.x) (&s_recij[0][0])[q] = -1;
+  if (with_v)
+    for (int q = threadIdx.x; q < 2 * JC_MAXP; q += blockDim.x) (&s_recij[0][0])[q] = -1;
   const float neg = DF ? (float)(fros * 1e-30) : 0.f;
   const double negd = fros * 1e-30;
   auto negligible = [&](S x) {
@@ -495,6 +497,7 @@ __global__ void __launch_bounds__(512, 1)
   int sweep = 0, par = 0;
   // with_v: the second half of the warps applies the rotations recorded in buffer b
   auto rotate_v = [&](int b) {
+    if constexpr (!V) return;
     for (int slot = warp - gwarps; slot < own; slot += gwarps) {
       const int ij = s_recij[b][slot];
       if (ij < 0) continue;
@@ -926,23 +929,28 @@ __global__ void __launch_bounds__(CL_THREADS)
 
 }  // namespace
 
-static const void* jacobi_fn(bool df, int m) {
-  if (df)
-    return m <= 128 ? (const void*)jacobi_cluster_kernel<true, 4>
-                    : (m <= 256 ? (const void*)jacobi_cluster_kernel<true, 8> : (const void*)jacobi_cluster_kernel<true, 0>);
-  return m <= 128 ? (const void*)jacobi_cluster_kernel<false, 4>
-                  : (m <= 256 ? (const void*)jacobi_cluster_kernel<false, 8> : (const void*)jacobi_cluster_kernel<false, 0>);
+template <bool DF, bool V>
+static const void* jacobi_fn(int m) {
+  return m <= 128 ? (const void*)jacobi_cluster_kernel<DF, 4, V>
+                  : (m <= 256 ? (const void*)jacobi_cluster_kernel<DF, 8, V> : (const void*)jacobi_cluster_kernel<DF, 0, V>);
+}
+
+// the kernel for rows of m elements; v: Vt beside the rows
+static const void* jacobi_fn(bool df, bool v, int m) {
+  return df ? jacobi_fn<true, true>(m) : (v ? jacobi_fn<false, true>(m) : jacobi_fn<false, false>(m));
 }
 
 static cudaError_t cluster_init() {
   if (g_csize) return cudaSuccess;
   cudaError_t e;
-  const void* fns[7] = {jacobi_fn(false, 128), jacobi_fn(false, 256), jacobi_fn(false, 257), jacobi_fn(true, 128),
-                        jacobi_fn(true, 256),  jacobi_fn(true, 257),  (const void*)chol_cluster_kernel};
-  for (const void* f : fns) {
-    if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, CL_SMEM)) != cudaSuccess) return e;
-  }
+  auto prepare = [](const void* f) {
+    cudaError_t r = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    return r != cudaSuccess ? r : cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, CL_SMEM);
+  };
+  for (int m : {128, 256, 257})
+    for (const void* f : {jacobi_fn(false, false, m), jacobi_fn(false, true, m), jacobi_fn(true, true, m)})
+      if ((e = prepare(f)) != cudaSuccess) return e;
+  if ((e = prepare((const void*)chol_cluster_kernel)) != cudaSuccess) return e;
   // 16 CTAs per cluster when the hardware can place such a cluster, else 8
   int csize = 8;
   cudaLaunchConfig_t cfg = {};
@@ -957,7 +965,7 @@ static cudaError_t cluster_init() {
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
   int nclusters = 0;
-  if (cudaOccupancyMaxActiveClusters(&nclusters, jacobi_fn(false, 257), &cfg) == cudaSuccess && nclusters >= 1)
+  if (cudaOccupancyMaxActiveClusters(&nclusters, jacobi_fn(false, false, 257), &cfg) == cudaSuccess && nclusters >= 1)
     csize = 16;
   cudaGetLastError();  // a refused query leaves no error behind
   g_csize = csize;
@@ -1035,7 +1043,7 @@ cudaError_t jacobi_cluster(cudaStream_t s, cplx* G, int n, int m, long long ldg,
   int warm = warm_v && Vt ? 1 : 0;
   long long stride = 0;
   void* args[] = {&G, &n, &m, &ldg, &stride, &Vin, &max_sweeps, &tol, &logp, &amap, &su, &st, &warm};
-  e = launch_cluster(jacobi_fn(df, m), args, smem, s, jacobi_threads(n, g_csize, v_in));
+  e = launch_cluster(jacobi_fn(df, v_in, m), args, smem, s, jacobi_threads(n, g_csize, v_in));
   count_launch();
   if (e != cudaSuccess || !replay) return e;
   const int npairs = ((n + 1) & ~1) / 2;
@@ -1064,7 +1072,7 @@ cudaError_t jacobi_cluster_batch(cudaStream_t s, cplx* G, int n, int m, long lon
   int *amap = nullptr, *su = nullptr, warm = 0;
   float tol = (float)((double)m * 2.220446049250313e-16);
   void* args[] = {&G, &n, &m, &ldg, &strideG, &Vin, &max_sweeps, &tol, &logp, &amap, &su, &st, &warm};
-  e = launch_cluster(jacobi_fn(false, m), args, smem, s, jacobi_threads(n, cs, false), cs, count);
+  e = launch_cluster(jacobi_fn(false, false, m), args, smem, s, jacobi_threads(n, cs, false), cs, count);
   count_launch();
   return e;
 }
