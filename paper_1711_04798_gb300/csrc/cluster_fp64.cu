@@ -13,6 +13,7 @@
 #include <algorithm>
 
 #include "ctm_internal.h"
+#include "dfloat.h"
 
 namespace cg = cooperative_groups;
 
@@ -42,110 +43,10 @@ __device__ __forceinline__ void pair_of(int r, int p, int np, int rounds, int* i
   *j = b;
 }
 
-// ---------------------------------------------------------------------------
-// Double-float arithmetic (a value is an unevaluated sum hi + lo of two FP32
-// numbers, about 48 significand bits; Dekker 1971, Knuth's TwoSum): the
-// precision form's Jacobi runs its dot products and row rotations on the
-// FP32 pipe, which this part executes at 64 times its FP64 rate.  The
-// intrinsics below are never contracted into fused multiply-adds, which the
-// error-free transformations rely on.
-// ---------------------------------------------------------------------------
-struct df2 {
-  float h, l;
-};
-
-__device__ __forceinline__ df2 df_of(double x) {
-  const float h = __double2float_rn(x);
-  return {h, __double2float_rn(x - (double)h)};
-}
-
-__device__ __forceinline__ double df_val(df2 a) { return (double)a.h + (double)a.l; }
-
-// s + e = a + b exactly
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-  s = __fadd_rn(a, b);
-  const float bb = __fadd_rn(s, -a);
-  e = __fadd_rn(__fadd_rn(a, -__fadd_rn(s, -bb)), __fadd_rn(b, -bb));
-}
-
-// acc += a b: the leading product exactly (its rounding error by an FMA), the
-// cross terms and the tails in FP32, the leading sum's rounding error carried
-// into acc.l
-__device__ __forceinline__ void acc_mul(df2& acc, df2 a, df2 b) {
-  const float p = __fmul_rn(a.h, b.h);
-  float e = __fmaf_rn(a.h, b.h, -p);
-  e = __fmaf_rn(a.h, b.l, e);
-  e = __fmaf_rn(a.l, b.h, e);
-  float s, t;
-  two_sum(acc.h, p, s, t);
-  acc.h = s;
-  acc.l = __fadd_rn(acc.l, __fadd_rn(t, e));
-}
-
-__device__ __forceinline__ df2 df_norm(df2 a) {
-  df2 r;
-  two_sum(a.h, a.l, r.h, r.l);
-  return r;
-}
-
-__device__ __forceinline__ df2 df_negate(df2 a) { return {-a.h, -a.l}; }
-
 // a complex element of a row: (Re hi, Re lo, Im hi, Im lo)
 __device__ __forceinline__ float4 df_elem(cplx x) {
   const df2 r = df_of(x.x), i = df_of(x.y);
   return make_float4(r.h, r.l, i.h, i.l);
-}
-
-// a b, the leading product exactly, the cross terms in FP32
-__device__ __forceinline__ df2 df_mul(df2 a, df2 b) {
-  const float p = __fmul_rn(a.h, b.h);
-  float e = __fmaf_rn(a.h, b.h, -p);
-  e = __fmaf_rn(a.h, b.l, e);
-  e = __fmaf_rn(a.l, b.h, e);
-  return {p, e};
-}
-
-__device__ __forceinline__ df2 df_add(df2 a, df2 b) {
-  df2 r;
-  two_sum(a.h, b.h, r.h, r.l);
-  r.l = __fadd_rn(r.l, __fadd_rn(a.l, b.l));
-  return df_norm(r);
-}
-
-// 1/sqrt(a) of a normalised a > 0: an FP32 root refined by one Householder step
-// of third order, x (1 + e/2 + 3 e^2/8) with e = 1 - a x^2 in double-float
-__device__ __forceinline__ df2 df_rsqrt(df2 a) {
-  const float x = rsqrtf(a.h);
-  const df2 xx = {x, 0.f};
-  const df2 ax2 = df_norm(df_mul(df_norm(df_mul(a, xx)), xx));
-  const float e = __fadd_rn(__fadd_rn(1.0f, -ax2.h), -ax2.l);
-  df2 r = {x, __fmul_rn(x, __fmul_rn(e, __fmaf_rn(0.375f, e, 0.5f)))};
-  return df_norm(r);
-}
-
-// 1/sqrt(a) of a finite a > 0 to FP64 rounding with five FP64 instructions:
-// the argument scaled into [1, 4) and converted on the integer pipe, an FP32
-// root, one Householder step of third order (its error (5/16) e^3 with |e| < 2^-21)
-__device__ __forceinline__ double rsqrt64(double a) {
-  const long long b = __double_as_longlong(a);
-  const int ex = (int)(b >> 52) - 1023, half = ex >> 1;                  // a = m 4^half, m in [1, 4)
-  const double m = __longlong_as_double(b - ((long long)half << 53));
-  const double x = f2d_bits(rsqrtf(d2f_bits(m)));
-  const double e = fma(-(m * x), x, 1.0);
-  const double r = fma(x * e, fma(0.375, e, 0.5), x);
-  return __longlong_as_double(__double_as_longlong(r) - ((long long)half << 52));
-}
-
-// 1/a of a normal a > 0 the same way: an FP32 reciprocal, one Householder
-// step of third order
-__device__ __forceinline__ double rcp64(double a) {
-  const long long b = __double_as_longlong(a);
-  const int ex = (int)(b >> 52) - 1023;
-  const double m = __longlong_as_double(b - ((long long)ex << 52));  // [1, 2)
-  const double x = f2d_bits(__frcp_rn(d2f_bits(m)));
-  const double e = fma(-m, x, 1.0);
-  const double r = fma(x, fma(e, e, e), x);
-  return __longlong_as_double(__double_as_longlong(r) - ((long long)ex << 52));
 }
 
 // the sums of a and b over the warp, in every lane: after the first butterfly
@@ -339,7 +240,7 @@ __device__ __forceinline__ int rotation(double al, double be, double gr, double 
   const df2 ur = df_norm(df_mul(u, dr)), ui = df_norm(df_mul(u, di));
   const double er = f2d_bits(ur.h) + f2d_bits(ur.l), ei = f2d_bits(ui.h) + f2d_bits(ui.l);  // t conj(phase), exactly
   const double w = fma(er, er, fma(ei, ei, 1.0));
-  rot.c = rsqrt64(w);
+  rot.c = rsqrt64_normal(w);  // 1 <= w <= 2
   rot.qr = rot.c * er;
   rot.qi = -(rot.c * ei);
   tg = fma(er, gr, ei * gi);
@@ -824,16 +725,24 @@ __global__ void __launch_bounds__(CL_THREADS)
         const double d = pj[j].x;
         // d > thr: the same in every thread; a dropped direction updates nothing
         if (d > thr && (int)(threadIdx.x & ~31u) < todo) {
-          const double inv = rcp64(d);
-          for (int e = threadIdx.x; e < todo; e += CH_PANEL) {
-            const int q = (int)((unsigned)e * rec >> 16), i = j + 1 + q, l = col(e - q * ncol);
-            if (l > j && l < i) continue;
-            cplx* w = pan + (long long)(i - j0) * n + l;
-            const bool diag = l == j;
-            const cplx g = pj[i], h = diag ? make_double2(1.0, 0.0) : pj[l];
-            const cplx v = diag ? make_double2(0.0, 0.0) : *w;
-            const double ax = g.x * inv, ay = g.y * inv;
-            *w = make_double2(fma(-ax, h.x, fma(-ay, h.y, v.x)), fma(-ax, h.y, fma(ay, h.x, v.y)));
+          auto update = [&](auto over_d) {
+            for (int e = threadIdx.x; e < todo; e += CH_PANEL) {
+              const int q = (int)((unsigned)e * rec >> 16), i = j + 1 + q, l = col(e - q * ncol);
+              if (l > j && l < i) continue;
+              cplx* w = pan + (long long)(i - j0) * n + l;
+              const bool diag = l == j;
+              const cplx g = pj[i], h = diag ? make_double2(1.0, 0.0) : pj[l];
+              const cplx v = diag ? make_double2(0.0, 0.0) : *w;
+              const double ax = over_d(g.x), ay = over_d(g.y);
+              *w = make_double2(fma(-ax, h.x, fma(-ay, h.y, v.x)), fma(-ax, h.y, fma(ay, h.x, v.y)));
+            }
+          };
+          if ((unsigned)(__double2hiint(d) >> 20) - 3u < 2040u) {  // 2^-1020 <= d < 2^1020, on the integer pipe
+            const double inv = rcp64_pos(d);
+            update([inv](double x) { return x * inv; });
+          } else {  // 1/d overflows or loses bits where x / d does not
+            const double inv = rsqrt(d);
+            update([inv](double x) { return x * inv * inv; });
           }
         }
         asm volatile("bar.sync 1, %0;" ::"n"(CH_PANEL) : "memory");

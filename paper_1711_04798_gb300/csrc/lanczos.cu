@@ -21,6 +21,7 @@
 #include <algorithm>
 
 #include "ctm_internal.h"
+#include "dfloat.h"
 
 namespace {
 
@@ -280,28 +281,16 @@ __global__ void scale_pair_kernel(const cplx* __restrict__ r, const cplx* __rest
   }
 }
 
-// 1/q of a normal q to FP64 rounding: an FP32 reciprocal refined by one step of
-// third order, x (1 + e + e^2) with e = 1 - q x below 2^-21
-__device__ __forceinline__ double rcp_signed(double q) {
-  const long long b = __double_as_longlong(q);
-  const long long sign = b & (long long)0x8000000000000000ull, mag = b ^ sign;
-  const int ex = (int)(mag >> 52) - 1023;
-  const double m = __longlong_as_double(mag - ((long long)ex << 52));  // [1, 2)
-  const double x = f2d_bits(__frcp_rn(d2f_bits(m)));
-  const double e = fma(-m, x, 1.0);
-  const double r = fma(x, fma(e, e, e), x);
-  return __longlong_as_double((__double_as_longlong(r) - ((long long)ex << 52)) | sign);
-}
-
 // eigenvalues of T below x: the negative pivots of T - x I (Wilkinson, "The
-// Algebraic Eigenvalue Problem", ch. 5)
+// Algebraic Eigenvalue Problem", ch. 5).  A pivot lies between pivmin (1e-30 of
+// T's scale) and 1e30 of the scale, so its reciprocal is the normal one.
 __device__ int sturm_below(const double* al, const double* b2, int m, double x, double pivmin) {
   int cnt = 0;
   double q = al[0] - x;
   if (fabs(q) < pivmin) q = -pivmin;
   cnt += __double_as_longlong(q) < 0;
   for (int i = 1; i < m; ++i) {
-    q = fma(-b2[i], rcp_signed(q), al[i] - x);
+    q = fma(-b2[i], rcp64_normal(q), al[i] - x);
     if (fabs(q) < pivmin) q = -pivmin;
     cnt += __double_as_longlong(q) < 0;
   }
@@ -366,13 +355,13 @@ __global__ void __launch_bounds__(32)
   const double shift = th + 1e-14 * fmax(scale, 1e-300);
   double d = al[0] - shift;
   if (fabs(d) < pivmin) d = pivmin;
-  id[0] = rcp_signed(d);
+  id[0] = rcp64_normal(d);
   for (int i = 1; i < m; ++i) {
     const double li = be[i] * id[i - 1];
     lw[i] = li;
     d = fma(-li, be[i], al[i] - shift);
     if (fabs(d) < pivmin) d = pivmin;
-    id[i] = rcp_signed(d);
+    id[i] = rcp64_normal(d);
   }
   for (int i = 0; i < m; ++i) y[i] = 1.0;
   double last = 0.0;
