@@ -87,7 +87,6 @@ struct Lane {
   cudaStream_t stream;
   cplx* Q[4];
   TcPacked Qp[4][2];
-  OzSquare Qo[4][2];
   void* Qpmem[4][2];
   cplx* thin[4];
   cplx* Vt;
@@ -122,7 +121,8 @@ struct ipeps_ctm_s {
   cplx* spareT[2];    // replacement T4 per row
   cplx* Q[4];
   TcPacked Qp[4][2];  // precision form: corners packed once per cut, [as is, transposed]
-  OzSquare Qo[4][2];  // FP64-accurate form: their digit planes
+  OzSquare Qo[4][2];  // FP64-accurate form: their digit planes, in the scratch of the cut being worked on
+  bool oz_planes;     // whether it held them
   void* Qpmem[4][2];
   cplx* omt;
   cplx* thin[4];      // k x K work
@@ -255,7 +255,6 @@ static void swap_lane(ipeps_ctm h) {
     std::swap(h->thin[i], h->alt.thin[i]);
     for (int v = 0; v < 2; ++v) {
       std::swap(h->Qp[i][v], h->alt.Qp[i][v]);
-      std::swap(h->Qo[i][v], h->alt.Qo[i][v]);
       std::swap(h->Qpmem[i][v], h->alt.Qpmem[i][v]);
     }
   }
@@ -295,25 +294,29 @@ static bool tc_form(int prec) {
   return prec == IPEPS_PREC_TF32 || prec == IPEPS_PREC_BF16X3 || prec == IPEPS_PREC_BF16X6;
 }
 
+// scratch of one projector's CholeskyQR passes and k x k core: five factors and
+// two bases, beside them a pass's four k x k matrices
+static long long core_scratch(long long k, long long K) { return 9 * k * k + 2 * k * K + 11 * 16; }
+
 // The range finder's bases by shifted CholeskyQR3 and the SVD of W through its
 // k x k core (all forms but plain FP64 always).  Plain FP64 takes the same
 // route for the truncations it resolves: its Grams see directions down to
 // about 1e-12 of the largest, so a cutoff below 1e-9, an orth_tol that asks
 // for directions to be dropped, or a Jacobi budget beyond the rotation log's
-// keeps one-sided Jacobi on the full rows.  At D = 4, chi = 64 that Jacobi took
-// 14 ms for each of the six k x K bases of a cut (80 rows of 1024) and 75 % of
-// the sweep; a CholeskyQR3 takes about 1 ms (sweep and spectra 1180 -> 522 ms).
+// keeps one-sided Jacobi on the full rows, and so does a scratch that the other
+// forms' sizes leave too small for the core (D = 1 only).  At D = 4, chi = 64 that
+// Jacobi took 14 ms for each of the six k x K bases of a cut (80 rows of 1024) and
+// 75 % of the sweep; a CholeskyQR3 takes about 1 ms (sweep and spectra 1180 -> 522 ms).
 constexpr int CHOL_MAX_SWEEPS = 64;
-static bool chol_route(const ipeps_options& o) {
+static bool chol_route(ipeps_ctm h) {
+  const ipeps_options& o = h->opt;
   return o.prec != IPEPS_PREC_FP64 ||
-         (o.orth_tol <= 1e-14 && o.svd_cutoff >= 1e-9 && o.jacobi_max_sweeps <= CHOL_MAX_SWEEPS);
+         (o.orth_tol <= 1e-14 && o.svd_cutoff >= 1e-9 && o.jacobi_max_sweeps <= CHOL_MAX_SWEEPS &&
+          h->scratch_elems - h->scratch_top >= core_scratch(h->k, h->K));
 }
 
-// bytes of one orientation of a packed corner, 0 for a form that packs none
-static size_t corner_pack_bytes(int prec, int K) {
-  if (tc_form(prec)) return tc_packed_bytes(prec, K);
-  return prec == IPEPS_PREC_FP64TC && K >= 64 ? oz_square_bytes(K) : 0;
-}
+// bytes of one orientation of a packed corner of the precision forms
+static size_t corner_pack_bytes(int prec, int K) { return tc_form(prec) ? tc_packed_bytes(prec, K) : 0; }
 
 // sizes of everything a handle carves from its memory
 struct Sizes {
@@ -321,7 +324,7 @@ struct Sizes {
   size_t total;
 };
 
-static Sizes plan_sizes(int Lx, int Ly, int d, int D, int chi, int k, int ntens, int prec, int max_sweeps) {
+static Sizes plan_sizes(int Lx, int Ly, int d, int D, int chi, int k, int ntens, int prec) {
   Sizes s;
   const long long D2 = (long long)D * D, K = chi * D2;
   s.tens = (long long)d * D2 * D2;
@@ -341,10 +344,6 @@ static Sizes plan_sizes(int Lx, int Ly, int d, int D, int chi, int k, int ntens,
   // digit planes of the FP64-accurate products: 28 B per complex element of
   // the A side, 56 B of the B side, and the exact split partials
   if (prec == IPEPS_PREC_FP64TC) s.scratch = s.scratch * 3 + (1 << 22);
-  // plain FP64: per projector lane the rotation log, the factors and the bases
-  // of the SVD of W beside the Grams' split sums
-  if (prec == IPEPS_PREC_FP64 && max_sweeps <= CHOL_MAX_SWEEPS)
-    s.scratch += 2 * (jacobi_log_elems(k, max_sweeps) + 10LL * k * k + 3 * s.thin);
   size_t tot = 0;
   auto add = [&](long long n, size_t el) { tot += align_up((size_t)n * el); };
   for (int i = 0; i < 2 * 4 * ntens; ++i) add(s.tens, 16);
@@ -892,8 +891,7 @@ extern "C" ipeps_status ipeps_ctm_workspace_size(const ipeps_cell* c, const ipep
                                                  size_t* bytes) {
   CKS(validate(c, o));
   if (!bytes) return fail(IPEPS_EINVAL, "null bytes");
-  Sizes s = plan_sizes(c->Lx, c->Ly, c->d, c->D, o->chi, o->chi + o->rsvd_oversample, c->n_tensors, o->prec,
-                       o->jacobi_max_sweeps);
+  Sizes s = plan_sizes(c->Lx, c->Ly, c->d, c->D, o->chi, o->chi + o->rsvd_oversample, c->n_tensors, o->prec);
   *bytes = s.total;
   return IPEPS_OK;
 }
@@ -1006,7 +1004,7 @@ extern "C" ipeps_status ipeps_ctm_create(const ipeps_cell* c, const ipeps_option
   if (!(h->opt.svd_cutoff > 0.0))  // automatic: above the noise floor of the contraction arithmetic
     h->opt.svd_cutoff = !tc_form(o->prec) ? 1e-8 : (o->prec == IPEPS_PREC_TF32 ? 1e-5 : 1e-6);
   h->stream = (cudaStream_t)o->stream;
-  Sizes sz = plan_sizes(h->Lx, h->Ly, h->d, h->D, h->chi, h->k, h->ntens, o->prec, o->jacobi_max_sweeps);
+  Sizes sz = plan_sizes(h->Lx, h->Ly, h->d, h->D, h->chi, h->k, h->ntens, o->prec);
   if (o->workspace) {
     if (o->workspace_bytes < sz.total) {
       delete h;
@@ -1306,9 +1304,7 @@ lower_left:
 // Whether a thin product of `rows` rows takes the corners' digit planes split
 // once per cut (FP64-accurate form; below, the planes' padding to 128 rows
 // and 64 columns outweighs them and the FP64 CUDA cores are as good).
-static bool oz_corners(ipeps_ctm h, int rows) {
-  return h->opt.prec == IPEPS_PREC_FP64TC && h->K >= 64 && rows >= 16;
-}
+static bool oz_corners(ipeps_ctm h, int rows) { return h->oz_planes && rows >= 16; }
 
 // thin (k x K, row-major = transposed K x k) times corner q, opQ applied to it
 static ipeps_status thin_mul(ipeps_ctm h, const cplx* in, int opin, cplx* out, int q, int opQ, int rows) {
@@ -1362,16 +1358,34 @@ static ipeps_status thin_chain(ipeps_ctm h, const cplx* in, bool conj_in, std::i
 
 static bool packed_path(ipeps_ctm h) { return tc_form(h->opt.prec); }
 
+// the corners packed for the thin products; FP64-accurate form: their digit
+// planes in scratch, where that leaves the projector's other steps their room
+// (at d = 8 it holds five times the planes; without them every product splits
+// its own operands)
 static ipeps_status pack_corners(ipeps_ctm h) {
-  for (int q = 0; q < 4; ++q) {
-    if (two_corners(h) && (q == 1 || q == 2)) continue;
-    if (!packed_path(h)) {
-      CK(oz_pack_square(h->stream, h->Q[q], h->K, h->Qpmem[q][0], h->Qpmem[q][1], &h->Qo[q][0], &h->Qo[q][1]));
-      continue;
-    }
-    CK(tc_pack_square(h->stream, (int)h->opt.prec, h->Q[q], h->K, corners_f32(h) ? h->D2 : 0, h->Qpmem[q][0], h->Qpmem[q][1], &h->Qp[q][0],
-                      &h->Qp[q][1]));
+  auto used = [&](int q) { return !two_corners(h) || q == 0 || q == 3; };
+  h->oz_planes = false;
+  if (packed_path(h)) {
+    for (int q = 0; q < 4; ++q)
+      if (used(q))
+        CK(tc_pack_square(h->stream, (int)h->opt.prec, h->Q[q], h->K, corners_f32(h) ? h->D2 : 0, h->Qpmem[q][0],
+                          h->Qpmem[q][1], &h->Qp[q][0], &h->Qp[q][1]));
+    return IPEPS_OK;
   }
+  if (h->opt.prec != IPEPS_PREC_FP64TC || h->K < 64 || h->k < 16) return IPEPS_OK;
+  const int k = h->k, K = h->K;
+  const long long plane = (long long)(oz_square_bytes(K) / sizeof(cplx)) + 1;
+  const size_t work = std::max({oz_work_bytes(k, k, K), oz_work_bytes(k, K, k), oz_thin_bytes(k, K)});
+  const long long rest = core_scratch(k, K) + jacobi_log_elems(k, h->opt.jacobi_max_sweeps) +
+                         (long long)(work / sizeof(cplx)) + 16;
+  if (h->scratch_elems - h->scratch_top < (two_corners(h) ? 4 : 8) * (plane + 16) + rest) return IPEPS_OK;
+  for (int q = 0; q < 4; ++q) {
+    if (!used(q)) continue;
+    cplx *n = scratch_alloc(h, plane), *t = scratch_alloc(h, plane);
+    if (!n || !t) return fail(IPEPS_ENOMEM, "scratch exhausted (corner planes)");
+    CK(oz_pack_square(h->stream, h->Q[q], K, n, t, &h->Qo[q][0], &h->Qo[q][1]));
+  }
+  h->oz_planes = true;
   return IPEPS_OK;
 }
 
@@ -1558,10 +1572,9 @@ static ipeps_status svd_rows_chol(ipeps_ctm h, const cplx* Wt, cplx* out, cplx* 
     cudaEvent_t a = nullptr;
     prof_begin(h, &a);
     const long long nlog = jacobi_log_elems(k, h->opt.jacobi_max_sweeps);
-    cplx* rotlog = scratch_alloc(h, nlog);
-    if (!rotlog) return fail(IPEPS_ENOMEM, "scratch exhausted (rotation log)");
+    cplx* rotlog = scratch_alloc(h, nlog);  // none: V is rotated beside the rows
     CK(jacobi_rows(h->stream, R1, k, k, k, Vt, h->sigma, h->opt.jacobi_max_sweeps, h->dwork, h->counters,
-                   h->st, rotlog, nlog, h->opt.wait_cycles, warm, !exact));
+                   h->st, rotlog, rotlog ? nlog : 0, h->opt.wait_cycles, warm, !exact));
     prof_end(h, a, 0.0, 1);
   }
   if (exact) {
@@ -1584,8 +1597,9 @@ static ipeps_status projectors(ipeps_ctm h, int f, int x, int y, cplx* PT, cplx*
   CKS(enlarged_corners(h, f, x, y, packed_path(h)));
   const int k = h->k, K = h->K, chi = h->chi;
   // CholeskyQR on FP64-accurate Grams, or Jacobi on the full rows (chol_route)
-  const bool jacobi_bases = !chol_route(h->opt);
-  if (packed_path(h) || oz_corners(h, k)) CKS(pack_corners(h));
+  const bool jacobi_bases = !chol_route(h);
+  const long long mark = h->scratch_top;
+  CKS(pack_corners(h));
   cplx* Qt = h->thin[0];
   cplx* Zt = h->thin[1];
   auto orth_any = [&](cplx* Y, bool last) -> ipeps_status {
@@ -1653,6 +1667,7 @@ static ipeps_status projectors(ipeps_ctm h, int f, int x, int y, cplx* PT, cplx*
     CKS(thin_mul(h, tmp, OP_N, Ptil, 0, OP_T, chi));
   }
   CK(scale_rows_isqrt(h->stream, Ptil, chi, K, K, h->s_sel));
+  h->scratch_top = mark;
   return IPEPS_OK;
 }
 

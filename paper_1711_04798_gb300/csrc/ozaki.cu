@@ -685,6 +685,11 @@ size_t oz_square_bytes(int K) {
   return 2 * oz_al(4 * Mp) + oz_al((size_t)OZ_DIGITS * Mp * Krp * 2) + 1024;
 }
 
+size_t oz_thin_bytes(int M, int K) {
+  const size_t rows = (2 * (size_t)M + 63) / 64 * 64, Krp = (2 * (size_t)K + OZ_CHUNK - 1) / OZ_CHUNK * OZ_CHUNK;
+  return oz_al((size_t)OZ_DIGITS * rows * Krp * 2) + oz_al(4 * rows) + 3072;
+}
+
 cudaError_t oz_pack_square(cudaStream_t s, const cplx* Q, int K, void* memN, void* memT, OzSquare* outN,
                            OzSquare* outT) {
   const int Mp = (K + OZ_BM - 1) / OZ_BM * OZ_BM, Krp = (2 * K + OZ_CHUNK - 1) / OZ_CHUNK * OZ_CHUNK;
@@ -717,8 +722,7 @@ cudaError_t oz_thin(cudaStream_t s, int M, const cplx* A, long long lda, bool co
   if (!timeouts || !work) return cudaErrorInvalidValue;
   const int K = Q.K, chunks = Q.Krp / OZ_CHUNK;
   char* base = (char*)(((uintptr_t)work + 1023) & ~(uintptr_t)1023);
-  const size_t fixed = oz_al((size_t)OZ_DIGITS * ((2 * (size_t)M + 63) / 64 * 64) * Q.Krp * 2) +
-                       oz_al(4 * ((2 * (size_t)M + 63) / 64 * 64)) + 3072;
+  const size_t fixed = oz_thin_bytes(M, K);
   if (work_bytes < fixed) return cudaErrorMemoryAllocation;
   int bn = 64, Nrp = 0, cps = chunks;
   oz_choose(Q.Mp, M, chunks, (double)(work_bytes - fixed), &bn, &Nrp, &cps);

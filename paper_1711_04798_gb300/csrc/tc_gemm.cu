@@ -1169,7 +1169,7 @@ void carve_parts(int prec, void* mem, size_t each, void* (&b)[3]) {
   b[2] = n == 3 ? p + 2 * each : b[1];
 }
 
-size_t parts_bytes(int prec, size_t each) { return (size_t)n_parts(prec) * (each + 1024) + 2048; }
+size_t parts_bytes(int prec, size_t each) { return (size_t)n_parts(prec) * ((each + 1023) & ~(size_t)1023) + 1024; }
 
 long long pad_k(int prec, int K) {
   long long Nrp, Krp;

@@ -136,6 +136,8 @@ size_t oz_square_bytes(int K);
 // Q (row-major K x K) for thin * Q (outN) and thin * Q^T (outT)
 cudaError_t oz_pack_square(cudaStream_t s, const cplx* Q, int K, void* memN, void* memT, OzSquare* outN,
                            OzSquare* outT);
+// the least work of oz_thin (without room for K splits)
+size_t oz_thin_bytes(int M, int K);
 // C = op(A) Q (op: conjugation with conj_in; the result conjugated with conj_out)
 cudaError_t oz_thin(cudaStream_t s, int M, const cplx* A, long long lda, bool conj_in, const OzSquare& Q, cplx* C,
                     long long ldc, bool conj_out, void* work, size_t work_bytes, int* timeouts);
