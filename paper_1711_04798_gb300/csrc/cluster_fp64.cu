@@ -22,6 +22,7 @@ namespace {
 constexpr int CL_THREADS = 256;         // 8 warps per CTA (Cholesky): FP64 pipe occupancy
 constexpr int CL_SMEM = 200 * 1024;     // dynamic shared memory bound per CTA
 int g_csize = 0;                        // CTAs per cluster (16 if schedulable, else 8)
+int g_clusters = 0;                     // clusters of 16 with CL_SMEM that the device holds at once
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
@@ -876,6 +877,7 @@ static cudaError_t cluster_init() {
   int nclusters = 0;
   if (cudaOccupancyMaxActiveClusters(&nclusters, jacobi_fn(false, false, 257), &cfg) == cudaSuccess && nclusters >= 1)
     csize = 16;
+  g_clusters = nclusters;
   cudaGetLastError();  // a refused query leaves no error behind
   g_csize = csize;
   return cudaSuccess;
@@ -966,15 +968,15 @@ cudaError_t jacobi_cluster(cudaStream_t s, cplx* G, int n, int m, long long ldg,
 bool jacobi_batch_fits(int n) { return n >= 1 && cluster_init() == cudaSuccess && jacobi_smem(n, n, false, g_csize) > 0; }
 
 // Singular values only of `count` matrices (matrix b at G + b * strideG), one
-// cluster each in one launch.  Clusters of 8 where 16-CTA ones would not all
-// be resident: the FP64 units of the SMs in use bound the kernel, and 16
-// corners on 8 CTAs each take 128 SMs at once.
+// cluster each in one launch.  Clusters of 8 where the device does not hold as
+// many of 16 at once: the FP64 units of the SMs in use bound the kernel, and the
+// 16 corners of a 2x2 cell on 8 CTAs each take 128 SMs in one wave.
 cudaError_t jacobi_cluster_batch(cudaStream_t s, cplx* G, int n, int m, long long ldg, long long strideG, int count,
                                  int max_sweeps, DevStatus* st) {
   cudaError_t e;
   if ((e = cluster_init()) != cudaSuccess) return e;
   int cs = g_csize;
-  if (count * cs > 144 && jacobi_smem(n, m, false, 8) > 0) cs = 8;
+  if (cs == 16 && count > g_clusters && jacobi_smem(n, m, false, 8) > 0) cs = 8;
   size_t smem = jacobi_smem(n, m, false, cs);
   cplx* Vin = nullptr;
   double4_16a* logp = nullptr;
