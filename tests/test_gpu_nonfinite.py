@@ -28,7 +28,8 @@ def test_nonfinite_element_of_a_square_operand(M, K, bad):
     size.restype = ctypes.c_size_t
     ptr, i64 = ctypes.c_void_p, ctypes.c_longlong
     pack.argtypes = [ptr, ptr, ctypes.c_int, ptr, ptr, ptr, ptr]
-    thin.argtypes = [ptr, ctypes.c_int, ptr, i64, ctypes.c_bool, ptr, ptr, i64, ctypes.c_bool, ptr, ctypes.c_size_t, ptr]
+    thin.argtypes = [ptr, ctypes.c_int, ptr, i64, ctypes.c_bool, ptr, ptr, i64, ctypes.c_bool, ptr, ctypes.c_size_t,
+                     ptr]
     rng = np.random.default_rng(K)
     A = rng.standard_normal((M, K)) + 1j * rng.standard_normal((M, K))
     Q = rng.standard_normal((K, K)) + 1j * rng.standard_normal((K, K))
