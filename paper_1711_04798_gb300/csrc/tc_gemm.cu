@@ -42,7 +42,7 @@ constexpr int PREC_TF32 = 1, PREC_BF16X3 = 2, PREC_BF16X6 = 3;
 // memory.  NOPS parts per operand (1 TF32, 2 BF16 hi/lo, 3 BF16 hi/mid/lo);
 // BF16x6 takes 64-byte k-blocks (64-byte swizzle) so that its three A and
 // three B parts fit four stages at BN = 128 and three at BN = 256.
-template <int PREC, int BN_>
+template <int PREC, int BN_, bool SPLIT_ACC_ = false>
 struct Cfg {
   static constexpr int BN = BN_;
   static constexpr int ELEM = PREC == PREC_TF32 ? 4 : 2;
@@ -58,14 +58,18 @@ struct Cfg {
   static constexpr int KSTEPS = BK / UMMA_K;
   // Accumulators.  The tensor cores round every FP32 accumulation towards zero, so
   // a run of n of them loses up to n ulps of the sum, always in the same direction.
-  // BF16x6 keeps the five products with a low part (2^-8 of the result and below)
-  // in an accumulator of their own, added at the end: one accumulation of the
-  // result's size per k-step instead of six.  69 x 848 x 848 complex, rms of the
-  // result: 1.2e-5 -> 1.7e-6 in one K split, 4.1e-7 -> 1.3e-7 in 27; RDMs of a 2x1
-  // cell at D = 4, chi = 53 with two-corner projectors, mean of 40 states: 1.2e-6 ->
-  // 5.7e-7 (largest 4.2e-6 -> 2.1e-6).  At BN = 256 that leaves tensor memory for one
-  // set, whose drain the next tile waits for: 1 to 2 % of a sweep.
-  static constexpr bool SPLIT_ACC = PREC == PREC_BF16X6;
+  // SPLIT_ACC keeps BF16x6's five products with a low part (2^-8 of the result and
+  // below) in an accumulator of their own, added at the end: one accumulation of
+  // the result's size per k-step instead of six.  69 x 848 x 848 complex in 27 K
+  // splits: 4.1e-7 -> 1.3e-7 of the result (rms).  For products whose K is split
+  // (the thin ones and the absorption's last, which the projectors' 1/sqrt(s)
+  // magnifies): RDMs of a 2x1 cell at D = 4, chi = 53 with two-corner projectors,
+  // mean of 40 states 1.2e-6 -> 6.3e-7, largest 4.2e-6 -> 1.8e-6.  At BN = 256 it leaves
+  // tensor memory for one set, whose drain the next tile waits for: 2.4 % of a
+  // D = 4, chi = 64 convergence; for the unsplit products too it would be another
+  // 2 % of a D = 5, chi = 100 step for 5.7e-7.
+  static constexpr bool SPLIT_ACC = SPLIT_ACC_;
+  static_assert(!SPLIT_ACC || PREC == PREC_BF16X6, "three parts");
   static constexpr int ACC_COLS = SPLIT_ACC ? 2 * BN : BN;  // tensor-memory columns of a set
   static constexpr int SETS = 2 * ACC_COLS <= 512 ? 2 : 1;  // 2: a tile drains under the next one's MMAs
   // stages, alignment, barriers, the epilogue warps' transpose buffers
@@ -99,7 +103,7 @@ __device__ __forceinline__ void umma(uint32_t dtmem, uint64_t a, uint64_t b, uin
 // the MMAs of tile i into accumulator set i % SETS (tensor-memory columns
 // ACC_COLS (i % SETS) ..), warps 2..5 drain that set to global memory, with two
 // sets while the MMAs of tile i + 1 run in the other one.
-template <int PREC, int BN>
+template <int PREC, int BN, bool SPLIT_ACC>
 __global__ void __launch_bounds__(NTHREADS, 1)
     tc_gemm_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ CUtensorMap mA1,
                    const __grid_constant__ CUtensorMap mA2, const __grid_constant__ CUtensorMap mB0,
@@ -107,7 +111,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                    int kb_total, int kb_per_split, int n_tiles, int m_tiles, int tiles, int M, int Nr, cplx alpha,
                    void* __restrict__ Cv, long long ldc, float* __restrict__ partial, int Nrp, long long pstride,
                    int unit_alpha, int out_f32, int* __restrict__ timeouts) {
-  using K_ = Cfg<PREC, BN>;
+  using K_ = Cfg<PREC, BN, SPLIT_ACC>;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint64_t* full = (uint64_t*)(smem + K_::STAGES * K_::STAGE_BYTES);
@@ -220,7 +224,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             umma<PREC, K_::IDESC>(dl, sdesc_kb<K_::KB_BYTES>(a2 + ko), sdesc_kb<K_::KB_BYTES>(b0 + ko), 1u);
             umma<PREC, K_::IDESC>(dl, sdesc_kb<K_::KB_BYTES>(a0 + ko), sdesc_kb<K_::KB_BYTES>(b1 + ko), 1u);
             umma<PREC, K_::IDESC>(dl, sdesc_kb<K_::KB_BYTES>(a1 + ko), sdesc_kb<K_::KB_BYTES>(b0 + ko), 1u);
-            umma<PREC, K_::IDESC>(d, sdesc_kb<K_::KB_BYTES>(a0 + ko), sdesc_kb<K_::KB_BYTES>(b0 + ko), acc);
+            umma<PREC, K_::IDESC>(d, sdesc_kb<K_::KB_BYTES>(a0 + ko), sdesc_kb<K_::KB_BYTES>(b0 + ko), SPLIT_ACC ? acc : 1u);
           } else {
             umma<PREC, K_::IDESC>(d, sdesc_kb<K_::KB_BYTES>(a0 + ko), sdesc_kb<K_::KB_BYTES>(b0 + ko), acc);
             if (K_::NOPS == 2) {
@@ -792,24 +796,24 @@ struct Operands {
 };
 
 // one-time kernel attribute (dynamic shared memory above 48 KB)
-template <int PREC, int BN>
+template <int PREC, int BN, bool SPLIT_ACC>
 cudaError_t ensure_attr() {
   static bool attr_set = false;
   if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(tc_gemm_kernel<PREC, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         Cfg<PREC, BN>::SMEM);
+    cudaError_t e = cudaFuncSetAttribute(tc_gemm_kernel<PREC, BN, SPLIT_ACC>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<PREC, BN>::SMEM);
     if (e != cudaSuccess) return e;
     attr_set = true;
   }
   return cudaSuccess;
 }
 
-template <int PREC, int BN>
-cudaError_t launch_main(cudaStream_t s, const Operands& o, int S, int M, int N, cplx alpha, void* C, long long ldc,
-                        bool c_f32, float* part, int* timeouts, TcProbe* probe, bool partials_only = false) {
-  using K_ = Cfg<PREC, BN>;
+template <int PREC, int BN, bool SPLIT_ACC>
+cudaError_t launch_tiles(cudaStream_t s, const Operands& o, int S, int M, int N, cplx alpha, void* C, long long ldc,
+                         bool c_f32, float* part, int* timeouts, TcProbe* probe, bool partials_only) {
+  using K_ = Cfg<PREC, BN, SPLIT_ACC>;
   cudaError_t e;
-  if ((e = ensure_attr<PREC, BN>()) != cudaSuccess) return e;
+  if ((e = ensure_attr<PREC, BN, SPLIT_ACC>()) != cudaSuccess) return e;
   if ((e = get_encoder()) != cudaSuccess) return e;
   CUtensorMap mA0, mA1, mA2, mB0, mB1, mB2;
   constexpr int KB = K_::KB_BYTES;
@@ -825,7 +829,6 @@ cudaError_t launch_main(cudaStream_t s, const Operands& o, int S, int M, int N, 
     if ((e = make_map(&mA2, o.a2, PREC, o.Mp, o.Krp, BM, KB)) != cudaSuccess) return e;
     if ((e = make_map(&mB2, o.b2, PREC, o.Nrp, o.Krp, BN, KB)) != cudaSuccess) return e;
   }
-  S = eff_splits(o.kb_total, S);
   const int kps = (o.kb_total + S - 1) / S;
   const int n_tiles = (int)(o.Nrp / BN), m_tiles = (int)(o.Mp / BM);
   const long long tiles = (long long)n_tiles * m_tiles * S;
@@ -848,10 +851,9 @@ cudaError_t launch_main(cudaStream_t s, const Operands& o, int S, int M, int N, 
     probe->elem_bytes = K_::ELEM;
     if ((e = cudaEventRecord(probe->ev[0], s)) != cudaSuccess) return e;
   }
-  tc_gemm_kernel<PREC, BN><<<grid, NTHREADS, K_::SMEM, s>>>(mA0, mA1, mA2, mB0, mB1, mB2, o.kb_total, kps, n_tiles,
-                                                             m_tiles, (int)tiles, M, 2 * N, alpha, C, ldc,
-                                                             S > 1 || partials_only ? part : nullptr, (int)o.Nrp,
-                                                             o.Mp * o.Nrp, unit, c_f32 ? 1 : 0, timeouts);
+  tc_gemm_kernel<PREC, BN, SPLIT_ACC><<<grid, NTHREADS, K_::SMEM, s>>>(
+      mA0, mA1, mA2, mB0, mB1, mB2, o.kb_total, kps, n_tiles, m_tiles, (int)tiles, M, 2 * N, alpha, C, ldc,
+      S > 1 || partials_only ? part : nullptr, (int)o.Nrp, o.Mp * o.Nrp, unit, c_f32 ? 1 : 0, timeouts);
   count_launch();
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (probe && (e = cudaEventRecord(probe->ev[1], s)) != cudaSuccess) return e;
@@ -868,6 +870,17 @@ cudaError_t launch_main(cudaStream_t s, const Operands& o, int S, int M, int N, 
   }
   if (probe && (e = cudaEventRecord(probe->ev[2], s)) != cudaSuccess) return e;
   return cudaSuccess;
+}
+
+// BF16x6 products whose K is split take two accumulators (Cfg)
+template <int PREC, int BN>
+cudaError_t launch_main(cudaStream_t s, const Operands& o, int S, int M, int N, cplx alpha, void* C, long long ldc,
+                        bool c_f32, float* part, int* timeouts, TcProbe* probe, bool partials_only = false) {
+  S = eff_splits(o.kb_total, S);
+  if constexpr (PREC == PREC_BF16X6)
+    if (S > 1 || partials_only)
+      return launch_tiles<PREC, BN, true>(s, o, S, M, N, alpha, C, ldc, c_f32, part, timeouts, probe, partials_only);
+  return launch_tiles<PREC, BN, false>(s, o, S, M, N, alpha, C, ldc, c_f32, part, timeouts, probe, partials_only);
 }
 
 template <int PREC>
@@ -1310,11 +1323,13 @@ cudaError_t tc_thin(cudaStream_t s, const TcThin& A, const TcPacked& Q, cplx* C,
 
 cudaError_t tc_init() {
   cudaError_t e;
-  if ((e = ensure_attr<PREC_TF32, 128>()) != cudaSuccess) return e;
-  if ((e = ensure_attr<PREC_TF32, 256>()) != cudaSuccess) return e;
-  if ((e = ensure_attr<PREC_BF16X3, 128>()) != cudaSuccess) return e;
-  if ((e = ensure_attr<PREC_BF16X3, 256>()) != cudaSuccess) return e;
-  if ((e = ensure_attr<PREC_BF16X6, 128>()) != cudaSuccess) return e;
-  if ((e = ensure_attr<PREC_BF16X6, 256>()) != cudaSuccess) return e;
+  if ((e = ensure_attr<PREC_TF32, 128, false>()) != cudaSuccess) return e;
+  if ((e = ensure_attr<PREC_TF32, 256, false>()) != cudaSuccess) return e;
+  if ((e = ensure_attr<PREC_BF16X3, 128, false>()) != cudaSuccess) return e;
+  if ((e = ensure_attr<PREC_BF16X3, 256, false>()) != cudaSuccess) return e;
+  if ((e = ensure_attr<PREC_BF16X6, 128, false>()) != cudaSuccess) return e;
+  if ((e = ensure_attr<PREC_BF16X6, 256, false>()) != cudaSuccess) return e;
+  if ((e = ensure_attr<PREC_BF16X6, 128, true>()) != cudaSuccess) return e;
+  if ((e = ensure_attr<PREC_BF16X6, 256, true>()) != cudaSuccess) return e;
   return get_encoder();
 }

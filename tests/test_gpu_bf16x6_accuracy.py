@@ -1,5 +1,5 @@
-"""Accuracy of the BF16x6 form's FP32 accumulation, in one product and in the
-RDMs of the case that magnifies it most."""
+"""Accuracy of the BF16x6 form's FP32 accumulation, in one product whose K is split
+and in the RDMs of the case that magnifies it most."""
 import numpy as np
 import pytest
 
@@ -10,7 +10,7 @@ from test_gpu_tc_gemm import _zgemm_tile
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("bn,splits", [(128, 1), (128, 27), (256, 1), (256, 5), (256, 27)])
+@pytest.mark.parametrize("bn,splits", [(128, 2), (128, 27), (256, 2), (256, 5), (256, 27)])
 @pytest.mark.parametrize("shape", [(848, 69, 848), (130, 100, 53), (1500, 256, 256)])
 def test_product_error_is_that_of_one_accumulation_per_k_step(shape, bn, splits):
     """An accumulation on the tensor cores cuts the running sum by half an ulp
@@ -36,8 +36,8 @@ def test_two_corner_rdms_of_a_2x1_cell():
     sweeps against the FP64-accurate form at the same cutoff, over 16 states: the
     case magnifies the products' rounding by a factor that differs from state to
     state, so the mean is held to a bound.  0.8e-6 lies between the means of one
-    accumulator for all six products (1.2e-6) and of the two in use (5.7e-7), both
-    over 40 other states."""
+    accumulator for all six products (1.2e-6) and of two (6e-7), both over 40 other
+    states."""
     err = []
     for seed in range(16):
         t = [synth.product_plus_noise(seed, i, 8, 4) for i in range(2)]
