@@ -6,8 +6,9 @@
 // barrier per step.  Here the rows are distributed over the CTAs of one
 // cluster (row i lives in the shared memory of CTA i mod csize), warps read
 // and write partner rows through distributed shared memory, and steps are
-// separated by the hardware cluster barrier.  The pair schedule and the
-// arithmetic are those of the grid-wide kernels (kernels.cu, cholqr.cu).
+// separated by the hardware cluster barrier.  The pair schedule is that of the
+// grid-wide kernels (kernels.cu), over the rows that take part; angles, carried
+// norms and the blocked Cholesky are this file's own.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -158,7 +159,8 @@ __device__ __forceinline__ int rotation(df2 al, df2 be, df2 gr, df2 gi, float to
   const float big = fmaxf(fabsf(gr.h), fabsf(gi.h));
   const int e = (int)(__float_as_uint(big) >> 23);
   if (!(big > 0.f) || e >= 255 || e < 8) return 0;
-  const float S = __uint_as_float((unsigned)(254 - e) << 23), iS = __uint_as_float((unsigned)e << 23);  // 2^(127-e), 1/S
+  const float S = __uint_as_float((unsigned)(254 - e) << 23);  // 2^(127-e)
+  const float iS = __uint_as_float((unsigned)e << 23);         // 1/S
   gr = {gr.h * S, gr.l * S};
   gi = {gi.h * S, gi.l * S};
   df2 g2 = df_mul(gr, gr);
@@ -569,7 +571,8 @@ __global__ void __launch_bounds__(512, 1)
       bool on = false;
       for (int a = threadIdx.x; a < na; a += blockDim.x) on |= s_act[a] == i;
       if (!__syncthreads_or(on))
-        for (int t = threadIdx.x; t < n; t += blockDim.x) Vt[(long long)i * n + t] = make_double2(t == i ? 1.0 : 0.0, 0.0);
+        for (int t = threadIdx.x; t < n; t += blockDim.x)
+          Vt[(long long)i * n + t] = make_double2(t == i ? 1.0 : 0.0, 0.0);
     }
   if (rank == 0) {
     if (amap) {
@@ -841,8 +844,8 @@ __global__ void __launch_bounds__(CL_THREADS)
 
 template <bool DF, bool V>
 static const void* jacobi_fn(int m) {
-  return m <= 128 ? (const void*)jacobi_cluster_kernel<DF, 4, V>
-                  : (m <= 256 ? (const void*)jacobi_cluster_kernel<DF, 8, V> : (const void*)jacobi_cluster_kernel<DF, 0, V>);
+  if (m <= 128) return (const void*)jacobi_cluster_kernel<DF, 4, V>;
+  return m <= 256 ? (const void*)jacobi_cluster_kernel<DF, 8, V> : (const void*)jacobi_cluster_kernel<DF, 0, V>;
 }
 
 // the kernel for rows of m elements; v: Vt beside the rows
@@ -965,7 +968,9 @@ cudaError_t jacobi_cluster(cudaStream_t s, cplx* G, int n, int m, long long ldg,
   return cudaGetLastError();
 }
 
-bool jacobi_batch_fits(int n) { return n >= 1 && cluster_init() == cudaSuccess && jacobi_smem(n, n, false, g_csize) > 0; }
+bool jacobi_batch_fits(int n) {
+  return n >= 1 && cluster_init() == cudaSuccess && jacobi_smem(n, n, false, g_csize) > 0;
+}
 
 // Singular values only of `count` matrices (matrix b at G + b * strideG), one
 // cluster each in one launch.  Clusters of 8 where the device does not hold as

@@ -729,8 +729,8 @@ static ipeps_status contract(ipeps_ctm h, const char* spec, TV A, bool conjA, TV
       TcProbe pr;
       TcProbe* p = tc_probe_begin(h, &pr);
       cudaError_t e = tc_zgemm_views(h->stream, (int)h->opt.prec, (int)M, (int)N, (int)Kd, direct ? alpha : ONE, VA,
-                                     pa, lda, opa, VB, pb, ldb, opb, out, N, direct && C.f32, h->scratch, h->scratch_elems,
-                                     h->scratch_top, &h->st->tc_timeouts, h->tuner, p);
+                                     pa, lda, opa, VB, pb, ldb, opb, out, N, direct && C.f32, h->scratch,
+                                     h->scratch_elems, h->scratch_top, &h->st->tc_timeouts, h->tuner, p);
       prof_end(h, ev, 8.0 * (double)M * (double)N * (double)Kd, 0);
       if (e == cudaSuccess) tc_probe_end(h, p, (int)M, (int)N, (int)Kd);
       CK(e);
@@ -1266,7 +1266,8 @@ static ipeps_status enlarged_corners(ipeps_ctm h, int f, int x, int y, bool raw)
   auto last = [&](const char* in, const char* xayb, const char* xyab, TV w, cplx* a, int q) -> ipeps_status {
     const std::string spec = std::string(in) + "->" + (q32 ? xyab : xayb);
     const TV A = tv(a, {D2, D2, D2, D2});
-    return contract(h, spec.c_str(), w, false, A, false, q32 ? tv(h->Q[q], {c, c, D2, D2}, true) : tv(h->Q[q], {c, D2, c, D2}));
+    return contract(h, spec.c_str(), w, false, A, false,
+                    q32 ? tv(h->Q[q], {c, c, D2, D2}, true) : tv(h->Q[q], {c, D2, c, D2}));
   };
   // Q1 = ((C1 T1) T4) a
   CKS(contract(h, "ab,bcr->acr", tv(envC(h, f, 0, x, y), {c, c}), false,
@@ -1531,9 +1532,12 @@ static ipeps_status orth_chol(ipeps_ctm h, cplx* Y, cplx* tmp, bool twice) {
 // rotated core is already nearly column-orthogonal and the sweeps converge
 // quadratically from there; the SVD found is the same (the Jacobi stops on
 // the same orthogonality test whatever its start).  The unitarity of the
-// accumulated V degrades like sqrt(rotations) x 2^-48 (the rotations are
-// replayed in double-float arithmetic), ~1e-12 after thousands of visits, far
-// below the 1e-6 truncation of the precision forms.
+// accumulated V degrades with every rotation of a row by what its c and q are off
+// c^2 + |q|^2 = 1, in double-float some 2^-45 (their root's correction is formed in
+// FP32): at k = 116 and four sweeps a visit 1e-11 after a thousand visits where the
+// errors' signs vary, 1e-8 where they do not, below the 1e-6 truncation of the
+// precision forms.  The FP64 forms' angles are good to 2^-45 too, their c and q
+// to FP64 rounding.
 static ipeps_status svd_rows_chol(ipeps_ctm h, const cplx* Wt, cplx* out, cplx* Vt) {
   const int k = h->k, K = h->K;
   const long long mark = h->scratch_top;

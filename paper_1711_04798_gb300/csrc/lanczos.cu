@@ -341,7 +341,8 @@ __global__ void __launch_bounds__(32)
     const double x = l + (h - l) * ((double)(lane + 1) * (1.0 / 33.0));
     const unsigned above = __ballot_sync(0xffffffffu, sturm_below(al, b2, m, x, pivmin) >= target);
     const int first = above ? __ffs(above) - 1 : 32;  // the eigenvalue lies below this point
-    const double xl = __shfl_sync(0xffffffffu, x, first > 0 ? first - 1 : 0), xh = __shfl_sync(0xffffffffu, x, first & 31);
+    const double xl = __shfl_sync(0xffffffffu, x, first > 0 ? first - 1 : 0);
+    const double xh = __shfl_sync(0xffffffffu, x, first & 31);
     const double nl = first > 0 ? xl : l, nh = first < 32 ? xh : h;
     if (nl == l && nh == h) break;  // no point strictly inside
     l = nl;
@@ -510,11 +511,9 @@ cudaError_t lanczos_leading(cudaStream_t s, const cplx* A, const cplx* B, long l
     // dropped
     if ((j + 1) % 10 != 0 && j + 1 < max_iter) continue;
     std::vector<double2> ha(j + 1 - m), hb(j + 1 - m);
-    if ((e = cudaMemcpyAsync(ha.data(), adot + m, ha.size() * sizeof(double2), cudaMemcpyDeviceToHost, s)) != cudaSuccess)
-      return e;
-    if ((e = cudaMemcpyAsync(hb.data(), bdot + m + 1, hb.size() * sizeof(double2), cudaMemcpyDeviceToHost, s)) !=
-        cudaSuccess)
-      return e;
+    const size_t bytes = ha.size() * sizeof(double2);
+    if ((e = cudaMemcpyAsync(ha.data(), adot + m, bytes, cudaMemcpyDeviceToHost, s)) != cudaSuccess) return e;
+    if ((e = cudaMemcpyAsync(hb.data(), bdot + m + 1, bytes, cudaMemcpyDeviceToHost, s)) != cudaSuccess) return e;
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
     for (size_t q = 0; q < ha.size() && !res->indefinite && !res->breakdown; ++q) {
       amax = fmax(amax, fabs(ha[q].x));

@@ -646,8 +646,8 @@ OzLayout oz_layout(int M, int N, int K) {
   return L;
 }
 
-cudaError_t oz_launch(cudaStream_t s, __nv_bfloat16* pa, __nv_bfloat16* pb, int Mp, int Nrp, int Krp, int bn, int chunks,
-                      int cps, int M, int N, const int* ea, const int* eb, cplx* C, long long ldc, bool trans,
+cudaError_t oz_launch(cudaStream_t s, __nv_bfloat16* pa, __nv_bfloat16* pb, int Mp, int Nrp, int Krp, int bn,
+                      int chunks, int cps, int M, int N, const int* ea, const int* eb, cplx* C, long long ldc, bool trans,
                       bool conj_out, long long* pI, float* pU, int* timeouts) {
   static bool attr = false;
   cudaError_t e;
@@ -707,8 +707,8 @@ cudaError_t oz_pack_square(cudaStream_t s, const cplx* Q, int K, void* memN, voi
     out[v]->p = p + 2 * oz_al(4 * (size_t)Mp);
     if ((e = cudaMemsetAsync(raw[v], 0, 4 * (size_t)Mp, s)) != cudaSuccess) return e;
   }
-  oz_square_exp_kernel<<<dim3((unsigned)((K + 31) / 32), (unsigned)((K + 127) / 128)), dim3(32, 8), 0, s>>>(Q, K, raw[1],
-                                                                                                     raw[0]);
+  oz_square_exp_kernel<<<dim3((unsigned)((K + 31) / 32), (unsigned)((K + 127) / 128)), dim3(32, 8), 0, s>>>(
+      Q, K, raw[1], raw[0]);
   // tiles cover Mp rows in both directions (Krp / 2 <= Mp)
   oz_square_prep_kernel<<<dim3((unsigned)(Mp / 32), (unsigned)(Mp / 32)), dim3(32, 8), 0, s>>>(
       Q, K, Mp, Krp, raw[1], raw[0], outT->e, outN->e, (__nv_bfloat16*)outT->p, (__nv_bfloat16*)outN->p);
@@ -733,8 +733,8 @@ cudaError_t oz_thin(cudaStream_t s, int M, const cplx* A, long long lda, bool co
   long long* pI = S > 1 ? (long long*)part : nullptr;
   float* pU = S > 1 ? (float*)(part + (size_t)S * Q.Mp * Nrp * 8) : nullptr;
   cudaError_t e;
-  oz_prep_kernel<false><<<(unsigned)(Nrp / 2), OZ_PREP_THREADS, 0, s>>>(nullptr, 0, OP_N, A, lda, OP_T | (conj_in ? OP_CONJ : 0),
-                                                               0, M, K, 0, Nrp, Q.Krp, nullptr, eb, nullptr, pb);
+  oz_prep_kernel<false><<<(unsigned)(Nrp / 2), OZ_PREP_THREADS, 0, s>>>(
+      nullptr, 0, OP_N, A, lda, OP_T | (conj_in ? OP_CONJ : 0), 0, M, K, 0, Nrp, Q.Krp, nullptr, eb, nullptr, pb);
   count_launch();
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if ((e = oz_launch(s, (__nv_bfloat16*)Q.p, pb, Q.Mp, Nrp, Q.Krp, bn, chunks, cps, K, M, Q.e, eb, C, ldc, true,

@@ -224,7 +224,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             umma<PREC, K_::IDESC>(dl, sdesc_kb<K_::KB_BYTES>(a2 + ko), sdesc_kb<K_::KB_BYTES>(b0 + ko), 1u);
             umma<PREC, K_::IDESC>(dl, sdesc_kb<K_::KB_BYTES>(a0 + ko), sdesc_kb<K_::KB_BYTES>(b1 + ko), 1u);
             umma<PREC, K_::IDESC>(dl, sdesc_kb<K_::KB_BYTES>(a1 + ko), sdesc_kb<K_::KB_BYTES>(b0 + ko), 1u);
-            umma<PREC, K_::IDESC>(d, sdesc_kb<K_::KB_BYTES>(a0 + ko), sdesc_kb<K_::KB_BYTES>(b0 + ko), SPLIT_ACC ? acc : 1u);
+            umma<PREC, K_::IDESC>(d, sdesc_kb<K_::KB_BYTES>(a0 + ko), sdesc_kb<K_::KB_BYTES>(b0 + ko),
+                                  SPLIT_ACC ? acc : 1u);
           } else {
             umma<PREC, K_::IDESC>(d, sdesc_kb<K_::KB_BYTES>(a0 + ko), sdesc_kb<K_::KB_BYTES>(b0 + ko), acc);
             if (K_::NOPS == 2) {
@@ -311,7 +312,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   fence_before();
   __syncthreads();
   if (warp == 0) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(K_::SETS * K_::ACC_COLS) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(K_::SETS * K_::ACC_COLS)
+                 : "memory");
   }
 }
 
@@ -1013,8 +1015,9 @@ cudaError_t tune_choice(cudaStream_t s, TcTuner* tuner, const TcTuner::Key& key,
 
 template <int PREC>
 cudaError_t run(cudaStream_t s, int M, int N, int K, cplx alpha, const cplx* A, long long lda, int opA,
-                const cplx* B, long long ldb, int opB, void* C, long long ldc, bool c_f32, char* scratch, size_t scratch_bytes, TcTuner* tuner, const TcChoice* force, int* timeouts,
-                TcProbe* probe, const TcView* va = nullptr, const TcView* vb = nullptr) {
+                const cplx* B, long long ldb, int opB, void* C, long long ldc, bool c_f32, char* scratch,
+                size_t scratch_bytes, TcTuner* tuner, const TcChoice* force, int* timeouts, TcProbe* probe,
+                const TcView* va = nullptr, const TcView* vb = nullptr) {
   if (!timeouts) return cudaErrorInvalidValue;
   using K_ = Cfg<PREC, 128>;  // element size, k-block and parts do not depend on the tile width
   Operands o;
@@ -1302,7 +1305,8 @@ cudaError_t run_thin(cudaStream_t s, const TcThin& A, const TcPacked& Q, cplx* C
       // never summing more than twice the default's run in FP32: the sums'
       // error grows with their length, and the timings do not see it
       const int S0 = eff_splits(o.kb_total, choice.splits);
-      cudaError_t e = tune_choice(s, tuner, key, o, choice, [&](int S) { return 2 * S >= S0 && room(S); }, [&](TcChoice c) { return launch(c, nullptr); }, &choice);
+      cudaError_t e = tune_choice(s, tuner, key, o, choice, [&](int S) { return 2 * S >= S0 && room(S); },
+                                  [&](TcChoice c) { return launch(c, nullptr); }, &choice);
       if (e != cudaSuccess) return e;
     }
   }

@@ -300,8 +300,8 @@ cudaError_t zgemm(cudaStream_t s, int M, int N, int K, cplx alpha, const cplx* A
       cfg.stream = s;
       cfg.attrs = &attr;
       cfg.numAttrs = 1;
-      const cudaError_t e = cudaLaunchKernelEx(&cfg, zgemm_kernel<1, true>, M, N, K, alpha, A, lda, opA, B, ldb, opB, beta,
-                                               C, ldc, 0LL, 0LL, 0LL, best_k, flags);
+      const cudaError_t e = cudaLaunchKernelEx(&cfg, zgemm_kernel<1, true>, M, N, K, alpha, A, lda, opA, B, ldb, opB,
+                                               beta, C, ldc, 0LL, 0LL, 0LL, best_k, flags);
       count_launch();
       return e;
     }
