@@ -463,7 +463,7 @@ def run_ours(args, rank, world, local_rank):
 # current kernel (the mean of the wide-product launches in the profile summary
 # of the default workload), keyed by (precision, bound); absent where no
 # capture of the current kernel exists
-TRAFFIC = {("bf16x6", "tensor"): 93.6e6}
+TRAFFIC = {("bf16x6", "tensor"): 55.9e6}
 
 
 def flops_per_move(D, chi, q=2, over=16):
